@@ -533,6 +533,124 @@ static LfErr setup_components(lfmm_ctx* ctx)
     return LfErr();
 }
 
+// Image rule of the remainders (LfImgRule): the fewest depths that reproduce
+// the image sums of the three near-field kernels to `tol` of their size.  The
+// hardest pairs are the closest: depth Z = 2 D (h = 0) and rho = 0, where
+// the summand 1/(1 + s) is singular one step left of the first image; wider
+// pairs are checked too.  A negative kappa is summed two terms at a time
+// (1/(1 - kappa y) = (1 + kappa y)/(1 - kappa^2 y^2)).  Depths and weights in
+// units of 2 D; returns the count, 0 where LFMM_IMG_RULE depths are not enough.
+// `gauss` keeps the Gauss rules of one kappa between calls.
+struct ImageGauss {
+    std::vector<double> nodes, weights;
+};
+static int image_rule(double kappa, double tol, std::vector<ImageGauss>& gauss, double* depth, double* weight)
+{
+    static const double A[2] = {1.0, 2.0}, B[4] = {0.0, 0.5, 1.5, 4.0};
+    auto term = [](double a, double b, double s, double* g) {
+        const double H = a + s, ir2 = 1.0 / (b * b + H * H), ir = sqrt(ir2);
+        g[0] = ir;
+        g[1] = H * ir * ir2;
+        g[2] = ir * ir2;  // the lateral kernel over rho
+    };
+    if (!(fabs(kappa) < 1.0)) return 0;
+    double exact[8][3];
+    for (int t = 0; t < 8; ++t) {
+        double* e = exact[t];
+        e[0] = e[1] = e[2] = 0.0;
+        const int nmax = kappa == 0.0 ? 1 : (int)std::min(40000.0, ceil(-40.0 / log(fabs(kappa))) + 1.0);
+        for (int n = nmax - 1; n >= 0; --n) {
+            double g[3];
+            term(A[t >> 2], B[t & 3], n, g);
+            for (int k = 0; k < 3; ++k) e[k] = g[k] + kappa * e[k];  // Horner from the far end
+        }
+    }
+    const bool neg = kappa < 0.0;
+    const double c = neg ? kappa * kappa : kappa;
+    const int qmax = neg ? 32 : 40;
+    gauss.resize(qmax + 1);
+    for (int tot = 1; tot <= LFMM_IMG_RULE; ++tot)
+        for (int q = 0; q <= qmax && q * (neg ? 2 : 1) <= tot; q += q < 4 ? 1 : 2) {
+            const int M = tot - q * (neg ? 2 : 1);
+            std::vector<double>&nodes = gauss[q].nodes, &wts = gauss[q].weights;
+            if (q > 0 && nodes.empty()) {
+                std::vector<double> a(q), b(q);
+                for (int k = 0; k < q; ++k) {
+                    a[k] = (c * (k + 1) + k) / (1.0 - c);
+                    b[k] = sqrt(c) * k / (1.0 - c);
+                }
+                nodes.resize(q);
+                wts.resize(q);
+                gauss_from_jacobi(q, a.data(), b.data(), 1.0 / (1.0 - c), nodes.data(), wts.data());
+            }
+            int n = 0;
+            double km = 1.0;
+            for (; n < M; ++n, km *= kappa) {
+                depth[n] = n;
+                weight[n] = km;
+            }
+            for (int i = 0; i < q; ++i) {
+                depth[n] = M + (neg ? 2.0 : 1.0) * nodes[i];
+                weight[n++] = km * wts[i];
+                if (neg) {
+                    depth[n] = depth[n - 1] + 1.0;
+                    weight[n] = kappa * weight[n - 1];
+                    ++n;
+                }
+            }
+            bool good = true;
+            for (int t = 0; t < 8 && good; ++t) {
+                double e[3] = {0.0, 0.0, 0.0};
+                for (int i = n - 1; i >= 0; --i) {
+                    double g[3];
+                    term(A[t >> 2], B[t & 3], depth[i], g);
+                    for (int k = 0; k < 3; ++k) e[k] += weight[i] * g[k];
+                }
+                for (int k = 0; k < 3; ++k) good = good && fabs(e[k] - exact[t][k]) <= tol * fabs(exact[t][k]);
+            }
+            if (good) return n;
+        }
+    return 0;
+}
+
+// The context's image rules, where every remainder is r0 / (1 - kappa x^2).
+static void setup_images(lfmm_ctx* ctx)
+{
+    ctx->img_ok = 0;
+    ctx->img64.n = ctx->img32.n = 0;
+    if (ctx->L > 2) return;
+    double kappa = 0.0;
+    bool any = false;
+    for (int c = 0; c < ctx->ncomp; ++c) {
+        const LfmmComp& cp = ctx->comp[c];
+        if (cp.is_free || !cp.has_rem) continue;
+        if (cp.den[1] != 0.0 || cp.rem[1] != 0.0 || cp.rem[2] != 0.0 || cp.rem[3] != 0.0 || cp.rem[4] != 0.0) return;
+        if (cp.zeta_r < 2.0 * cp.D * (1.0 - 1e-12)) return;  // the rule's range of depths
+        if (any && fabs(cp.den[2] + kappa) > 1e-14) return;
+        kappa = -cp.den[2];
+        any = true;
+    }
+    if (any) {
+        const double step = 2.0 * (ctx->d[0] - ctx->d[1]);
+        double s[LFMM_IMG_RULE], w[LFMM_IMG_RULE];
+        std::vector<ImageGauss> gauss;
+        const int n64 = image_rule(kappa, 2e-14, gauss, s, w);
+        for (int i = 0; i < n64; ++i) {
+            ctx->img64.c[i] = step * s[i];
+            ctx->img64.w[i] = w[i];
+        }
+        const int n32 = image_rule(kappa, 5e-9, gauss, s, w);
+        for (int i = 0; i < n32; ++i) {
+            ctx->img32.c[i] = (float)(step * s[i]);
+            ctx->img32.w[i] = (float)w[i];
+        }
+        if (n64 == 0 || n32 == 0) return;
+        ctx->img64.n = n64;
+        ctx->img32.n = n32;
+    }
+    ctx->img_ok = 1;
+}
+
 // Free-space M2L tables: T_N^mu of the offset (t - s)/h in the rotated half
 // plane (rho = |offset_xy|, z = offset_z), for |offset|_inf in [2, TR]: TR = 3
 // (classic separation) or 5 (wider separation of high orders, whose finer-level
@@ -729,6 +847,7 @@ lfmm_status lfmm_create(const double* d, int L, const double* eps, int p, lfmm_c
         e = lf_cuda(cudaMemcpy(ctx->comp_dev.ptr, ctx->comp, sizeof(LfmmComp) * ctx->ncomp, cudaMemcpyHostToDevice),
                     "components");
     if (e.empty()) e = setup_rules(ctx);
+    if (e.empty()) setup_images(ctx);
     if (e.empty()) e = setup_tables(ctx);
     if (e.empty()) e = lf_setup_m2l_ops(ctx);
     // the setup tables travel by pageable copies on the legacy stream, which
@@ -839,8 +958,8 @@ static lfmm_status set_option(lfmm_ctx* ctx, int opt, double v)
 // tables are built here once per context, outside any evaluation.
 static LfErr auto_near_tables(lfmm_ctx* ctx)
 {
-    if (ctx->use_near_tab != 2 || ctx->precision != 1 || !ctx->built || ctx->near_reaction_entries == 0 ||
-        ctx->near_tab_ready)
+    if (ctx->use_near_tab != 2 || ctx->precision != 1 || ctx->img_ok || !ctx->built ||
+        ctx->near_reaction_entries == 0 || ctx->near_tab_ready)
         return LfErr();
     return lf_near_tables(ctx, nullptr);
 }

@@ -53,6 +53,11 @@ struct lfmm_ctx {
     // components
     int ncomp = 0;
     LfmmComp comp[LFMM_MAXCOMP];
+    // image rules of the remainders (lfmm_internal.cuh), to FP64 and to float32
+    // accuracy; img_ok 0: the medium has none (four or more layers, slow series)
+    int img_ok = 0;
+    LfImgRule<double> img64 = {};
+    LfImgRule<float> img32 = {};
 
     // device and streams
     int device = 0;

@@ -103,6 +103,20 @@ struct LfmmComp {
     double me[LFMM_MAXL + 1];        // permittivities
 };
 
+// Remainder of a geometric density, rem(x)/den(x) = r0 / (1 - kappa x^2)
+// (every component of two or three layers, kappa the product of the middle
+// layer's two reflection coefficients): its integrals are sums over images,
+//   int J_mu(k rho) k^N e^{-k Z} r0 / (1 - kappa x^2) dk = r0 sum_n kappa^n T_N^mu(rho, Z + 2 n D),
+// and the sum is taken by a rule of n depths c_i = 2 D s_i and weights w_i: the
+// first terms as they are, the tail by Gauss quadrature for the discrete
+// weight kappa^n on n = 0, 1, 2, ... (Meixner polynomials, beta = 1).
+#define LFMM_IMG_RULE 96
+template <typename R>
+struct LfImgRule {
+    int n;  // 0: no remainder anywhere in the medium
+    R c[LFMM_IMG_RULE], w[LFMM_IMG_RULE];
+};
+
 __host__ __device__ __forceinline__ int lf_nre(int p) { return (p + 1) * (p + 2) / 2; }
 __host__ __device__ __forceinline__ int lf_nc(int p) { return (p + 1) * (p + 1); }
 __host__ __device__ __forceinline__ int lf_re(int n, int m) { return n * (n + 1) / 2 + m; }
@@ -642,6 +656,37 @@ __device__ __forceinline__ bool lf_nt_remainder4(const float4* __restrict__ ctab
     r10 = a1 * iZ * iZ;
     r11 = a2 * iZ * iZ;
     return true;
+}
+
+// Reaction pair kernel by the image rule: I_00, I_10 and I_11 / rho of the
+// leading image (depth zeta, amplitude C) and of the remainder's images
+// (depths zeta_r + c_i, weights r0 w_i).
+template <typename R>
+__device__ __forceinline__ void lf_image_pair(R C, R zeta, R zeta_r, R r0, R rho2, R h, const LfImgRule<R>& rule,
+                                              R& k00, R& k10, R& g)
+{
+    typedef LfMath<R> F;
+    R s0 = R(0), s1 = R(0), s2 = R(0);
+    if (r0 != R(0)) {
+        const R Z = h + zeta_r;
+#pragma unroll 2
+        for (int i = 0; i < rule.n; ++i) {
+            const R H = Z + rule.c[i];
+            const R ir = F::Rsqrt(rho2 + H * H);
+            const R wi = rule.w[i] * ir;
+            const R w3 = wi * ir * ir;
+            s0 += wi;
+            s1 += w3 * H;
+            s2 += w3;
+        }
+    }
+    const R H = h + zeta;
+    const R ir = F::Rsqrt(rho2 + H * H);
+    const R ci = C * ir;
+    const R c3 = ci * ir * ir;
+    k00 = ci + r0 * s0;
+    k10 = c3 * H + r0 * s1;
+    g = c3 + r0 * s2;
 }
 
 template <typename R, bool GEN = false>

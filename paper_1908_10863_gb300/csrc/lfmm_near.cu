@@ -396,6 +396,236 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_p2p_warp(P2PArgs a, const flo
     }
 }
 
+// Near field with lists of sources: the FP64 form, and the float32 form where
+// the near lists hold reaction pairs, in media whose remainders are image
+// sums (LfImgRule) or without any reaction pair.  One warp per target leaf
+// (or per part of its list).  For a pass of T targets the warp walks its list
+// twice, free-space entries first, then the reaction entries: 32 entries at a
+// time, one per lane, a warp scan places their sources in one flat range, and
+// chunks of PL_CAP of them are staged in shared memory (position relative to
+// the target box, charges, component).  The 32 lanes are T target slots times
+// 32 / T slices of the staged chunk; T is the width that pads the leaf's
+// charges least.
+// A reaction pair costs one inverse square root and about ten operations per
+// image of the rule (14 to 60 images in FP64, 8 to 36 in float32) where the
+// quadrature costs exp, J0, J1 and a division at each of 32 to 80 nodes, and
+// the float32 tables 16 gathered 16-byte loads.  The FP64 pipe (2 multiply-adds
+// per clock and SM) bounds the FP64 form, so what counts there is that every
+// lane of a warp instruction holds a pair.
+// Measured, eps (1, 5, 10): 1,000 charges in FP64, 86k reaction pairs, 6.27 ms
+// by one block of 128 threads per leaf and the quadrature, 0.48 ms here; 2,848
+// charges at p = 20, 538k reaction pairs, 33.0 and 1.67 ms; float32, 50,001
+// charges beside the interfaces, 30M reaction pairs, 0.95 ms by the tables
+// (k_p2p_warp), 0.57 ms here.
+#define PL_CAP 64
+#define PL_WARPS 4
+
+// slots of target charges per pass: the padded passes, plus the staging's share
+__device__ __forceinline__ int pl_targets(int nt)
+{
+    int best = 1 << 30, T = 32;
+    for (int t = 32; t >= 4; t >>= 1) {
+        const int cost = ((nt + t - 1) / t) * (t + 2);
+        if (cost < best) {
+            best = cost;
+            T = t;
+        }
+    }
+    return T;
+}
+
+template <typename R>
+struct PlComp {  // one component's pair constants: leading image, remainder, polarization map
+    R C, zeta, zeta_r, r0;
+};
+
+template <typename R, int RB>
+__global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const float4* __restrict__ rel, int nleaf,
+                                                            int ncomp, const __grid_constant__ LfImgRule<R> rule)
+{
+    typedef LfMath<R> F;
+    constexpr bool DBL = sizeof(R) == 8;
+    __shared__ R s_x[PL_WARPS][PL_CAP], s_y[PL_WARPS][PL_CAP], s_z[PL_WARPS][PL_CAP], s_q[PL_WARPS][RB][PL_CAP];
+    __shared__ short s_c[PL_WARPS][PL_CAP];  // component, bit 8: targets above (a = 1: h = z - z'')
+    __shared__ PlComp<R> s_comp[LFMM_MAXCOMP];
+    __shared__ double2 s_map[LFMM_MAXCOMP];  // z'' = s z' + o
+    __shared__ short s_kind[LFMM_MAXCOMP];   // 0: free space; else 1 + 256 (a == 1)
+    for (int c = threadIdx.x; c < ncomp; c += 32 * PL_WARPS) {
+        const LfmmComp& cp = a.comps[c];
+        s_comp[c] = PlComp<R>{(R)cp.C, (R)cp.zeta, (R)cp.zeta_r, cp.has_rem ? (R)cp.rem[0] : R(0)};
+        s_map[c] = cp.is_free ? make_double2(1.0, 0.0) : make_double2(cp.s, cp.o);
+        s_kind[c] = cp.is_free ? 0 : (cp.a == 1 ? 257 : 1);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int wi = blockIdx.x * PL_WARPS + w;
+    if (wi >= nleaf * a.split) return;  // whole warp, after the block's only barrier
+    const int li = wi / a.split, part0 = wi - li * a.split;
+    const R* q = reinterpret_cast<const R*>(a.q);
+    const int t = a.leaf_off + li;
+    const bool cells = !DBL && a.grid;
+    const LfD4 ct = cells ? LfD4{0.0, 0.0, 0.0, 0.0} : a.cen[t];
+    const int4 gt = cells ? a.grid[t] : make_int4(0, 0, 0, 0);
+    const int tb = a.pbeg[t], te = a.pend[t];
+    const int eb = a.nbeg[t], ee = a.nend[t];
+    const int nmine = (ee - eb > part0) ? (ee - eb - part0 + a.split - 1) / a.split : 0;
+    const int T = pl_targets(te - tb), G = 32 / T;
+    const int ti = lane & (T - 1), slice = lane / T;
+    for (int base = tb; base < te; base += T) {
+        const int i = base + ti;
+        const bool valid = i < te;
+        R xi = 0, yi = 0, zi = 0;
+        if (valid) {
+            if constexpr (DBL) {
+                xi = (R)(a.xs[i] - ct.x);
+                yi = (R)(a.ys[i] - ct.y);
+                zi = (R)(a.zs[i] - ct.z);
+            } else {
+                const float4 r = rel[i];
+                xi = r.x;
+                yi = r.y;
+                zi = r.z;
+            }
+        }
+        P2PAcc<R, RB> A;
+        P2PPart<R, RB> part;
+#pragma unroll 1
+        for (int react = 0; react < 2; ++react) {
+#pragma unroll 1
+            for (int k0 = 0; k0 < nmine; k0 += 32) {
+                // this lane's entry: first source, sources, centre offset of its (image) box
+                int b0 = 0, n = 0, c = 0;
+                float dx0 = 0.f, dy0 = 0.f, dz0 = 0.f, szs = 1.f;
+                const int j = k0 + lane;
+                if (j < nmine) {
+                    const uint32_t ent = a.nent[eb + part0 + j * a.split];
+                    const int s = (int)(ent & LFMM_ENT_MASK);
+                    c = (int)(ent >> LFMM_ENT_SHIFT);
+                    if ((s_kind[c] != 0) == (react != 0)) {
+                        b0 = a.pbeg[s];
+                        n = a.pend[s] - b0;
+                        if constexpr (!DBL) {
+                            if (cells) {
+                                const int4 gs = a.grid[s];
+                                const float4 pc = a.pcon[c];
+                                szs = pc.x;
+                                dx0 = (float)(gs.x - gt.x) * a.hleaf;
+                                dy0 = (float)(gs.y - gt.y) * a.hleaf;
+                                dz0 = (pc.x * ((float)gs.z + 0.5f) - ((float)gt.z + 0.5f) + pc.y) * a.hleaf;
+                            } else {
+                                const LfD4 cs = a.cen[s];
+                                szs = (float)s_map[c].x;
+                                dx0 = (float)(cs.x - ct.x);
+                                dy0 = (float)(cs.y - ct.y);
+                                dz0 = (float)(s_map[c].x * cs.z + s_map[c].y - ct.z);
+                            }
+                        }
+                    }
+                }
+                int incl = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                const int excl = incl - n;
+                const int tot = __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll 1
+                for (int f0 = 0; f0 < tot; f0 += PL_CAP) {
+                    const int cnt = min(PL_CAP, tot - f0);
+                    __syncwarp();  // the previous chunk has been read
+#pragma unroll 1
+                    for (int h = 0; h < cnt; h += 32) {
+                        // flat source f0 + h + lane belongs to the last entry that starts at or
+                        // before it (entries without sources start where the next one does)
+                        const int u = f0 + h + lane;
+                        int lo = 0;
+#pragma unroll
+                        for (int step = 16; step > 0; step >>= 1) {
+                            const int ex = __shfl_sync(0xffffffffu, excl, (lo + step) & 31);
+                            if (ex <= u) lo += step;
+                        }
+                        const int src = __shfl_sync(0xffffffffu, b0, lo) + (u - __shfl_sync(0xffffffffu, excl, lo));
+                        const int cc = __shfl_sync(0xffffffffu, c, lo);
+                        float ox, oy, oz, sz;
+                        if constexpr (!DBL) {
+                            ox = __shfl_sync(0xffffffffu, dx0, lo);
+                            oy = __shfl_sync(0xffffffffu, dy0, lo);
+                            oz = __shfl_sync(0xffffffffu, dz0, lo);
+                            sz = __shfl_sync(0xffffffffu, szs, lo);
+                        }
+                        if (u < f0 + cnt) {
+                            const int d = h + lane;
+                            if constexpr (DBL) {
+                                s_x[w][d] = a.xs[src] - ct.x;
+                                s_y[w][d] = a.ys[src] - ct.y;
+                                const double2 m = s_map[cc];
+                                s_z[w][d] = (react ? m.x * a.zs[src] + m.y : a.zs[src]) - ct.z;
+                            } else {
+                                const float4 r = rel[src];
+                                s_x[w][d] = r.x + ox;
+                                s_y[w][d] = r.y + oy;
+                                s_z[w][d] = sz * r.z + oz;
+                            }
+#pragma unroll
+                            for (int k = 0; k < RB; ++k)
+                                if (k < a.nr) s_q[w][k][d] = q[(size_t)k * a.qstride + src];
+                            s_c[w][d] = (short)(cc | (s_kind[cc] & 256));
+                        }
+                    }
+                    __syncwarp();
+                    if (valid) {
+                        if (!react) {
+                            for (int u = slice; u < cnt; u += G)
+                                p2p_free_add<R, RB>(xi - s_x[w][u], yi - s_y[w][u], zi - s_z[w][u], &s_q[w][0][u],
+                                                    PL_CAP, a.nr, part);
+                        } else {
+                            for (int u = slice; u < cnt; u += G) {
+                                const int ck = s_c[w][u];
+                                const PlComp<R> pc = s_comp[ck & 255];
+                                const R dx = xi - s_x[w][u], dy = yi - s_y[w][u], dz = zi - s_z[w][u];
+                                const R sg = (ck & 256) ? R(1) : R(-1);
+                                const R rho2 = dx * dx + dy * dy;
+                                R k00, k10, g;
+                                lf_image_pair<R>(pc.C, pc.zeta, pc.zeta_r, pc.r0, rho2, sg * dz, rule, k00, k10, g);
+                                k10 *= sg;
+#pragma unroll
+                                for (int k = 0; k < RB; ++k) {
+                                    if (k >= a.nr) break;
+                                    const R qv = s_q[w][k][u];
+                                    part.P[k].add(qv * k00);
+                                    part.Ez[k].add(qv * k10);
+                                    const R qg = qv * g;
+                                    part.Ex[k].add(qg * dx);
+                                    part.Ey[k].add(qg * dy);
+                                }
+                            }
+                        }
+                        p2p_flush<R, RB>(part, A);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < RB; ++k) {
+            // the slices of a target slot meet (every lane takes part in the shuffles)
+            R v0 = A.P[k].s - A.P[k].c, v1 = A.Ex[k].s - A.Ex[k].c;
+            R v2 = A.Ey[k].s - A.Ey[k].c, v3 = A.Ez[k].s - A.Ez[k].c;
+            for (int off = T; off < 32; off <<= 1) {
+                v0 += __shfl_xor_sync(0xffffffffu, v0, off);
+                v1 += __shfl_xor_sync(0xffffffffu, v1, off);
+                v2 += __shfl_xor_sync(0xffffffffu, v2, off);
+                v3 += __shfl_xor_sync(0xffffffffu, v3, off);
+            }
+            A.P[k].s = v0;
+            A.Ex[k].s = v1;
+            A.Ey[k].s = v2;
+            A.Ez[k].s = v3;
+        }
+        if (valid && slice == 0) p2p_store<R, RB>(a, i, A);
+    }
+}
+
 // Float32 free-space near field, one charge vector, when no near list holds
 // a reaction entry (the benchmark-size trees): one warp per target leaf, as
 // k_p2p_warp, but the warp first stages its whole near list in shared memory
@@ -727,7 +957,7 @@ template <typename R>
 __device__ __forceinline__ void p2p_drain(const LfmmComp& cp, const uint16_t* qe, int count, int lane, int wbase,
                                           const R* tx, const R* ty, const R* tz, const R* sx, const R* sy,
                                           const R* sz, const R* sq, R (*acc)[4], int Qn, const double* gl_t,
-                                          const double* gl_w, const double* ctab)
+                                          const double* gl_w, const double* ctab, const LfImgRule<R>& rule)
 {
     typedef LfMath<R> F;
     if (lane >= count) return;
@@ -737,7 +967,13 @@ __device__ __forceinline__ void p2p_drain(const LfmmComp& cp, const uint16_t* qe
     R h = (cp.a == 1) ? dz : -dz;
     R rho = F::Sqrt(dx * dx + dy * dy);
     R k00, k10, k11;
-    lf_reaction_pair<R>(cp, rho, h, Qn, gl_t, gl_w, k00, k10, k11, ctab);
+    if (rule.n >= 0) {
+        lf_image_pair<R>((R)cp.C, (R)cp.zeta, (R)cp.zeta_r, cp.has_rem ? (R)cp.rem[0] : R(0), dx * dx + dy * dy, h,
+                         rule, k00, k10, k11);
+        k11 *= rho;
+    } else {
+        lf_reaction_pair<R>(cp, rho, h, Qn, gl_t, gl_w, k00, k10, k11, ctab);
+    }
     R qs = sq[u];
     atomicAdd(&acc[o][0], qs * k00);
     atomicAdd(&acc[o][3], (cp.a == 1) ? qs * k10 : -qs * k10);
@@ -749,7 +985,7 @@ __device__ __forceinline__ void p2p_drain(const LfmmComp& cp, const uint16_t* qe
 }
 
 template <typename R>
-__global__ void __launch_bounds__(P2P_T) k_p2p_net(P2PArgs a)
+__global__ void __launch_bounds__(P2P_T) k_p2p_net(P2PArgs a, const __grid_constant__ LfImgRule<R> rule)
 {
     typedef LfMath<R> F;
     __shared__ R sx[P2P_T], sy[P2P_T], sz[P2P_T], sq[P2P_T];
@@ -859,14 +1095,14 @@ __global__ void __launch_bounds__(P2P_T) k_p2p_net(P2PArgs a)
                         if (qn >= 32) {
                             __syncwarp();
                             qn -= 32;
-                            p2p_drain<R>(cp, &qbuf[wid][qn], 32, lane, wbase, tx, ty, tz, sx, sy, sz, sq, acc, a.Qn, a.gl_t, a.gl_w, LF_CTAB(a, c));
+                            p2p_drain<R>(cp, &qbuf[wid][qn], 32, lane, wbase, tx, ty, tz, sx, sy, sz, sq, acc, a.Qn, a.gl_t, a.gl_w, LF_CTAB(a, c), rule);
                             __syncwarp();
                         }
                     }
                 }
                 if (qn > 0) {
                     __syncwarp();
-                    p2p_drain<R>(cp, &qbuf[wid][0], qn, lane, wbase, tx, ty, tz, sx, sy, sz, sq, acc, a.Qn, a.gl_t, a.gl_w, LF_CTAB(a, c));
+                    p2p_drain<R>(cp, &qbuf[wid][0], qn, lane, wbase, tx, ty, tz, sx, sy, sz, sq, acc, a.Qn, a.gl_t, a.gl_w, LF_CTAB(a, c), rule);
                     __syncwarp();
                 }
             }
@@ -947,7 +1183,16 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
     // of the near lists (counted at every build); without any, the kernels of
     // thinner media compute the free-space pairs alone and are exact
     const bool general = ctx->L >= 3 && ctx->near_reaction_entries > 0;
-    const bool warp_kernel = !net && !general && ctx->precision;
+    // Reaction pairs by the image rule (k_p2p_list) where the medium has one,
+    // unless the tables are asked for.  The FP64 form of a context that holds
+    // trained networks keeps the quadrature for the pairs outside the network
+    // runs (test_surrogate_gain_in_near_field states the network's gain over
+    // it).  FP64 lists without reaction pairs take the same kernel.
+    const bool react = ctx->near_reaction_entries > 0;
+    const bool img = ctx->img_ok && ctx->use_near_tab != 1;
+    const bool list = !net && !general &&
+                      (react ? img && (ctx->precision || !ctx->surr_ready) : ctx->precision == 0);
+    const bool warp_kernel = list || (!net && !general && ctx->precision);
     int split = ctx->p2p_split;
     if (split <= 0) {
         const int want = warp_kernel ? 152 * 32 : 152 * 8;  // warps, or blocks of P2P_T threads
@@ -959,6 +1204,10 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
         LF_CHECK(cudaMemsetAsync(a.phi, 0, sizeof(double) * (size_t)ctx->n * nr, st));
         LF_CHECK(cudaMemsetAsync(a.fld, 0, 3 * sizeof(double) * (size_t)ctx->n * nr, st));
     }
+    // the network's rejected pairs go by the image rule too (n = -1: quadrature or tables)
+    LfImgRule<float> net32 = ctx->img32;
+    LfImgRule<double> net64 = ctx->img64;
+    if (!img) net32.n = net64.n = -1;
     const double* phi0 = a.phi;
     double* fld0 = a.fld;
     const char* q0 = reinterpret_cast<const char*>(a.q);
@@ -968,16 +1217,32 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
         a.q = q0 + (size_t)r0 * qs;
         a.phi = const_cast<double*>(phi0) + (size_t)r0 * ctx->n;
         a.fld = fld0 + (size_t)r0 * ctx->n * 3;
-        if (general) {
+        if (list) {
+            const int g = lf_blocks((int64_t)leaf.nbox * split, PL_WARPS), T = 32 * PL_WARPS;
+            const float4* rel = ctx->pos_rel.as<float4>();
+            const int nb = leaf.nbox, nc = ctx->ncomp;
+#define PL_LAUNCH(R, RB, RULE) ++ctx->launches, k_p2p_list<R, RB><<<g, T, 0, st>>>(a, rel, nb, nc, ctx->RULE)
+            if (ctx->precision) {
+                if (a.nr == 1) PL_LAUNCH(float, 1, img32);
+                else if (a.nr == 2) PL_LAUNCH(float, 2, img32);
+                else PL_LAUNCH(float, 4, img32);
+            } else {
+                if (a.nr == 1) PL_LAUNCH(double, 1, img64);
+                else if (a.nr == 2) PL_LAUNCH(double, 2, img64);
+                else if (a.nr <= 4) PL_LAUNCH(double, 4, img64);
+                else PL_LAUNCH(double, 8, img64);
+            }
+#undef PL_LAUNCH
+        } else if (general) {
             if (ctx->precision)
                 ++ctx->launches, k_p2p<float, 1, true><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
             else
                 ++ctx->launches, k_p2p<double, 1, true><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
         } else if (net) {
             if (ctx->precision)
-                ++ctx->launches, k_p2p_net<float><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
+                ++ctx->launches, k_p2p_net<float><<<leaf.nbox * split, P2P_T, 0, st>>>(a, net32);
             else
-                ++ctx->launches, k_p2p_net<double><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
+                ++ctx->launches, k_p2p_net<double><<<leaf.nbox * split, P2P_T, 0, st>>>(a, net64);
         } else if (ctx->precision) {
             const int g = lf_blocks((int64_t)leaf.nbox * split, PW_WARPS), T = 32 * PW_WARPS;
             const float4* rel = ctx->pos_rel.as<float4>();

@@ -1118,7 +1118,7 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
     int* rbeg = ctx->m2r_off.as<int>();
     int* rend = rbeg + nb;
     // level 0: near(root_t) = root of the source layer of every component
-    int64_t near_used = 0;
+    int64_t near_used = 0, root_react = 0;  // entries, reaction entries
     {
         const LfmmLevel& r = ctx->levels[0];
         if (r.nbox > 128) return "internal: more than 128 root boxes";
@@ -1151,6 +1151,7 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
                 if (src < 0) continue;
                 if (ne >= MAXE) return "internal: too many root list entries";
                 ent[ne++] = ((uint32_t)c << LFMM_ENT_SHIFT) | (uint32_t)src;
+                root_react += !cp.is_free;
             }
             he[i] = ne;
         }
@@ -1264,7 +1265,8 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
     ctx->stats[LFMM_STAT_M2L_REACTION] = (int64_t)hs[1];
     // particle-pair counts only on request (lf_p2p_pair_stats); the near field
     // needs to know whether any leaf's near list holds a reaction entry
-    ctx->near_reaction_entries = (int64_t)hs[4];
+    // (counted by the list kernel; the roots are the leaves of a tree of depth 0)
+    ctx->near_reaction_entries = depth > 0 ? (int64_t)hs[4] : root_react;
     ctx->p2p_stats_stale = 1;
     ctx->stats[LFMM_STAT_P2P_FREE] = 0;
     ctx->stats[LFMM_STAT_P2P_REACTION] = 0;
