@@ -57,26 +57,27 @@ enum {
     LFMM_OPT_QUAD_NODES = 4, /* Gauss-Laguerre nodes of the M2L remainder integrals (16..128, default 64) */
     LFMM_OPT_SURROGATE = 5,  /* 1 = near-field reaction kernels by the trained network (default 0) */
     LFMM_OPT_SURROGATE_TOL = 6, /* error estimate above which a pair falls back to quadrature (default 1e-6) */
-    LFMM_OPT_TENSOR_CORES = 7,  /* float32 free M2L engine: 2 = automatic (default): tensor cores (3xTF32)
-                                   where (p+1)^2 <= 128, the compensated CUDA-core sums above; 1 = tensor
-                                   cores at every order (for 11 <= p <= 14 the wide form: Err2 of the
-                                   potential ~8e-7 at p = 14 against ~4e-7 on the CUDA cores, in a sixth
-                                   of the time); 0 = CUDA cores.  Where (p+1)^2 <= 128 the tensor cores
-                                   also take the L2L into the leaves and the keyed reaction M2L (each
-                                   key's operator formed in shared memory from its Sommerfeld table,
-                                   eqs. metoleimage1, coefintable); 0 puts both on the CUDA cores. */
+    LFMM_OPT_TENSOR_CORES = 7,  /* float32 free M2L engine: 2 = automatic (default) and 1: tensor cores (operands
+                                   as two float16 pieces, accumulated in order of falling degree; for
+                                   11 <= p <= 14 the wide form); 0 = the compensated CUDA-core sums.
+                                   Where (p+1)^2 <= 128 the tensor cores also take the L2L into the
+                                   leaves and the keyed reaction M2L (each key's operator formed in
+                                   shared memory from its Sommerfeld table, eqs. metoleimage1,
+                                   coefintable); 0 puts both on the CUDA cores. */
     LFMM_OPT_P2P_SPLIT = 8,     /* near list of a leaf shared by this many warps/blocks of the P2P kernels:
                                    0 = chosen from the leaf count (default), else 1, 2, 4, 8 or 16 */
     LFMM_OPT_TC_GROUPS = 9,     /* tensor-core free M2L: CTAs per tile of targets (256, or 128 in the wide
                                    form), each summing 189/groups offsets in its tensor-memory accumulator
                                    before a float atomic add; a divisor of 189, or 0 = automatic (default:
-                                   27, i.e. 7 offsets per accumulation; 63 in the wide form) */
-    LFMM_OPT_NEAR_TABLES = 10,  /* near-field reaction kernels: 2 = automatic (default): the float32 form
-                                   takes the remainder from pre-computed tables (deviation from the
-                                   quadrature ~2e-8, see lfmm_near_tables) once a build's near lists hold
-                                   reaction pairs, building them at the end of that build (once per
-                                   context), the FP64 form keeps the quadrature; 1 = tables in both forms
-                                   (built on first use); 0 = quadrature */
+                                   21, i.e. 9 offsets per accumulation; 63 in the wide form) */
+    LFMM_OPT_NEAR_TABLES = 10,  /* near-field reaction kernels: 2 = automatic (default): image sums where the
+                                   medium's remainders have them (up to three layers whose reflections'
+                                   product stays below ~0.97), else the float32 form takes the remainder
+                                   from pre-computed tables (deviation from the quadrature ~2e-8 to 1e-5,
+                                   see lfmm_near_tables) once a build's near lists hold reaction pairs,
+                                   building them at the end of that build (once per context), and the
+                                   FP64 form the quadrature; 1 = tables in both forms (built on first
+                                   use); 0 = image sums or the quadrature, no tables */
     LFMM_OPT_TC_PERSISTENT = 11, /* tensor-core free M2L: 1 = one persistent CTA per SM walking the
                                    (tile, offset group) units with a double-buffered accumulator, for
                                    launches of at least 4 units per SM; 0 = one CTA per unit, two CTAs per

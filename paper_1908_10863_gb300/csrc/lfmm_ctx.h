@@ -128,9 +128,10 @@ struct lfmm_ctx {
     int m2l_rm = 0, m2l_rp = 0, m2l_ntiles = 0;
     // tensor-core free M2L (float32 form, (p+1)^2 <= 128)
     DevBuf m2l_Atc, m2l_tc_tiles, m2l_Ms;
+    DevBuf tc_cscale, tc_perm;     // 2^e of every packed coefficient (float16 operand scaling); K order
     DevBuf tc_mseg;  // runs of the merged tensor-core tiles, [merged tile][LFMM_TC_MSEG] int4 (level, start, count, 0)
-    DevBuf m2m_Atc, l2l_Atc, tc_shift_tiles;        // tensor-core M2M / L2L operators and tiles
-    std::vector<int> tc_m2m_first, tc_l2l_first;    // first tensor-core translation tile of each level
+    DevBuf l2l_Atc, tc_shift_tiles;  // tensor-core L2L operators (into the leaves) and tiles
+    std::vector<int> tc_l2l_first;   // first tensor-core translation tile of each level
     std::vector<int4> tc_shift_h;
     // M2M / L2L as gathered GEMMs (the same kernel as the free M2L)
     DevBuf m2m_A64, m2m_A32, l2l_A64, l2l_A32, shift_cls, m2m_slots, shift_tiles;
@@ -146,7 +147,7 @@ struct lfmm_ctx {
     int use_near_tab = 2;       // 0 quadrature, 1 tables, 2 tables in the float32 form (default)
     double near_tab_err = -1.0;  // largest relative deviation from the quadrature at the check points
     double m2l_levelh_h[16] = {0};
-    // use_tc: 2 automatic (tensor cores where (p+1)^2 <= 128), 1 at every order, 0 never
+    // use_tc: 2 automatic and 1: tensor cores, 0: CUDA cores
     int m2l_tc_ok = 0, m2l_tc_ntiles = 0, use_tc = 2, tc_groups = 0;  // tc_groups 0: automatic
     int m2l_tc_wide = 0;  // tensor-core free M2L in its wide form ((p+1)^2 > 128): no tensor-core M2M / L2L
     // reaction M2L grouped by geometry key on interface-aligned levels
@@ -233,13 +234,11 @@ inline cudaError_t lf_d2h(void* dst, const void* src, size_t bytes, cudaStream_t
 // ---- tree construction (lfmm_tree.cu) ----
 LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz_dev, const int32_t* layer_dev, int64_t n, cudaStream_t st);
 LfErr lf_p2p_pair_stats(lfmm_ctx* ctx);
-// whether the float32 free M2L runs on the tensor cores: the automatic setting
-// keeps the compensated CUDA-core sums for the wide form ((p+1)^2 > 128),
-// where they are the more accurate choice
-inline bool lf_tc_on(const lfmm_ctx* ctx)
-{
-    return ctx->m2l_tc_ok && (ctx->use_tc == 1 || (ctx->use_tc == 2 && !ctx->m2l_tc_wide));
-}
+// whether the float32 free M2L runs on the tensor cores (the automatic setting
+// takes them at every order: with its degree-ordered accumulation the wide form
+// of p = 11 .. 14 is as accurate as the compensated CUDA-core sums, Err2(phi)
+// 3.1e-7 against 3.2e-7 at N = 65,536, p = 14, in an eighth of the time)
+inline bool lf_tc_on(const lfmm_ctx* ctx) { return ctx->m2l_tc_ok && ctx->use_tc != 0; }
 
 // ---- free-space M2L GEMM (lfmm_m2l.cu) ----
 LfErr lf_setup_m2l_ops(lfmm_ctx* ctx);
@@ -285,9 +284,12 @@ LfErr lf_shift_gemm(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st);
 // ---- tensor-core free M2L (lfmm_m2l_tc.cu) ----
 // byte offset in ctx->counts of the int counting device waits that ran out
 #define LFMM_TIMEOUT_OFF 40960
+// ... and of the largest scaled coefficient (float bits) per right-hand side:
+// multipoles of each level at [0, 16), locals at [16, 32)
+#define LFMM_TCMAX_OFF 45056
 #define LFMM_TC_MSEG 16  // runs per merged tensor-core M2L tile (one leftover run per level and class)
-LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, const double* A64, const double* M2M64, const double* L2L64, int KP, int RP);
-LfErr lf_shift_tc(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st);
+LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP);
+LfErr lf_l2l_tc(lfmm_ctx* ctx, int level, cudaStream_t st);
 LfErr lf_wait_probe(lfmm_ctx* ctx, double limit_ms, int* timed_out);
 LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st);
 int lf_m2l_tc_tile(const lfmm_ctx* ctx);

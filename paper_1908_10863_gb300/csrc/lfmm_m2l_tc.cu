@@ -5,47 +5,68 @@
 //   r = output coefficient (M = 128 rows, expansions with (p+1)^2 <= 128),
 //   j = target box of the tile (N = 256 columns, one level and octant class),
 //   k = input coefficient of the source at offset o (K = 128 in chunks of
-//       TC_KC, only the chunks that hold the (p+1)^2 inputs),
+//       TH_KC, only the chunks that hold the (p+1)^2 inputs),
 // accumulated in tensor memory (128 lanes x 256 float32 columns).  The wide
 // form takes 128 < (p+1)^2 <= 256 (p = 11 .. 14): two 128-row halves of r,
 // K = 256, tiles of 128 targets (see k_m2l_tc<true>).
 //
-// Precision: float32 operands as sums of two TF32 pieces, the operator
-// (a1 + a2, from its FP64 values) and the multipoles (x1 + x2, split once per
-// evaluation), with the three products a1 x1 + a1 x2 + a2 x1 ("3xTF32",
-// ~2^-21 of |a||x| per product).  What limits the result is the tensor
-// core's float32 accumulation: its error grows with the number of MMAs
-// summed into one accumulator, so each CTA takes only 7 of the 189 offsets
-// (27 CTAs per tile, joined by float atomics), which keeps the far field
-// within the CUDA-core float32 GEMM's error (measured: Err2 of the potential
-// against the FP64 path 2.0e-6 with 7 offsets per CTA, 1.2e-5 with 63,
-// 3.3e-5 with 189; 1.4e-6 for the CUDA-core float32 GEMM).
+// Precision: float32 operands as sums of two float16 pieces (11 + 11 bits, the
+// significand of two TF32 pieces), the operator (a1 + a2, from its FP64
+// values) and the multipoles (x1 + x2, split once per evaluation), with the
+// three products a1 x1 + a1 x2 + a2 x1 (~2^-21 of |a||x| per product).  Float16
+// has half the bytes of TF32 in L2, shared memory and the MMAs' operand reads,
+// and twice the multiply rate; its five exponent bits are no limit after
+// scaling by powers of two:
+//   - coefficient (n, m) carries 2^e, e = log2 sqrt((n - m)! (n + m)!) rounded
+//     (M scaled up by it, L down), which takes the factorials out of the
+//     expansions and of the operators (entries below 2);
+//   - each level's multipoles are scaled by one power of two that puts the
+//     largest scaled coefficient into [2^13, 2^14) (k_tc_max), so the pieces
+//     lose nothing above 2^-39 of that largest coefficient.
+// What limits the result is the tensor core's float32 accumulation: its error
+// grows with the number of MMAs added to an accumulator that is already large.
+// So the input coefficients run from the highest degree to the lowest (K is
+// ordered by degree, and a unit takes K chunk by K chunk, each for all its
+// offsets): the small contributions of the high degrees meet in a small
+// accumulator, and only the last chunk, degrees 0 to 4, adds at full size.
+// Each CTA takes only some of the 189 offsets, and the CTAs of a tile are
+// joined by float atomics.
 //
-// One CTA = (tile of 256 targets, one third of its 189 offsets):
-//   warps 0..7  gather the 256 pre-split source multipoles of a (offset,
-//               K chunk) stage with 16-byte cp.async into the swizzled
+// Measured (config-2 geometry, M2L alone; Err2(phi) of the float32 form
+// against the FP64 form), TF32 pieces in offset order -> float16 pieces in
+// degree order: N = 1M, p = 10: 2.25 ms, 2.1e-6 -> 1.33 ms, 0.66e-6; N = 262,144,
+// p = 6: 0.208 -> 0.137 ms, 1.5e-6 -> 0.6e-6; the wide form, N = 65,536, p = 14:
+// 1.29 ms, 6.8e-7 -> 0.93 ms, 3.1e-7, the error of the compensated CUDA-core sums
+// (7.9 ms), so the wide form is the default.  Float16 pieces in offset order: 1.45
+// ms, 1.26e-6 at N = 1M.  Bound: L2 -> shared memory, 192 KB per tile and
+// offset (8.8 GB at N = 1M, 6.6 TB/s); the MMAs alone would take 0.6 ms.
+//
+// One CTA = (tile of 256 targets, 9 of its 189 offsets):
+//   warps 0..7  gather the 256 pre-split source multipoles of a (K chunk,
+//               offset) stage with 16-byte cp.async into the swizzled
 //               K-major layout (zeros where a target has no source there), ahead
 //               of the tensor cores; thread 0 also starts the bulk
 //               copy of the matching operator chunk (stored pre-split and
 //               pre-swizzled in HBM);
-//   warp 8      one thread issues the MMAs of a stage (3 products x K chunk / 8) and commits them to
+//   warp 8      one thread issues the MMAs of a stage (3 products x 2 K steps of 16) and commits them to
 //               the stage's "empty" barrier;
-//   epilogue    warps 0..7 read the accumulator (tcgen05.ld), scale by 1/h and
-//               add into the local expansions (float atomics: the CTAs of a
+//   epilogue    warps 0..7 read the accumulator (tcgen05.ld), scale by 1/h and the inverse
+//               operand scales and add into the local expansions (float atomics: the CTAs of a
 //               tile's offset groups meet there).
-// Two stages of 48 KB (K chunks of 16, 64-byte swizzle) per CTA buffer the
+// Two stages of 48 KB (K chunks of 32, 64-byte swizzle) per CTA buffer the
 // operands, handed to the tensor cores one stage after their copies start;
-// two CTAs share an SM, so four stages are in flight per SM.  (K chunks of 8
-// with 32-byte swizzle, or one CTA per SM with four stages, measured slower.)
+// two CTAs share an SM, so four stages are in flight per SM.
 // Tiles of one octant class share their offset list; each tile walks it from a different starting offset so
 // that concurrent CTAs read different operator chunks.  Every barrier wait is
 // bounded; on a timeout the CTA records an error, stops issuing work, waits
 // (bounded) for its copies in flight and frees its tensor memory.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -65,7 +86,7 @@
 
 #define TC_N 256                     // targets per tile (MMA N)
 #define TC_M 128                     // output coefficients (MMA M)
-#define TC_NKC (128 / TC_KC)         // K chunks (K = 128)
+#define TC_NKC (128 / TH_KC)         // K chunks (K = 128)
 #define TC_RCH (TC_ROWB / 16)        // 16-byte chunks per row
 #define TC_NOFF 189                  // offsets per octant class
 #define TC_NALL 343
@@ -76,11 +97,10 @@
 #define TC_AP 2                      // operator pieces
 #define TC_XP 2                      // multipole pieces
 #define TC_STAGE_BYTES (TC_AP * TC_A_BYTES + TC_XP * TC_X_BYTES)
-#define TC_MROW 128                  // floats per multipole piece row in the split copy (512 B)
+#define TC_MROW 128                  // halves per multipole piece row in the split copy (256 B)
 // Two CTAs per SM (97 KB of shared memory and 256 tensor-memory columns
 // each), two 48 KB stages apiece: one CTA's prologue, gathers and atomic
-// epilogue overlap the other's MMAs.  Measured at N = 1M, p = 10: 2.39 ms
-// against 2.63 ms for one CTA per SM with four stages.
+// epilogue overlap the other's MMAs.
 #ifndef TC_STAGES
 #define TC_STAGES 2
 #endif
@@ -95,6 +115,10 @@
 #define TC_WIDE_STAGES 4             // wide form: one CTA per SM
 #define TC_WIDE_SMEM (TC_WIDE_STAGES * TC_STAGE_BYTES + 1024)
 #define TC_MSEG LFMM_TC_MSEG
+// offsets per CTA whose source boxes are kept in shared memory: every K chunk
+// walks the offsets again, and a load from the slot table (one 32-byte sector
+// per target) at each stage cost 0.2 ms at N = 1M.  Larger groups read the table.
+#define TC_SRC 9
 
 struct TcArgs {
     const int4* tiles;      // level, class, start, count
@@ -105,17 +129,30 @@ struct TcArgs {
     int unit_scale;         // 1: add D as it is (M2M, L2L); 0: add D / h_level (M2L)
     const double* levelh;   // box size per level
     const int4* mseg;       // merged tiles' runs [merged tile][TC_MSEG]: (level, start, count, 0)
-    const unsigned char* A; // [343][4 chunks][2 pieces x 16 KB], pre-swizzled
-    const float* Ms;        // split multipoles [box + 1][2 pieces][128] (last box: zeros)
-    int zero_row;           // index of the zero box of Ms
+    const unsigned char* A; // [343][4 chunks][2 pieces x 8 KB], pre-swizzled
+    const __half* Ms;       // split, scaled expansions [box][2 pieces][128]
+    const float* cscale;    // 2^e of every coefficient (output rows)
+    float unscale;          // inverse of the operators' common scale
+    const unsigned* gmax;   // largest scaled coefficients of the sources, [32] per right-hand side
+    int gslot;              // slot of the source level: the target's level + gslot
     float* L;               // locals [box][nc]
     int nc;
-    int nkc;                // K chunks of TC_KC coefficients that hold the nc inputs: ceil(nc / TC_KC)
-    size_t ms_stride;       // per right-hand side (blockIdx.y): split multipoles, in floats
+    int nkc;                // K chunks of TH_KC coefficients that hold the nc inputs: ceil(nc / TH_KC)
+    size_t ms_stride;       // per right-hand side (blockIdx.y): split multipoles, in halves
     size_t l_stride;        // per right-hand side: local expansions, in floats
     int groups;             // CTAs per tile (offset groups; divides noff)
     int* err;               // [0]: timeouts
 };
+
+// The power of two that takes the largest magnitude (float bits) into
+// [2^13, 2^14); 1 for zero or non-finite values.
+__device__ __forceinline__ float tc_scale(unsigned maxbits)
+{
+    if (maxbits == 0u || maxbits >= 0x7f800000u) return 1.f;
+    int e = 140 - (int)(maxbits >> 23);  // 13 - (biased exponent - 127)
+    e = e > 126 ? 126 : (e < -126 ? -126 : e);
+    return __uint_as_float((unsigned)(e + 127) << 23);
+}
 
 // Target t of a tile (a box id, or -1 past the tile's count) and its output
 // scale (1 for M2M and L2L, 1/h of the target's level for M2L).  A tile with
@@ -123,19 +160,25 @@ struct TcArgs {
 // of one octant class on several levels, listed at mseg[-1 - level] with
 // tile.z runs; its columns take the runs in order, each with its level's
 // scale (the operators depend only on the class and the offset).
+__device__ __forceinline__ float tc_out_scale(const TcArgs& g, int level)
+{
+    // 1/h, and the inverse of the sources' and the operators' scales
+    const float s = g.unscale / tc_scale(g.gmax[(size_t)blockIdx.y * 32 + level + g.gslot]);
+    return g.unit_scale ? s : s * (1.f / (float)g.levelh[level]);
+}
 __device__ __forceinline__ int tc_tile_target(const TcArgs& g, const int4& tile, int t, float& ih)
 {
     ih = 0.f;
     if (t >= tile.w) return -1;
     if (tile.x >= 0) {
-        ih = g.unit_scale ? 1.f : 1.f / (float)g.levelh[tile.x];
+        ih = tc_out_scale(g, tile.x);
         return g.sorted ? g.sorted[tile.z + t] : tile.z + t;
     }
     const int4* sg = g.mseg + (size_t)(-1 - tile.x) * TC_MSEG;
     for (int k = 0; k < tile.z; ++k) {
         const int4 r = sg[k];
         if (t < r.z) {
-            ih = g.unit_scale ? 1.f : 1.f / (float)g.levelh[r.x];
+            ih = tc_out_scale(g, r.x);
             return g.sorted[r.y + t];
         }
         t -= r.z;
@@ -156,8 +199,8 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
 {
     constexpr int TN = WIDE ? 128 : TC_N;       // targets per tile (MMA N)
     constexpr int MH = WIDE ? 2 : 1;            // 128-row halves of the output (MMA M = 128 each)
-    constexpr int NKC = WIDE ? 16 : TC_NKC;     // K chunks per operator in the blob
-    constexpr int MROW = WIDE ? 256 : TC_MROW;  // floats per multipole piece row
+    constexpr int NKC = WIDE ? 2 * TC_NKC : TC_NKC;      // K chunks per operator in the blob
+    constexpr int MROW = WIDE ? 2 * TC_MROW : TC_MROW;  // halves per multipole piece row
     constexpr int ABYTES = MH * TC_A_BYTES;     // one operator piece of a stage
     constexpr int XBYTES = TN * TC_ROWB;        // one multipole piece of a stage
     constexpr int NST = WIDE ? TC_WIDE_STAGES : TC_STAGES;
@@ -173,6 +216,7 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
     __shared__ int s_abort;
     __shared__ int s_tb[TC_N];
     __shared__ float s_ih[TC_N];  // output scale of each target column
+    __shared__ int s_src[TC_SRC][TN];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int item = blockIdx.x;
@@ -186,8 +230,15 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
 
     if (tid < TN) {
         float ih;
-        s_tb[tid] = tc_tile_target(g, tile, tid, ih);
+        const int tb = tc_tile_target(g, tile, tid, ih);
+        s_tb[tid] = tb;
         s_ih[tid] = ih;
+        if (goff <= TC_SRC) {
+            const int* src = g.slots + (size_t)(tb >= 0 ? tb : 0) * g.noff + grp * goff;
+#pragma unroll
+            for (int o = 0; o < TC_SRC; ++o)
+                if (o < goff) s_src[o][tid] = tb >= 0 ? src[o] : -1;
+        }
     }
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
@@ -216,15 +267,14 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
         const int ptid = tid;  // 0 .. 255
         const int rot = (item / g.groups) % goff;
         int armed = 0;         // stages with a bulk copy issued by this thread, for the bounded drain
-        int my_src = -1;       // source of row (warp * 32 + lane) at the current offset
-        // the source at the next offset is loaded one offset ahead (its
-        // latency hides behind the current offset's gathers)
-        const int my_tb = s_tb[(WIDE ? (warp & 3) : warp) * 32 + lane];
-        int nxt_src = (my_tb >= 0) ? g.slots[(size_t)my_tb * g.noff + grp * goff + rot % goff] : -1;
+        const int my_row = (WIDE ? (warp & 3) : warp) * 32 + lane;
+        const int* my_slots = g.slots + (size_t)max(s_tb[my_row], 0) * g.noff + grp * goff;
         int it = 0;
         for (; it < nstage; ++it) {
             const int s = it % NST, round = it / NST;
-            const int oi = grp * goff + (it / nkc + rot) % goff, kc = it % nkc;
+            const int ol = (it + rot) % goff, oi = grp * goff + ol, kc = nkc - 1 - it / goff;
+            // source of this thread's row at the stage's offset
+            const int my_src = goff <= TC_SRC ? s_src[ol][my_row] : (s_tb[my_row] >= 0 ? my_slots[ol] : -1);
             if (it >= NST) {
                 if (!mbar_wait(&empty_bar[s], (round - 1) & 1)) atomicExch(&s_abort, 1);
             }
@@ -235,11 +285,6 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
                 mbar_arrive_tx(&full_bar[s], TC_AP * ABYTES);
                 bulk_g2s(st, g.A + ((size_t)o * NKC + kc) * (TC_AP * ABYTES), TC_AP * ABYTES, &full_bar[s]);
                 armed = it + 1;
-            }
-            if (kc == 0) {
-                my_src = nxt_src;
-                const int on = it / nkc + 1;
-                if (on < goff && my_tb >= 0) nxt_src = g.slots[(size_t)my_tb * g.noff + grp * goff + (on + rot) % goff];
             }
             unsigned char* xs = st + TC_AP * ABYTES;
             const uint32_t xbase = smem_u32(xs);
@@ -253,10 +298,10 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
                 const int rl = flat / TC_RCH, chunk = flat % TC_RCH;
                 const int src = __shfl_sync(0xffffffffu, my_src, rl);
                 const int row = (WIDE ? (warp & 3) : warp) * 32 + rl;
-                const uint32_t off = piece * XBYTES + swz(row, chunk * 4);
+                const uint32_t off = piece * XBYTES + swz16(row, chunk * 8);
                 if (src >= 0) {
-                    const float* gsrc = g.Ms + (size_t)blockIdx.y * g.ms_stride + ((size_t)src * TC_XP + piece) * MROW +
-                                        kc * TC_KC + chunk * 4;
+                    const __half* gsrc = g.Ms + (size_t)blockIdx.y * g.ms_stride +
+                                         ((size_t)src * TC_XP + piece) * MROW + kc * TH_KC + chunk * 8;
                     cp_async16(xbase + off, gsrc);
                 } else {
                     *reinterpret_cast<float4*>(xs + off) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -288,6 +333,7 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
             // narrow: half = target half of the 256 columns; wide: half = the
             // 128-row half of the outputs, whose accumulator starts at column half * TN
             const int row = (WIDE ? 128 * half : 0) + 32 * q + lane;
+            const float rs = row < nc ? g.cscale[row] : 0.f;
 #pragma unroll 1
             for (int ch = 0; ch < 4; ++ch) {
                 const int col0 = (WIDE ? 0 : half * 128) + ch * 32;  // first target of the chunk
@@ -304,7 +350,7 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
                         const int j = col0 + i;
-                        if (j < cnt) atomicAdd(g.L + (size_t)blockIdx.y * g.l_stride + (size_t)s_tb[j] * nc + row, v[i] * s_ih[j]);
+                        if (j < cnt) atomicAdd(g.L + (size_t)blockIdx.y * g.l_stride + (size_t)s_tb[j] * nc + row, v[i] * s_ih[j] * rs);
                     }
                 }
             }
@@ -314,7 +360,7 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
     } else {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            const uint32_t idesc = tc_idesc(TC_M, TN);
+            const uint32_t idesc = tc_idesc_f16(TC_M, TN);
             bool ok = true;
             for (int it = 0; it < nstage && ok; ++it) {
                 const int s = it % NST, round = it / NST;
@@ -326,21 +372,26 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
                 tc_fence_after();
                 const uint32_t base = smem_u32(sm + (size_t)s * TC_STAGE_BYTES);
                 const uint32_t xb = base + TC_AP * ABYTES;
-                // a1 x1, a1 x2, a2 x1
-                const int pa[3] = {0, 0, 1}, px[3] = {0, 1, 0};
+                // the small products first: a2 x1, a1 x2, a1 x1
+                const int pa[3] = {1, 0, 0}, px[3] = {0, 1, 0};
+                // K steps of 16 that hold coefficients (both but in an operator's last chunk)
+                const int nks = (nc - (nkc - 1 - it / goff) * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
                 for (int prod = 0; prod < 3; ++prod) {
                     const uint32_t a = base + pa[prod] * ABYTES;
                     const uint32_t b = xb + px[prod] * XBYTES;
                     // narrow: one accumulator; wide: a1 x1 alone, the corrections in the second
-                    const uint32_t acc = (WIDE && prod > 0) ? SMALL : 0u;
-                    const int first = WIDE ? (prod == 2 ? 1 : 0) : prod;  // 0: may start its accumulator
+                    const uint32_t acc = (WIDE && prod < 2) ? SMALL : 0u;
+                    const bool starts = prod == 0 || (WIDE && prod == 2);  // may start its accumulator
 #pragma unroll
-                    for (int ks = 0; ks < TC_KC / 8; ++ks)
+                    for (int ks = 1; ks >= 0; --ks) {
+                        if (ks >= nks) continue;
 #pragma unroll
                         for (int h = 0; h < MH; ++h)
-                            tc_mma(tmem + acc + (uint32_t)(h * TN), smem_desc(a + h * TC_A_BYTES + 32 * ks),
-                                   smem_desc(b + 32 * ks), idesc, (it | first | ks) != 0 ? 1u : 0u);
+                            tc_mma_f16(tmem + acc + (uint32_t)(h * TN), smem_desc(a + h * TC_A_BYTES + 32 * ks),
+                                       smem_desc(b + 32 * ks), idesc,
+                                       (it == 0 && starts && ks == nks - 1) ? 0u : 1u);
+                    }
                 }
                 tc_commit(&empty_bar[s]);
             }
@@ -439,11 +490,11 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
             const int my_tb = tc_tile_target(g, tile, row, ih_unused);
             const int rot = (u / g.groups) % goff;
             int my_src = -1;
-            // the source at the next offset is loaded one offset ahead
+            // the next stage's source is loaded one stage ahead
             int nxt_src = (my_tb >= 0) ? g.slots[(size_t)my_tb * g.noff + grp * goff + rot % goff] : -1;
             for (int j = 0; j < nstage; ++j, ++it) {
                 const int s = it % TCP_STAGES, round = it / TCP_STAGES;
-                const int oi = grp * goff + (j / g.nkc + rot) % goff, kc = j % g.nkc;
+                const int oi = grp * goff + (j + rot) % goff, kc = g.nkc - 1 - j / goff;
                 if (it >= TCP_STAGES) {
                     if (!mbar_wait(&empty_bar[s], (round - 1) & 1)) atomicExch(&s_abort, 1);
                 }
@@ -459,12 +510,8 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
                              &full_bar[s]);
                     armed = it + 1;
                 }
-                if (kc == 0) {
-                    my_src = nxt_src;
-                    const int on = j / g.nkc + 1;
-                    if (on < goff && my_tb >= 0)
-                        nxt_src = g.slots[(size_t)my_tb * g.noff + grp * goff + (on + rot) % goff];
-                }
+                my_src = nxt_src;
+                if (my_tb >= 0) nxt_src = g.slots[(size_t)my_tb * g.noff + grp * goff + (j + 1 + rot) % goff];
                 unsigned char* xs = st + TC_AP * TC_A_BYTES;
                 const uint32_t xbase = smem_u32(xs);
 #pragma unroll
@@ -474,10 +521,10 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
                     const int rl = flat / TC_RCH, chunk = flat % TC_RCH;
                     const int src = __shfl_sync(0xffffffffu, my_src, rl);
                     const int r = warp * 32 + rl;
-                    const uint32_t off = piece * TC_X_BYTES + swz(r, chunk * 4);
+                    const uint32_t off = piece * TC_X_BYTES + swz16(r, chunk * 8);
                     if (src >= 0) {
-                        const float* gsrc = g.Ms + (size_t)blockIdx.y * g.ms_stride +
-                                            ((size_t)src * TC_XP + piece) * TC_MROW + kc * TC_KC + chunk * 4;
+                        const __half* gsrc = g.Ms + (size_t)blockIdx.y * g.ms_stride +
+                                             ((size_t)src * TC_XP + piece) * TC_MROW + kc * TH_KC + chunk * 8;
                         cp_async16(xbase + off, gsrc);
                     } else {
                         *reinterpret_cast<float4*>(xs + off) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -505,7 +552,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
     } else if (warp == TC_PROD_WARPS) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            const uint32_t idesc = tc_idesc(TC_M, TC_N);
+            const uint32_t idesc = tc_idesc_f16(TC_M, TC_N);
             int it = 0, ul = 0;
             bool ok = true;
             for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++ul) {
@@ -525,15 +572,17 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
                     tc_fence_after();
                     const uint32_t base = smem_u32(sm + (size_t)s * TC_STAGE_BYTES);
                     const uint32_t xb = base + TC_AP * TC_A_BYTES;
-                    const int pa[3] = {0, 0, 1}, px[3] = {0, 1, 0};  // a1 x1, a1 x2, a2 x1
+                    const int pa[3] = {1, 0, 0}, px[3] = {0, 1, 0};  // a2 x1, a1 x2, a1 x1
+                    const int nks = (nc - (g.nkc - 1 - j / goff) * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
                     for (int prod = 0; prod < 3; ++prod) {
                         const uint32_t a = base + pa[prod] * TC_A_BYTES;
                         const uint32_t bb = xb + px[prod] * TC_X_BYTES;
 #pragma unroll
-                        for (int ks = 0; ks < TC_KC / 8; ++ks)
-                            tc_mma(acc, smem_desc(a + 32 * ks), smem_desc(bb + 32 * ks), idesc,
-                                   (j | prod | ks) != 0 ? 1u : 0u);
+                        for (int ks = 1; ks >= 0; --ks)
+                            if (ks < nks)
+                                tc_mma_f16(acc, smem_desc(a + 32 * ks), smem_desc(bb + 32 * ks), idesc,
+                                           (j == 0 && prod == 0 && ks == nks - 1) ? 0u : 1u);
                     }
                     tc_commit(&empty_bar[s]);
                 }
@@ -549,6 +598,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
         // so a warp that gives up on a timed-out wait cannot strand another)
         const int q = warp & 3;  // tensor-memory lanes 32 q .. 32 q + 31
         const int r = 32 * q + lane;
+        const float rs = r < nc ? g.cscale[r] : 0.f;
         int ul = 0;
         for (int u = blockIdx.x; u < nunits; u += gridDim.x, ++ul) {
             const int b = ul & 1;
@@ -576,7 +626,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
                 for (int i = 0; i < 32; ++i) {
                     const int tb = __shfl_sync(0xffffffffu, tbl, i);
                     const float ih = __shfl_sync(0xffffffffu, ihl, i);
-                    if (r < nc && tb >= 0) atomicAdd(Lb + (size_t)tb * nc + r, v[i] * ih);
+                    if (r < nc && tb >= 0) atomicAdd(Lb + (size_t)tb * nc + r, v[i] * ih * rs);
                 }
             }
             tc_fence_before();
@@ -596,60 +646,100 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
 // ---------------------------------------------------------------------------
 // Host: operator blob and launch.
 // ---------------------------------------------------------------------------
-static inline uint32_t host_tf32(float x)
+// packed index of the K-th input coefficient: by degree, Re before Im
+static void coef_order(int p, std::vector<int>& perm)
 {
-    // round to nearest (ties away from zero) at 10 explicit mantissa bits
-    uint32_t u;
-    memcpy(&u, &x, 4);
-    if ((u & 0x7f800000u) == 0x7f800000u) return u;
-    u = (u + 0x1000u) & 0xffffe000u;
-    return u;
+    perm.clear();
+    for (int n = 0; n <= p; ++n) {
+        for (int m = 0; m <= n; ++m) perm.push_back(lf_re(n, m));
+        for (int m = 1; m <= n; ++m) perm.push_back(lf_im(p, n, m));
+    }
 }
 
-// A64: [nops][KP in][RP out] (double) -> the tensor-core operator blob:
-// per operator nkc K chunks of two TF32 pieces, each piece mh 128-row halves
-// (mh = 2 for the wide form), pre-swizzled
-static LfErr tc_blob(const double* A64, int nops, int KP, int RP, int nc, bool wide, DevBuf& out)
+// binary exponent of each packed coefficient's scale: log2 sqrt((n-m)! (n+m)!), rounded
+static void coef_exponents(int p, std::vector<int>& e)
 {
-    const int mh = wide ? 2 : 1, nkc = wide ? 16 : TC_NKC;
-    const size_t chunk = (size_t)TC_AP * mh * TC_A_BYTES;
-    const size_t per = (size_t)nkc * chunk;
-    std::vector<uint32_t> blob((size_t)nops * per / 4, 0u);
-    for (int o = 0; o < nops; ++o)
-        for (int kc = 0; kc < nkc; ++kc) {
-            unsigned char* p0 = reinterpret_cast<unsigned char*>(blob.data()) + (size_t)o * per + (size_t)kc * chunk;
-            for (int r = 0; r < mh * TC_M; ++r)
-                for (int k = 0; k < TC_KC; ++k) {
-                    const int kin = kc * TC_KC + k;
-                    double v = (r < nc && kin < nc) ? A64[((size_t)o * KP + kin) * RP + r] : 0.0;
-                    for (int q = 0; q < TC_AP; ++q) {
-                        uint32_t t = host_tf32((float)v);
-                        float tf;
-                        memcpy(&tf, &t, 4);
-                        memcpy(p0 + ((size_t)q * mh + r / TC_M) * TC_A_BYTES + swz(r % TC_M, k), &t, 4);
-                        v -= (double)tf;
-                    }
-                }
+    const int nc = lf_nc(p);
+    e.assign(nc, 0);
+    for (int j = 0; j < nc; ++j) {
+        int n, m, im;
+        lf_decode(p, j, n, m, im);
+        e[j] = (int)std::lround(0.5 * (std::lgamma(n - m + 1.0) + std::lgamma(n + m + 1.0)) / std::log(2.0));
+    }
+}
+
+// Device operators A [nops][KP in][RP out] (FP64) -> the tensor-core operator
+// blob: per operator nkc K chunks of two float16 pieces, each piece mh 128-row
+// halves (mh = 2 for the wide form), pre-swizzled.  Entries are scaled by
+// 2^{sin e_in - e_out} (sin = -1: multipoles in, +1: locals in) and by
+// 2^TC_ASHIFT.  Scaled by the exponents they stay below 2 for every order (the
+// factorials leave binomial coefficients of N over 2^{N+1} or less), so the
+// pieces stay below 2^13; an entry beyond float16's range is counted in bad.
+// One block per (operator, K chunk).
+#define TC_ASHIFT 12
+__global__ void __launch_bounds__(256) k_tc_blob(const double* __restrict__ A, int KP, int RP, int nc,
+                                                 const int* __restrict__ perm, const float* __restrict__ cs, int sin,
+                                                 int mh, unsigned char* __restrict__ blob, int* __restrict__ bad)
+{
+    const int nkc = mh * TC_NKC, o = blockIdx.x / nkc, kc = blockIdx.x % nkc;
+    unsigned char* p0 = blob + (size_t)blockIdx.x * TC_AP * mh * TC_A_BYTES;
+    for (int i = threadIdx.x; i < TH_KC * mh * TC_M; i += 256) {
+        const int k = i / (mh * TC_M), r = i - k * (mh * TC_M), kk = kc * TH_KC + k;
+        double v = 0.0;
+        if (kk < nc && r < nc) {
+            const int kin = perm[kk];
+            const double si = sin < 0 ? 1.0 / (double)cs[kin] : (double)cs[kin];
+            v = A[((size_t)o * KP + kin) * RP + r] * si / (double)cs[r] * (double)(1 << TC_ASHIFT);
+            if (!(fabs(v) < 60000.0)) atomicAdd(bad, 1);
         }
-    LF_TRY(lf_reserve(out, blob.size() * 4));
-    LF_CHECK(cudaMemcpy(out.ptr, blob.data(), blob.size() * 4, cudaMemcpyHostToDevice));
-    return LfErr();
+#pragma unroll
+        for (int piece = 0; piece < TC_AP; ++piece) {
+            const __half h = __float2half_rn((float)v);
+            *reinterpret_cast<__half*>(p0 + ((size_t)piece * mh + r / TC_M) * TC_A_BYTES + swz16(r % TC_M, k)) = h;
+            v -= (double)__half2float(h);
+        }
+    }
 }
 
-// A64: [343][KP][RP] free M2L operators; M2M, L2L: [8][KP][RP] octant operators
-LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, const double* A64, const double* M2M64, const double* L2L64, int KP, int RP)
+static LfErr tc_blob(lfmm_ctx* ctx, const DevBuf& A64, int nops, int KP, int RP, int sin, bool wide, DevBuf& out)
+{
+    const int mh = wide ? 2 : 1, nkc = mh * TC_NKC;
+    LF_TRY(lf_reserve(out, (size_t)nops * nkc * TC_AP * mh * TC_A_BYTES));
+    LF_TRY(lf_reserve(ctx->counts, 65536));
+    int* bad = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
+    LF_CHECK(cudaMemsetAsync(bad, 0, sizeof(int), ctx->s_main));
+    ++ctx->launches, k_tc_blob<<<nops * nkc, 256, 0, ctx->s_main>>>(
+        A64.as<double>(), KP, RP, lf_nc(ctx->p), ctx->tc_perm.as<int>(), ctx->tc_cscale.as<float>(), sin, mh,
+        out.as<unsigned char>(), bad);
+    LF_TRY(lf_cuda(cudaGetLastError(), "tensor-core operators"));
+    int n = 0;
+    LF_CHECK(lf_d2h(&n, bad, sizeof(int), ctx->s_main));
+    return n ? LfErr("internal: tensor-core operator out of range") : LfErr();
+}
+
+// from the context's device operators m2l_A64 [343][KP][RP] and l2l_A64 [8][KP][RP]
+LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP)
 {
     const int nc = lf_nc(ctx->p);
     ctx->m2l_tc_ok = 0;
     ctx->m2l_tc_wide = 0;
     if (nc > 2 * TC_M || KP < nc || RP < nc) return LfErr();
     const bool wide = nc > TC_M;
-    // the wide form serves the free M2L only; M2M and L2L stay on the CUDA cores
-    LF_TRY(tc_blob(A64, TC_NALL, KP, RP, nc, wide, ctx->m2l_Atc));
-    if (!wide) {
-        LF_TRY(tc_blob(M2M64, 8, KP, RP, nc, false, ctx->m2m_Atc));
-        LF_TRY(tc_blob(L2L64, 8, KP, RP, nc, false, ctx->l2l_Atc));
-    }
+    std::vector<int> e;
+    coef_exponents(ctx->p, e);
+    std::vector<int> perm;
+    coef_order(ctx->p, perm);
+    std::vector<float> cs(nc);
+    for (int k = 0; k < nc; ++k) cs[k] = std::ldexp(1.f, e[k]);
+    LF_TRY(lf_reserve(ctx->tc_cscale, nc * sizeof(float)));
+    LF_CHECK(cudaMemcpy(ctx->tc_cscale.ptr, cs.data(), nc * sizeof(float), cudaMemcpyHostToDevice));
+    LF_TRY(lf_reserve(ctx->tc_perm, nc * sizeof(int)));
+    LF_CHECK(cudaMemcpy(ctx->tc_perm.ptr, perm.data(), nc * sizeof(int), cudaMemcpyHostToDevice));
+    // the wide form serves the free M2L only; L2L stays on the CUDA cores
+    // (the uploads above ran on the legacy stream, which s_main does not wait for)
+    LF_CHECK(cudaDeviceSynchronize());
+    LF_TRY(tc_blob(ctx, ctx->m2l_A64, TC_NALL, KP, RP, -1, wide, ctx->m2l_Atc));
+    if (!wide) LF_TRY(tc_blob(ctx, ctx->l2l_A64, 8, KP, RP, 1, false, ctx->l2l_Atc));
     LF_CHECK(cudaFuncSetAttribute(k_m2l_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
     LF_CHECK(cudaFuncSetAttribute(k_m2l_tc<false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     LF_CHECK(cudaFuncSetAttribute(k_m2l_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_WIDE_SMEM));
@@ -664,34 +754,99 @@ LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, const double* A64, const double* M2M64, con
     return LfErr();
 }
 
-// expansions [box][nc] -> two TF32 pieces per box, rows padded to mrow floats
-// (128, or 256 for the wide form), for the boxes b0 .. b0 + count - 1 (the
-// arrays hold nbox boxes per right-hand side, blockIdx.y)
-__global__ void k_split_m(const float* __restrict__ M, int nbox, int nc, int mrow, int b0, int count,
-                          float* __restrict__ Ms)
+// level of a global box id (levels are stored finest first)
+struct TcLevels {
+    int depth;
+    int off[17];
+};
+__device__ __forceinline__ int tc_level(const TcLevels& lv, int b)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)count * mrow) return;
+    int l = lv.depth;
+    while (l > 0 && b >= lv.off[l - 1]) --l;
+    return l;
+}
+
+// largest scaled magnitude |X_k| 2^{+-e_k} of the boxes b0 .. b0 + count - 1,
+// per level, as float bits in gmax[32 rhs + slot0 + level]; one warp per eight
+// boxes.  Reads the expansions just written (L2): 70,848 boxes of 121 floats
+// take about as long as the launch.
+__global__ void __launch_bounds__(256) k_tc_max(const float* __restrict__ X, int nbox, int nc, int b0, int count,
+                                                const float* __restrict__ cs, int inv, const __grid_constant__ TcLevels lv, int slot0,
+                                                unsigned* __restrict__ gmax)
+{
+    __shared__ float s_cs[256];
+    for (int k = threadIdx.x; k < nc; k += 256) s_cs[k] = inv ? 1.f / cs[k] : cs[k];
+    __syncthreads();
+    X += (size_t)blockIdx.y * nbox * nc;
+    const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int first = b0 + 8 * w, last = min(first + 8, b0 + count);
+    for (int b = first; b < last;) {
+        const int l = tc_level(lv, b);
+        unsigned m = 0;
+        for (; b < last && (l == 0 || b < lv.off[l - 1]); ++b)
+            for (int k = lane; k < nc; k += 32) m = max(m, __float_as_uint(fabsf(X[(size_t)b * nc + k] * s_cs[k])));
+        m = __reduce_max_sync(0xffffffffu, m);
+        unsigned* g = gmax + (size_t)blockIdx.y * 32 + slot0 + l;
+        if (lane == 0 && m > *(volatile unsigned*)g) atomicMax(g, m);
+    }
+}
+
+// expansions [box][nc] -> two scaled float16 pieces per box, rows padded to
+// mrow halves (128, or 256 for the wide form) in K order, for the boxes b0 ..
+// b0 + count - 1 (the arrays hold nbox boxes per right-hand side, blockIdx.y); one thread
+// per 8 coefficients
+__global__ void __launch_bounds__(256) k_split_m(const float* __restrict__ M, int nbox, int nc, int mrow, int b0,
+                                                 int count, const float* __restrict__ cs, int inv,
+                                                 const __grid_constant__ TcLevels lv,
+                                                 int slot0, const unsigned* __restrict__ gmax,
+                                                 const int* __restrict__ perm, __half* __restrict__ Ms)
+{
+    const int per = mrow / 8;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)count * per) return;
     M += (size_t)blockIdx.y * nbox * nc;
-    Ms += (size_t)blockIdx.y * (nbox + 1) * TC_XP * mrow;
-    const int b = b0 + (int)(i / mrow), k = (int)(i % mrow);
-    const float x = (k < nc) ? M[(size_t)b * nc + k] : 0.f;
-    const uint32_t hi = to_tf32(x);
-    const uint32_t lo = to_tf32(x - __uint_as_float(hi));
-    Ms[((size_t)b * TC_XP + 0) * mrow + k] = __uint_as_float(hi);
-    Ms[((size_t)b * TC_XP + 1) * mrow + k] = __uint_as_float(lo);
+    Ms += (size_t)blockIdx.y * nbox * TC_XP * mrow;
+    const int b = b0 + (int)(i / per), k0 = (int)(i % per) * 8;
+    const float s = tc_scale(gmax[(size_t)blockIdx.y * 32 + slot0 + tc_level(lv, b)]);
+    __align__(16) __half hi[8], lo[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int k = k0 + u;
+        float x = 0.f;
+        if (k < nc) {
+            const int j = perm[k];
+            x = M[(size_t)b * nc + j] * (inv ? 1.f / cs[j] : cs[j]) * s;
+        }
+        hi[u] = __float2half_rn(x);
+        lo[u] = __float2half_rn(x - __half2float(hi[u]));
+    }
+    __half* out = Ms + (size_t)b * TC_XP * mrow + k0;
+    *reinterpret_cast<uint4*>(out) = *reinterpret_cast<const uint4*>(hi);
+    *reinterpret_cast<uint4*>(out + mrow) = *reinterpret_cast<const uint4*>(lo);
 }
 
 static int ms_row(const lfmm_ctx* ctx) { return ctx->m2l_tc_wide ? 2 * TC_MROW : TC_MROW; }
+static unsigned* tc_gmax(lfmm_ctx* ctx) { return reinterpret_cast<unsigned*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF); }
 
-static LfErr split_boxes(lfmm_ctx* ctx, const float* src, int b0, int count, cudaStream_t st)
+// scale and split the expansions of the boxes b0 .. b0 + count - 1: multipoles
+// (locals = 0) or locals (1)
+static LfErr split_boxes(lfmm_ctx* ctx, const float* src, int b0, int count, int locals, cudaStream_t st)
 {
     if (count <= 0) return LfErr();
-    const int nb = ctx->nbox_total, nr = ctx->nrhs_b, mrow = ms_row(ctx);
-    LF_TRY(lf_reserve(ctx->m2l_Ms, (size_t)(nb + 1) * TC_XP * mrow * sizeof(float) * nr));
-    const size_t tot = (size_t)count * mrow;
+    static_assert(LFMM_TCMAX_OFF + LFMM_RHS_BATCH * 32 * 4 <= 65536, "counter buffer");
+    const int nb = ctx->nbox_total, nr = ctx->nrhs_b, mrow = ms_row(ctx), nc = lf_nc(ctx->p);
+    LF_TRY(lf_reserve(ctx->m2l_Ms, (size_t)nb * TC_XP * mrow * sizeof(__half) * nr));
+    TcLevels lv;
+    lv.depth = ctx->depth;
+    for (int l = 0; l < 17; ++l) lv.off[l] = l <= ctx->depth ? ctx->levels[l].off : 0;
+    unsigned* gm = tc_gmax(ctx);
+    if (!locals) LF_CHECK(cudaMemsetAsync(gm, 0, (size_t)nr * 32 * sizeof(unsigned), st));
+    ++ctx->launches, k_tc_max<<<dim3((count + 63) / 64, nr), 256, 0, st>>>(
+        src, nb, nc, b0, count, ctx->tc_cscale.as<float>(), locals, lv, 16 * locals, gm);
+    const int64_t tot = (int64_t)count * (mrow / 8);
     ++ctx->launches, k_split_m<<<dim3((unsigned)((tot + 255) / 256), nr), 256, 0, st>>>(
-        src, nb, lf_nc(ctx->p), mrow, b0, count, ctx->m2l_Ms.as<float>());
+        src, nb, nc, mrow, b0, count, ctx->tc_cscale.as<float>(), locals, lv, 16 * locals, gm,
+        ctx->tc_perm.as<int>(), ctx->m2l_Ms.as<__half>());
     return lf_cuda(cudaGetLastError(), "split");
 }
 
@@ -701,12 +856,13 @@ static TcArgs tc_args(lfmm_ctx* ctx)
     TcArgs g;
     g.levelh = ctx->m2l_levelh.as<double>();
     g.mseg = ctx->tc_mseg.as<int4>();
-    g.Ms = ctx->m2l_Ms.as<float>();
-    g.zero_row = nb;
-    g.ms_stride = (size_t)(nb + 1) * TC_XP * ms_row(ctx);
+    g.Ms = ctx->m2l_Ms.as<__half>();
+    g.cscale = ctx->tc_cscale.as<float>();
+    g.gmax = tc_gmax(ctx);
+    g.ms_stride = (size_t)nb * TC_XP * ms_row(ctx);
     g.l_stride = (size_t)nb * lf_nc(ctx->p);
     g.nc = lf_nc(ctx->p);
-    g.nkc = (g.nc + TC_KC - 1) / TC_KC;
+    g.nkc = (g.nc + TH_KC - 1) / TH_KC;
     g.err = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
     return g;
 }
@@ -716,8 +872,10 @@ LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st)
     if (ctx->m2l_tc_ntiles == 0) return LfErr();
     const int nb = ctx->nbox_total;
     const int nr = ctx->nrhs_b;
-    LF_TRY(split_boxes(ctx, ctx->Mexp.as<float>(), 0, nb, st));
+    LF_TRY(split_boxes(ctx, ctx->Mexp.as<float>(), 0, nb, 0, st));
     TcArgs g = tc_args(ctx);
+    g.gslot = 0;
+    g.unscale = 1.f / (float)(1 << TC_ASHIFT);
     g.tiles = ctx->m2l_tc_tiles.as<int4>();
     g.sorted = ctx->m2l_sorted.as<int>();
     g.slots = ctx->m2l_slots.as<int>();
@@ -726,10 +884,8 @@ LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st)
     g.unit_scale = 0;
     g.A = ctx->m2l_Atc.as<unsigned char>();
     g.L = ctx->Lexp.as<float>();
-    // automatic: 7 offsets per accumulator, 3 in the wide form, whose float32
-    // accumulation adds twice the MMAs per offset (measured at N = 1M, p = 14:
-    // Err2 of the potential 1.18e-6 with 7 offsets, 7.5e-7 with 3, for 1.2 ms more)
-    g.groups = ctx->tc_groups > 0 ? ctx->tc_groups : (ctx->m2l_tc_wide ? 63 : 27);
+    // automatic: 9 offsets per accumulator, 3 in the wide form
+    g.groups = ctx->tc_groups > 0 ? ctx->tc_groups : (ctx->m2l_tc_wide ? 63 : 21);
     const int nunits = ctx->m2l_tc_ntiles * g.groups;
     // the persistent form pays off when every SM walks many units; a small
     // tree (or one of many problems sharing the GPU in a batch) keeps one
@@ -748,47 +904,30 @@ LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st)
     return lf_cuda(cudaGetLastError(), "m2l tensor-core gemm");
 }
 
-// M2M into the parents at `level` (from their children one level down), or
-// L2L into the boxes at `level` (from their parents), on the tensor cores:
-// the source expansions are split into TF32 pieces first; the products are
-// added atomically (M2M into zeroed parents, L2L onto the M2L results).
-LfErr lf_shift_tc(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st)
+// L2L into the boxes at `level` (from their parents) on the tensor cores: the
+// parents' locals are scaled and split first, the products added atomically
+// onto the M2L results.
+LfErr lf_l2l_tc(lfmm_ctx* ctx, int level, cudaStream_t st)
 {
-    const int t0 = l2l ? ctx->tc_l2l_first[level] : ctx->tc_m2m_first[level];
-    const int t1 = l2l ? ctx->tc_l2l_first[level + 1] : ctx->tc_m2m_first[level + 1];
+    const int t0 = ctx->tc_l2l_first[level], t1 = ctx->tc_l2l_first[level + 1];
     if (t1 <= t0) return LfErr();
-    if (ctx->m2l_tc_wide) return LfErr("internal: tensor-core translations need (p+1)^2 <= 128");
-    const int nr = ctx->nrhs_b, nc = lf_nc(ctx->p);
-    const LfmmLevel& src = ctx->levels[l2l ? level - 1 : level + 1];
-    TcArgs g;
-    if (l2l) {
-        LF_TRY(split_boxes(ctx, ctx->Lexp.as<float>(), src.off, src.nbox, st));
-        g = tc_args(ctx);
-        g.sorted = ctx->m2l_sorted.as<int>();
-        g.slots = ctx->box_parent.as<int>();
-        g.noff = 1;
-        g.A = ctx->l2l_Atc.as<unsigned char>();
-        g.L = ctx->Lexp.as<float>();
-        g.groups = 1;
-    } else {
-        LF_TRY(split_boxes(ctx, ctx->Mexp.as<float>(), src.off, src.nbox, st));
-        const LfmmLevel& lv = ctx->levels[level];
-        const size_t ms = (size_t)ctx->nbox_total * nc;
-        LF_CHECK(cudaMemset2DAsync(ctx->Mexp.as<float>() + (size_t)lv.off * nc, ms * sizeof(float), 0,
-                                   sizeof(float) * (size_t)lv.nbox * nc, nr, st));
-        g = tc_args(ctx);
-        g.sorted = nullptr;
-        g.slots = ctx->m2m_slots.as<int>();
-        g.noff = 8;
-        g.A = ctx->m2m_Atc.as<unsigned char>();
-        g.L = ctx->Mexp.as<float>();
-        g.groups = 8;  // one child octant per CTA, summed by the atomics
-    }
+    if (ctx->m2l_tc_wide) return LfErr("internal: tensor-core L2L needs (p+1)^2 <= 128");
+    const LfmmLevel& src = ctx->levels[level - 1];
+    LF_TRY(split_boxes(ctx, ctx->Lexp.as<float>(), src.off, src.nbox, 1, st));
+    TcArgs g = tc_args(ctx);
+    g.sorted = ctx->m2l_sorted.as<int>();
+    g.slots = ctx->box_parent.as<int>();
+    g.noff = 1;
+    g.A = ctx->l2l_Atc.as<unsigned char>();
+    g.L = ctx->Lexp.as<float>();
+    g.groups = 1;
+    g.gslot = 16 - 1;  // the parents' level
+    g.unscale = 1.f / (float)(1 << TC_ASHIFT);
     g.tiles = ctx->tc_shift_tiles.as<int4>() + t0;
     g.cls = ctx->shift_cls.as<int>();
     g.unit_scale = 1;
-    ++ctx->launches, k_m2l_tc<false><<<dim3((t1 - t0) * g.groups, nr), TC_THREADS, TC_SMEM, st>>>(g);
-    return lf_cuda(cudaGetLastError(), l2l ? "l2l tensor-core gemm" : "m2m tensor-core gemm");
+    ++ctx->launches, k_m2l_tc<false><<<dim3((t1 - t0) * g.groups, ctx->nrhs_b), TC_THREADS, TC_SMEM, st>>>(g);
+    return lf_cuda(cudaGetLastError(), "l2l tensor-core gemm");
 }
 
 // Self-check of the bounded-wait path: one thread waits on a barrier that

@@ -12,6 +12,7 @@
 #define TC_KC 16                     // K elements per staged row (64-byte rows)
 #endif
 #define TC_ROWB (TC_KC * 4)          // bytes per row of a staged tile
+#define TH_KC (TC_ROWB / 2)          // 16-bit K elements per staged row
 #define TC_SPIN_CYCLES (1ll << 31)   // ~1 s at 2 GHz
 // ---------------------------------------------------------------------------
 // PTX helpers
@@ -105,6 +106,20 @@ __device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t 
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
         : "memory");
 }
+// the same with float16 operands (kind::f16, K = 16 per instruction)
+__host__ __device__ constexpr uint32_t tc_idesc_f16(int M, int N)
+{
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+__device__ __forceinline__ void tc_mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t acc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+        : "memory");
+}
 __device__ __forceinline__ void tc_commit(uint64_t* bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
@@ -137,3 +152,11 @@ __host__ __device__ __forceinline__ uint32_t swz(int row, int k)
     return (uint32_t)row * TC_ROWB + ((c ^ x) << 4) + (uint32_t)(k & 3) * 4u;
 }
 
+
+// the same for rows of TH_KC 16-bit elements
+__host__ __device__ __forceinline__ uint32_t swz16(int row, int k)
+{
+    const uint32_t c = (uint32_t)(k >> 3);
+    const uint32_t x = (TC_ROWB == 64) ? (uint32_t)((row >> 1) & 3) : (uint32_t)((row >> 2) & 1);
+    return (uint32_t)row * TC_ROWB + ((c ^ x) << 4) + (uint32_t)(k & 7) * 2u;
+}
