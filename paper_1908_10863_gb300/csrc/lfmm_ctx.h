@@ -167,13 +167,13 @@ struct lfmm_ctx {
     std::vector<int> m2r_ktab_h;
     double m2r_levelh_h[16] = {0};
     int m2r_nkeys = 0, m2r_nbatch = 0, m2r_keyed_from = 0, m2r_ntab = 0;
-    DevBuf m2r_ops;         // assembled operator per key, [nkeys][RP][RP] in the precision below
+    DevBuf m2r_phase64;     // FP64 e^{i m phi}, m <= LFMM_PMAX (rotated form)
+    int m2r_phase64_ready = 0;
     DevBuf m2r_phase;       // float32 e^{i m phi} of the 225 lateral key offsets, m <= 2p (tensor-core form)
     int m2r_phase_p = -1;   // order the phase table holds
     DevBuf m2r_pairs;       // int2 (source box, target box) per sorted reaction entry
     int m2r_nent = 0;       // sorted reaction entries
-    int m2r_ops_prec = -1;  // 0 FP64, 1 FP32, -1 not assembled for this build
-    int m2r_dev_pending = 0;  // 1: the keys' tables and operators are still to be computed (first evaluation)
+    int m2r_dev_pending = 0;  // 1: the keys' tables are still to be computed (first evaluation)
     cudaEvent_t ev_m2r = nullptr;  // recorded after them on the stream that computed them
     int m2r_wait = 0;              // 1: the far field must wait for ev_m2r before the reaction M2L
 
@@ -248,7 +248,6 @@ LfErr lf_m2l_gemm(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_prepare_m2r(lfmm_ctx* ctx, cudaStream_t st);         // enqueue (no synchronisation)
 LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st);  // synchronise st, host part
 LfErr lf_m2r_apply(lfmm_ctx* ctx, cudaStream_t st);
-LfErr lf_m2r_ops(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st);
 // stable LSD radix sort of uint32 (key, value) pairs (lfmm_tree.cu); uses keys_tmp, vals_tmp, hist
 // (set 1: keys_tmp2, vals_tmp2, hist2)

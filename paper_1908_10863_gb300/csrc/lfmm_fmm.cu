@@ -690,7 +690,7 @@ LfErr lf_evaluate_sorted(lfmm_ctx* ctx, int nrhs, const double* q_dev, double* p
         ++ctx->launches, k_gather_q<double><<<g1, 256, 0, st>>>(q_dev, ctx->perm.as<int32_t>(), n,
                                                                ctx->q_sorted.as<double>());
     LF_TRY(lf_cuda(cudaGetLastError(), "gather q"));
-    // the reaction M2L's tables and operators of a fresh build: on the
+    // the reaction M2L's tables of a fresh build: on the
     // near-field stream ahead of the near field, beside the far field's
     // upward pass; the far field waits for them before the reaction M2L
     const bool m2r_dev = ctx->m2r_dev_pending != 0;

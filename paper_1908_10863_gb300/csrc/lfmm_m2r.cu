@@ -1,17 +1,19 @@
 // lfmm_m2r.cu -- reaction-component M2L (eqs. metoleimage1, coefintable)
 // grouped by geometry key.
 //
-// On a level whose grid planes contain the interfaces, every polarization
-// box is a grid box, so the offset o = (t - P(s))/h of a reaction M2L pair is
-// an integer vector in [-3,3]^3.  The translation operator then depends only
-// on the key (component, level, offset): the Sommerfeld table of the pair
-// (leading image in closed form + Gauss-Laguerre remainder, all (N, mu)) is
-// computed once per key at build time, and at evaluation time the pairs of
-// one key are applied as batched GEMMs Y = A_key X (X = 64 gathered source
+// The offset o = (t - P(s))/h of a reaction M2L pair, P the polarization map
+// of the source box, is an integer vector up to a vertical fraction fixed per
+// (component, level).  The translation then depends only on the key
+// (component, level, offset): the Sommerfeld table of the pair (leading image
+// in closed form + Gauss-Laguerre remainder, all (N, mu)) is computed once per
+// (component, level, rho^2, oz) after a build, and at evaluation time the pairs
+// of one key are applied together (Y = A_key X, X the gathered source
 // multipoles), added atomically into the targets' local expansions.  The
 // reflection sign (-1)^{n+m} of the multipole (s = -1 maps) and the
-// (-1)^{N+mu} of an a = 2 component are folded into A_key.
-// Pairs on coarser, non-aligned levels keep the per-pair kernel.
+// (-1)^{N+mu} of an a = 2 component belong to A_key.
+// The float32 form with p <= 10 applies the keys on the tensor cores
+// (k_m2r_tc), every other case in the rotated frame (k_m2r_rot).  A level with
+// an entry outside the key range, and the coarser ones, keep the per-pair kernel.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -150,16 +152,13 @@ LfErr lf_prepare_m2r(lfmm_ctx* ctx, cudaStream_t st)
     ctx->m2r_nkeys = 0;
     ctx->m2r_nbatch = 0;
     ctx->m2r_ntab = 0;
-    ctx->m2r_ops_prec = -1;
     ctx->m2r_dev_pending = 0;
     ctx->stats[LFMM_STAT_REACTION_KEYS] = 0;
     ctx->stats[LFMM_STAT_REACTION_TABLES] = 0;
     ctx->m2r_keyed_from = ctx->depth + 1;
     ctx->m2r_pending_ne = 0;
     ctx->m2r_nent = 0;
-    // the keyed GEMM holds a whole operator in shared memory (p <= 10) or
-    // stages it in chunks (p <= 15)
-    if (ctx->m2l_rm == 0 || ctx->m2l_rm > 16 || ctx->m2r_total == 0) return LfErr();
+    if (ctx->m2r_total == 0) return LfErr();
     // every level with reaction entries is keyed; a level some of whose
     // entries fall outside the key's offset range stays per pair (found at
     // lf_prepare_m2r_finish)
@@ -353,14 +352,14 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
     // (the host staging vectors live in the context; the build synchronises at its end)
     ctx->stats[LFMM_STAT_REACTION_KEYS] = nku;
     ctx->stats[LFMM_STAT_REACTION_TABLES] = ntab;
-    // the tables and operators themselves are device work of the first
+    // the tables themselves are device work of the first
     // evaluation after this build (lf_m2r_device), beside its upward pass
     ctx->m2r_dev_pending = 1;
     return LfErr();
 }
 
-// Sommerfeld tables of the keys (FP64) and the keys' operators in the
-// current precision, enqueued on `st` (the first evaluation after a build
+// Sommerfeld tables of the keys (FP64) and the keys' (source, target) pairs,
+// enqueued on `st` (the first evaluation after a build
 // runs this on the near-field stream, so it overlaps the far field's upward
 // pass and free M2L; the reaction M2L waits for it).
 // (source box, target box) of every reaction M2L entry in key order
@@ -396,346 +395,176 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
             ctx->m2r_pairs.as<int2>());
         LF_TRY(lf_cuda(cudaGetLastError(), "m2r pairs"));
     }
-    LF_TRY(lf_m2r_ops(ctx, st));
     ctx->m2r_dev_pending = 0;  // only once both are enqueued
     return LfErr();
 }
 
 // ---------------------------------------------------------------------------
-// Evaluation: one operator per key (assembled once per build and precision),
-// then batched GEMMs with atomic accumulation.
+// Evaluation in the rotated frame (FP64, and float32 off the tensor cores).
+//
+// Turned about z by the key's azimuth phi (M' = M e^{i m phi}, a diagonal),
+// the coefficients of eq. coefintable are the real table T(N, |mu|), so the
+// real parts of the locals see only real parts and the imaginary ones only
+// imaginary parts:
+//   Re L'(k, l) = (-1)^k sum_n [ T(n+k, l) Re M'(n, 0) + sum_m (T(n+k, m+l) + s T(n+k, |l-m|)) Re M'(n, m) ]
+//   Im L'(k, l) = (-1)^k sum_n             sum_m (T(n+k, m+l) - s T(n+k, |l-m|)) Im M'(n, m)
+// with s = (-1)^m for m <= l, (-1)^l beyond.  That is half the multiply-adds of
+// the dense (p+1)^2 x (p+1)^2 operator, and the two entries come from two table
+// values, so no operator is stored: the table (a few KB) stays in shared
+// memory, and a pair of additions serves C columns.  One block per batch of
+// pairs of one key (and part of the rows); an item is one (k, l) for C columns,
+// C the width in {2, 4, 8} that pads the batch least.
+// FP64 (2 multiply-adds per clock and SM) bounds it.  Against one stored dense
+// operator per key (assembled after every build, 720 MB at N = 65,536) and a
+// GEMM: 6.44 + 1.79 ms -> 3.76 ms there, FP64, p = 10; float32, p = 14: 1.04 +
+// 0.74 -> 0.83 ms; and orders above 15, which integrated a table per pair
+// before, 27.0 -> 3.0 ms (2,848 charges, 6,910 pairs, p = 20).
 // ---------------------------------------------------------------------------
-struct ROpArgs {
-    int p, nc;
-    const uint32_t* kval;
-    const double* tables;   // one per (component, level, rho^2, oz)
-    const int* ktab;        // table of each key
-    const LfmmComp* comps;  // the context's components
-    void* ops;              // [nkeys][RP][RP]: A_key[k_in][r_out], zero padded
-};
+#define RR_PH (LFMM_PMAX + 1)
 
-// One block per key: A_key from its table, the lateral phases e^{i mu phi}
-// and the signs (eq. coefintable with the reflection of the multipole).
-template <typename R, int RP>
-__global__ void __launch_bounds__(R_T) k_m2r_ops(ROpArgs g)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int p = g.p, nc = g.nc, TS = 2 * p + 1;
-    R* sT = reinterpret_cast<R*>(smem_raw);  // [TS*TS]
-    R* sC = sT + TS * TS;                    // cos(m phi), m <= 2p
-    R* sS = sC + TS;
-    __shared__ unsigned char s_n[RP], s_m[RP], s_im[RP];  // (n, m, imaginary part) of each packed index
-    const int tid = threadIdx.x;
-    const int kidx = blockIdx.x;
-    if (tid < RP) {
-        int n = 0, m = 0, im = 0;
-        if (tid < nc) lf_decode(p, tid, n, m, im);
-        s_n[tid] = (unsigned char)n;
-        s_m[tid] = (unsigned char)m;
-        s_im[tid] = (unsigned char)im;
-    }
-    int c, lev, ox, oy, oz;
-    rkey_decode(g.kval[kidx], c, lev, ox, oy, oz);
-    (void)lev;
-    (void)oz;
-    const LfmmComp& cp = g.comps[c];
-    const double phi = (ox == 0 && oy == 0) ? 0.0 : atan2((double)oy, (double)ox);
-    if (tid < TS) {
-        double sn, cs;
-        sincos(tid * phi, &sn, &cs);
-        sC[tid] = (R)cs;
-        sS[tid] = (R)sn;
-    }
-    const double* Tk = g.tables + (size_t)g.ktab[kidx] * TS * TS;
-    for (int j = tid; j < TS * TS; j += R_T) sT[j] = (R)Tk[j];
-    __syncthreads();
-    R* A = reinterpret_cast<R*>(g.ops) + (size_t)kidx * RP * RP;
-    for (int idx = tid; idx < RP * RP; idx += R_T) {
-        const int kin = idx / RP, rout = idx - kin * RP;
-        R v = 0;
-        if (kin < nc && rout < nc) {
-            const int n = s_n[kin], mp = s_m[kin], bim = s_im[kin];
-            const int k = s_n[rout], l = s_m[rout], aim = s_im[rout];
-            // T_N^mu (complex) = e^{i mu phi} T(N, |mu|) with T_N^{-mu} = (-1)^mu conj
-            const int N = n + k;
-            const int mu1 = mp + l;
-            const R c1 = sT[N * TS + mu1] * sC[mu1], d1 = sT[N * TS + mu1] * sS[mu1];
-            R c2 = 0, d2 = 0, sg = 0;
-            if (mp > 0) {
-                const int mu2 = l - mp, a2 = mu2 < 0 ? -mu2 : mu2;
-                const R tv = sT[N * TS + a2];
-                c2 = tv * sC[a2];
-                d2 = tv * sS[a2];
-                if (mu2 < 0) {
-                    if (a2 & 1) c2 = -c2; else d2 = -d2;
-                }
-                sg = (mp & 1) ? R(-1) : R(1);
-            }
-            const R sk = (k & 1) ? R(-1) : R(1);
-            if (!aim && !bim) v = sk * (c1 + sg * c2);
-            else if (!aim && bim) v = sk * (-d1 + sg * d2);
-            else if (aim && !bim) v = sk * (d1 + sg * d2);
-            else v = sk * (c1 - sg * c2);
-            if (cp.refl && ((n + mp) & 1)) v = -v;
-        }
-        A[idx] = v;
-    }
-}
-
-struct RGemmArgs {
-    int p, nc;
-    const int4* batches;    // key, first sorted entry, count
-    const uint32_t* kval;
-    const void* ops;        // [nkeys][RP][RP]
-    const uint32_t* order;  // sorted entry indices
-    const uint32_t* ent;    // m2r entries (component | source box)
-    const int* tgt;         // target box per entry
+struct RRotArgs {
+    int p, nc, cb;          // order, coefficients, columns staged at a time
+    const int4* batches;    // key index, first sorted entry, count | key << 8, table
+    const double* tables;   // [table][TS][TS]
+    const LfmmComp* comps;
+    const double* phase;    // [225 lateral offsets][cos | sin][RR_PH]
+    const int2* pairs;      // (source box, target box) per sorted entry
     const double* levelh;
     const void* M;
     void* L;
     size_t stride;          // expansions per right-hand side, in elements
-    int nr;                 // right-hand sides, applied in turn with the operator staged once
+    int nr;
 };
 
-// Y = A X over the first 4 * CG columns (CG column groups of 4; the rest of
-// the 256 threads split the RP rows), scaled by 1/h and added into the
-// targets' local expansions.
-template <typename R, int RP, int CG>
-__device__ __forceinline__ void m2r_tile(const R* __restrict__ sA, const R* __restrict__ sX, int cnt,
-                                         const int* s_tgt, R ih, R* __restrict__ L, int nc)
+// e^{i m phi}, m <= p, of every lateral key offset, FP64
+__global__ void k_m2r_phase64(double* out)
 {
-    constexpr int KP = RP, XS = KP + 1;
-    constexpr int RG = R_T / CG;  // row groups
-    constexpr int RM = RP / RG;   // rows per thread
-    static_assert(RM >= 1 && RM * RG == RP, "tile shape");
-    const int tid = threadIdx.x;
-    const int cg = tid % CG, rg = tid / CG;
-    R acc[RM][4];
+    const int b = blockIdx.x, m = threadIdx.x;
+    if (m >= RR_PH) return;
+    const int ox = b / R_OW - R_OR, oy = b % R_OW - R_OR;
+    const double phi = (ox == 0 && oy == 0) ? 0.0 : atan2((double)oy, (double)ox);
+    double sn, cs;
+    sincos(m * phi, &sn, &cs);
+    out[(size_t)b * 2 * RR_PH + m] = cs;
+    out[(size_t)b * 2 * RR_PH + RR_PH + m] = sn;
+}
+
+// columns [0, cnt) of the staged chunk, rows part of nparts
+template <typename R, int C>
+__device__ __forceinline__ void rr_apply(int p, int nc, const R* sT, const R* sXr, const R* sXi, int cb, int cnt,
+                                         const int* s_tgt, const R* sC, const R* sS, R ih, R* __restrict__ L, int part,
+                                         int nparts)
+{
+    const int nre = lf_nre(p), TS = 2 * p + 1;
+    const int ng = (cnt + C - 1) / C, items = nre * ng;
+    for (int it = part * R_T + threadIdx.x; it < items; it += R_T * nparts) {
+        const int row = it / ng, c0 = (it - row * ng) * C;
+        int k, l, dummy;
+        lf_decode(p, row, k, l, dummy);
+        R ar[C], ai[C];
 #pragma unroll
-    for (int r = 0; r < RM; ++r)
+        for (int c = 0; c < C; ++c) ar[c] = ai[c] = R(0);
+        const R* xr = sXr + c0;
+        const R* xi = sXi + c0;
+        for (int n = 0; n <= p; ++n) {
+            const R* Tr = sT + (n + k) * TS;
+            {
+                const R e = Tr[l];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] = 0;
-#pragma unroll 4
-    for (int kk = 0; kk < KP; ++kk) {
-        R a[RM];
+                for (int c = 0; c < C; ++c) ar[c] += e * xr[c];
+                xr += cb;
+                xi += cb;
+            }
+#pragma unroll 2
+            for (int m = 1; m <= n; ++m) {
+                const int d = l - m;
+                const R t1 = Tr[m + l];
+                R t2 = Tr[d < 0 ? -d : d];
+                if ((d < 0 ? l : m) & 1) t2 = -t2;
+                const R er = t1 + t2, ei = t1 - t2;
 #pragma unroll
-        for (int r = 0; r < RM; ++r) a[r] = sA[kk * RP + rg * RM + r];
-        R x[4];
+                for (int c = 0; c < C; ++c) {
+                    ar[c] += er * xr[c];
+                    ai[c] += ei * xi[c];
+                }
+                xr += cb;
+                xi += cb;
+            }
+        }
+        const R cr = (k & 1) ? -sC[l] * ih : sC[l] * ih, sr = (k & 1) ? -sS[l] * ih : sS[l] * ih;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = sX[(4 * cg + q) * XS + kk];
-#pragma unroll
-        for (int r = 0; r < RM; ++r)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[r][q] += a[r] * x[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = 4 * cg + q;
-        if (j >= cnt) continue;
-        R* Lt = L + (size_t)s_tgt[j] * nc;
-#pragma unroll
-        for (int r = 0; r < RM; ++r) {
-            const int row = rg * RM + r;
-            if (row < nc) atomicAdd(Lt + row, acc[r][q] * ih);
+        for (int c = 0; c < C; ++c) {
+            if (c0 + c >= cnt) break;
+            R* Lt = L + (size_t)s_tgt[c0 + c] * nc;
+            atomicAdd(Lt + row, cr * ar[c] - sr * ai[c]);
+            if (l > 0) atomicAdd(Lt + lf_im(p, k, l), sr * ar[c] + cr * ai[c]);
         }
     }
 }
 
-// One block per batch of up to R_TB pairs of one key.
-template <typename R, int RP>
-__global__ void __launch_bounds__(R_T) k_m2r_gemm(RGemmArgs g)
+template <typename R>
+__global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int KP = RP;
-    constexpr int XS = KP + 1;
-    constexpr int CG_MIN = (R_T / RP) > 4 ? (R_T / RP) : 4;  // at least one row per thread
-    const int nc = g.nc;
-    R* sA = reinterpret_cast<R*>(smem_raw);  // [KP][RP]
-    R* sX = sA + KP * RP;                    // [R_TB][XS]
     __shared__ int s_src[R_TB], s_tgt[R_TB];
-    const int tid = threadIdx.x;
+    __shared__ R sC[RR_PH], sS[RR_PH];
+    const int p = g.p, nc = g.nc, nre = lf_nre(p), TS = 2 * p + 1, cb = g.cb, tid = threadIdx.x;
+    R* sXr = reinterpret_cast<R*>(smem_raw);  // [(n, m)][cb]
+    R* sXi = sXr + nre * cb;
+    R* sT = sXi + nre * cb;  // [TS][TS]
     const int4 b = g.batches[blockIdx.x];
-    const int kidx = b.x, start = b.y, cnt = b.z & 255;
+    const int start = b.y, cnt = b.z & 255;
     int c, lev, ox, oy, oz;
-    rkey_decode(g.kval[kidx], c, lev, ox, oy, oz);
-    // the key's operator: a contiguous copy in 16-byte pieces
-    {
-        const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const R*>(g.ops) +
-                                                            (size_t)kidx * KP * RP);
-        float4* dst = reinterpret_cast<float4*>(sA);
-        constexpr int NV = KP * RP * (int)sizeof(R) / 16;
-        for (int i = tid; i < NV; i += R_T) dst[i] = src[i];
-    }
-    if (tid < R_TB) {
-        if (tid < cnt) {
-            const uint32_t e = g.order[start + tid];
-            s_src[tid] = (int)(g.ent[e] & LFMM_ENT_MASK);
-            s_tgt[tid] = g.tgt[e];
-        } else {
-            s_src[tid] = -1;
-            s_tgt[tid] = -1;
-        }
-    }
-    __syncthreads();
-    // columns the tile shape below reads (block-uniform)
-    const int cgs = cnt > 32 ? 16 : (cnt > 16 ? 8 : 4);
-    const int ncol = 4 * (cgs > CG_MIN ? cgs : CG_MIN);
+    rkey_decode((uint32_t)b.z >> 8, c, lev, ox, oy, oz);
+    const bool refl = g.comps[c].refl != 0;
     const R ih = (R)(1.0 / g.levelh[lev]);
-    const int tot = ncol * KP;
-    for (int r = 0; r < g.nr; ++r) {
-        if (r > 0) __syncthreads();  // the previous vector's products are read out of sX
-        const R* M = reinterpret_cast<const R*>(g.M) + (size_t)r * g.stride;
-        // eight loads in flight per thread before their stores
-        for (int b0 = tid; b0 < tot; b0 += 8 * R_T) {
-            R v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = b0 + u * R_T;
-                v[u] = R(0);
-                if (idx < tot) {
-                    const int j = idx / KP, k = idx - j * KP;
-                    const int s = s_src[j];
-                    if (s >= 0 && k < nc) v[u] = M[(size_t)s * nc + k];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = b0 + u * R_T;
-                if (idx < tot) {
-                    const int j = idx / KP, k = idx - j * KP;
-                    sX[j * XS + k] = v[u];
-                }
-            }
-        }
-        __syncthreads();
-        R* L = reinterpret_cast<R*>(g.L) + (size_t)r * g.stride;
-        if (cgs == 16 || CG_MIN >= 16)
-            m2r_tile<R, RP, 16>(sA, sX, cnt, s_tgt, ih, L, nc);
-        else if (cgs == 8 || CG_MIN >= 8)
-            m2r_tile<R, RP, (CG_MIN > 8 ? CG_MIN : 8)>(sA, sX, cnt, s_tgt, ih, L, nc);
-        else
-            m2r_tile<R, RP, CG_MIN>(sA, sX, cnt, s_tgt, ih, L, nc);
-    }
-}
-
-// Orders 11 .. 15 ((p+1)^2 up to 256): the key's operator is too large for
-// shared memory, so it is staged in chunks of R_KC input rows while the
-// gathered multipoles stay resident; the same tile shapes as m2r_tile.
-#define R_KC 32
-
-template <typename R, int RP, int CG>
-__device__ __forceinline__ void m2r_tile_kc(const R* __restrict__ A, R* __restrict__ sA, const R* __restrict__ sX,
-                                            int cnt, const int* s_tgt, R ih, R* __restrict__ L, int nc)
-{
-    constexpr int KP = RP, XS = KP + 1;
-    constexpr int RG = R_T / CG;  // row groups
-    constexpr int RM = RP / RG;   // rows per thread
-    static_assert(RM >= 1 && RM * RG == RP, "tile shape");
-    const int tid = threadIdx.x;
-    const int cg = tid % CG, rg = tid / CG;
-    R acc[RM][4];
-#pragma unroll
-    for (int r = 0; r < RM; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] = 0;
-    for (int kc = 0; kc < KP; kc += R_KC) {
-        __syncthreads();  // the previous chunk has been read
-        {
-            const float4* src = reinterpret_cast<const float4*>(A + (size_t)kc * RP);
-            float4* dst = reinterpret_cast<float4*>(sA);
-            constexpr int NV = R_KC * RP * (int)sizeof(R) / 16;
-            for (int i = tid; i < NV; i += R_T) dst[i] = src[i];
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < R_KC; ++kk) {
-            R a[RM];
-#pragma unroll
-            for (int r = 0; r < RM; ++r) a[r] = sA[kk * RP + rg * RM + r];
-            R x[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) x[q] = sX[(4 * cg + q) * XS + kc + kk];
-#pragma unroll
-            for (int r = 0; r < RM; ++r)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[r][q] += a[r] * x[q];
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = 4 * cg + q;
-        if (j >= cnt) continue;
-        R* Lt = L + (size_t)s_tgt[j] * nc;
-#pragma unroll
-        for (int r = 0; r < RM; ++r) {
-            const int row = rg * RM + r;
-            if (row < nc) atomicAdd(Lt + row, acc[r][q] * ih);
-        }
-    }
-}
-
-template <typename R, int RP>
-__global__ void __launch_bounds__(R_T) k_m2r_gemm_kc(RGemmArgs g)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int KP = RP;
-    constexpr int XS = KP + 1;
-    const int nc = g.nc;
-    R* sA = reinterpret_cast<R*>(smem_raw);  // [R_KC][RP]
-    R* sX = sA + R_KC * RP;                  // [R_TB][XS]
-    __shared__ int s_src[R_TB], s_tgt[R_TB];
-    const int tid = threadIdx.x;
-    const int4 b = g.batches[blockIdx.x];
-    const int kidx = b.x, start = b.y, cnt = b.z & 255;
-    int c, lev, ox, oy, oz;
-    rkey_decode(g.kval[kidx], c, lev, ox, oy, oz);
-    const R* A = reinterpret_cast<const R*>(g.ops) + (size_t)kidx * KP * RP;
     if (tid < R_TB) {
-        if (tid < cnt) {
-            const uint32_t e = g.order[start + tid];
-            s_src[tid] = (int)(g.ent[e] & LFMM_ENT_MASK);
-            s_tgt[tid] = g.tgt[e];
-        } else {
-            s_src[tid] = -1;
-            s_tgt[tid] = -1;
-        }
+        const int2 pr = (tid < cnt) ? g.pairs[start + tid] : make_int2(-1, -1);
+        s_src[tid] = pr.x;
+        s_tgt[tid] = pr.y;
     }
-    __syncthreads();
-    const int cgs = cnt > 32 ? 16 : (cnt > 16 ? 8 : 4);
-    const int ncol = 4 * cgs;
-    const R ih = (R)(1.0 / g.levelh[lev]);
-    const int tot = ncol * KP;
+    if (tid >= 64 && tid < 64 + RR_PH) {
+        const double* ph = g.phase + (size_t)((ox + R_OR) * R_OW + (oy + R_OR)) * 2 * RR_PH + (tid - 64);
+        sC[tid - 64] = (R)ph[0];
+        sS[tid - 64] = (R)ph[RR_PH];
+    }
+    const double* Tk = g.tables + (size_t)b.w * TS * TS;
+    for (int j = tid; j < TS * TS; j += R_T) sT[j] = (R)Tk[j];
     for (int r = 0; r < g.nr; ++r) {
-        if (r > 0) __syncthreads();  // the previous vector's products are read out of sX
         const R* M = reinterpret_cast<const R*>(g.M) + (size_t)r * g.stride;
-        for (int b0 = tid; b0 < tot; b0 += 8 * R_T) {
-            R v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = b0 + u * R_T;
-                v[u] = R(0);
-                if (idx < tot) {
-                    const int j = idx / KP, k = idx - j * KP;
-                    const int s = s_src[j];
-                    if (s >= 0 && k < nc) v[u] = M[(size_t)s * nc + k];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int idx = b0 + u * R_T;
-                if (idx < tot) {
-                    const int j = idx / KP, k = idx - j * KP;
-                    sX[j * XS + k] = v[u];
-                }
-            }
-        }
         R* L = reinterpret_cast<R*>(g.L) + (size_t)r * g.stride;
-        if (cgs == 16)
-            m2r_tile_kc<R, RP, 16>(A, sA, sX, cnt, s_tgt, ih, L, nc);
-        else if (cgs == 8)
-            m2r_tile_kc<R, RP, 8>(A, sA, sX, cnt, s_tgt, ih, L, nc);
-        else
-            m2r_tile_kc<R, RP, 4>(A, sA, sX, cnt, s_tgt, ih, L, nc);
+        for (int q0 = 0; q0 < cnt; q0 += cb) {
+            const int nq = min(cb, cnt - q0);
+            __syncthreads();  // the tables are in shared memory; the previous chunk has been read
+            // rotated (and for reflections sign-flipped) multipoles; columns past the batch: zeros
+            for (int i = tid; i < nre * cb; i += R_T) {
+                const int j = i / nre, x = i - j * nre;  // column, (n, m)
+                R vr = R(0), vi = R(0);
+                if (j < nq) {
+                    int n, m, dummy;
+                    lf_decode(p, x, n, m, dummy);
+                    const R* Ms = M + (size_t)s_src[q0 + j] * nc;
+                    const R mr = Ms[x], mi = m > 0 ? Ms[lf_im(p, n, m)] : R(0);
+                    vr = mr * sC[m] - mi * sS[m];
+                    vi = mr * sS[m] + mi * sC[m];
+                    if (refl && ((n + m) & 1)) {
+                        vr = -vr;
+                        vi = -vi;
+                    }
+                }
+                sXr[x * cb + j] = vr;
+                sXi[x * cb + j] = vi;
+            }
+            __syncthreads();
+            // padded cost of each width: two additions and 2 C multiply-adds per (n, m)
+            const int w2 = ((nq + 1) / 2) * 6, w4 = ((nq + 3) / 4) * 10, w8 = ((nq + 7) / 8) * 18;
+            if (w8 <= w4 && w8 <= w2)
+                rr_apply<R, 8>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, sC, sS, ih, L, blockIdx.y, gridDim.y);
+            else if (w4 <= w2)
+                rr_apply<R, 4>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, sC, sS, ih, L, blockIdx.y, gridDim.y);
+            else
+                rr_apply<R, 2>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, sC, sS, ih, L, blockIdx.y, gridDim.y);
+        }
     }
 }
 
@@ -743,7 +572,7 @@ __global__ void __launch_bounds__(R_T) k_m2r_gemm_kc(RGemmArgs g)
 // Tensor-core form (float32, (p+1)^2 <= 128): one CTA per batch of up to
 // R_TB pairs of one key.  The key's operator is never stored: the CTA forms
 // it in shared memory from the key's Sommerfeld table and the lateral phases
-// (the same entries as k_m2r_ops), directly as two TF32 pieces a1 + a2 in the
+// directly as two TF32 pieces a1 + a2 in the
 // 64-byte-swizzled K-major layout of the MMA's A operand (M = 128 output
 // coefficients, K = the input coefficients in chunks of 16).  The batch's
 // source multipoles (B operand: N = the batch rounded up to 16 columns) are
@@ -1030,74 +859,39 @@ __global__ void __launch_bounds__(RT_THREADS, RT_MINB) k_m2r_tc(RTcArgs g)
                      : "memory");
 }
 
-template <typename R, int RP>
-static LfErr m2r_build_ops(lfmm_ctx* ctx, cudaStream_t st)
+template <typename R>
+static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
 {
-    const int nk = ctx->m2r_nkeys;
-    LF_TRY(lf_reserve(ctx->m2r_ops, (size_t)nk * RP * RP * sizeof(R) + 16));
-    ROpArgs g;
+    RRotArgs g;
     g.p = ctx->p;
     g.nc = lf_nc(ctx->p);
-    g.kval = ctx->m2r_kval.as<uint32_t>() + ctx->m2r_kfirst;
+    // 32 columns (16 above p = 10) keep several blocks per SM
+    g.cb = ctx->p <= 10 ? 32 : 16;
+    g.batches = ctx->m2r_batches.as<int4>();
     g.tables = ctx->m2r_tables.as<double>();
-    g.ktab = ctx->m2r_ktab.as<int>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
-    g.ops = ctx->m2r_ops.ptr;
+    if (!ctx->m2r_phase64_ready) {
+        // once per context (the first evaluation; a captured batch graph never sees it)
+        LF_TRY(lf_reserve(ctx->m2r_phase64, (size_t)R_OW * R_OW * 2 * RR_PH * sizeof(double)));
+        ++ctx->launches, k_m2r_phase64<<<R_OW * R_OW, 32, 0, st>>>(ctx->m2r_phase64.as<double>());
+        LF_TRY(lf_cuda(cudaGetLastError(), "m2r phases"));
+        ctx->m2r_phase64_ready = 1;
+    }
+    g.phase = ctx->m2r_phase64.as<double>();
+    g.pairs = ctx->m2r_pairs.as<int2>();
+    g.levelh = ctx->m2r_levelh.as<double>();
+    g.M = ctx->Mexp.ptr;
+    g.L = ctx->Lexp.ptr;
+    g.stride = (size_t)ctx->nbox_total * g.nc;
+    g.nr = ctx->nrhs_b;
     const int TS = 2 * ctx->p + 1;
-    const size_t sm = sizeof(R) * ((size_t)TS * TS + 2 * (size_t)TS) + 16;
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_ops<R, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    ++ctx->launches, k_m2r_ops<R, RP><<<nk, R_T, sm, st>>>(g);
-    LF_TRY(lf_cuda(cudaGetLastError(), "m2r operators"));
-    ctx->m2r_ops_prec = sizeof(R) == 4 ? 1 : 0;
-    return LfErr();
-}
-
-template <typename R, int RP>
-static LfErr m2r_apply_rp(lfmm_ctx* ctx, cudaStream_t st)
-{
-    if (ctx->m2r_ops_prec != (sizeof(R) == 4 ? 1 : 0)) LF_TRY((m2r_build_ops<R, RP>(ctx, st)));
-    RGemmArgs g;
-    g.p = ctx->p;
-    g.nc = lf_nc(ctx->p);
-    g.batches = ctx->m2r_batches.as<int4>();
-    g.kval = ctx->m2r_kval.as<uint32_t>() + ctx->m2r_kfirst;
-    g.ops = ctx->m2r_ops.ptr;
-    g.order = ctx->m2r_order.as<uint32_t>();
-    g.ent = ctx->m2r_ent.as<uint32_t>();
-    g.tgt = ctx->m2r_tgt.as<int>();
-    g.levelh = ctx->m2r_levelh.as<double>();
-    g.M = ctx->Mexp.ptr;
-    g.L = ctx->Lexp.ptr;
-    g.stride = (size_t)ctx->nbox_total * g.nc;
-    g.nr = ctx->nrhs_b;
-    const size_t sm = sizeof(R) * ((size_t)RP * RP + (size_t)R_TB * (RP + 1)) + 16;
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_gemm<R, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    ++ctx->launches, k_m2r_gemm<R, RP><<<ctx->m2r_nbatch, R_T, sm, st>>>(g);
-    return lf_cuda(cudaGetLastError(), "m2r gemm");
-}
-
-template <typename R, int RP>
-static LfErr m2r_apply_kc(lfmm_ctx* ctx, cudaStream_t st)
-{
-    if (ctx->m2r_ops_prec != (sizeof(R) == 4 ? 1 : 0)) LF_TRY((m2r_build_ops<R, RP>(ctx, st)));
-    RGemmArgs g;
-    g.p = ctx->p;
-    g.nc = lf_nc(ctx->p);
-    g.batches = ctx->m2r_batches.as<int4>();
-    g.kval = ctx->m2r_kval.as<uint32_t>() + ctx->m2r_kfirst;
-    g.ops = ctx->m2r_ops.ptr;
-    g.order = ctx->m2r_order.as<uint32_t>();
-    g.ent = ctx->m2r_ent.as<uint32_t>();
-    g.tgt = ctx->m2r_tgt.as<int>();
-    g.levelh = ctx->m2r_levelh.as<double>();
-    g.M = ctx->Mexp.ptr;
-    g.L = ctx->Lexp.ptr;
-    g.stride = (size_t)ctx->nbox_total * g.nc;
-    g.nr = ctx->nrhs_b;
-    const size_t sm = sizeof(R) * ((size_t)R_KC * RP + (size_t)R_TB * (RP + 1)) + 16;
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_gemm_kc<R, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    ++ctx->launches, k_m2r_gemm_kc<R, RP><<<ctx->m2r_nbatch, R_T, sm, st>>>(g);
-    return lf_cuda(cudaGetLastError(), "m2r gemm (operator chunks)");
+    const size_t sm = sizeof(R) * ((size_t)2 * lf_nre(ctx->p) * g.cb + (size_t)TS * TS);
+    // few batches (small trees): share the rows of each between blocks
+    int parts = 1;
+    while (parts < 8 && (int64_t)ctx->m2r_nbatch * parts < 8 * 152) parts *= 2;
+    LF_CHECK(cudaFuncSetAttribute(k_m2r_rot<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ++ctx->launches, k_m2r_rot<R><<<dim3(ctx->m2r_nbatch, parts), R_T, sm, st>>>(g);
+    return lf_cuda(cudaGetLastError(), "m2r rotated");
 }
 
 // the float32 form with (p+1)^2 <= 128 applies the keys on the tensor cores
@@ -1133,38 +927,9 @@ static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
     return lf_cuda(cudaGetLastError(), "m2r tensor-core GEMM");
 }
 
-template <typename R>
-static LfErr m2r_apply_t(lfmm_ctx* ctx, cudaStream_t st)
-{
-    if (sizeof(R) == 4 && m2r_tc_on(ctx)) return m2r_apply_tc(ctx, st);
-    switch (ctx->m2l_rm) {
-    case 2: return m2r_apply_rp<R, 32>(ctx, st);
-    case 4: return m2r_apply_rp<R, 64>(ctx, st);
-    case 8: return m2r_apply_rp<R, 128>(ctx, st);
-    case 12: return m2r_apply_kc<R, 192>(ctx, st);
-    case 16: return m2r_apply_kc<R, 256>(ctx, st);
-    default: return "internal: reaction GEMM supports p <= 15";
-    }
-}
-
-// assemble the operators of the keys for the current precision (build time)
-LfErr lf_m2r_ops(lfmm_ctx* ctx, cudaStream_t st)
-{
-    // the tensor-core form assembles each operator where it is applied; the
-    // CUDA-core GEMM builds them on first use if the option changes later
-    if (ctx->m2r_nbatch == 0 || m2r_tc_on(ctx)) return LfErr();
-    switch (ctx->m2l_rm) {
-    case 2: return ctx->precision ? m2r_build_ops<float, 32>(ctx, st) : m2r_build_ops<double, 32>(ctx, st);
-    case 4: return ctx->precision ? m2r_build_ops<float, 64>(ctx, st) : m2r_build_ops<double, 64>(ctx, st);
-    case 8: return ctx->precision ? m2r_build_ops<float, 128>(ctx, st) : m2r_build_ops<double, 128>(ctx, st);
-    case 12: return ctx->precision ? m2r_build_ops<float, 192>(ctx, st) : m2r_build_ops<double, 192>(ctx, st);
-    case 16: return ctx->precision ? m2r_build_ops<float, 256>(ctx, st) : m2r_build_ops<double, 256>(ctx, st);
-    default: return "internal: reaction GEMM supports p <= 15";
-    }
-}
-
 LfErr lf_m2r_apply(lfmm_ctx* ctx, cudaStream_t st)
 {
     if (ctx->m2r_nbatch == 0) return LfErr();
-    return ctx->precision ? m2r_apply_t<float>(ctx, st) : m2r_apply_t<double>(ctx, st);
+    if (m2r_tc_on(ctx)) return m2r_apply_tc(ctx, st);
+    return ctx->precision ? m2r_apply_rot<float>(ctx, st) : m2r_apply_rot<double>(ctx, st);
 }
