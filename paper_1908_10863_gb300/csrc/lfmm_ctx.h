@@ -149,6 +149,10 @@ struct lfmm_ctx {
     double m2l_levelh_h[16] = {0};
     // use_tc: 2 automatic and 1: tensor cores, 0: CUDA cores
     int m2l_tc_ok = 0, m2l_tc_ntiles = 0, use_tc = 2, tc_groups = 0;  // tc_groups 0: automatic
+    // FP64 free M2L by digit products (lfmm_m2l_oz.cu)
+    DevBuf oz_A, oz_Ms, oz_cscale, oz_tiles, oz_mseg;
+    std::vector<int4> oz_tiles_h, oz_mseg_h;
+    int oz_ntiles = 0, oz_ready = 0;
     int m2l_tc_wide = 0;  // tensor-core free M2L in its wide form ((p+1)^2 > 128): no tensor-core M2M / L2L
     // reaction M2L grouped by geometry key on interface-aligned levels
     DevBuf m2r_keys, m2r_order, m2r_tgt, m2r_kstart, m2r_kval, m2r_tables, m2r_levelh, m2r_batches;
@@ -286,11 +290,16 @@ LfErr lf_shift_gemm(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st);
 // ... and of the largest scaled coefficient (float bits) per right-hand side:
 // multipoles of each level at [0, 16), locals at [16, 32)
 #define LFMM_TCMAX_OFF 45056
+#define LFMM_OZ_BAD_OFF 40976  // in ctx->counts: operator entries out of the digit range (set-up)
+#define LFMM_OZ_TILE 64        // targets per tile of the FP64 digit-product M2L
 #define LFMM_TC_MSEG 16  // runs per merged tensor-core M2L tile (one leftover run per level and class)
 LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP);
 LfErr lf_l2l_tc(lfmm_ctx* ctx, int level, cudaStream_t st);
 LfErr lf_wait_probe(lfmm_ctx* ctx, double limit_ms, int* timed_out);
 LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st);
+// ---- FP64 free M2L by digit products (lfmm_m2l_oz.cu) ----
+bool lf_m2l_oz_ok(const lfmm_ctx* ctx);
+LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st);
 int lf_m2l_tc_tile(const lfmm_ctx* ctx);
 LfErr lf_surrogate_alloc(lfmm_ctx* ctx);
 LfErr lf_surrogate_pack(lfmm_ctx* ctx, int comp);

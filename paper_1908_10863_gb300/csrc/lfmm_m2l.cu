@@ -13,6 +13,9 @@
 // its tile in registers and, for each of the 189 offsets, gathers the 64
 // source multipoles (zero where a target has no source at that offset) and
 // multiplies them by A_o: 189 register-tiled GEMMs of (p+1)^2 x (p+1)^2 x 64.
+// This CUDA-core GEMM serves the float32 form on request; by default the
+// float32 form runs in lfmm_m2l_tc.cu and the FP64 form in lfmm_m2l_oz.cu,
+// over the tiles and slots set up here.
 //
 // The same gathered GEMM runs the translations between levels: M2M (eq.
 // metome) with the 8 child-octant maps (each parent gathers its children,
@@ -453,6 +456,20 @@ LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
         LF_CHECK(cudaMemcpyAsync(ctx->m2l_tiles.ptr, tiles.data(), tiles.size() * sizeof(int4),
                                  cudaMemcpyHostToDevice, st));
     }
+    // merged tiles of the same runs for the FP64 digit-product kernel
+    ctx->oz_ntiles = 0;
+    if (lf_m2l_oz_ok(ctx)) {
+        m2l_tc_tiles(hcnt, depth, LFMM_OZ_TILE, ctx->oz_tiles_h, ctx->oz_mseg_h);
+        ctx->oz_ntiles = (int)ctx->oz_tiles_h.size();
+        LF_TRY(lf_reserve(ctx->oz_tiles, ctx->oz_tiles_h.size() * sizeof(int4) + 16));
+        LF_TRY(lf_reserve(ctx->oz_mseg, ctx->oz_mseg_h.size() * sizeof(int4) + 16));
+        if (!ctx->oz_tiles_h.empty())
+            LF_CHECK(cudaMemcpyAsync(ctx->oz_tiles.ptr, ctx->oz_tiles_h.data(), ctx->oz_tiles_h.size() * sizeof(int4),
+                                     cudaMemcpyHostToDevice, st));
+        if (!ctx->oz_mseg_h.empty())
+            LF_CHECK(cudaMemcpyAsync(ctx->oz_mseg.ptr, ctx->oz_mseg_h.data(), ctx->oz_mseg_h.size() * sizeof(int4),
+                                     cudaMemcpyHostToDevice, st));
+    }
     // wider tiles of the same (level, class) runs for the tensor-core kernel
     std::vector<int4>& tct = ctx->tc_tiles_h;
     tct.clear();
@@ -781,5 +798,5 @@ LfErr lf_shift_gemm(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st)
 LfErr lf_m2l_gemm(lfmm_ctx* ctx, cudaStream_t st)
 {
     if (ctx->m2l_ntiles == 0) return LfErr();
-    return ctx->precision ? m2l_gemm_t<float>(ctx, st) : m2l_gemm_t<double>(ctx, st);
+    return ctx->precision ? m2l_gemm_t<float>(ctx, st) : lf_m2l_oz(ctx, st);
 }
