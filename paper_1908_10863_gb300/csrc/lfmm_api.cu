@@ -958,7 +958,7 @@ static lfmm_status set_option(lfmm_ctx* ctx, int opt, double v)
 // tables are built here once per context, outside any evaluation.
 static LfErr auto_near_tables(lfmm_ctx* ctx)
 {
-    if (ctx->use_near_tab != 2 || ctx->precision != 1 || ctx->img_ok || !ctx->built ||
+    if (ctx->use_near_tab != 2 || ctx->precision != 1 || lf_img32_on(ctx) || !ctx->built ||
         ctx->near_reaction_entries == 0 || ctx->near_tab_ready)
         return LfErr();
     return lf_near_tables(ctx, nullptr);

@@ -244,6 +244,16 @@ LfErr lf_p2p_pair_stats(lfmm_ctx* ctx);
 // 3.1e-7 against 3.2e-7 at N = 65,536, p = 14, in an eighth of the time)
 inline bool lf_tc_on(const lfmm_ctx* ctx) { return ctx->m2l_tc_ok && ctx->use_tc != 0; }
 
+// whether the float32 near field takes its reaction remainders from the image
+// rule: unless the tables are asked for, and while the rule is short.  A pair
+// costs ~9 instructions per image against 16 gathered loads and ~100
+// instructions of the tables.
+#define LFMM_IMG32_MAX 20
+inline bool lf_img32_on(const lfmm_ctx* ctx)
+{
+    return ctx->img_ok && ctx->use_near_tab != 1 && (ctx->img32.n <= LFMM_IMG32_MAX || ctx->use_near_tab == 0);
+}
+
 // ---- free-space M2L GEMM (lfmm_m2l.cu) ----
 LfErr lf_setup_m2l_ops(lfmm_ctx* ctx);
 LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st);
@@ -296,6 +306,7 @@ LfErr lf_shift_gemm(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st);
 LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP);
 LfErr lf_l2l_tc(lfmm_ctx* ctx, int level, cudaStream_t st);
 LfErr lf_wait_probe(lfmm_ctx* ctx, double limit_ms, int* timed_out);
+LfErr lf_tc_split(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st);
 // ---- FP64 free M2L by digit products (lfmm_m2l_oz.cu) ----
 bool lf_m2l_oz_ok(const lfmm_ctx* ctx);

@@ -475,11 +475,13 @@ __global__ void __launch_bounds__(128) k_l2p(int64_t n, int p, const int* __rest
 // ---------------------------------------------------------------------------
 template <typename R>
 __global__ void k_gather_q(const double* __restrict__ q, const int32_t* __restrict__ perm, int64_t n,
-                           R* __restrict__ qs)
+                           R* __restrict__ qs, unsigned* __restrict__ gmax)
 {
-    // blockIdx.y: right-hand side (vectors of n, caller order in, sorted order out)
+    // blockIdx.y: right-hand side (vectors of n, caller order in, sorted order out);
+    // gmax: the pass's largest-coefficient slots (LFMM_TCMAX_OFF), 32 words each, start at zero
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t r = blockIdx.y;
+    if (i < 32) gmax[r * 32 + i] = 0u;
     if (i < n) qs[r * n + i] = (R)q[r * n + perm[i]];
 }
 
@@ -580,9 +582,12 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
     const int lth = ((nre + 31) / 32) * 32;
     LF_CHECK(cudaMemsetAsync(L, 0, sizeof(R) * ms * nr, st));
     const bool gemm = ctx->m2l_ntiles > 0;
+    const bool tc = sizeof(R) == 4 && lf_tc_on(ctx);
+    if (tc && !(gemm && ctx->m2l_tc_ntiles > 0) && ctx->m2r_nbatch > 0) LF_TRY(lf_tc_split(ctx, st));
     if (gemm) {
         ph = lf_prof_start(ctx, LFMM_TIME_M2L_FREE, st);
-        if (sizeof(R) == 4 && lf_tc_on(ctx) && ctx->m2l_tc_ntiles > 0)
+        if (tc && ctx->m2l_tc_ntiles > 0) LF_TRY(lf_tc_split(ctx, st));
+        if (tc && ctx->m2l_tc_ntiles > 0)
             LF_TRY(lf_m2l_tc(ctx, st));
         else
             LF_TRY(lf_m2l_gemm(ctx, st));
@@ -684,11 +689,13 @@ LfErr lf_evaluate_sorted(lfmm_ctx* ctx, int nrhs, const double* q_dev, double* p
     LF_TRY(lf_reserve(ctx->fld_near, (size_t)n * 24 * nr));
     const int ptot = lf_prof_start(ctx, LFMM_TIME_TOTAL, st);
     const dim3 g1(lf_blocks(n, 256), (unsigned)nrhs);
+    unsigned* gmax = reinterpret_cast<unsigned*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
     if (ctx->precision)
-        ++ctx->launches, k_gather_q<float><<<g1, 256, 0, st>>>(q_dev, ctx->perm.as<int32_t>(), n, ctx->q_sorted.as<float>());
+        ++ctx->launches, k_gather_q<float><<<g1, 256, 0, st>>>(q_dev, ctx->perm.as<int32_t>(), n,
+                                                              ctx->q_sorted.as<float>(), gmax);
     else
         ++ctx->launches, k_gather_q<double><<<g1, 256, 0, st>>>(q_dev, ctx->perm.as<int32_t>(), n,
-                                                               ctx->q_sorted.as<double>());
+                                                               ctx->q_sorted.as<double>(), gmax);
     LF_TRY(lf_cuda(cudaGetLastError(), "gather q"));
     // the reaction M2L's tables of a fresh build: on the
     // near-field stream ahead of the near field, beside the far field's

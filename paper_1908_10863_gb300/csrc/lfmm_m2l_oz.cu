@@ -387,29 +387,35 @@ __device__ __forceinline__ int oz_level(const OzLevels& lv, int b)
     return l;
 }
 
-// largest scaled multipole |M_k| 2^{e_k} of each level, as double bits; one
-// warp per eight boxes
+// largest scaled multipole |M_k| 2^{e_k} of each level, as double bits in
+// gmax[16 rhs + level] (zeroed when the charges were sorted); one block per 32
+// boxes, met in shared memory
 __global__ void __launch_bounds__(256) k_oz_max(const double* __restrict__ M, int nbox, int nc,
                                                 const double* __restrict__ cs, const __grid_constant__ OzLevels lv,
                                                 unsigned long long* __restrict__ gmax)
 {
+    __shared__ unsigned long long s_max[16];
+    if (threadIdx.x < 16) s_max[threadIdx.x] = 0ull;
+    __syncthreads();
     M += (size_t)blockIdx.y * nbox * nc;
-    const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const int last = min(8 * w + 8, nbox);
-    for (int b = 8 * w; b < last;) {
-        const int l = oz_level(lv, b);
+    const int lane = threadIdx.x & 31, i0 = blockIdx.x * 32 + (threadIdx.x >> 5) * 4;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int b = i0 + u;
+        if (b >= nbox) break;
         unsigned long long m = 0;
-        for (; b < last && (l == 0 || b < lv.off[l - 1]); ++b)
-            for (int k = lane; k < nc; k += 32) {
-                const unsigned long long v =
-                    (unsigned long long)__double_as_longlong(fabs(M[(size_t)b * nc + k] * cs[k]));
-                m = v > m ? v : m;
-            }
+        for (int k = lane; k < nc; k += 32) {
+            const unsigned long long v = (unsigned long long)__double_as_longlong(fabs(M[(size_t)b * nc + k] * cs[k]));
+            m = v > m ? v : m;
+        }
         const unsigned h = __reduce_max_sync(0xffffffffu, (unsigned)(m >> 32));
         const unsigned lw = __reduce_max_sync(0xffffffffu, (unsigned)(m >> 32) == h ? (unsigned)m : 0u);
-        m = ((unsigned long long)h << 32) | lw;
-        unsigned long long* g = gmax + (size_t)blockIdx.y * 16 + l;
-        if (lane == 0 && m > *(volatile unsigned long long*)g) atomicMax(g, m);
+        if (lane == 0) atomicMax(&s_max[oz_level(lv, b)], ((unsigned long long)h << 32) | lw);
+    }
+    __syncthreads();
+    if (threadIdx.x < 16 && s_max[threadIdx.x] != 0ull) {
+        unsigned long long* g = gmax + (size_t)blockIdx.y * 16 + threadIdx.x;
+        if (s_max[threadIdx.x] > *(volatile unsigned long long*)g) atomicMax(g, s_max[threadIdx.x]);
     }
 }
 
@@ -487,9 +493,8 @@ LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st)
     OzLevels lv;
     lv.depth = ctx->depth;
     for (int l = 0; l < 17; ++l) lv.off[l] = l <= ctx->depth ? ctx->levels[l].off : 0;
-    LF_CHECK(cudaMemsetAsync(gm, 0, (size_t)nr * 16 * sizeof(unsigned long long), st));
     const double* M = ctx->Mexp.as<double>();
-    ++ctx->launches, k_oz_max<<<dim3((nb + 63) / 64, nr), 256, 0, st>>>(M, nb, nc, ctx->oz_cscale.as<double>(), lv, gm);
+    ++ctx->launches, k_oz_max<<<dim3((nb + 31) / 32, nr), 256, 0, st>>>(M, nb, nc, ctx->oz_cscale.as<double>(), lv, gm);
     const int64_t tot = (int64_t)nb * (g.mrow / 2);
     ++ctx->launches, k_oz_split<<<dim3((unsigned)((tot + 255) / 256), nr), 256, 0, st>>>(
         M, nb, nc, g.mrow, ctx->oz_cscale.as<double>(), lv, gm, ctx->oz_Ms.as<__half>());

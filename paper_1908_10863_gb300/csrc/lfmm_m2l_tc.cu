@@ -144,16 +144,6 @@ struct TcArgs {
     int* err;               // [0]: timeouts
 };
 
-// The power of two that takes the largest magnitude (float bits) into
-// [2^13, 2^14); 1 for zero or non-finite values.
-__device__ __forceinline__ float tc_scale(unsigned maxbits)
-{
-    if (maxbits == 0u || maxbits >= 0x7f800000u) return 1.f;
-    int e = 140 - (int)(maxbits >> 23);  // 13 - (biased exponent - 127)
-    e = e > 126 ? 126 : (e < -126 ? -126 : e);
-    return __uint_as_float((unsigned)(e + 127) << 23);
-}
-
 // Target t of a tile (a box id, or -1 past the tile's count) and its output
 // scale (1 for M2M and L2L, 1/h of the target's level for M2L).  A tile with
 // level < 0 is a merged tile: the leftover runs (fewer targets than a tile)
@@ -217,6 +207,8 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
     __shared__ int s_tb[TC_N];
     __shared__ float s_ih[TC_N];  // output scale of each target column
     __shared__ int s_src[TC_SRC][TN];
+    __shared__ unsigned s_mask;     // offsets with a source (groups of at most TC_SRC offsets)
+    __shared__ int s_act[TC_SRC];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int item = blockIdx.x;
@@ -226,20 +218,37 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
     const int cl = tile.y, cnt = tile.w;
     const int nc = g.nc;
     const int nkc = g.nkc;  // K chunks that hold coefficients (the rest are zero)
-    const int nstage = goff * nkc;
+    const bool listed = goff <= TC_SRC;
 
+    if (tid == 0) s_mask = 0u;
+    __syncthreads();
     if (tid < TN) {
         float ih;
         const int tb = tc_tile_target(g, tile, tid, ih);
         s_tb[tid] = tb;
         s_ih[tid] = ih;
-        if (goff <= TC_SRC) {
+        if (listed) {
             const int* src = g.slots + (size_t)(tb >= 0 ? tb : 0) * g.noff + grp * goff;
+            unsigned any = 0;
 #pragma unroll
             for (int o = 0; o < TC_SRC; ++o)
-                if (o < goff) s_src[o][tid] = tb >= 0 ? src[o] : -1;
+                if (o < goff) {
+                    const int s = tb >= 0 ? src[o] : -1;
+                    s_src[o][tid] = s;
+                    any |= s >= 0 ? 1u << o : 0u;
+                }
+            any = __reduce_or_sync(0xffffffffu, any);
+            if (lane == 0 && any) atomicOr(&s_mask, any);
         }
     }
+    __syncthreads();
+    // offsets at which some target of the tile has a source; the others (thin
+    // layers, small trees) are skipped
+    const unsigned mask = s_mask;
+    const int nact = listed ? __popc(mask) : goff;
+    if (nact == 0) return;  // block-uniform, before anything is allocated
+    if (listed && tid < goff && ((mask >> tid) & 1u)) s_act[__popc(mask & ((1u << tid) - 1u))] = tid;
+    const int nstage = nact * nkc;
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             mbar_init(&full_bar[s], TC_PROD_WARPS + 1);  // one arrival per producer warp + the bulk copy's
@@ -265,16 +274,17 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
         // stage it is filled at iteration it and handed to the tensor cores at
         // iteration it + TC_LAG, once its copies have landed
         const int ptid = tid;  // 0 .. 255
-        const int rot = (item / g.groups) % goff;
+        const int rot = (item / g.groups) % nact;
         int armed = 0;         // stages with a bulk copy issued by this thread, for the bounded drain
         const int my_row = (WIDE ? (warp & 3) : warp) * 32 + lane;
         const int* my_slots = g.slots + (size_t)max(s_tb[my_row], 0) * g.noff + grp * goff;
         int it = 0;
         for (; it < nstage; ++it) {
             const int s = it % NST, round = it / NST;
-            const int ol = (it + rot) % goff, oi = grp * goff + ol, kc = nkc - 1 - it / goff;
+            const int oa = (it + rot) % nact, ol = listed ? s_act[oa] : oa;
+            const int oi = grp * goff + ol, kc = nkc - 1 - it / nact;
             // source of this thread's row at the stage's offset
-            const int my_src = goff <= TC_SRC ? s_src[ol][my_row] : (s_tb[my_row] >= 0 ? my_slots[ol] : -1);
+            const int my_src = listed ? s_src[ol][my_row] : (s_tb[my_row] >= 0 ? my_slots[ol] : -1);
             if (it >= NST) {
                 if (!mbar_wait(&empty_bar[s], (round - 1) & 1)) atomicExch(&s_abort, 1);
             }
@@ -375,7 +385,7 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
                 // the small products first: a2 x1, a1 x2, a1 x1
                 const int pa[3] = {1, 0, 0}, px[3] = {0, 1, 0};
                 // K steps of 16 that hold coefficients (both but in an operator's last chunk)
-                const int nks = (nc - (nkc - 1 - it / goff) * TH_KC) > 16 ? 2 : 1;
+                const int nks = (nc - (nkc - 1 - it / nact) * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
                 for (int prod = 0; prod < 3; ++prod) {
                     const uint32_t a = base + pa[prod] * ABYTES;
@@ -767,27 +777,39 @@ __device__ __forceinline__ int tc_level(const TcLevels& lv, int b)
 }
 
 // largest scaled magnitude |X_k| 2^{+-e_k} of the boxes b0 .. b0 + count - 1,
-// per level, as float bits in gmax[32 rhs + slot0 + level]; one warp per eight
-// boxes.  Reads the expansions just written (L2): 70,848 boxes of 121 floats
-// take about as long as the launch.
+// per level, as float bits in gmax[32 rhs + slot0 + level] (zeroed when the
+// charges were sorted); one warp per box, the block's boxes met in shared
+// memory (one global atomic per box, or eight boxes per warp one after the
+// other, took 10 to 15 us on any tree).
 __global__ void __launch_bounds__(256) k_tc_max(const float* __restrict__ X, int nbox, int nc, int b0, int count,
-                                                const float* __restrict__ cs, int inv, const __grid_constant__ TcLevels lv, int slot0,
+                                                const float* __restrict__ cs, int inv,
+                                                const __grid_constant__ TcLevels lv, int slot0,
                                                 unsigned* __restrict__ gmax)
 {
-    __shared__ float s_cs[256];
-    for (int k = threadIdx.x; k < nc; k += 256) s_cs[k] = inv ? 1.f / cs[k] : cs[k];
+    __shared__ unsigned s_max[8];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 8 + w;
+    unsigned m = 0u;
+    if (i < count) {
+        const float* Xb = X + ((size_t)blockIdx.y * nbox + b0 + i) * nc;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int k = lane + 32 * q;
+            if (k < nc) {
+                const float c = cs[k];
+                m = max(m, __float_as_uint(fabsf(Xb[k] * (inv ? 1.f / c : c))));
+            }
+        }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) s_max[w] = m;
     __syncthreads();
-    X += (size_t)blockIdx.y * nbox * nc;
-    const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const int first = b0 + 8 * w, last = min(first + 8, b0 + count);
-    for (int b = first; b < last;) {
-        const int l = tc_level(lv, b);
-        unsigned m = 0;
-        for (; b < last && (l == 0 || b < lv.off[l - 1]); ++b)
-            for (int k = lane; k < nc; k += 32) m = max(m, __float_as_uint(fabsf(X[(size_t)b * nc + k] * s_cs[k])));
-        m = __reduce_max_sync(0xffffffffu, m);
+    // the first warp of each level in the block takes the level's maximum on
+    if (lane == 0 && i < count) {
+        const int l = tc_level(lv, b0 + i);
+        if (w > 0 && tc_level(lv, b0 + i - 1) == l) return;
+        for (int v = w + 1; v < 8 && i + v - w < count && tc_level(lv, b0 + i + v - w) == l; ++v) m = max(m, s_max[v]);
         unsigned* g = gmax + (size_t)blockIdx.y * 32 + slot0 + l;
-        if (lane == 0 && m > *(volatile unsigned*)g) atomicMax(g, m);
+        if (m > *(volatile unsigned*)g) atomicMax(g, m);
     }
 }
 
@@ -840,8 +862,7 @@ static LfErr split_boxes(lfmm_ctx* ctx, const float* src, int b0, int count, int
     lv.depth = ctx->depth;
     for (int l = 0; l < 17; ++l) lv.off[l] = l <= ctx->depth ? ctx->levels[l].off : 0;
     unsigned* gm = tc_gmax(ctx);
-    if (!locals) LF_CHECK(cudaMemsetAsync(gm, 0, (size_t)nr * 32 * sizeof(unsigned), st));
-    ++ctx->launches, k_tc_max<<<dim3((count + 63) / 64, nr), 256, 0, st>>>(
+    ++ctx->launches, k_tc_max<<<dim3((count + 7) / 8, nr), 256, 0, st>>>(
         src, nb, nc, b0, count, ctx->tc_cscale.as<float>(), locals, lv, 16 * locals, gm);
     const int64_t tot = (int64_t)count * (mrow / 8);
     ++ctx->launches, k_split_m<<<dim3((unsigned)((tot + 255) / 256), nr), 256, 0, st>>>(
@@ -867,12 +888,17 @@ static TcArgs tc_args(lfmm_ctx* ctx)
     return g;
 }
 
+// the multipoles of every box as float16 pieces, for the free M2L and the
+// keyed reaction M2L of this evaluation
+LfErr lf_tc_split(lfmm_ctx* ctx, cudaStream_t st)
+{
+    return split_boxes(ctx, ctx->Mexp.as<float>(), 0, ctx->nbox_total, 0, st);
+}
+
 LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st)
 {
     if (ctx->m2l_tc_ntiles == 0) return LfErr();
-    const int nb = ctx->nbox_total;
     const int nr = ctx->nrhs_b;
-    LF_TRY(split_boxes(ctx, ctx->Mexp.as<float>(), 0, nb, 0, st));
     TcArgs g = tc_args(ctx);
     g.gslot = 0;
     g.unscale = 1.f / (float)(1 << TC_ASHIFT);

@@ -14,6 +14,7 @@
 // The float32 form with p <= 10 applies the keys on the tensor cores
 // (k_m2r_tc), every other case in the rotated frame (k_m2r_rot).  A level with
 // an entry outside the key range, and the coarser ones, keep the per-pair kernel.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -571,58 +572,62 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 // ---------------------------------------------------------------------------
 // Tensor-core form (float32, (p+1)^2 <= 128): one CTA per batch of up to
 // R_TB pairs of one key.  The key's operator is never stored: the CTA forms
-// it in shared memory from the key's Sommerfeld table and the lateral phases
-// directly as two TF32 pieces a1 + a2 in the
-// 64-byte-swizzled K-major layout of the MMA's A operand (M = 128 output
-// coefficients, K = the input coefficients in chunks of 16).  The batch's
-// source multipoles (B operand: N = the batch rounded up to 16 columns) are
-// loaded into registers up front and split the same way.  K runs in rounds
-// of RT_KQ chunks through two buffers: while the tensor cores take one round
-// (3xTF32: a1 x1 + a1 x2 + a2 x1, issued by one thread into one accumulator
-// of 64 tensor-memory columns), the threads form the next.  The operator
-// entries come from a table of the reaction coefficient extended to negative
-// orders, so each is two shared-memory loads and a fused multiply-add with
-// signs and offsets precomputed per output row and input coefficient.  Each
-// batch carries its key and table index, so one dependent load reaches the
-// table, the phases and the batch's (source, target) pairs.  With 61 KB of
-// shared memory the kernel shares its SMs with the near field that runs
-// beside it.  The eight warps then read the accumulator back (warp w:
-// lanes 32 (w mod 4) .., columns 32 (w / 4) ..), scale it by 1/h and add it
-// into the targets' local expansions.  Several right-hand sides repeat the
-// rounds per vector.  Every wait is bounded: on a timeout the CTA counts it
-// in err and skips its read-backs.
+// it in shared memory from the key's Sommerfeld table and the lateral phases,
+// directly as two float16 pieces a1 + a2 in the 64-byte-swizzled K-major layout
+// of the MMA's A operand (M = 128 output coefficients, K = the input
+// coefficients by falling degree in chunks of 32), scaled like the free M2L's
+// operators (lfmm_m2l_tc.cu: 2^{-e} per coefficient, folded into the signs
+// below).  The source multipoles (B operand) are the scaled float16 pieces
+// which that M2L split once per evaluation, gathered by 16-byte cp.async;
+// products a2 x1 + a1 x2 + a1 x1.  Operator entries come from a table of the
+// reaction coefficient extended to negative orders, so each is two
+// shared-memory loads and a fused multiply-add with signs and offsets
+// precomputed per output row and input coefficient; forming them bounds the
+// kernel.  While the tensor cores take one chunk the threads form the next.
+//   V = 1: one vector, A and X of a chunk in two buffers (48 KB), three CTAs
+// per SM, which leaves room for the near field beside it.
+//   V = 2: several vectors; the whole operator (64 KB) is formed once and kept,
+// and the vectors stream past it two at a time, two CTAs per SM.
+// The eight warps read the accumulator back (warp w: lanes 32 (w mod 4) ..,
+// every second 32-column block), scale it by 1/h and the inverse operand
+// scales and add it into the targets' local expansions.  Every wait is
+// bounded: on a timeout the CTA counts it in err and skips its read-backs.
+// Measured, p = 10, float16 pieces against TF32 pieces with the operator formed
+// again for every vector: 64 vectors of 262,144 charges 13.8 -> 4.95 ms; one
+// vector 0.258 -> 0.250 ms (operator formation).
 // ---------------------------------------------------------------------------
 #define RT_THREADS 256
 #define RT_TS 21                        // table side 2p + 1 for p <= 10
 #define RT_WS 41                        // 4p + 1: orders -2p .. 2p
-// one K chunk per round and three CTAs per SM (61 KB of shared memory, 64
-// registers each) measured 0.26 ms at N = 1M, p = 10, against 0.31 ms for
-// rounds of two chunks at two CTAs per SM
-#ifndef RT_KQ
-#define RT_KQ 1                         // K chunks per round
-#endif
-#ifndef RT_MINB
-#define RT_MINB 3                       // resident CTAs per SM
-#endif
+#define RT_NKC 4                        // K chunks at most
 #define RT_A_CHUNK (128 * TC_ROWB)      // one K chunk of one operator piece: 128 rows x 64 B
-#define RT_X_CHUNK (R_TB * TC_ROWB)     // one K chunk of one multipole piece: 64 rows x 64 B
-#define RT_A_ROUND (RT_KQ * RT_A_CHUNK)
-#define RT_X_ROUND (RT_KQ * RT_X_CHUNK)
-#define RT_BUF (2 * RT_A_ROUND + 2 * RT_X_ROUND)  // a1, a2, x1, x2 of one round
-#define RT_SMEM (2 * RT_BUF + 512)
-#define RT_TMEM_COLS 64
+#define RT_X_CHUNK (R_TB * TC_ROWB)     // one K chunk of one multipole piece and vector: 64 rows x 64 B
+#define RT_ASHIFT 8                     // operators carry 2^8: entries (reflections and image sums included) stay
+                                        // far inside float16's range
+template <int V>
+struct RtShape {
+    static constexpr bool KEEP = V > 1;                        // operator kept for all vectors
+    static constexpr int NA = KEEP ? RT_NKC : 2;               // operator chunks in shared memory
+    static constexpr int XB = 2 * V * RT_X_CHUNK;              // multipole bytes of a chunk: two pieces
+    static constexpr int SMEM = NA * 2 * RT_A_CHUNK + 2 * XB + 512;
+    static constexpr int MINB = KEEP ? 2 : 3;                  // resident CTAs per SM
+    static constexpr uint32_t COLS = 64 * V;                   // tensor-memory columns
+};
 
 struct RTcArgs {
-    int p, nc, nkc;         // order, coefficients, K chunks of 16 that hold them
+    int p, nc, nkc;         // order, coefficients, K chunks of 32 that hold them
     const int4* batches;    // key index, first sorted entry, count | key << 8, table
     const double* tables;   // [table][TS][TS]
     const LfmmComp* comps;
     const float* phase;     // [225 lateral offsets][cos | sin][RT_TS] (k_m2r_phase)
     const int2* pairs;      // (source box, target box) per sorted entry (k_m2r_pairs)
     const double* levelh;
-    const float* M;
+    const __half* Ms;       // split multipoles [box][2 pieces][128]
+    const float* cscale;    // 2^e per packed coefficient
+    const int* perm;        // packed index of each K position
+    const unsigned* gmax;   // largest scaled multipole per level (float bits), [32] per right-hand side
     float* L;
-    size_t stride;          // expansions per right-hand side, in floats
+    size_t ms_stride, stride;  // per right-hand side: halves of Ms, floats of L
     int nr;
     int* err;               // [0]: timeouts
 };
@@ -641,58 +646,70 @@ __global__ void k_m2r_phase(int p, float* out)
     out[(size_t)b * 2 * RT_TS + RT_TS + m] = (float)sn;
 }
 
-__global__ void __launch_bounds__(RT_THREADS, RT_MINB) k_m2r_tc(RTcArgs g)
+template <int V>
+__global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs g)
 {
+    typedef RtShape<V> S;
     extern __shared__ unsigned char smem_raw[];
     // 512-byte alignment: the period of the 64-byte swizzle
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 511) &
                                                          ~(uintptr_t)511);
+    unsigned char* smx = sm + S::NA * 2 * RT_A_CHUNK;
     // W(N, mu) = T(N, |mu|) e^{i mu phi} for mu in [-2p, 2p], extended to
     // negative orders by W(N, -mu) = (-1)^mu conj W(N, mu); real parts, then
     // imaginary parts, each [N][mu + 2p] with rows of 4p + 1
     __shared__ float sW[2 * RT_TS * RT_WS];
     __shared__ float sPh[2 * RT_TS];
-    __shared__ int2 s_off[2][128];   // per output parity aim and input: offsets of the two W terms
-    __shared__ float2 s_cf[2][128];  // their signs (0: no second term, or no such input)
+    __shared__ int2 s_off[2][128];   // per output parity aim and K position: offsets of the two W terms
+    __shared__ float2 s_cf[2][128];  // their signs and scales (0: no second term, or no such input)
     __shared__ int s_roff[128];      // per output coefficient (k, l): k (4p + 1) + l + 2p
-    __shared__ float s_sk[128];      // (-1)^k, 0 past the last coefficient
+    __shared__ float s_sk[128];      // (-1)^k with the row's scale, 0 past the last coefficient
     __shared__ unsigned char s_aim[128];
     __shared__ int s_src[R_TB], s_tgt[R_TB];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
-    __shared__ float s_ih;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int p = g.p, nc = g.nc, nkc = g.nkc, TS = 2 * p + 1, WS = 4 * p + 1, TSZ = TS * WS;
     const int4 b = g.batches[blockIdx.x];
     // the batch carries its key and table: one dependent load to everything else
     const int start = b.y, cnt = b.z & 255, tab = b.w;
     if (cnt <= 0 || cnt > R_TB) return;
-    const int N = (cnt + 15) & ~15;  // MMA columns
-    const int nq = (nkc + RT_KQ - 1) / RT_KQ;
+    const int Np = (cnt + 15) & ~15;  // columns per vector
     int c, lev, ox, oy, oz;
     rkey_decode((uint32_t)b.z >> 8, c, lev, ox, oy, oz);
     const bool refl = g.comps[c].refl != 0;
 
     if (tid < 128) {
-        // output coefficient tid as a row, input coefficient tid as a column
+        // packed coefficient tid as an output row
         int n = 0, m = 0, im = 0;
         const bool in = tid < nc;
         if (in) lf_decode(p, tid, n, m, im);
         s_roff[tid] = in ? n * WS + m + 2 * p : 0;
-        s_sk[tid] = in ? ((n & 1) ? -1.f : 1.f) : 0.f;
+        s_sk[tid] = in ? ((n & 1) ? -1.f : 1.f) * (float)(1 << RT_ASHIFT) / g.cscale[tid] : 0.f;
         s_aim[tid] = (unsigned char)im;
+    } else {
+        // K position k as an input column
+        const int k = tid - 128;
+        const bool in = k < nc;
+        int n = 0, m = 0, im = 0;
+        float sc = 0.f;
+        if (in) {
+            const int j = g.perm[k];
+            lf_decode(p, j, n, m, im);
+            sc = 1.f / g.cscale[j];
+        }
         // the multipole's reflection sign (-1)^{n+m} for s = -1 maps
-        const float rs = (refl && ((n + m) & 1)) ? -1.f : 1.f;
+        const float rs = (refl && ((n + m) & 1)) ? -sc : sc;
         const float sg = (m & 1) ? -1.f : 1.f;  // (-1)^m of the second term
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
             const int t = (a ^ im) * TSZ;  // real parts where the parities agree, else imaginary
-            s_off[a][tid] = in ? make_int2(t + n * WS + m, t + n * WS - m) : make_int2(0, 0);
+            s_off[a][k] = in ? make_int2(t + n * WS + m, t + n * WS - m) : make_int2(0, 0);
             // (re,re): W1 + sg W2; (re out, im in): -W1 + sg W2; (im, re): W1 + sg W2; (im, im): W1 - sg W2
             const float c1 = (a == 0 && im == 1) ? -1.f : 1.f;
             const float c2 = m > 0 ? ((a == 1 && im == 1) ? -sg : sg) : 0.f;
-            s_cf[a][tid] = in ? make_float2(rs * c1, rs * c2) : make_float2(0.f, 0.f);
+            s_cf[a][k] = make_float2(rs * c1, rs * c2);
         }
     }
     if (tid < R_TB) {
@@ -702,10 +719,9 @@ __global__ void __launch_bounds__(RT_THREADS, RT_MINB) k_m2r_tc(RTcArgs g)
     }
     if (tid >= 128 && tid < 128 + 2 * RT_TS)
         sPh[tid - 128] = g.phase[(size_t)((ox + R_OR) * R_OW + (oy + R_OR)) * 2 * RT_TS + (tid - 128)];
-    if (tid == 192) s_ih = (float)(1.0 / g.levelh[lev]);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(RT_TMEM_COLS)
+                     "r"(S::COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -732,93 +748,82 @@ __global__ void __launch_bounds__(RT_THREADS, RT_MINB) k_m2r_tc(RTcArgs g)
             sW[TSZ + j] = wi;
         }
     }
-    const float ih = s_ih;
-    // gather unit of every K chunk: column xj (rows >= N are not read), 16-byte
-    // quarter xq; a warp covers 8 columns = 512 contiguous bytes of a chunk.
-    // Operator units: rows xj and xj + 64, quarter xq.
+    const double hl = g.levelh[lev];
+    __syncthreads();  // W is in shared memory
+    // gather and operator unit of every chunk: row xj (and xj + 64 of the operator), 16-byte quarter xq
     const int xj = tid >> 2, xq = tid & 3;
-    const uint32_t idesc = tc_idesc(128, N);
+    const int src = xj < Np ? s_src[xj] : -1;
     bool ok = true;
-    for (int r = 0; r < g.nr && ok; ++r) {
-        float xv[8][4];
-        {
-            const float* M = g.M + (size_t)r * g.stride;
-            const int s = (xj < N) ? s_src[xj] : -1;
-#pragma unroll
-            for (int kc = 0; kc < 8; ++kc)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int k = kc * 16 + 4 * xq + e;
-                    xv[kc][e] = (kc < nkc && s >= 0 && k < nc) ? M[(size_t)s * nc + k] : 0.f;
-                }
-        }
-        if (r == 0) __syncthreads();  // W is in shared memory
-#pragma unroll
-        for (int i = 0; i < 8 / RT_KQ; ++i) {
-            if (i >= nq) break;
-            const int gr = r * nq + i, buf = gr & 1;  // round counter over the vectors
+    int gr = 0;  // round counter over the vectors
+    for (int r0 = 0; r0 < g.nr && ok; r0 += V) {
+        const int nv = min(V, g.nr - r0);  // vectors of this pass
+        const uint32_t idesc = tc_idesc_f16(128, nv * Np);
+        for (int i = 0; i < nkc; ++i, ++gr) {
+            const int kc = nkc - 1 - i, buf = gr & 1;  // falling degree
             if (gr >= 2 && !mbar_wait(&bar[buf], (uint32_t)(((gr - 2) >> 1) & 1))) s_abort = 1;
-            unsigned char* sb = sm + (size_t)buf * RT_BUF;
+            unsigned char* sa = sm + (size_t)(S::KEEP ? kc : buf) * 2 * RT_A_CHUNK;
+            unsigned char* sx = smx + (size_t)buf * S::XB;
+            if (xj < Np) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int row = xj + 64 * h;
-                const float* W = sW + s_roff[row];
-                const float sk = s_sk[row];
-                const int a = s_aim[row];
+                for (int v = 0; v < V; ++v) {
+                    if (v >= nv) break;
+                    const __half* gs = g.Ms + (size_t)(r0 + v) * g.ms_stride + (size_t)(src >= 0 ? src : 0) * 256 +
+                                       kc * TH_KC + xq * 8;
+                    const uint32_t off = swz16(v * Np + xj, xq * 8);
 #pragma unroll
-                for (int kl = 0; kl < RT_KQ; ++kl) {
-                    const int kc = i * RT_KQ + kl;
-                    if (kc >= nkc) break;
-                    float hi[4], lo[4];
+                    for (int piece = 0; piece < 2; ++piece) {
+                        unsigned char* dst = sx + piece * V * RT_X_CHUNK + off;
+                        if (src >= 0)
+                            cp_async16(smem_u32(dst), gs + piece * 128);
+                        else
+                            *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+            }
+            cp_async_commit();
+            if (!S::KEEP || r0 == 0) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int kin = kc * 16 + 4 * xq + e;
+                for (int h = 0; h < 2; ++h) {
+                    const int row = xj + 64 * h;
+                    const float* W = sW + s_roff[row];
+                    const float sk = s_sk[row];
+                    const int a = s_aim[row];
+                    __align__(16) __half hi[8], lo[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int kin = kc * TH_KC + 8 * xq + e;
                         const int2 o = s_off[a][kin];
                         const float2 cf = s_cf[a][kin];
                         const float v = sk * fmaf(cf.x, W[o.x], cf.y * W[o.y]);
-                        hi[e] = __uint_as_float(to_tf32(v));
-                        lo[e] = __uint_as_float(to_tf32(v - hi[e]));
+                        hi[e] = __float2half_rn(v);
+                        lo[e] = __float2half_rn(v - __half2float(hi[e]));
                     }
-                    const uint32_t off = (uint32_t)kl * RT_A_CHUNK + swz(row, 4 * xq);
-                    *reinterpret_cast<float4*>(sb + off) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-                    *reinterpret_cast<float4*>(sb + RT_A_ROUND + off) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+                    const uint32_t off = swz16(row, 8 * xq);
+                    *reinterpret_cast<uint4*>(sa + off) = *reinterpret_cast<const uint4*>(hi);
+                    *reinterpret_cast<uint4*>(sa + RT_A_CHUNK + off) = *reinterpret_cast<const uint4*>(lo);
                 }
             }
-            if (xj < N) {
-#pragma unroll
-                for (int kl = 0; kl < RT_KQ; ++kl) {
-                    const int kc = i * RT_KQ + kl;
-                    if (kc >= nkc) break;
-                    float hi[4], lo[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        hi[e] = __uint_as_float(to_tf32(xv[kc][e]));
-                        lo[e] = __uint_as_float(to_tf32(xv[kc][e] - hi[e]));
-                    }
-                    const uint32_t off = 2 * RT_A_ROUND + (uint32_t)kl * RT_X_CHUNK + swz(xj, 4 * xq);
-                    *reinterpret_cast<float4*>(sb + off) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-                    *reinterpret_cast<float4*>(sb + RT_X_ROUND + off) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-                }
-            }
+            cp_async_wait<0>();
             fence_async_smem();
             tc_fence_before();
             __syncthreads();
-            if (*(volatile int*)&s_abort) break;  // block-uniform after the barrier
+            if (*(volatile int*)&s_abort) {  // block-uniform after the barrier
+                ok = false;
+                break;
+            }
             if (tid == 0) {
                 tc_fence_after();
-                const uint32_t a0 = smem_u32(sb), x0 = a0 + 2 * RT_A_ROUND;
+                const uint32_t a0 = smem_u32(sa), x0 = smem_u32(sx);
+                const int nks = (nc - kc * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
-                for (int prod = 0; prod < 3; ++prod) {
-                    const uint32_t a = a0 + (prod == 2 ? RT_A_ROUND : 0), x = x0 + (prod == 1 ? RT_X_ROUND : 0);
+                for (int prod = 0; prod < 3; ++prod) {  // a2 x1, a1 x2, a1 x1
+                    const uint32_t a = a0 + (prod == 0 ? RT_A_CHUNK : 0);
+                    const uint32_t x = x0 + (prod == 1 ? V * RT_X_CHUNK : 0);
 #pragma unroll
-                    for (int kl = 0; kl < RT_KQ; ++kl) {
-                        if (i * RT_KQ + kl >= nkc) break;
-#pragma unroll
-                        for (int ks = 0; ks < 2; ++ks)
-                            tc_mma(tmem, smem_desc(a + kl * RT_A_CHUNK + 32 * ks),
-                                   smem_desc(x + kl * RT_X_CHUNK + 32 * ks), idesc,
-                                   (i | prod | kl | ks) != 0 ? 1u : 0u);
-                    }
+                    for (int ks = 1; ks >= 0; --ks)
+                        if (ks < nks)
+                            tc_mma_f16(tmem, smem_desc(a + 32 * ks), smem_desc(x + 32 * ks), idesc,
+                                       (i == 0 && prod == 0 && ks == nks - 1) ? 0u : 1u);
                 }
                 tc_commit(&bar[buf]);
             }
@@ -826,24 +831,27 @@ __global__ void __launch_bounds__(RT_THREADS, RT_MINB) k_m2r_tc(RTcArgs g)
         }
         // the last round's commit covers every MMA before it
         bool got = false;
-        if (!*(volatile int*)&s_abort) {
-            const int gl = r * nq + nq - 1;
-            got = mbar_wait(&bar[gl & 1], (uint32_t)((gl >> 1) & 1));
-        }
+        if (ok) got = mbar_wait(&bar[(gr - 1) & 1], (uint32_t)(((gr - 1) >> 1) & 1));
         ok = __syncthreads_and(got) != 0;  // block-uniform
         tc_fence_after();
         if (ok) {
-            const int q4 = warp & 3, half = warp >> 2;
-            if (half * 32 < N) {
+            const int q4 = warp & 3, row = 32 * q4 + lane;
+            const float rs = row < nc ? g.cscale[row] : 0.f;
+            float sc[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                sc[v] = rs * (float)(1.0 / hl) /
+                        (tc_scale(g.gmax[(size_t)min(r0 + v, g.nr - 1) * 32 + lev]) * (float)(1 << RT_ASHIFT));
+            for (int c0 = 32 * (warp >> 2); c0 < nv * Np; c0 += 64) {
                 float v[32];
-                tc_ld32(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(half * 32), v);
-                const int row = 32 * q4 + lane;
+                tc_ld32(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)c0, v);
                 if (row < nc) {
-                    float* L = g.L + (size_t)r * g.stride;
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
-                        const int j = half * 32 + i;
-                        if (j < cnt) atomicAdd(L + (size_t)s_tgt[j] * nc + row, v[i] * ih);
+                        const int vj = (V > 1 && c0 + i >= Np) ? 1 : 0, j = c0 + i - vj * Np;
+                        if (vj < nv && j < cnt)
+                            atomicAdd(g.L + (size_t)(r0 + vj) * g.stride + (size_t)s_tgt[j] * nc + row,
+                                      v[i] * (V > 1 && vj ? sc[V - 1] : sc[0]));
                     }
                 }
             }
@@ -855,7 +863,7 @@ __global__ void __launch_bounds__(RT_THREADS, RT_MINB) k_m2r_tc(RTcArgs g)
         tc_fence_after();
     }
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(RT_TMEM_COLS)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::COLS)
                      : "memory");
 }
 
@@ -896,20 +904,27 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
 
 // the float32 form with (p+1)^2 <= 128 applies the keys on the tensor cores
 // whenever the free M2L does (tensor-core option)
-static bool m2r_tc_on(const lfmm_ctx* ctx) { return ctx->precision == 1 && ctx->p <= 10 && lf_tc_on(ctx); }
+static bool m2r_tc_on(const lfmm_ctx* ctx)
+{
+    return ctx->precision == 1 && ctx->p <= 10 && lf_tc_on(ctx);
+}
 
 static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
 {
     RTcArgs g;
     g.p = ctx->p;
     g.nc = lf_nc(ctx->p);
-    g.nkc = (g.nc + 15) / 16;
+    g.nkc = (g.nc + TH_KC - 1) / TH_KC;
     g.batches = ctx->m2r_batches.as<int4>();
     g.tables = ctx->m2r_tables.as<double>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
     g.pairs = ctx->m2r_pairs.as<int2>();
     g.levelh = ctx->m2r_levelh.as<double>();
-    g.M = ctx->Mexp.as<float>();
+    g.Ms = ctx->m2l_Ms.as<__half>();
+    g.cscale = ctx->tc_cscale.as<float>();
+    g.perm = ctx->tc_perm.as<int>();
+    g.gmax = reinterpret_cast<unsigned*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
+    g.ms_stride = (size_t)ctx->nbox_total * 256;
     g.L = ctx->Lexp.as<float>();
     g.stride = (size_t)ctx->nbox_total * g.nc;
     g.nr = ctx->nrhs_b;
@@ -922,8 +937,13 @@ static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
         ctx->m2r_phase_p = ctx->p;
     }
     g.phase = ctx->m2r_phase.as<float>();
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, RT_SMEM));
-    ++ctx->launches, k_m2r_tc<<<ctx->m2r_nbatch, RT_THREADS, RT_SMEM, st>>>(g);
+    if (g.nr == 1) {
+        LF_CHECK(cudaFuncSetAttribute(k_m2r_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, RtShape<1>::SMEM));
+        ++ctx->launches, k_m2r_tc<1><<<ctx->m2r_nbatch, RT_THREADS, RtShape<1>::SMEM, st>>>(g);
+    } else {
+        LF_CHECK(cudaFuncSetAttribute(k_m2r_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, RtShape<2>::SMEM));
+        ++ctx->launches, k_m2r_tc<2><<<ctx->m2r_nbatch, RT_THREADS, RtShape<2>::SMEM, st>>>(g);
+    }
     return lf_cuda(cudaGetLastError(), "m2r tensor-core GEMM");
 }
 

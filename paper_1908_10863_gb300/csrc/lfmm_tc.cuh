@@ -1,17 +1,14 @@
 // lfmm_tc.cuh -- inline-PTX building blocks of the tcgen05 kernels: shared-
-// memory mbarriers with bounded waits, bulk and cp.async copies, the TF32
-// split, shared-memory matrix descriptors (K-major, 64-byte swizzle), the
-// instruction descriptor of kind::tf32, MMA issue and commit, and the
+// memory mbarriers with bounded waits, bulk and cp.async copies, the operand
+// scale, shared-memory matrix descriptors (K-major, 64-byte swizzle), the
+// instruction descriptor of kind::f16, MMA issue and commit, and the
 // 32-lane tensor-memory load.  Included by the free-space and reaction M2L
 // kernels.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#ifndef TC_KC
-#define TC_KC 16                     // K elements per staged row (64-byte rows)
-#endif
-#define TC_ROWB (TC_KC * 4)          // bytes per row of a staged tile
+#define TC_ROWB 64                   // bytes per row of a staged tile (64-byte swizzle)
 #define TH_KC (TC_ROWB / 2)          // 16-bit K elements per staged row
 #define TC_SPIN_CYCLES (1ll << 31)   // ~1 s at 2 GHz
 // ---------------------------------------------------------------------------
@@ -73,14 +70,18 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ uint32_t to_tf32(float x)
-{
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// The power of two that takes the largest magnitude (float bits) into
+// [2^13, 2^14); 1 for zero or non-finite values.
+__device__ __forceinline__ float tc_scale(unsigned maxbits)
+{
+    if (maxbits == 0u || maxbits >= 0x7f800000u) return 1.f;
+    int e = 140 - (int)(maxbits >> 23);  // 13 - (biased exponent - 127)
+    e = e > 126 ? 126 : (e < -126 ? -126 : e);
+    return __uint_as_float((unsigned)(e + 127) << 23);
+}
 
 // shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups 512 B apart
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr)
@@ -90,23 +91,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr)
     d |= (uint64_t)1 << 16;                   // leading byte offset (unused for swizzled K-major)
     d |= (uint64_t)((8 * TC_ROWB) >> 4) << 32;  // stride byte offset: 8 rows
     d |= (uint64_t)1 << 46;                   // descriptor version
-    d |= (uint64_t)(TC_ROWB == 64 ? 4 : 6) << 61;  // 64-byte or 32-byte swizzle
+    d |= (uint64_t)4 << 61;                     // 64-byte swizzle
     return d;
 }
-// instruction descriptor: D float32, A and B TF32, both K-major, M x N
-__host__ __device__ constexpr uint32_t tc_idesc(int M, int N)
-{
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
-}
-// the same with float16 operands (kind::f16, K = 16 per instruction)
+// instruction descriptor of kind::f16: D float32, A and B float16, both K-major, M x N (K = 16 per instruction)
 __host__ __device__ constexpr uint32_t tc_idesc_f16(int M, int N)
 {
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -154,22 +142,12 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float v[16])
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// byte offset of element (row, k) of a swizzled K-major tile with TC_ROWB-byte
-// rows: the 16-byte chunk index is XORed with the address bits just above the
-// swizzle span -- 64-byte swizzle: chunk (bits 4-5) ^ bits 7-8 = (row / 2) mod 4;
-// 32-byte swizzle: chunk (bit 4) ^ bit 7 = (row / 4) mod 2
-__host__ __device__ __forceinline__ uint32_t swz(int row, int k)
-{
-    const uint32_t c = (uint32_t)(k >> 2);
-    const uint32_t x = (TC_ROWB == 64) ? (uint32_t)((row >> 1) & 3) : (uint32_t)((row >> 2) & 1);
-    return (uint32_t)row * TC_ROWB + ((c ^ x) << 4) + (uint32_t)(k & 3) * 4u;
-}
-
-
-// the same for rows of TH_KC 16-bit elements
+// byte offset of element (row, k) of a swizzled K-major tile with rows of TH_KC
+// 16-bit elements (64 bytes): the 16-byte chunk index (bits 4-5) is XORed with
+// the address bits just above the swizzle span, bits 7-8 = (row / 2) mod 4
 __host__ __device__ __forceinline__ uint32_t swz16(int row, int k)
 {
     const uint32_t c = (uint32_t)(k >> 3);
-    const uint32_t x = (TC_ROWB == 64) ? (uint32_t)((row >> 1) & 3) : (uint32_t)((row >> 2) & 1);
+    const uint32_t x = (uint32_t)((row >> 1) & 3);
     return (uint32_t)row * TC_ROWB + ((c ^ x) << 4) + (uint32_t)(k & 7) * 2u;
 }
