@@ -253,17 +253,13 @@ __global__ void k_rel_pos(int leaf_off, int nleaf, const LfD4* __restrict__ cen,
     }
 }
 
-// A leaf of at most 16 (8) charges gives each target 2 (4) lanes, each
-// taking a contiguous part of every staged source box; their sums meet by
-// shuffles at the end.
-template <int RB>
+// Free-space near field, one charge vector, staging per source box (leaf levels
+// whose images are no grid cells, or LFMM_OPT_P2P_STAGED = 0).  A leaf of at
+// most 16 (8) charges gives each target 2 (4) lanes, each taking a contiguous
+// part of every staged source box; their sums meet by shuffles at the end.
 __global__ void __launch_bounds__(32 * PW_WARPS) k_p2p_warp(P2PArgs a, const float4* __restrict__ rel, int nleaf)
 {
-    // one charge vector: sources staged as (x, y, z, q), one 16-byte shared load per pair
-    constexpr bool ONE = (RB == 1);
-    __shared__ float sx[PW_WARPS][ONE ? 1 : 32], sy[PW_WARPS][ONE ? 1 : 32], sz[PW_WARPS][ONE ? 1 : 32],
-        sq[PW_WARPS][RB][ONE ? 1 : 32];
-    __shared__ float4 sp[PW_WARPS][ONE ? 32 : 1];
+    __shared__ float4 sp[PW_WARPS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int wi = blockIdx.x * PW_WARPS + w;
     if (wi >= nleaf * a.split) return;  // whole warp
@@ -288,29 +284,22 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_p2p_warp(P2PArgs a, const flo
             yi = r.y;
             zi = r.z;
         }
-        P2PAcc<float, RB> A;
-        P2PPart<float, RB> part;
+        P2PAcc<float, 1> A;
+        P2PPart<float, 1> part;
         for (int e = eb + part0; e < ee; e += a.split) {
-            const uint32_t ent = a.nent[e];
-            const int c = (int)(ent >> LFMM_ENT_SHIFT);
-            const int s = (int)(ent & LFMM_ENT_MASK);
-            const LfmmComp& cp = a.comps[c];
-            // source box centre (free) or its polarization image (reaction), relative to the target box
-            float dx0, dy0, dz0, szs;
+            const int s = (int)(a.nent[e] & LFMM_ENT_MASK);
+            // source box centre relative to the target box
+            float dx0, dy0, dz0;
             if (a.grid) {
-                // (z_t - z'') / h = (iz_t + 1/2) - s (iz_s + 1/2) - K with K an integer on this level
                 const int4 gs = a.grid[s];
-                const float4 pc = a.pcon[c];
-                szs = pc.x;
                 dx0 = (float)(gs.x - gt.x) * a.hleaf;
                 dy0 = (float)(gs.y - gt.y) * a.hleaf;
-                dz0 = (pc.x * ((float)gs.z + 0.5f) - ((float)gt.z + 0.5f) + pc.y) * a.hleaf;
+                dz0 = (float)(gs.z - gt.z) * a.hleaf;
             } else {
                 const LfD4 cs = a.cen[s];
                 dx0 = (float)(cs.x - ct.x);
                 dy0 = (float)(cs.y - ct.y);
-                dz0 = (float)(cp.is_free ? cs.z - ct.z : cp.s * cs.z + cp.o - ct.z);
-                szs = cp.is_free ? 1.f : (float)cp.s;
+                dz0 = (float)(cs.z - ct.z);
             }
             const int sb = a.pbeg[s], se = a.pend[s];
             for (int cb = sb; cb < se; cb += 32) {
@@ -318,92 +307,61 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_p2p_warp(P2PArgs a, const flo
                 __syncwarp();
                 if (j < se) {
                     const float4 r = rel[j];
-                    if constexpr (ONE) {
-                        sp[w][lane] = make_float4(r.x + dx0, r.y + dy0, szs * r.z + dz0, q[j]);
-                    } else {
-                        sx[w][lane] = r.x + dx0;
-                        sy[w][lane] = r.y + dy0;
-                        sz[w][lane] = szs * r.z + dz0;
-#pragma unroll
-                        for (int k = 0; k < RB; ++k)
-                            if (k < a.nr) sq[w][k][lane] = q[(size_t)k * a.qstride + j];
-                    }
+                    sp[w][lane] = make_float4(r.x + dx0, r.y + dy0, r.z + dz0, q[j]);
                 }
                 __syncwarp();
                 if (!valid) continue;
                 const int cnt = min(32, se - cb);
                 // this lane's contiguous share of the staged sources
                 const int u0 = (slice * cnt) / G, u1 = ((slice + 1) * cnt) / G;
-                if constexpr (ONE) {
-                    if (cp.is_free) {
-                        float& P = part.P[0].s;
-                        float& Ex = part.Ex[0].s;
-                        float& Ey = part.Ey[0].s;
-                        float& Ez = part.Ez[0].s;
+                float& P = part.P[0].s;
+                float& Ex = part.Ex[0].s;
+                float& Ey = part.Ey[0].s;
+                float& Ez = part.Ez[0].s;
 #pragma unroll 4
-                        for (int u = u0; u < u1; ++u) {
-                            const float4 v = sp[w][u];
-                            const float dx = xi - v.x, dy = yi - v.y, dz = zi - v.z;
-                            const float r2 = dx * dx + dy * dy + dz * dz;
-                            const float ir = (r2 > 0.f) ? rsqrtf(r2) : 0.f;  // the target itself: no term
-                            const float q3 = v.w * ir * ir * ir;
-                            P += v.w * ir;
-                            Ex += q3 * dx;
-                            Ey += q3 * dy;
-                            Ez += q3 * dz;
-                        }
-                    } else {
-                        for (int u = u0; u < u1; ++u) {
-                            const float4 v = sp[w][u];
-                            p2p_reaction_add<float, 1>(cp, xi - v.x, yi - v.y, zi - v.z, &sp[w][u].w, 0, 1, a.Qn,
-                                                       a.gl_t, a.gl_w, part, LF_CTAB(a, c), LF_CTAB4(a, c));
-                        }
-                    }
-                    continue;
-                }
-                if (cp.is_free) {
-                    for (int u = u0; u < u1; ++u)
-                        p2p_free_add<float, RB>(xi - sx[w][u], yi - sy[w][u], zi - sz[w][u], &sq[w][0][u], 32, a.nr,
-                                                part);
-                } else {
-                    for (int u = u0; u < u1; ++u)
-                        p2p_reaction_add<float, RB>(cp, xi - sx[w][u], yi - sy[w][u], zi - sz[w][u], &sq[w][0][u],
-                                                    32, a.nr, a.Qn, a.gl_t, a.gl_w, part, LF_CTAB(a, c),
-                                                    LF_CTAB4(a, c));
+                for (int u = u0; u < u1; ++u) {
+                    const float4 v = sp[w][u];
+                    const float dx = xi - v.x, dy = yi - v.y, dz = zi - v.z;
+                    const float r2 = dx * dx + dy * dy + dz * dz;
+                    const float ir = (r2 > 0.f) ? rsqrtf(r2) : 0.f;  // the target itself: no term
+                    const float q3 = v.w * ir * ir * ir;
+                    P += v.w * ir;
+                    Ex += q3 * dx;
+                    Ey += q3 * dy;
+                    Ez += q3 * dz;
                 }
             }
-            p2p_flush<float, RB>(part, A);
+            p2p_flush<float, 1>(part, A);
         }
         if (G > 1) {
             // the lanes of one target meet (every lane takes part in the shuffles)
-#pragma unroll
-            for (int k = 0; k < RB; ++k) {
-                float v0 = A.P[k].s - A.P[k].c, v1 = A.Ex[k].s - A.Ex[k].c;
-                float v2 = A.Ey[k].s - A.Ey[k].c, v3 = A.Ez[k].s - A.Ez[k].c;
-                for (int off = T; off < 32; off <<= 1) {
-                    v0 += __shfl_xor_sync(0xffffffffu, v0, off);
-                    v1 += __shfl_xor_sync(0xffffffffu, v1, off);
-                    v2 += __shfl_xor_sync(0xffffffffu, v2, off);
-                    v3 += __shfl_xor_sync(0xffffffffu, v3, off);
-                }
-                A.P[k].s = v0;
-                A.Ex[k].s = v1;
-                A.Ey[k].s = v2;
-                A.Ez[k].s = v3;
+            float v0 = A.P[0].s - A.P[0].c, v1 = A.Ex[0].s - A.Ex[0].c;
+            float v2 = A.Ey[0].s - A.Ey[0].c, v3 = A.Ez[0].s - A.Ez[0].c;
+            for (int off = T; off < 32; off <<= 1) {
+                v0 += __shfl_xor_sync(0xffffffffu, v0, off);
+                v1 += __shfl_xor_sync(0xffffffffu, v1, off);
+                v2 += __shfl_xor_sync(0xffffffffu, v2, off);
+                v3 += __shfl_xor_sync(0xffffffffu, v3, off);
             }
+            A.P[0].s = v0;
+            A.Ex[0].s = v1;
+            A.Ey[0].s = v2;
+            A.Ez[0].s = v3;
         }
-        if (valid && slice == 0) p2p_store<float, RB>(a, i, A);
+        if (valid && slice == 0) p2p_store<float, 1>(a, i, A);
     }
 }
 
-// Near field with lists of sources: the FP64 form, and the float32 form where
-// the near lists hold reaction pairs, in media whose remainders are image
-// sums (LfImgRule) or without any reaction pair.  One warp per target leaf
+// Near field with lists of sources: the FP64 form, and the float32 form with
+// several charge vectors or reaction pairs in the near lists, in media whose
+// remainders are image sums (LfImgRule) or without any reaction pair.  One warp per target leaf
 // (or per part of its list).  For a pass of T targets the warp walks its list
 // twice, free-space entries first, then the reaction entries: 32 entries at a
 // time, one per lane, a warp scan places their sources in one flat range, and
 // chunks of PL_CAP of them are staged in shared memory (position relative to
-// the target box, charges, component).  The 32 lanes are T target slots times
+// the target box, charges, component).  Where several warps share a leaf, each
+// takes its share of the flat range (whole entries would leave one warp most
+// of the reaction pairs).  The 32 lanes are T target slots times
 // 32 / T slices of the staged chunk; T is the width that pads the leaf's
 // charges least.
 // A reaction pair costs one inverse square root and about ten operations per
@@ -416,16 +374,20 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_p2p_warp(P2PArgs a, const flo
 // by one block of 128 threads per leaf and the quadrature, 0.48 ms here; 2,848
 // charges at p = 20, 538k reaction pairs, 33.0 and 1.67 ms; float32, 50,001
 // charges beside the interfaces, 30M reaction pairs, 0.95 ms by the tables
-// (k_p2p_warp), 0.57 ms here.
+// (k_p2p_warp), 0.57 ms here.  Several vectors share a pair's kernels: eight
+// per batch in float32 (four multiply-adds per pair and vector, charges read
+// as float4s), all batches in one launch; 64 vectors of 262,144 charges,
+// 21.4 ms (k_p2p_warp, batches of 4, one source box at a time) -> 6.95 ms.
 #define PL_CAP 64
 #define PL_WARPS 4
 
-// slots of target charges per pass: the padded passes, plus the staging's share
-__device__ __forceinline__ int pl_targets(int nt)
+// slots of target charges per pass: the padded passes, plus the staging's
+// share (2 of a target's pairs, or 6 with many charges to stage)
+__device__ __forceinline__ int pl_targets(int nt, int stage)
 {
     int best = 1 << 30, T = 32;
     for (int t = 32; t >= 4; t >>= 1) {
-        const int cost = ((nt + t - 1) / t) * (t + 2);
+        const int cost = ((nt + t - 1) / t) * (t + stage);
         if (cost < best) {
             best = cost;
             T = t;
@@ -439,14 +401,53 @@ struct PlComp {  // one component's pair constants: leading image, remainder, po
     R C, zeta, zeta_r, r0;
 };
 
+template <typename R>
+struct __align__(16) PlSrc {  // a staged source: position, and component (bit 8: h = z - z'')
+    R x, y, z;
+    int c;
+};
+
+// the RB charges of one staged source
 template <typename R, int RB>
+__device__ __forceinline__ void pl_charges(const R* s, R* q)
+{
+    if constexpr (sizeof(R) == 4 && RB % 4 == 0) {
+#pragma unroll
+        for (int k = 0; k < RB; k += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(s + k);
+            q[k] = v.x;
+            q[k + 1] = v.y;
+            q[k + 2] = v.z;
+            q[k + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < RB; ++k) q[k] = s[k];
+    }
+}
+
+// blockIdx.y: batch of RB right-hand sides.  phases: 1 free-space entries, 2
+// reaction entries, 3 both; add: add to the outputs instead of storing them.
+// MODE: reaction pairs by the image rule (PL_IMG), by the pair routine (tables
+// or quadrature; PL_PAIR), or by the one of media of four and five layers
+// (PL_GEN; PL_GFREE: the free-space entries of such a medium).  The last two
+// take positions relative to the target box from the FP64 coordinates, rounded
+// once; float32 otherwise adds the charges' float offsets from their own leaf
+// centres to the centre offset, which next to several interfaces loses part of
+// a digit of the field (2.3e-5 against 9.6e-6, five layers).
+#define PL_IMG 0
+#define PL_PAIR 1
+#define PL_GEN 2
+#define PL_GFREE 3
+template <typename R, int RB, int MODE = PL_IMG>
 __global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const float4* __restrict__ rel, int nleaf,
-                                                            int ncomp, const __grid_constant__ LfImgRule<R> rule)
+                                                            int ncomp, int phases, int add,
+                                                            const __grid_constant__ LfImgRule<R> rule)
 {
     typedef LfMath<R> F;
     constexpr bool DBL = sizeof(R) == 8;
-    __shared__ R s_x[PL_WARPS][PL_CAP], s_y[PL_WARPS][PL_CAP], s_z[PL_WARPS][PL_CAP], s_q[PL_WARPS][RB][PL_CAP];
-    __shared__ short s_c[PL_WARPS][PL_CAP];  // component, bit 8: targets above (a = 1: h = z - z'')
+    __shared__ PlSrc<R> s_p[PL_WARPS][PL_CAP];
+    __shared__ __align__(16) R s_q[PL_WARPS][PL_CAP][RB];  // charges (zero past the last right-hand side)
     __shared__ PlComp<R> s_comp[LFMM_MAXCOMP];
     __shared__ double2 s_map[LFMM_MAXCOMP];  // z'' = s z' + o
     __shared__ short s_kind[LFMM_MAXCOMP];   // 0: free space; else 1 + 256 (a == 1)
@@ -461,22 +462,24 @@ __global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const flo
     const int wi = blockIdx.x * PL_WARPS + w;
     if (wi >= nleaf * a.split) return;  // whole warp, after the block's only barrier
     const int li = wi / a.split, part0 = wi - li * a.split;
-    const R* q = reinterpret_cast<const R*>(a.q);
+    const int r0 = (int)blockIdx.y * RB, nr = min(RB, a.nr - r0);
+    const R* q = reinterpret_cast<const R*>(a.q) + (size_t)r0 * a.qstride;
     const int t = a.leaf_off + li;
-    const bool cells = !DBL && a.grid;
+    constexpr bool dp = DBL || MODE >= PL_GEN;
+    const bool cells = !dp && a.grid;
     const LfD4 ct = cells ? LfD4{0.0, 0.0, 0.0, 0.0} : a.cen[t];
     const int4 gt = cells ? a.grid[t] : make_int4(0, 0, 0, 0);
     const int tb = a.pbeg[t], te = a.pend[t];
     const int eb = a.nbeg[t], ee = a.nend[t];
-    const int nmine = (ee - eb > part0) ? (ee - eb - part0 + a.split - 1) / a.split : 0;
-    const int T = pl_targets(te - tb), G = 32 / T;
+    const int nent = ee - eb;
+    const int T = pl_targets(te - tb, RB >= 4 ? 6 : 2), G = 32 / T;
     const int ti = lane & (T - 1), slice = lane / T;
     for (int base = tb; base < te; base += T) {
         const int i = base + ti;
         const bool valid = i < te;
         R xi = 0, yi = 0, zi = 0;
         if (valid) {
-            if constexpr (DBL) {
+            if constexpr (dp) {
                 xi = (R)(a.xs[i] - ct.x);
                 yi = (R)(a.ys[i] - ct.y);
                 zi = (R)(a.zs[i] - ct.z);
@@ -490,21 +493,21 @@ __global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const flo
         P2PAcc<R, RB> A;
         P2PPart<R, RB> part;
 #pragma unroll 1
-        for (int react = 0; react < 2; ++react) {
+        for (int react = (phases & 1) ? 0 : 1; react < ((phases & 2) ? 2 : 1); ++react) {
 #pragma unroll 1
-            for (int k0 = 0; k0 < nmine; k0 += 32) {
+            for (int k0 = 0; k0 < nent; k0 += 32) {
                 // this lane's entry: first source, sources, centre offset of its (image) box
                 int b0 = 0, n = 0, c = 0;
                 float dx0 = 0.f, dy0 = 0.f, dz0 = 0.f, szs = 1.f;
                 const int j = k0 + lane;
-                if (j < nmine) {
-                    const uint32_t ent = a.nent[eb + part0 + j * a.split];
+                if (j < nent) {
+                    const uint32_t ent = a.nent[eb + j];
                     const int s = (int)(ent & LFMM_ENT_MASK);
                     c = (int)(ent >> LFMM_ENT_SHIFT);
                     if ((s_kind[c] != 0) == (react != 0)) {
                         b0 = a.pbeg[s];
                         n = a.pend[s] - b0;
-                        if constexpr (!DBL) {
+                        if constexpr (!dp) {
                             if (cells) {
                                 const int4 gs = a.grid[s];
                                 const float4 pc = a.pcon[c];
@@ -530,9 +533,11 @@ __global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const flo
                 }
                 const int excl = incl - n;
                 const int tot = __shfl_sync(0xffffffffu, incl, 31);
+                // this part's share of the flat range
+                const int fb = (int)((int64_t)tot * part0 / a.split), fe = (int)((int64_t)tot * (part0 + 1) / a.split);
 #pragma unroll 1
-                for (int f0 = 0; f0 < tot; f0 += PL_CAP) {
-                    const int cnt = min(PL_CAP, tot - f0);
+                for (int f0 = fb; f0 < fe; f0 += PL_CAP) {
+                    const int cnt = min(PL_CAP, fe - f0);
                     __syncwarp();  // the previous chunk has been read
 #pragma unroll 1
                     for (int h = 0; h < cnt; h += 32) {
@@ -547,57 +552,83 @@ __global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const flo
                         }
                         const int src = __shfl_sync(0xffffffffu, b0, lo) + (u - __shfl_sync(0xffffffffu, excl, lo));
                         const int cc = __shfl_sync(0xffffffffu, c, lo);
-                        float ox, oy, oz, sz;
-                        if constexpr (!DBL) {
+                        float ox = 0.f, oy = 0.f, oz = 0.f, sz = 0.f;
+                        if constexpr (!dp) {
                             ox = __shfl_sync(0xffffffffu, dx0, lo);
                             oy = __shfl_sync(0xffffffffu, dy0, lo);
                             oz = __shfl_sync(0xffffffffu, dz0, lo);
                             sz = __shfl_sync(0xffffffffu, szs, lo);
                         }
                         if (u < f0 + cnt) {
-                            const int d = h + lane;
-                            if constexpr (DBL) {
-                                s_x[w][d] = a.xs[src] - ct.x;
-                                s_y[w][d] = a.ys[src] - ct.y;
+                            PlSrc<R> sp;
+                            if constexpr (dp) {
+                                sp.x = (R)(a.xs[src] - ct.x);
+                                sp.y = (R)(a.ys[src] - ct.y);
                                 const double2 m = s_map[cc];
-                                s_z[w][d] = (react ? m.x * a.zs[src] + m.y : a.zs[src]) - ct.z;
+                                sp.z = (R)((react ? m.x * a.zs[src] + m.y : a.zs[src]) - ct.z);
                             } else {
                                 const float4 r = rel[src];
-                                s_x[w][d] = r.x + ox;
-                                s_y[w][d] = r.y + oy;
-                                s_z[w][d] = sz * r.z + oz;
+                                sp.x = r.x + ox;
+                                sp.y = r.y + oy;
+                                sp.z = sz * r.z + oz;
                             }
+                            sp.c = cc | (s_kind[cc] & 256);
+                            s_p[w][h + lane] = sp;
 #pragma unroll
                             for (int k = 0; k < RB; ++k)
-                                if (k < a.nr) s_q[w][k][d] = q[(size_t)k * a.qstride + src];
-                            s_c[w][d] = (short)(cc | (s_kind[cc] & 256));
+                                s_q[w][h + lane][k] = k < nr ? q[(size_t)k * a.qstride + src] : R(0);
                         }
                     }
                     __syncwarp();
                     if (valid) {
                         if (!react) {
-                            for (int u = slice; u < cnt; u += G)
-                                p2p_free_add<R, RB>(xi - s_x[w][u], yi - s_y[w][u], zi - s_z[w][u], &s_q[w][0][u],
-                                                    PL_CAP, a.nr, part);
-                        } else {
+#pragma unroll 2
                             for (int u = slice; u < cnt; u += G) {
-                                const int ck = s_c[w][u];
-                                const PlComp<R> pc = s_comp[ck & 255];
-                                const R dx = xi - s_x[w][u], dy = yi - s_y[w][u], dz = zi - s_z[w][u];
-                                const R sg = (ck & 256) ? R(1) : R(-1);
-                                const R rho2 = dx * dx + dy * dy;
-                                R k00, k10, g;
-                                lf_image_pair<R>(pc.C, pc.zeta, pc.zeta_r, pc.r0, rho2, sg * dz, rule, k00, k10, g);
-                                k10 *= sg;
+                                const PlSrc<R> sp = s_p[w][u];
+                                R qv[RB];
+                                pl_charges<R, RB>(s_q[w][u], qv);
+                                const R dx = xi - sp.x, dy = yi - sp.y, dz = zi - sp.z;
+                                const R r2 = dx * dx + dy * dy + dz * dz;
+                                const R ir = r2 > R(0) ? F::Rsqrt(r2) : R(0);  // the target itself: no term
+                                const R ir3 = ir * ir * ir;
+                                const R gx = ir3 * dx, gy = ir3 * dy, gz = ir3 * dz;
 #pragma unroll
                                 for (int k = 0; k < RB; ++k) {
-                                    if (k >= a.nr) break;
-                                    const R qv = s_q[w][k][u];
-                                    part.P[k].add(qv * k00);
-                                    part.Ez[k].add(qv * k10);
-                                    const R qg = qv * g;
-                                    part.Ex[k].add(qg * dx);
-                                    part.Ey[k].add(qg * dy);
+                                    part.P[k].s += qv[k] * ir;
+                                    part.Ex[k].s += qv[k] * gx;
+                                    part.Ey[k].s += qv[k] * gy;
+                                    part.Ez[k].s += qv[k] * gz;
+                                }
+                            }
+                        } else if constexpr (MODE != PL_GFREE) {
+                            for (int u = slice; u < cnt; u += G) {
+                                const PlSrc<R> sp = s_p[w][u];
+                                const R dx = xi - sp.x, dy = yi - sp.y, dz = zi - sp.z;
+                                const R sg = (sp.c & 256) ? R(1) : R(-1);
+                                const R rho2 = dx * dx + dy * dy;
+                                R k00, k10, g;
+                                if constexpr (MODE == PL_IMG) {
+                                    const PlComp<R> pc = s_comp[sp.c & 255];
+                                    lf_image_pair<R>(pc.C, pc.zeta, pc.zeta_r, pc.r0, rho2, sg * dz, rule, k00, k10,
+                                                     g);
+                                } else {
+                                    const int c = sp.c & 255;
+                                    const R rho = F::Sqrt(rho2);
+                                    lf_reaction_pair<R, MODE == PL_GEN>(a.comps[c], rho, sg * dz, a.Qn, a.gl_t, a.gl_w,
+                                                                        k00, k10, g, LF_CTAB(a, c),
+                                                                        sizeof(R) == 4 ? LF_CTAB4(a, c) : nullptr);
+                                    g = rho > R(0) ? g / rho : R(0);
+                                }
+                                k10 *= sg;
+                                R qv[RB];
+                                pl_charges<R, RB>(s_q[w][u], qv);
+                                const R gx = g * dx, gy = g * dy;
+#pragma unroll
+                                for (int k = 0; k < RB; ++k) {
+                                    part.P[k].s += qv[k] * k00;
+                                    part.Ex[k].s += qv[k] * gx;
+                                    part.Ey[k].s += qv[k] * gy;
+                                    part.Ez[k].s += qv[k] * k10;
                                 }
                             }
                         }
@@ -622,7 +653,24 @@ __global__ void __launch_bounds__(32 * PL_WARPS) k_p2p_list(P2PArgs a, const flo
             A.Ey[k].s = v2;
             A.Ez[k].s = v3;
         }
-        if (valid && slice == 0) p2p_store<R, RB>(a, i, A);
+        if (valid && slice == 0) {
+#pragma unroll
+            for (int k = 0; k < RB; ++k) {
+                if (k >= nr) break;
+                const size_t o = (size_t)(r0 + k) * a.qstride + i;
+                if (a.split > 1) {
+                    atomicAdd(a.phi + o, (double)A.P[k].s);
+                    atomicAdd(a.fld + 3 * o + 0, (double)A.Ex[k].s);
+                    atomicAdd(a.fld + 3 * o + 1, (double)A.Ey[k].s);
+                    atomicAdd(a.fld + 3 * o + 2, (double)A.Ez[k].s);
+                } else {
+                    a.phi[o] = (add ? a.phi[o] : 0.0) + (double)A.P[k].s;
+                    a.fld[3 * o + 0] = (add ? a.fld[3 * o + 0] : 0.0) + (double)A.Ex[k].s;
+                    a.fld[3 * o + 1] = (add ? a.fld[3 * o + 1] : 0.0) + (double)A.Ey[k].s;
+                    a.fld[3 * o + 2] = (add ? a.fld[3 * o + 2] : 0.0) + (double)A.Ez[k].s;
+                }
+            }
+        }
     }
 }
 
@@ -1172,9 +1220,7 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
     const int ph = lf_prof_start(ctx, LFMM_TIME_P2P, st);
     // the network variant only where the near field holds reaction pairs (it
     // needs far more registers, which slows the free-space part); one launch
-    // per right-hand side.  The quadrature kernels take batches of up to 4
-    // (float32: more registers per thread cost more than the shared pair
-    // geometry saves) or 8 (FP64).
+    // per right-hand side.  The FP64 quadrature kernel takes batches of up to 8.
     const bool net = a.sv.ready != 0 && ctx->near_reaction_entries > 0;
     // Few leaves (small problems) leave most SMs idle with one warp or block
     // per leaf: share each near list between `split` of them.  A set value
@@ -1183,21 +1229,27 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
     // of the near lists (counted at every build); without any, the kernels of
     // thinner media compute the free-space pairs alone and are exact
     const bool general = ctx->L >= 3 && ctx->near_reaction_entries > 0;
-    // Reaction pairs by the image rule (k_p2p_list) where the medium has one,
-    // unless the tables are asked for.  The FP64 form of a context that holds
-    // trained networks keeps the quadrature for the pairs outside the network
-    // runs (test_surrogate_gain_in_near_field states the network's gain over
-    // it).  FP64 lists without reaction pairs take the same kernel.
+    // Float32: reaction pairs in k_p2p_list, by the image rule where it is
+    // short (lf_img32_on), else from the tables (media of four and five layers,
+    // slow image series) or the quadrature.  FP64: by the image rule in the same
+    // kernel, unless the tables are asked for or the medium has no rule; the
+    // FP64 form of a context that holds trained networks keeps the quadrature
+    // for the pairs outside the network runs (test_surrogate_gain_in_near_field
+    // states the network's gain over it).  Lists without reaction pairs take
+    // k_p2p_list in FP64 and with several charge vectors.
     const bool react = ctx->near_reaction_entries > 0;
-    const bool img = ctx->img_ok && ctx->use_near_tab != 1;
-    const bool list = !net && !general &&
-                      (react ? img && (ctx->precision || !ctx->surr_ready) : ctx->precision == 0);
-    const bool warp_kernel = list || (!net && !general && ctx->precision);
+    const bool img = ctx->precision ? lf_img32_on(ctx) : ctx->img_ok && ctx->use_near_tab != 1 && !ctx->surr_ready;
+    const bool list = !net && (ctx->precision ? react || nr > 1 : !react || (img && !general));
+    const int list_rb = nr == 1 ? 1 : (nr == 2 ? 2 : (nr <= 4 ? 4 : 8));  // right-hand sides per batch
+    const int list_ny = (nr + list_rb - 1) / list_rb;
+    const bool warp_kernel = list || (!net && ctx->precision);
     int split = ctx->p2p_split;
     if (split <= 0) {
-        const int want = warp_kernel ? 152 * 32 : 152 * 8;  // warps, or blocks of P2P_T threads
+        // warps (twice as many where reaction pairs make the leaves uneven), or blocks of P2P_T threads
+        const int want = list && react ? 152 * 64 : (warp_kernel ? 152 * 32 : 152 * 8);
         split = 1;
-        while (split < LFMM_P2P_SPLIT_MAX && (int64_t)leaf.nbox * split * 2 <= want) split *= 2;
+        const int64_t units = (int64_t)leaf.nbox * (list ? list_ny : 1);
+        while (split < LFMM_P2P_SPLIT_MAX && units * split * 2 <= want) split *= 2;
     }
     a.split = split;
     if (split > 1) {
@@ -1207,56 +1259,67 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
     // the network's rejected pairs go by the image rule too (n = -1: quadrature or tables)
     LfImgRule<float> net32 = ctx->img32;
     LfImgRule<double> net64 = ctx->img64;
-    if (!img) net32.n = net64.n = -1;
+    if (!lf_img32_on(ctx)) net32.n = -1;
+    if (!ctx->img_ok || ctx->use_near_tab == 1) net64.n = -1;
+    if (list) {
+        const dim3 g(lf_blocks((int64_t)leaf.nbox * split, PL_WARPS), list_ny);
+        const int T = 32 * PL_WARPS, nb = leaf.nbox, nc = ctx->ncomp;
+        const float4* rel = ctx->pos_rel.as<float4>();
+        a.nr = nr;
+#define PL_LAUNCH(R, RB, MODE, PH, ADD, RULE) \
+    ++ctx->launches, k_p2p_list<R, RB, MODE><<<g, T, 0, st>>>(a, rel, nb, nc, PH, ADD, ctx->RULE)
+#define PL_LAUNCH_RB(R, MODE, PH, ADD, RULE)                          \
+    do {                                                              \
+        if (list_rb == 1) PL_LAUNCH(R, 1, MODE, PH, ADD, RULE);       \
+        else if (list_rb == 2) PL_LAUNCH(R, 2, MODE, PH, ADD, RULE);  \
+        else if (list_rb == 4) PL_LAUNCH(R, 4, MODE, PH, ADD, RULE);  \
+        else PL_LAUNCH(R, 8, MODE, PH, ADD, RULE);                    \
+    } while (0)
+        if (!ctx->precision) {
+            PL_LAUNCH_RB(double, PL_IMG, 3, 0, img64);
+        } else if (!react || img) {
+            PL_LAUNCH_RB(float, PL_IMG, 3, 0, img32);
+        } else {
+            // the pair routine needs far more registers: the free-space pairs
+            // in a launch of their own
+            if (general) {
+                PL_LAUNCH_RB(float, PL_GFREE, 1, 0, img32);
+                PL_LAUNCH_RB(float, PL_GEN, 2, 1, img32);
+            } else {
+                PL_LAUNCH_RB(float, PL_IMG, 1, 0, img32);
+                PL_LAUNCH_RB(float, PL_PAIR, 2, 1, img32);
+            }
+        }
+#undef PL_LAUNCH_RB
+#undef PL_LAUNCH
+        LF_TRY(lf_cuda(cudaGetLastError(), "p2p"));
+        lf_prof_stop(ctx, ph, st);
+        return LfErr();
+    }
     const double* phi0 = a.phi;
     double* fld0 = a.fld;
     const char* q0 = reinterpret_cast<const char*>(a.q);
-    const int step = (net || general) ? 1 : (ctx->precision ? 4 : 8);
+    const int step = (net || general) ? 1 : 8;
     for (int r0 = 0; r0 < nr; r0 += step) {
         a.nr = nr - r0 < step ? nr - r0 : step;
         a.q = q0 + (size_t)r0 * qs;
         a.phi = const_cast<double*>(phi0) + (size_t)r0 * ctx->n;
         a.fld = fld0 + (size_t)r0 * ctx->n * 3;
-        if (list) {
-            const int g = lf_blocks((int64_t)leaf.nbox * split, PL_WARPS), T = 32 * PL_WARPS;
-            const float4* rel = ctx->pos_rel.as<float4>();
-            const int nb = leaf.nbox, nc = ctx->ncomp;
-#define PL_LAUNCH(R, RB, RULE) ++ctx->launches, k_p2p_list<R, RB><<<g, T, 0, st>>>(a, rel, nb, nc, ctx->RULE)
-            if (ctx->precision) {
-                if (a.nr == 1) PL_LAUNCH(float, 1, img32);
-                else if (a.nr == 2) PL_LAUNCH(float, 2, img32);
-                else PL_LAUNCH(float, 4, img32);
-            } else {
-                if (a.nr == 1) PL_LAUNCH(double, 1, img64);
-                else if (a.nr == 2) PL_LAUNCH(double, 2, img64);
-                else if (a.nr <= 4) PL_LAUNCH(double, 4, img64);
-                else PL_LAUNCH(double, 8, img64);
-            }
-#undef PL_LAUNCH
-        } else if (general) {
-            if (ctx->precision)
-                ++ctx->launches, k_p2p<float, 1, true><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
-            else
-                ++ctx->launches, k_p2p<double, 1, true><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
+        if (general) {
+            ++ctx->launches, k_p2p<double, 1, true><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
         } else if (net) {
             if (ctx->precision)
                 ++ctx->launches, k_p2p_net<float><<<leaf.nbox * split, P2P_T, 0, st>>>(a, net32);
             else
                 ++ctx->launches, k_p2p_net<double><<<leaf.nbox * split, P2P_T, 0, st>>>(a, net64);
-        } else if (ctx->precision) {
-            const int g = lf_blocks((int64_t)leaf.nbox * split, PW_WARPS), T = 32 * PW_WARPS;
+        } else if (ctx->precision) {  // one charge vector, no reaction pairs
             const float4* rel = ctx->pos_rel.as<float4>();
-            if (a.nr == 1 && a.grid && ctx->near_reaction_entries == 0 && ctx->p2p_staged)
+            if (a.grid && ctx->p2p_staged)
                 ++ctx->launches, k_p2p_free_staged<<<lf_blocks((int64_t)leaf.nbox * split, PF_WARPS), 32 * PF_WARPS, 0,
                                                      st>>>(a, rel, leaf.nbox);
-            else if (a.nr == 1)
-                ++ctx->launches, k_p2p_warp<1><<<g, T, 0, st>>>(a, rel, leaf.nbox);
-            else if (a.nr == 2)
-                ++ctx->launches, k_p2p_warp<2><<<g, T, 0, st>>>(a, rel, leaf.nbox);
-            else if (a.nr <= 4)
-                ++ctx->launches, k_p2p_warp<4><<<g, T, 0, st>>>(a, rel, leaf.nbox);
             else
-                ++ctx->launches, k_p2p_warp<8><<<g, T, 0, st>>>(a, rel, leaf.nbox);
+                ++ctx->launches, k_p2p_warp<<<lf_blocks((int64_t)leaf.nbox * split, PW_WARPS), 32 * PW_WARPS, 0, st>>>(
+                    a, rel, leaf.nbox);
         } else {
             if (a.nr == 1)
                 ++ctx->launches, k_p2p<double, 1><<<leaf.nbox * split, P2P_T, 0, st>>>(a);
