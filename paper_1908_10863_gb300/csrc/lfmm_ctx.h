@@ -219,7 +219,7 @@ LfErr lf_cuda(cudaError_t e, const char* what);
 #define LFMM_PIN_SCAN 512       // a scan's last input and output (2 ints)
 #define LFMM_PIN_LIST 1024      // list statistics, overflow, counters, per-level snapshots (< 1 KB)
 #define LFMM_PIN_M2L 2048       // free M2L class counts (144 ints)
-#define LFMM_PIN_ROOT 2688      // root box keys (up to 128)
+#define LFMM_PIN_ROOT 2688      // (end of the class counts)
 #define LFMM_PIN_BOUNDS 4096    // bounding-box partials (256 blocks x 6 doubles)
 #define LFMM_PIN_UP 4096        // later in the build: root lists and list counters to upload (12 KB)
 #define LFMM_PIN_M2R 16384      // reaction M2L key starts and values (the rest)
@@ -256,6 +256,7 @@ inline bool lf_img32_on(const lfmm_ctx* ctx)
 
 // ---- free-space M2L GEMM (lfmm_m2l.cu) ----
 LfErr lf_setup_m2l_ops(lfmm_ctx* ctx);
+LfErr lf_prepare_m2l_classes(lfmm_ctx* ctx, cudaStream_t st);  // enqueue (no synchronisation)
 LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2l_gemm(lfmm_ctx* ctx, cudaStream_t st);
 // ---- reaction M2L by geometry key (lfmm_m2r.cu) ----

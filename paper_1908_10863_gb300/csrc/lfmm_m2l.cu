@@ -367,7 +367,10 @@ static void m2l_tc_tiles(const int* hcnt, int depth, int tn, std::vector<int4>& 
     }
 }
 
-LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
+// Device part that needs only the boxes: targets grouped by (level, octant
+// class), the counts of the classes (read back into pinned memory), and the
+// children of each parent.  Enqueued beside the interaction lists.
+LfErr lf_prepare_m2l_classes(lfmm_ctx* ctx, cudaStream_t st)
 {
     ctx->m2l_ntiles = 0;
     ctx->shift_ready = 0;
@@ -375,9 +378,7 @@ LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
     const int depth = ctx->depth;
     if (depth < 2) return LfErr();
     const size_t nb = (size_t)ctx->nbox_total;
-    // the slot table was filled with the lists; errors counted at `err`
-    int* err = reinterpret_cast<int*>(ctx->counts.as<char>() + 24576);
-    int* cnt = err + 16;  // [16 levels][8]
+    int* cnt = reinterpret_cast<int*>(ctx->counts.as<char>() + 24576) + 16;  // [16 levels][8]
     LF_CHECK(cudaMemsetAsync(cnt, 0, sizeof(int) * 16 * 8, st));
     int nsort = 0;
     for (int l = 1; l <= depth; ++l) nsort += ctx->levels[l].nbox;
@@ -395,6 +396,9 @@ LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
     if (nsort > 0)
         ++ctx->launches, k_class_keys<<<lf_blocks(nsort, 256), 256, 0, st>>>(
             cl, nsort, ctx->box_key.as<uint32_t>(), ctx->m2l_keys.as<uint32_t>(), ctx->m2l_sorted.as<uint32_t>(), cnt);
+    static_assert(LFMM_PIN_M2L + (16 + 16 * 8) * sizeof(int) <= LFMM_PIN_ROOT, "pinned regions");
+    LF_CHECK(cudaMemcpyAsync(lf_pin<int>(ctx, LFMM_PIN_M2L) + 16, cnt, 16 * 8 * sizeof(int), cudaMemcpyDeviceToHost,
+                             st));
     // M2M slots: children of each parent by octant (every box of levels
     // 1 .. depth, which hold the ids below the roots', in one launch)
     LF_TRY(lf_reserve(ctx->m2m_slots, nb * 8 * sizeof(int)));
@@ -406,14 +410,19 @@ LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
     // keys are level << 28 | class << 25 | index: with fewer than 2^24 boxes the
     // top byte alone orders them (stable within a level and class)
     if (nsort < (1 << 24))
-        LF_TRY(lf_radix_sort(ctx, ctx->m2l_keys.as<uint32_t>(), ctx->m2l_sorted.as<uint32_t>(), nsort, st, 3, 1));
+        LF_TRY(lf_radix_sort(ctx, ctx->m2l_keys.as<uint32_t>(), ctx->m2l_sorted.as<uint32_t>(), nsort, st, 3, 1, 1));
     else
-        LF_TRY(lf_radix_sort(ctx, ctx->m2l_keys.as<uint32_t>(), ctx->m2l_sorted.as<uint32_t>(), nsort, st));
-    static_assert(LFMM_PIN_M2L + (16 + 16 * 8) * sizeof(int) <= LFMM_PIN_ROOT, "pinned regions");
-    const int* hcnt = lf_pin<int>(ctx, LFMM_PIN_M2L);
-    LF_CHECK(cudaMemcpyAsync(lf_pin<int>(ctx, LFMM_PIN_M2L), err, (16 + 16 * 8) * sizeof(int), cudaMemcpyDeviceToHost,
-                             st));
-    LF_CHECK(cudaStreamSynchronize(st));
+        LF_TRY(lf_radix_sort(ctx, ctx->m2l_keys.as<uint32_t>(), ctx->m2l_sorted.as<uint32_t>(), nsort, st, 0, 4, 1));
+    return LfErr();
+}
+
+// Tiles, once the lists and the class counts have been read back.
+LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
+{
+    if (ctx->m2l_rm == 0) return LfErr();
+    const int depth = ctx->depth;
+    if (depth < 2) return LfErr();
+    const int* hcnt = lf_pin<int>(ctx, LFMM_PIN_M2L);  // [0]: entries outside their class; [16 ..]: class counts
     if (hcnt[0] != 0) return "internal: free M2L entry outside its offset class";
     std::vector<int4>& tiles = ctx->m2l_tiles_h;
     std::vector<int4>& l2l_tiles = ctx->l2l_tiles_h;

@@ -68,16 +68,21 @@ __host__ __device__ __forceinline__ void rkey_decode(uint32_t key, int& c, int& 
 // (component, level) (0 on levels where the interfaces are grid planes); the
 // key holds n, the table is taken at n + f.  An entry outside the key's
 // offset range counts in bad[level] (its level then stays per pair).
-__global__ void k_m2r_keys(const LfmmComp* __restrict__ comps, int off, int nb, const int4* __restrict__ grid,
-                           const int* __restrict__ zbase,
+struct RkLevels {
+    int depth;
+    int off[17];  // first box of each level (finest first)
+};
+__global__ void k_m2r_keys(const LfmmComp* __restrict__ comps, int nb, const __grid_constant__ RkLevels lv,
+                           const int4* __restrict__ grid, const int* __restrict__ zbase,
                            const int* __restrict__ rbeg, const int* __restrict__ rend,
-                           const uint32_t* __restrict__ rent, int level, uint32_t* __restrict__ keys,
+                           const uint32_t* __restrict__ rent, uint32_t* __restrict__ keys,
                            uint32_t* __restrict__ vals, int* __restrict__ tgt, int* __restrict__ bad)
 {
-    // one warp per target box, lanes over its entries
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= nb) return;
-    const int t = off + i;
+    // one warp per target box of the keyed levels, lanes over its entries
+    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (t >= nb) return;
+    int level = lv.depth;
+    while (level > 0 && t >= lv.off[level - 1]) --level;
     const int4 gt = grid[t];
     for (int e = rbeg[t] + (threadIdx.x & 31); e < rend[t]; e += 32) {
         uint32_t v = rent[e];
@@ -213,13 +218,16 @@ LfErr lf_prepare_m2r(lfmm_ctx* ctx, cudaStream_t st)
     // entries of levels la .. depth are contiguous: index them relative to `first`
     uint32_t* keys = ctx->m2r_keys.as<uint32_t>();
     uint32_t* vals = ctx->m2r_order.as<uint32_t>();
-    for (int l = la; l <= ctx->depth; ++l) {
-        const LfmmLevel& lv = ctx->levels[l];
-        if (lv.nbox == 0 || lv.m2r_count == 0) continue;
-        ++ctx->launches, k_m2r_keys<<<lf_blocks(lv.nbox, 4), 128, 0, st>>>(
-            ctx->comp_dev.as<LfmmComp>(), lv.off, lv.nbox, ctx->box_grid.as<int4>(), ctx->m2r_zbase.as<int>(), ctx->m2r_off.as<int>(),
-            ctx->m2r_off.as<int>() + ctx->nbox_total, ctx->m2r_ent.as<uint32_t>(), l, keys - first, vals - first,
-            ctx->m2r_tgt.as<int>(), bad);
+    {
+        // levels la .. depth hold the box ids [0, end of la), finest first
+        RkLevels lv;
+        lv.depth = ctx->depth;
+        for (int l = 0; l < 17; ++l) lv.off[l] = l <= ctx->depth ? ctx->levels[l].off : 0;
+        const int nb = ctx->levels[la].off + ctx->levels[la].nbox;
+        ++ctx->launches, k_m2r_keys<<<lf_blocks(nb, 4), 128, 0, st>>>(
+            ctx->comp_dev.as<LfmmComp>(), nb, lv, ctx->box_grid.as<int4>(), ctx->m2r_zbase.as<int>(),
+            ctx->m2r_off.as<int>(), ctx->m2r_off.as<int>() + ctx->nbox_total, ctx->m2r_ent.as<uint32_t>(),
+            keys - first, vals - first, ctx->m2r_tgt.as<int>(), bad);
     }
     LF_TRY(lf_cuda(cudaGetLastError(), "m2r keys"));
     // vals hold absolute entry indices (e), keys sorted ascending

@@ -135,38 +135,106 @@ LfErr lf_scan_i32(lfmm_ctx* ctx, const int* in, int* out, int64_t n, int64_t* to
 }
 
 // ---------------------------------------------------------------------------
-// Stable LSD radix sort of (key, value) uint32 pairs, 8 bits per pass.
+// Stable LSD radix sort of (key, value) uint32 pairs, 8 bits per pass.  A pass
+// is a histogram per block, [digit][block], and a scatter whose blocks find
+// their own offsets: thread d sums row d (all blocks for the digit's total, the
+// blocks before it for its own part) and the totals are scanned in shared
+// memory.  Up to RS_FUSE blocks that is all; above, one launch of 256 blocks
+// scans the rows first.  (A recursive scan between the two took three more
+// launches per pass, 8 us of 24 at 65,536 keys.)
 // ---------------------------------------------------------------------------
 #define RS_T 256
-#define RS_ROUNDS 8
-#define RS_TILE (RS_T * RS_ROUNDS)
+#define RS_ROUNDS 8   // most rounds of RS_T keys per block
+#define RS_FUSE 128   // most blocks whose rows the scatter reads itself
 
-__global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, int* __restrict__ hist,
-                             int nblocks)
+__global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, int rounds,
+                             int* __restrict__ hist, int nblocks)
 {
     __shared__ int h[256];
     const int tid = threadIdx.x;
     h[tid] = 0;
     __syncthreads();
-    for (int r = 0; r < RS_ROUNDS; ++r) {
-        int64_t i = (int64_t)blockIdx.x * RS_TILE + r * RS_T + tid;
+#pragma unroll 4
+    for (int r = 0; r < rounds; ++r) {
+        int64_t i = ((int64_t)blockIdx.x * rounds + r) * RS_T + tid;
         if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1);
     }
     __syncthreads();
     hist[tid * nblocks + blockIdx.x] = h[tid];
 }
 
-__global__ void k_radix_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, int64_t n, int shift,
-                                const int* __restrict__ hoff, int nblocks)
+// exclusive prefix sums of the rows of hist, in place, and their totals
+__global__ void __launch_bounds__(256) k_radix_rows(int* __restrict__ hist, int nblocks, int* __restrict__ total)
+{
+    __shared__ int s_w[8];
+    int* row = hist + (size_t)blockIdx.x * nblocks;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int base = 0;
+    for (int j0 = 0; j0 < nblocks; j0 += 256) {
+        const int j = j0 + tid;
+        const int v = j < nblocks ? row[j] : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_w[w] = x;
+        __syncthreads();
+        int before = 0, all = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k < w) before += s_w[k];
+            all += s_w[k];
+        }
+        if (j < nblocks) row[j] = base + before + x - v;
+        base += all;
+        __syncthreads();
+    }
+    if (tid == 0) total[blockIdx.x] = base;
+}
+
+__global__ void __launch_bounds__(RS_T) k_radix_scatter(const uint32_t* __restrict__ kin,
+                                                        const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
+                                                        uint32_t* __restrict__ vout, int64_t n, int shift, int rounds,
+                                                        const int* __restrict__ hist, int nblocks,
+                                                        const int* __restrict__ total)
 {
     __shared__ int s_off[256];
     __shared__ int s_wcnt[RS_T / 32][256];
-    __shared__ int s_rtot[256];
+    __shared__ int s_w[RS_T / 32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    s_off[tid] = hoff[tid * nblocks + blockIdx.x];
-    for (int r = 0; r < RS_ROUNDS; ++r) {
-        int64_t i = (int64_t)blockIdx.x * RS_TILE + r * RS_T + tid;
+    {
+        // this block's first position of digit tid
+        const int* row = hist + (size_t)tid * nblocks;
+        int tot = 0, pre = 0;
+        if (total) {
+            tot = total[tid];
+            pre = row[blockIdx.x];
+        } else {
+#pragma unroll 8
+            for (int j = 0; j < nblocks; ++j) {
+                const int v = row[j];
+                tot += v;
+                pre += j < (int)blockIdx.x ? v : 0;
+            }
+        }
+        int x = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_w[wid] = x;
+        __syncthreads();
+        int before = 0;
+#pragma unroll
+        for (int k = 0; k < RS_T / 32; ++k)
+            if (k < wid) before += s_w[k];
+        s_off[tid] = before + x - tot + pre;
+    }
+    for (int r = 0; r < rounds; ++r) {
+        int64_t i = ((int64_t)blockIdx.x * rounds + r) * RS_T + tid;
         bool valid = i < n;
         uint32_t key = valid ? kin[i] : 0u;
         uint32_t val = valid ? vin[i] : 0u;
@@ -179,15 +247,12 @@ __global__ void k_radix_scatter(const uint32_t* __restrict__ kin, const uint32_t
         int leader = __ffs(peers) - 1;
         if (valid && lane == leader) s_wcnt[wid][digit] = __popc(peers);
         __syncthreads();
-        {
-            int run = 0;
+        int run = 0;
 #pragma unroll
-            for (int w = 0; w < RS_T / 32; ++w) {
-                int t = s_wcnt[w][tid];
-                s_wcnt[w][tid] = run;
-                run += t;
-            }
-            s_rtot[tid] = run;
+        for (int w = 0; w < RS_T / 32; ++w) {
+            int t = s_wcnt[w][tid];
+            s_wcnt[w][tid] = run;
+            run += t;
         }
         __syncthreads();
         if (valid) {
@@ -196,8 +261,7 @@ __global__ void k_radix_scatter(const uint32_t* __restrict__ kin, const uint32_t
             vout[pos] = val;
         }
         __syncthreads();
-        s_off[tid] += s_rtot[tid];
-        __syncthreads();
+        s_off[tid] += run;
     }
 }
 
@@ -206,22 +270,24 @@ __global__ void k_radix_scatter(const uint32_t* __restrict__ kin, const uint32_t
 LfErr lf_radix_sort(lfmm_ctx* ctx, uint32_t* keys, uint32_t* vals, int64_t n, cudaStream_t st, int first_pass,
                     int npass, int set)
 {
-    int nb = lf_blocks(n, RS_TILE);
+    // as few keys per block as keep the rows short enough for the scatter
+    const int rounds = (int)std::min<int64_t>(RS_ROUNDS, std::max<int64_t>(1, (n + RS_T * RS_FUSE - 1) / (RS_T * RS_FUSE)));
+    const int nb = lf_blocks(n, RS_T * rounds);
     DevBuf& kt = set ? ctx->keys_tmp2 : ctx->keys_tmp;
     DevBuf& vt = set ? ctx->vals_tmp2 : ctx->vals_tmp;
     DevBuf& ht = set ? ctx->hist2 : ctx->hist;
     LF_TRY(lf_reserve(kt, (size_t)n * 4));
     LF_TRY(lf_reserve(vt, (size_t)n * 4));
-    LF_TRY(lf_reserve(ht, (size_t)256 * nb * 4));
+    LF_TRY(lf_reserve(ht, ((size_t)256 * nb + 256) * 4));
     uint32_t *ka = keys, *va = vals, *kb = kt.as<uint32_t>(), *vb = vt.as<uint32_t>();
     int* h = ht.as<int>();
+    int* total = nb > RS_FUSE ? h + (size_t)256 * nb : nullptr;
     for (int pass = first_pass; pass < first_pass + npass; ++pass) {
         int shift = 8 * pass;
-        ++ctx->launches, k_radix_hist<<<nb, RS_T, 0, st>>>(ka, n, shift, h, nb);
-        LF_TRY(lf_cuda(cudaGetLastError(), "radix hist"));
-        LF_TRY(lf_scan_i32(ctx, h, h, (int64_t)256 * nb, nullptr, st, set));
-        ++ctx->launches, k_radix_scatter<<<nb, RS_T, 0, st>>>(ka, va, kb, vb, n, shift, h, nb);
-        LF_TRY(lf_cuda(cudaGetLastError(), "radix scatter"));
+        ++ctx->launches, k_radix_hist<<<nb, RS_T, 0, st>>>(ka, n, shift, rounds, h, nb);
+        if (total) ++ctx->launches, k_radix_rows<<<256, 256, 0, st>>>(h, nb, total);
+        ++ctx->launches, k_radix_scatter<<<nb, RS_T, 0, st>>>(ka, va, kb, vb, n, shift, rounds, h, nb, total);
+        LF_TRY(lf_cuda(cudaGetLastError(), "radix pass"));
         std::swap(ka, kb);
         std::swap(va, vb);
     }
@@ -318,6 +384,8 @@ __global__ void k_level_counts(const uint32_t* __restrict__ keys, int64_t n, int
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
         uint32_t k = keys[i], kp = (i > 0) ? keys[i - 1] : 0u;
+        // counts[15]: the layers that hold charges, one bit each
+        if (i == 0 || (k >> (3 * fine)) != (kp >> (3 * fine))) atomicOr(&counts[15], 1 << (k >> (3 * fine)));
         for (int l = 0; l <= fine; ++l) {
             int sh = 3 * (fine - l);
             if (i == 0 || (k >> sh) != (kp >> sh)) atomicAdd(&s[l], 1);
@@ -1070,6 +1138,16 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
             ctx->box_center.as<LfD4>(), ctx->box_grid.as<int4>());
     }
     LF_TRY(lf_cuda(cudaGetLastError(), "boxes"));
+    // what follows from the boxes alone goes on the second stream, beside the
+    // lists: the M2L and translation classes, the near field's positions (their
+    // scratch buffers and pinned read-back regions are disjoint)
+    cudaStream_t s2 = ctx->s_near;
+    ctx->n = n;
+    LF_CHECK(cudaEventRecord(ctx->ev_fork, st));
+    LF_CHECK(cudaStreamWaitEvent(s2, ctx->ev_fork, 0));
+    LF_TRY(lf_prepare_m2l_classes(ctx, s2));
+    LF_TRY(lf_near_prepare(ctx, s2));
+    LF_CHECK(cudaEventRecord(ctx->ev_join, s2));
     {
         // per (component, level) constants of the admissibility test
         // host staging owned by the context: the copy needs no synchronisation
@@ -1121,11 +1199,12 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
     int64_t near_used = 0, root_react = 0;  // entries, reaction entries
     {
         const LfmmLevel& r = ctx->levels[0];
-        if (r.nbox > 128) return "internal: more than 128 root boxes";
-        const uint32_t* rk = lf_pin<uint32_t>(ctx, LFMM_PIN_ROOT);
-        LF_CHECK(cudaMemcpyAsync(lf_pin<uint32_t>(ctx, LFMM_PIN_ROOT), bkey + r.off, 4 * r.nbox, cudaMemcpyDeviceToHost,
-                                 st));
-        LF_CHECK(cudaStreamSynchronize(st));
+        // the root boxes' keys are their layers, in order: read with the level counts
+        uint32_t rk[LFMM_MAXL + 1] = {0};
+        int nroot_l = 0;
+        for (int l = 0; l <= LFMM_MAXL; ++l)
+            if ((hc[15] >> l) & 1) rk[nroot_l++] = (uint32_t)l;
+        if (r.nbox != nroot_l) return "internal: root boxes";
         int root_of[LFMM_MAXL + 1];
         for (int l = 0; l <= LFMM_MAXL; ++l) root_of[l] = -1;
         for (int i = 0; i < r.nbox; ++i) root_of[rk[i]] = r.off + i;
@@ -1232,6 +1311,8 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
         LF_CHECK(cudaMemcpyAsync(hovp, overflow, sizeof(int), cudaMemcpyDeviceToHost, st));
         LF_CHECK(cudaMemcpyAsync(hused, used, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
         LF_CHECK(cudaMemcpyAsync(hsnap, snap, sizeof(unsigned) * 3 * (size_t)(depth + 1), cudaMemcpyDeviceToHost, st));
+        LF_CHECK(cudaMemcpyAsync(lf_pin<int>(ctx, LFMM_PIN_M2L), slot_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+        LF_CHECK(cudaStreamWaitEvent(st, ctx->ev_join, 0));  // (the class counts are read back by then)
         LF_CHECK(cudaStreamSynchronize(st));
         if (!*hovp) break;
         if (attempt >= 8) return "internal: interaction lists keep overflowing";
@@ -1274,14 +1355,8 @@ LfErr lf_build_tree(lfmm_ctx* ctx, const double* xyz, const int32_t* layer, int6
     ctx->stats[LFMM_STAT_M2M_EDGES] = tot - ctx->levels[0].nbox;
     ctx->n = n;
     ctx->stats[LFMM_STAT_REACTION_KEYS] = 0;
-    // the reaction M2L keys and the near field's relative positions go on the
-    // second stream, beside the free M2L classes and slots on this one (their
-    // scratch buffers and pinned read-back regions are disjoint)
-    cudaStream_t s2 = ctx->s_near;
-    LF_CHECK(cudaEventRecord(ctx->ev_fork, st));
-    LF_CHECK(cudaStreamWaitEvent(s2, ctx->ev_fork, 0));
+    // the reaction M2L keys go on the second stream, beside the free M2L tiles
     LF_TRY(lf_prepare_m2r(ctx, s2));
-    LF_TRY(lf_near_prepare(ctx, s2));
     LF_TRY(lf_prepare_m2l(ctx, st));
     LF_TRY(lf_prepare_m2r_finish(ctx, s2));
     LF_CHECK(cudaEventRecord(ctx->ev_join, s2));
