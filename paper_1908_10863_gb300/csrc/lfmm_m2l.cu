@@ -528,9 +528,13 @@ LfErr lf_prepare_m2l(lfmm_ctx* ctx, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------------------
-// The GEMM kernel.  Thread (rg, cg): rows rg*RM .. rg*RM+RM-1 of the packed
-// output, columns 4cg .. 4cg+3 of the tile.  X is stored column-major
-// [j][k] with stride KP+1 (conflict-free gathers and reads).
+// The GEMM kernel.  Thread (rg, cg): rows rg*RM .. rg*RM+RM-1 of the block's
+// 16 RM output rows (part blockIdx.z of the RP), columns 4cg .. 4cg+3 of the
+// tile.  X is stored column-major [j][k] with stride KP+1 (conflict-free
+// gathers and reads).  Where a launch has few tiles (the translations between
+// coarse levels, FP64 everywhere: a 128 x 128 x 64 tile is 270 us on one SM's
+// FP64 pipe) the rows are shared by RP / 32 blocks of RM = 2; the whole chain of
+// translations is serial, so their latency is what counts.
 // ---------------------------------------------------------------------------
 struct GemmArgs {
     int p, nc, RP;
@@ -549,15 +553,16 @@ struct GemmArgs {
     size_t mstride, lstride;  // per right-hand side (blockIdx.y), in elements
 };
 
-template <typename R, int RM, bool COMPF = false>
+template <typename R, int RP, int RM, bool COMPF = false>
 __global__ void __launch_bounds__(G_T) k_m2l_gemm(GemmArgs g)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int RP = 16 * RM;
+    constexpr int RB = 16 * RM;  // rows of this block
     constexpr int KP = RP;
     constexpr int XS = KP + 1;
-    R* sA = reinterpret_cast<R*>(smem_raw);  // [G_KC][RP]
-    R* sX = sA + G_KC * RP;                  // [G_TB][XS]
+    R* sA = reinterpret_cast<R*>(smem_raw);  // [G_KC][RB]
+    R* sX = sA + G_KC * RB;                  // [G_TB][XS]
+    const int row0 = (int)blockIdx.z * RB;
     __shared__ int s_tb[G_TB];
     __shared__ int s_src[G_TB];
     const int tid = threadIdx.x;
@@ -621,15 +626,16 @@ __global__ void __launch_bounds__(G_T) k_m2l_gemm(GemmArgs g)
         const R* Ao = A + (size_t)o * KP * RP;
         for (int kc = 0; kc < KP; kc += G_KC) {
             __syncthreads();
-            // stage A_o[kc .. kc+KC][0 .. RP) (contiguous)
-            const R* src = Ao + (size_t)kc * RP;
-            for (int idx = tid; idx < G_KC * RP; idx += G_T) sA[idx] = src[idx];
+            // stage A_o[kc .. kc+KC][row0 .. row0 + RB)
+            const R* src = Ao + (size_t)kc * RP + row0;
+#pragma unroll
+            for (int idx = tid; idx < G_KC * RB; idx += G_T) sA[idx] = src[(idx / RB) * RP + idx % RB];
             __syncthreads();
 #pragma unroll 4
             for (int kk = 0; kk < G_KC; ++kk) {
                 R a[RM];
 #pragma unroll
-                for (int r = 0; r < RM; ++r) a[r] = sA[kk * RP + rg * RM + r];
+                for (int r = 0; r < RM; ++r) a[r] = sA[kk * RB + rg * RM + r];
                 R x[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) x[c] = sX[(4 * cg + c) * XS + kc + kk];
@@ -672,7 +678,7 @@ __global__ void __launch_bounds__(G_T) k_m2l_gemm(GemmArgs g)
         R* Lt = L + (size_t)s_tb[j] * nc;
 #pragma unroll
         for (int r = 0; r < RM; ++r) {
-            int row = rg * RM + r;
+            int row = row0 + rg * RM + r;
             if (row < nc) {
                 if (g.mode == 1)
                     Lt[row] = acc[r][c];
@@ -687,27 +693,32 @@ __global__ void __launch_bounds__(G_T) k_m2l_gemm(GemmArgs g)
     }
 }
 
+template <typename R, int RP, int RM, bool COMPF>
+static LfErr launch_one(lfmm_ctx* ctx, cudaStream_t st, const GemmArgs& g, int nblk)
+{
+    const size_t sm = sizeof(R) * ((size_t)G_KC * 16 * RM + (size_t)G_TB * (RP + 1));
+    LF_CHECK(cudaFuncSetAttribute(k_m2l_gemm<R, RP, RM, COMPF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ++ctx->launches, k_m2l_gemm<R, RP, RM, COMPF><<<dim3(nblk, ctx->nrhs_b, RP / (16 * RM)), G_T, sm, st>>>(g);
+    return lf_cuda(cudaGetLastError(), "gathered gemm");
+}
+
 template <typename R, int RM>
 static LfErr launch_gemm(lfmm_ctx* ctx, cudaStream_t st, const GemmArgs& g, int ntiles)
 {
     if (ntiles <= 0) return LfErr();
     constexpr int RP = 16 * RM;
-    size_t sm = sizeof(R) * ((size_t)G_KC * RP + (size_t)G_TB * (RP + 1));
     const int nblk = g.split ? ntiles * g.noff : ntiles;
     // compensated sums where one block adds many offsets into one output
     if constexpr (sizeof(R) == 4) {
-        if (g.noff == G_NOFF && !g.split) {
-            LF_CHECK(cudaFuncSetAttribute(k_m2l_gemm<R, RM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sm));
-            ++ctx->launches, k_m2l_gemm<R, RM, true><<<dim3(nblk, ctx->nrhs_b), G_T, sm, st>>>(g);
-            return lf_cuda(cudaGetLastError(), "gathered gemm");
-        }
+        if (g.noff == G_NOFF && !g.split) return launch_one<R, RP, RM, true>(ctx, st, g, nblk);
     }
-    {
-        LF_CHECK(cudaFuncSetAttribute(k_m2l_gemm<R, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        ++ctx->launches, k_m2l_gemm<R, RM><<<dim3(nblk, ctx->nrhs_b), G_T, sm, st>>>(g);
+    // shared rows: FP64, or too few blocks for two per SM
+    if constexpr (sizeof(R) == 8) {
+        return launch_one<R, RP, 2, false>(ctx, st, g, nblk);
+    } else {
+        if (RM > 2 && (int64_t)nblk * ctx->nrhs_b < 2 * 152) return launch_one<R, RP, 2, false>(ctx, st, g, nblk);
+        return launch_one<R, RP, RM, false>(ctx, st, g, nblk);
     }
-    return lf_cuda(cudaGetLastError(), "gathered gemm");
 }
 
 template <typename R>
