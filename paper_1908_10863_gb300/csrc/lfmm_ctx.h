@@ -156,8 +156,9 @@ struct lfmm_ctx {
     int m2l_tc_wide = 0;  // tensor-core free M2L in its wide form ((p+1)^2 > 128): no tensor-core M2M / L2L
     // reaction M2L grouped by geometry key on interface-aligned levels
     DevBuf m2r_keys, m2r_order, m2r_tgt, m2r_kstart, m2r_kval, m2r_tables, m2r_levelh, m2r_batches;
-    DevBuf m2r_tdesc, m2r_ktab;  // table descriptors (component, level, rho^2, oz); table of each key
-    std::vector<int4> m2r_tdesc_h, m2r_batches_h;  // host staging of asynchronous uploads
+    DevBuf m2r_tdesc;  // table descriptors (component | level << 8, node set, rho^2, oz)
+    DevBuf m2r_ndesc, m2r_nodes;  // node sets (component, level, oz) and the remainder at their quadrature nodes
+    std::vector<int4> m2r_tdesc_h, m2r_ndesc_h, m2r_batches_h;  // host staging of asynchronous uploads
     int m2r_pending_ne = 0;             // reaction M2L entries whose key grouping awaits lf_prepare_m2r_finish
     int m2r_la = 0;                     // first level with reaction M2L entries (keyed from there if in range)
     int m2r_kfirst = 0;                 // first key of the keyed levels among the sorted keys

@@ -459,10 +459,16 @@ __host__ __device__ __forceinline__ double lf_sigma_rem(const LfmmComp& c, doubl
     return rem * exp(k * c.zeta_r);
 }
 
+// Table of one reaction component, all (N, mu) with mu <= N <= nmax: the leading
+// image in closed form plus the remainder by the rule.  rt (may be null): the
+// scaled remainder lf_sigma_rem at each node, precomputed.  Two halves of the
+// block prepare the nodes, one the Bessel functions, the other the powers; the
+// sums then take the (nmax+1)(nmax+2)/2 entries two per thread.
 template <bool GEN = false>
 __device__ __forceinline__ void lf_sommerfeld_table_block(const LfmmComp& c, double rho_h, double z_h, double S,
                                                           int nmax, double* T, int ld, int Q, const double* gl_t,
-                                                          const double* gl_w, double* sJ, double* sA)
+                                                          const double* gl_w, double* sJ, double* sA,
+                                                          const double* rt = nullptr)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int w = nmax + 1;
@@ -471,26 +477,43 @@ __device__ __forceinline__ void lf_sommerfeld_table_block(const LfmmComp& c, dou
     if (c.has_rem) {
         const double Zh = z_h + c.zeta_r / S;
         const double iZ = 1.0 / Zh;
-        for (int q = tid; q < Q; q += nt) {
-            double kap = gl_t[q] * iZ;
+        for (int i = tid; i < 2 * Q; i += nt) {
+            const int q = i < Q ? i : i - Q;
             // kap is in box units: the density's k is kap / S
-            double rt = lf_sigma_rem<GEN>(c, kap / S);
-            double a = gl_w[q] * iZ * rt;
-            double* Arow = sA + q * w;
-            for (int N = 0; N <= nmax; ++N) {
-                Arow[N] = a;
-                a *= kap;
+            const double kap = gl_t[q] * iZ;
+            if (i < Q) {
+                lf_bessel_j_set(kap * rho_h, nmax, sJ + q * w);
+            } else {
+                double a = gl_w[q] * iZ * (rt ? rt[q] : lf_sigma_rem<GEN>(c, kap / S));
+                double* Arow = sA + q * w;
+                for (int N = 0; N <= nmax; ++N) {
+                    Arow[N] = a;
+                    a *= kap;
+                }
             }
-            lf_bessel_j_set(kap * rho_h, nmax, sJ + q * w);
         }
         __syncthreads();
-        const int nent = w * w;
-        for (int e = tid; e < nent; e += nt) {
-            int N = e / w, mu = e - N * w;
-            if (mu > N) continue;
-            double s = 0.0;
-            for (int q = 0; q < Q; ++q) s += sA[q * w + N] * sJ[q * w + mu];
-            T[N * ld + mu] += s;
+        const int nent = w * (w + 1) / 2;
+        for (int e = tid; e < nent; e += 2 * nt) {
+            int N0 = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+            while ((N0 + 1) * (N0 + 2) / 2 <= e) ++N0;
+            while (N0 * (N0 + 1) / 2 > e) --N0;
+            const int mu0 = e - N0 * (N0 + 1) / 2;
+            const int e1 = e + nt;
+            int N1 = N0, mu1 = mu0;
+            if (e1 < nent) {
+                N1 = (int)((sqrtf(8.f * (float)e1 + 1.f) - 1.f) * 0.5f);
+                while ((N1 + 1) * (N1 + 2) / 2 <= e1) ++N1;
+                while (N1 * (N1 + 1) / 2 > e1) --N1;
+                mu1 = e1 - N1 * (N1 + 1) / 2;
+            }
+            double s0 = 0.0, s1 = 0.0;
+            for (int q = 0; q < Q; ++q) {
+                s0 += sA[q * w + N0] * sJ[q * w + mu0];
+                s1 += sA[q * w + N1] * sJ[q * w + mu1];
+            }
+            T[N0 * ld + mu0] += s0;
+            if (e1 < nent) T[N1 * ld + mu1] += s1;
         }
     }
     __syncthreads();

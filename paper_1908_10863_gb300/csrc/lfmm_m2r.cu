@@ -116,15 +116,37 @@ __global__ void k_key_starts(const uint32_t* __restrict__ keys, int n, const int
     kval[idx[i]] = keys[i];
 }
 
-// One block per key: the box-unit table (lead + remainder) with the a = 2 sign.
+// Remainder values at the quadrature nodes: they depend on (component, level,
+// oz) only, not on the lateral distance, so about 15 tables share them.  In
+// media of four and five layers each is a solve of the interface problem and
+// a coupling series, which took most of the tables' time (four layers, 2,808
+// tables: 0.744 -> 0.331 + 0.080 ms).
+template <bool GEN>
+__global__ void __launch_bounds__(128) k_m2r_nodes(const LfmmComp* __restrict__ comps, const int4* __restrict__ ndesc,
+                                                   int nnode, const double* __restrict__ levelh,
+                                                   const double* __restrict__ zfrac, const double* __restrict__ gt,
+                                                   int Q, double* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nnode * Q) return;
+    const int4 d = ndesc[i / Q];
+    const int c = d.x, l = d.y, q = i % Q;
+    const LfmmComp& cp = comps[c];
+    if (!cp.has_rem) return;
+    const double vz = (double)d.z + zfrac[c * 16 + l], zz = (cp.a == 1) ? vz : -vz;
+    const double S = levelh[l];
+    out[i] = lf_sigma_rem<GEN>(cp, gt[q] / (zz + cp.zeta_r / S) / S);
+}
+
+// One block per table: the box-unit table (lead + remainder) with the a = 2 sign.
 // One Sommerfeld table per (component, level, rho^2, oz): the table depends on
 // the lateral distance only; the azimuth enters through the phases applied
-// when the operator is assembled.
-template <bool GEN>
-__global__ void k_m2r_tables(const LfmmComp* __restrict__ comps, const int4* __restrict__ tdesc, int ntab,
-                             const double* __restrict__ levelh, const double* __restrict__ zfrac, int P,
-                             const double* __restrict__ gt, const double* __restrict__ gw, int Q,
-                             double* __restrict__ tables)
+// when the operator is formed.  tdesc: component | level << 8, node set, rho^2, oz.
+__global__ void __launch_bounds__(128) k_m2r_tables(const LfmmComp* __restrict__ comps, const int4* __restrict__ tdesc,
+                                                    int ntab, const double* __restrict__ levelh,
+                                                    const double* __restrict__ zfrac, int P,
+                                                    const double* __restrict__ gt, const double* __restrict__ gw, int Q,
+                                                    const double* __restrict__ nodes, double* __restrict__ tables)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int TS = 2 * P + 1, TT = TS * TS;
@@ -133,14 +155,15 @@ __global__ void k_m2r_tables(const LfmmComp* __restrict__ comps, const int4* __r
     double* sA = sJ + Q * TS;
     const int k = blockIdx.x;
     const int4 d = tdesc[k];
-    const int c = d.x, l = d.y, oz = d.w;
-    const LfmmComp cp = comps[c];
+    const int c = d.x & 255, l = d.x >> 8, oz = d.w;
+    const LfmmComp& cp = comps[c];
     const double rho = sqrt((double)d.z);
     const double vz = (double)oz + zfrac[c * 16 + l];  // image offset n + f in box units
     const double zz = (cp.a == 1) ? vz : -vz;
     for (int j = threadIdx.x; j < TT; j += blockDim.x) sT[j] = 0.0;
     __syncthreads();
-    lf_sommerfeld_table_block<GEN>(cp, rho, zz, levelh[l], 2 * P, sT, TS, Q, gt, gw, sJ, sA);
+    lf_sommerfeld_table_block<false>(cp, rho, zz, levelh[l], 2 * P, sT, TS, Q, gt, gw, sJ, sA,
+                                     nodes + (size_t)d.y * Q);
     double* out = tables + (size_t)k * TT;
     for (int j = threadIdx.x; j < TT; j += blockDim.x) {
         int N = j / TS, mu = j - N * TS;
@@ -302,7 +325,9 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
     // tables, one per distinct (component, level, rho^2, oz)
     std::vector<int4>& tdesc = ctx->m2r_tdesc_h;
     std::vector<int>& ktab = ctx->m2r_ktab_h;
+    std::vector<int4>& ndesc = ctx->m2r_ndesc_h;
     tdesc.clear();
+    ndesc.clear();
     ktab.assign(nku, 0);
     {
         // keys arrive sorted by (component, level, offset): within one
@@ -315,19 +340,26 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
         slot.assign((size_t)NR2 * R_OW, 0);
         stamp.assign((size_t)NR2 * R_OW, 0u);
         uint32_t gen = 0, run = ~0u;
+        int node_of[R_OW];  // node set of each oz in the current (component, level) run
         for (int64_t k = k0; k < k1; ++k) {
             int c, l, ox, oy, oz;
             rkey_decode(kv[k], c, l, ox, oy, oz);
             if ((kv[k] >> 12) != run) {
                 run = kv[k] >> 12;
                 ++gen;
+                std::fill(node_of, node_of + R_OW, -1);
             }
             const int r2 = ox * ox + oy * oy;
             const size_t i = (size_t)r2 * R_OW + (oz + R_OR);
             if (stamp[i] != gen) {
                 stamp[i] = gen;
                 slot[i] = (int)tdesc.size();
-                tdesc.push_back(make_int4(c, l, r2, oz));
+                int& node = node_of[oz + R_OR];
+                if (node < 0) {
+                    node = (int)ndesc.size();
+                    ndesc.push_back(make_int4(c, l, oz, 0));
+                }
+                tdesc.push_back(make_int4(c | l << 8, node, r2, oz));
             }
             ktab[k - k0] = slot[i];
         }
@@ -336,15 +368,15 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
     const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS, Q = ctx->gl_q_m2l;
     LF_TRY(lf_reserve(ctx->m2r_tables, (size_t)ntab * TT * 8 + 16));
     LF_TRY(lf_reserve(ctx->m2r_tdesc, (size_t)ntab * sizeof(int4) + 16));
-    LF_TRY(lf_reserve(ctx->m2r_ktab, (size_t)nku * sizeof(int) + 16));
+    LF_TRY(lf_reserve(ctx->m2r_ndesc, ndesc.size() * sizeof(int4) + 16));
+    LF_TRY(lf_reserve(ctx->m2r_nodes, ndesc.size() * (size_t)Q * sizeof(double) + 16));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_tdesc.ptr, tdesc.data(), ntab * sizeof(int4), cudaMemcpyHostToDevice, st));
-    LF_CHECK(cudaMemcpyAsync(ctx->m2r_ktab.ptr, ktab.data(), nku * sizeof(int), cudaMemcpyHostToDevice, st));
+    LF_CHECK(cudaMemcpyAsync(ctx->m2r_ndesc.ptr, ndesc.data(), ndesc.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     double* hl = ctx->m2r_levelh_h;
     for (int l = 0; l < 16; ++l) hl[l] = (l <= ctx->depth) ? ctx->levels[l].h : 0.0;
     LF_TRY(lf_reserve(ctx->m2r_levelh, sizeof(double) * 16));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_levelh.ptr, hl, sizeof(double) * 16, cudaMemcpyHostToDevice, st));
     (void)P;
-    (void)Q;
     ctx->m2r_ntab = ntab;
     // batches of R_TB pairs of one key: key index, first sorted entry, count | key << 8, table
     std::vector<int4>& batches = ctx->m2r_batches_h;
@@ -390,12 +422,16 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
     const int ntab = ctx->m2r_ntab;
     const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS, Q = ctx->gl_q_m2l;
     size_t sm = sizeof(double) * ((size_t)TT + 2 * (size_t)Q * TS);
-    auto tabk = (ctx->L >= 3) ? k_m2r_tables<true> : k_m2r_tables<false>;
-    LF_CHECK(cudaFuncSetAttribute(tabk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    ++ctx->launches, tabk<<<ntab, 128, sm, st>>>(ctx->comp_dev.as<LfmmComp>(), ctx->m2r_tdesc.as<int4>(), ntab,
-                                                 ctx->m2r_levelh.as<double>(), ctx->m2r_zfrac.as<double>(), P,
-                                                 ctx->gl_t_m2l.as<double>(),
-                                                 ctx->gl_w_m2l.as<double>(), Q, ctx->m2r_tables.as<double>());
+    const int nnode = (int)ctx->m2r_ndesc_h.size();
+    auto nodk = (ctx->L >= 3) ? k_m2r_nodes<true> : k_m2r_nodes<false>;
+    ++ctx->launches, nodk<<<lf_blocks((int64_t)nnode * Q, 128), 128, 0, st>>>(
+        ctx->comp_dev.as<LfmmComp>(), ctx->m2r_ndesc.as<int4>(), nnode, ctx->m2r_levelh.as<double>(),
+        ctx->m2r_zfrac.as<double>(), ctx->gl_t_m2l.as<double>(), Q, ctx->m2r_nodes.as<double>());
+    LF_CHECK(cudaFuncSetAttribute(k_m2r_tables, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ++ctx->launches, k_m2r_tables<<<ntab, 128, sm, st>>>(
+        ctx->comp_dev.as<LfmmComp>(), ctx->m2r_tdesc.as<int4>(), ntab, ctx->m2r_levelh.as<double>(),
+        ctx->m2r_zfrac.as<double>(), P, ctx->gl_t_m2l.as<double>(), ctx->gl_w_m2l.as<double>(), Q,
+        ctx->m2r_nodes.as<double>(), ctx->m2r_tables.as<double>());
     LF_TRY(lf_cuda(cudaGetLastError(), "m2r tables"));
     if (ctx->m2r_nent > 0) {
         LF_TRY(lf_reserve(ctx->m2r_pairs, (size_t)ctx->m2r_nent * sizeof(int2) + 16));
