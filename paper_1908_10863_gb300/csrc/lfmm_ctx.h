@@ -129,6 +129,7 @@ struct lfmm_ctx {
     // tensor-core free M2L (float32 form, (p+1)^2 <= 128)
     DevBuf m2l_Atc, m2l_tc_tiles, m2l_Ms;
     DevBuf tc_cscale, tc_perm;     // 2^e of every packed coefficient (float16 operand scaling); K order
+    int tc_nk = 0;                 // K positions (coefficients, and one hole for even p)
     DevBuf tc_mseg;  // runs of the merged tensor-core tiles, [merged tile][LFMM_TC_MSEG] int4 (level, start, count, 0)
     DevBuf l2l_Atc, tc_shift_tiles;  // tensor-core L2L operators (into the leaves) and tiles
     std::vector<int> tc_l2l_first;   // first tensor-core translation tile of each level

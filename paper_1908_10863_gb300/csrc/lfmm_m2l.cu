@@ -713,11 +713,12 @@ static LfErr launch_gemm(lfmm_ctx* ctx, cudaStream_t st, const GemmArgs& g, int 
         if (g.noff == G_NOFF && !g.split) return launch_one<R, RP, RM, true>(ctx, st, g, nblk);
     }
     // shared rows: FP64, or too few blocks for two per SM
-    if constexpr (RM > 2) {
-        if (sizeof(R) == 8 || (int64_t)nblk * ctx->nrhs_b < 2 * 152)
-            return launch_one<R, RP, 2, false>(ctx, st, g, nblk);
+    if constexpr (sizeof(R) == 8) {
+        return launch_one<R, RP, 2, false>(ctx, st, g, nblk);
+    } else {
+        if (RM > 2 && (int64_t)nblk * ctx->nrhs_b < 2 * 152) return launch_one<R, RP, 2, false>(ctx, st, g, nblk);
+        return launch_one<R, RP, RM, false>(ctx, st, g, nblk);
     }
-    return launch_one<R, RP, RM, false>(ctx, st, g, nblk);
 }
 
 template <typename R>

@@ -137,7 +137,7 @@ struct TcArgs {
     int gslot;              // slot of the source level: the target's level + gslot
     float* L;               // locals [box][nc]
     int nc;
-    int nkc;                // K chunks of TH_KC coefficients that hold the nc inputs: ceil(nc / TH_KC)
+    int nk, nkc;            // K positions in use, and chunks of TH_KC that hold them
     size_t ms_stride;       // per right-hand side (blockIdx.y): split multipoles, in halves
     size_t l_stride;        // per right-hand side: local expansions, in floats
     int groups;             // CTAs per tile (offset groups; divides noff)
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(TC_THREADS, WIDE ? 1 : TC_MINB) k_m2l_tc(TcArg
                 // the small products first: a2 x1, a1 x2, a1 x1
                 const int pa[3] = {1, 0, 0}, px[3] = {0, 1, 0};
                 // K steps of 16 that hold coefficients (both but in an operator's last chunk)
-                const int nks = (nc - (nkc - 1 - it / nact) * TH_KC) > 16 ? 2 : 1;
+                const int nks = (g.nk - (nkc - 1 - it / nact) * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
                 for (int prod = 0; prod < 3; ++prod) {
                     const uint32_t a = base + pa[prod] * ABYTES;
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
                     const uint32_t base = smem_u32(sm + (size_t)s * TC_STAGE_BYTES);
                     const uint32_t xb = base + TC_AP * TC_A_BYTES;
                     const int pa[3] = {1, 0, 0}, px[3] = {0, 1, 0};  // a2 x1, a1 x2, a1 x1
-                    const int nks = (nc - (g.nkc - 1 - j / goff) * TH_KC) > 16 ? 2 : 1;
+                    const int nks = (g.nk - (g.nkc - 1 - j / goff) * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
                     for (int prod = 0; prod < 3; ++prod) {
                         const uint32_t a = base + pa[prod] * TC_A_BYTES;
@@ -656,13 +656,27 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
 // ---------------------------------------------------------------------------
 // Host: operator blob and launch.
 // ---------------------------------------------------------------------------
-// packed index of the K-th input coefficient: by degree, Re before Im
+// Packed index of the K-th input coefficient, by degree, in pairs at even
+// positions: Re and Im of (n, m) for m >= 1, and the real (n, 0) of two
+// successive degrees (-1: no coefficient).  The reaction M2L forms its operators
+// pair by pair (lfmm_m2r.cu).
 static void coef_order(int p, std::vector<int>& perm)
 {
     perm.clear();
     for (int n = 0; n <= p; ++n) {
-        for (int m = 0; m <= n; ++m) perm.push_back(lf_re(n, m));
-        for (int m = 1; m <= n; ++m) perm.push_back(lf_im(p, n, m));
+        if (n & 1) {
+            perm.push_back(lf_re(n - 1, 0));
+            perm.push_back(lf_re(n, 0));
+        }
+        // (the pair of singles goes before the larger of its two degrees)
+        for (int m = 1; m <= n; ++m) {
+            perm.push_back(lf_re(n, m));
+            perm.push_back(lf_im(p, n, m));
+        }
+    }
+    if (!(p & 1)) {
+        perm.push_back(lf_re(p, 0));
+        perm.push_back(-1);
     }
 }
 
@@ -687,7 +701,7 @@ static void coef_exponents(int p, std::vector<int>& e)
 // pieces stay below 2^13; an entry beyond float16's range is counted in bad.
 // One block per (operator, K chunk).
 #define TC_ASHIFT 12
-__global__ void __launch_bounds__(256) k_tc_blob(const double* __restrict__ A, int KP, int RP, int nc,
+__global__ void __launch_bounds__(256) k_tc_blob(const double* __restrict__ A, int KP, int RP, int nc, int nk,
                                                  const int* __restrict__ perm, const float* __restrict__ cs, int sin,
                                                  int mh, unsigned char* __restrict__ blob, int* __restrict__ bad)
 {
@@ -696,7 +710,7 @@ __global__ void __launch_bounds__(256) k_tc_blob(const double* __restrict__ A, i
     for (int i = threadIdx.x; i < TH_KC * mh * TC_M; i += 256) {
         const int k = i / (mh * TC_M), r = i - k * (mh * TC_M), kk = kc * TH_KC + k;
         double v = 0.0;
-        if (kk < nc && r < nc) {
+        if (kk < nk && r < nc && perm[kk] >= 0) {
             const int kin = perm[kk];
             const double si = sin < 0 ? 1.0 / (double)cs[kin] : (double)cs[kin];
             v = A[((size_t)o * KP + kin) * RP + r] * si / (double)cs[r] * (double)(1 << TC_ASHIFT);
@@ -719,7 +733,7 @@ static LfErr tc_blob(lfmm_ctx* ctx, const DevBuf& A64, int nops, int KP, int RP,
     int* bad = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
     LF_CHECK(cudaMemsetAsync(bad, 0, sizeof(int), ctx->s_main));
     ++ctx->launches, k_tc_blob<<<nops * nkc, 256, 0, ctx->s_main>>>(
-        A64.as<double>(), KP, RP, lf_nc(ctx->p), ctx->tc_perm.as<int>(), ctx->tc_cscale.as<float>(), sin, mh,
+        A64.as<double>(), KP, RP, lf_nc(ctx->p), ctx->tc_nk, ctx->tc_perm.as<int>(), ctx->tc_cscale.as<float>(), sin, mh,
         out.as<unsigned char>(), bad);
     LF_TRY(lf_cuda(cudaGetLastError(), "tensor-core operators"));
     int n = 0;
@@ -743,8 +757,9 @@ LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP)
     for (int k = 0; k < nc; ++k) cs[k] = std::ldexp(1.f, e[k]);
     LF_TRY(lf_reserve(ctx->tc_cscale, nc * sizeof(float)));
     LF_CHECK(cudaMemcpy(ctx->tc_cscale.ptr, cs.data(), nc * sizeof(float), cudaMemcpyHostToDevice));
-    LF_TRY(lf_reserve(ctx->tc_perm, nc * sizeof(int)));
-    LF_CHECK(cudaMemcpy(ctx->tc_perm.ptr, perm.data(), nc * sizeof(int), cudaMemcpyHostToDevice));
+    ctx->tc_nk = (int)perm.size();
+    LF_TRY(lf_reserve(ctx->tc_perm, perm.size() * sizeof(int)));
+    LF_CHECK(cudaMemcpy(ctx->tc_perm.ptr, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice));
     // the wide form serves the free M2L only; L2L stays on the CUDA cores
     // (the uploads above ran on the legacy stream, which s_main does not wait for)
     LF_CHECK(cudaDeviceSynchronize());
@@ -817,7 +832,7 @@ __global__ void __launch_bounds__(256) k_tc_max(const float* __restrict__ X, int
 // mrow halves (128, or 256 for the wide form) in K order, for the boxes b0 ..
 // b0 + count - 1 (the arrays hold nbox boxes per right-hand side, blockIdx.y); one thread
 // per 8 coefficients
-__global__ void __launch_bounds__(256) k_split_m(const float* __restrict__ M, int nbox, int nc, int mrow, int b0,
+__global__ void __launch_bounds__(256) k_split_m(const float* __restrict__ M, int nbox, int nc, int nk, int mrow, int b0,
                                                  int count, const float* __restrict__ cs, int inv,
                                                  const __grid_constant__ TcLevels lv,
                                                  int slot0, const unsigned* __restrict__ gmax,
@@ -835,8 +850,8 @@ __global__ void __launch_bounds__(256) k_split_m(const float* __restrict__ M, in
     for (int u = 0; u < 8; ++u) {
         const int k = k0 + u;
         float x = 0.f;
-        if (k < nc) {
-            const int j = perm[k];
+        const int j = k < nk ? perm[k] : -1;
+        if (j >= 0) {
             x = M[(size_t)b * nc + j] * (inv ? 1.f / cs[j] : cs[j]) * s;
         }
         hi[u] = __float2half_rn(x);
@@ -866,7 +881,7 @@ static LfErr split_boxes(lfmm_ctx* ctx, const float* src, int b0, int count, int
         src, nb, nc, b0, count, ctx->tc_cscale.as<float>(), locals, lv, 16 * locals, gm);
     const int64_t tot = (int64_t)count * (mrow / 8);
     ++ctx->launches, k_split_m<<<dim3((unsigned)((tot + 255) / 256), nr), 256, 0, st>>>(
-        src, nb, nc, mrow, b0, count, ctx->tc_cscale.as<float>(), locals, lv, 16 * locals, gm,
+        src, nb, nc, ctx->tc_nk, mrow, b0, count, ctx->tc_cscale.as<float>(), locals, lv, 16 * locals, gm,
         ctx->tc_perm.as<int>(), ctx->m2l_Ms.as<__half>());
     return lf_cuda(cudaGetLastError(), "split");
 }
@@ -883,7 +898,8 @@ static TcArgs tc_args(lfmm_ctx* ctx)
     g.ms_stride = (size_t)nb * TC_XP * ms_row(ctx);
     g.l_stride = (size_t)nb * lf_nc(ctx->p);
     g.nc = lf_nc(ctx->p);
-    g.nkc = (g.nc + TH_KC - 1) / TH_KC;
+    g.nk = ctx->tc_nk;
+    g.nkc = (g.nk + TH_KC - 1) / TH_KC;
     g.err = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
     return g;
 }

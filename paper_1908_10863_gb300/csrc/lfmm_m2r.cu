@@ -623,11 +623,15 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 // operators (lfmm_m2l_tc.cu: 2^{-e} per coefficient, folded into the signs
 // below).  The source multipoles (B operand) are the scaled float16 pieces
 // which that M2L split once per evaluation, gathered by 16-byte cp.async;
-// products a2 x1 + a1 x2 + a1 x1.  Operator entries come from a table of the
-// reaction coefficient extended to negative orders, so each is two
-// shared-memory loads and a fused multiply-add with signs and offsets
-// precomputed per output row and input coefficient; forming them bounds the
-// kernel.  While the tensor cores take one chunk the threads form the next.
+// products a2 x1 + a1 x2 + a1 x1.  Operator entries come from a table W of the
+// complex reaction coefficient extended to negative orders.  They are formed in
+// blocks of two rows (Re and Im of an output (k, l)) by two columns (Re and Im
+// of an input (n, m)): the four entries are sums and differences of the parts
+// of W(n+k, l+m) and W(n+k, l-m), so a block costs two 8-byte loads (one entry
+// at a time took two 4-byte loads and two of offsets and signs each, and the
+// shared-memory pipe bounded the kernel).  Orders m = 0 have one part only; two
+// of them share a row or column pair.  While the tensor cores take one chunk
+// the threads form the next.
 //   V = 1: one vector, A and X of a chunk in two buffers (48 KB), three CTAs
 // per SM, which leaves room for the near field beside it.
 //   V = 2: several vectors; the whole operator (64 KB) is formed once and kept,
@@ -637,8 +641,8 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 // scales and add it into the targets' local expansions.  Every wait is
 // bounded: on a timeout the CTA counts it in err and skips its read-backs.
 // Measured, p = 10, float16 pieces against TF32 pieces with the operator formed
-// again for every vector: 64 vectors of 262,144 charges 13.8 -> 4.95 ms; one
-// vector 0.258 -> 0.250 ms (operator formation).
+// again for every vector: 64 vectors of 262,144 charges 13.8 -> 4.95 ms.  One
+// vector, N = 1M: 0.258 ms with entries formed one at a time, 0.170 ms in blocks.
 // ---------------------------------------------------------------------------
 #define RT_THREADS 256
 #define RT_TS 21                        // table side 2p + 1 for p <= 10
@@ -659,7 +663,7 @@ struct RtShape {
 };
 
 struct RTcArgs {
-    int p, nc, nkc;         // order, coefficients, K chunks of 32 that hold them
+    int p, nc, nk, nkc;     // order, coefficients, K positions, chunks of 32 that hold them
     const int4* batches;    // key index, first sorted entry, count | key << 8, table
     const double* tables;   // [table][TS][TS]
     const LfmmComp* comps;
@@ -700,15 +704,16 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
                                                          ~(uintptr_t)511);
     unsigned char* smx = sm + S::NA * 2 * RT_A_CHUNK;
     // W(N, mu) = T(N, |mu|) e^{i mu phi} for mu in [-2p, 2p], extended to
-    // negative orders by W(N, -mu) = (-1)^mu conj W(N, mu); real parts, then
-    // imaginary parts, each [N][mu + 2p] with rows of 4p + 1
-    __shared__ float sW[2 * RT_TS * RT_WS];
+    // negative orders by W(N, -mu) = (-1)^mu conj W(N, mu); [N][mu + 2p], rows of 4p + 1
+    __shared__ float2 sW[RT_TS * RT_WS];
     __shared__ float sPh[2 * RT_TS];
-    __shared__ int2 s_off[2][128];   // per output parity aim and K position: offsets of the two W terms
-    __shared__ float2 s_cf[2][128];  // their signs and scales (0: no second term, or no such input)
-    __shared__ int s_roff[128];      // per output coefficient (k, l): k (4p + 1) + l + 2p
-    __shared__ float s_sk[128];      // (-1)^k with the row's scale, 0 past the last coefficient
-    __shared__ unsigned char s_aim[128];
+    // column pairs: offsets of the two W terms from the row's, their signs and
+    // scales; y < 0: two real inputs (n, 0), -1 - offset of the second
+    __shared__ int2 s_co[64];
+    __shared__ float2 s_cf[64];
+    // row pairs: packed rows (y = -1: none), offsets; z == w: Re and Im of one (k, l)
+    __shared__ int4 s_row[64];
+    __shared__ float2 s_rk[64];  // (-1)^k with the rows' scales
     __shared__ int s_src[R_TB], s_tgt[R_TB];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t s_tmem;
@@ -724,37 +729,62 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
     rkey_decode((uint32_t)b.z >> 8, c, lev, ox, oy, oz);
     const bool refl = g.comps[c].refl != 0;
 
-    if (tid < 128) {
-        // packed coefficient tid as an output row
-        int n = 0, m = 0, im = 0;
-        const bool in = tid < nc;
-        if (in) lf_decode(p, tid, n, m, im);
-        s_roff[tid] = in ? n * WS + m + 2 * p : 0;
-        s_sk[tid] = in ? ((n & 1) ? -1.f : 1.f) * (float)(1 << RT_ASHIFT) / g.cscale[tid] : 0.f;
-        s_aim[tid] = (unsigned char)im;
-    } else {
-        // K position k as an input column
-        const int k = tid - 128;
-        const bool in = k < nc;
-        int n = 0, m = 0, im = 0;
-        float sc = 0.f;
-        if (in) {
-            const int j = g.perm[k];
-            lf_decode(p, j, n, m, im);
-            sc = 1.f / g.cscale[j];
+    if (tid < 64) {
+        // row pair tid: the (k, l) with l >= 1, then the (k, 0) two at a time
+        const int nl = p * (p + 1) / 2;
+        int4 r = make_int4(-1, -1, 0, 0);
+        float2 sk = make_float2(0.f, 0.f);
+        const float as = (float)(1 << RT_ASHIFT);
+        if (tid < nl) {
+            int k = 1, t = tid;
+            while (t >= k) t -= k++;
+            const int l = t + 1;
+            r = make_int4(lf_re(k, l), lf_im(p, k, l), k * WS + l + 2 * p, k * WS + l + 2 * p);
+            sk.x = sk.y = ((k & 1) ? -as : as) / g.cscale[r.x];
+        } else {
+            const int k = 2 * (tid - nl);
+            if (k <= p) {
+                r.x = lf_re(k, 0);
+                r.z = k * WS + 2 * p;
+                r.w = -1;  // (not an Re / Im pair)
+                sk.x = as / g.cscale[r.x];
+            }
+            if (k + 1 <= p) {
+                r.y = lf_re(k + 1, 0);
+                r.w = (k + 1) * WS + 2 * p;
+                sk.y = -as / g.cscale[r.y];
+            }
         }
-        // the multipole's reflection sign (-1)^{n+m} for s = -1 maps
-        const float rs = (refl && ((n + m) & 1)) ? -sc : sc;
-        const float sg = (m & 1) ? -1.f : 1.f;  // (-1)^m of the second term
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const int t = (a ^ im) * TSZ;  // real parts where the parities agree, else imaginary
-            s_off[a][k] = in ? make_int2(t + n * WS + m, t + n * WS - m) : make_int2(0, 0);
-            // (re,re): W1 + sg W2; (re out, im in): -W1 + sg W2; (im, re): W1 + sg W2; (im, im): W1 - sg W2
-            const float c1 = (a == 0 && im == 1) ? -1.f : 1.f;
-            const float c2 = m > 0 ? ((a == 1 && im == 1) ? -sg : sg) : 0.f;
-            s_cf[a][k] = make_float2(rs * c1, rs * c2);
+        s_row[tid] = r;
+        s_rk[tid] = sk;
+    } else if (tid < 128) {
+        // column pair: K positions 2c and 2c + 1
+        const int c2 = 2 * (tid - 64);
+        int2 o = make_int2(0, 0);
+        float2 f = make_float2(0.f, 0.f);
+        if (c2 < g.nk) {
+            const int j0 = g.perm[c2], j1 = g.perm[c2 + 1];
+            int n, m, im;
+            lf_decode(p, j0, n, m, im);
+            // the multipole's reflection sign (-1)^{n+m} for s = -1 maps, and (-1)^m of the second term
+            const float c = (refl && ((n + m) & 1) ? -1.f : 1.f) / g.cscale[j0];
+            if (m > 0) {
+                o = make_int2(n * WS + m, n * WS - m);
+                f = make_float2(c, (m & 1) ? -c : c);
+            } else {
+                o.x = n * WS;
+                f.x = c;
+                o.y = -1;
+                if (j1 >= 0) {
+                    int n1;
+                    lf_decode(p, j1, n1, m, im);
+                    o.y = -1 - n1 * WS;
+                    f.y = (refl && (n1 & 1) ? -1.f : 1.f) / g.cscale[j1];
+                }
+            }
         }
+        s_co[tid - 64] = o;
+        s_cf[tid - 64] = f;
     }
     if (tid < R_TB) {
         const int2 pr = (tid < cnt) ? g.pairs[start + tid] : make_int2(-1, -1);
@@ -788,15 +818,16 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
             if (mu < 0) {
                 if (a & 1) wr = -wr; else wi = -wi;
             }
-            sW[j] = wr;
-            sW[TSZ + j] = wi;
+            sW[j] = make_float2(wr, wi);
         }
     }
     const double hl = g.levelh[lev];
     __syncthreads();  // W is in shared memory
-    // gather and operator unit of every chunk: row xj (and xj + 64 of the operator), 16-byte quarter xq
+    // gather unit of every chunk: row xj, 16-byte quarter xq; operator unit: row pair xj, quarter xq
     const int xj = tid >> 2, xq = tid & 3;
     const int src = xj < Np ? s_src[xj] : -1;
+    const int4 rw = s_row[xj];
+    const float2 rk = s_rk[xj];
     bool ok = true;
     int gr = 0;  // round counter over the vectors
     for (int r0 = 0; r0 < g.nr && ok; r0 += V) {
@@ -825,26 +856,49 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
                 }
             }
             cp_async_commit();
-            if (!S::KEEP || r0 == 0) {
+            if ((!S::KEEP || r0 == 0) && rw.x >= 0) {
+                __align__(16) __half2 ha[4], la[4], hb[4], lb[4];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int row = xj + 64 * h;
-                    const float* W = sW + s_roff[row];
-                    const float sk = s_sk[row];
-                    const int a = s_aim[row];
-                    __align__(16) __half hi[8], lo[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int kin = kc * TH_KC + 8 * xq + e;
-                        const int2 o = s_off[a][kin];
-                        const float2 cf = s_cf[a][kin];
-                        const float v = sk * fmaf(cf.x, W[o.x], cf.y * W[o.y]);
-                        hi[e] = __float2half_rn(v);
-                        lo[e] = __float2half_rn(v - __half2float(hi[e]));
+                for (int e = 0; e < 4; ++e) {
+                    const int cp = kc * (TH_KC / 2) + 4 * xq + e;
+                    const int2 o = s_co[cp];
+                    const float2 f = s_cf[cp];
+                    const bool sg = o.y < 0;  // two real inputs
+                    const int o2 = sg ? -1 - o.y : o.y;
+                    const float2 x = sW[rw.z + o.x], y = sW[rw.z + o2];
+                    float a0, a1, b0, b1;
+                    if (rw.z == rw.w) {  // Re and Im of one output
+                        const float fy = sg ? 0.f : f.y;
+                        a0 = fmaf(f.x, x.x, fy * y.x);
+                        b0 = fmaf(f.x, x.y, fy * y.y);
+                        a1 = sg ? f.y * y.x : fmaf(-f.x, x.y, f.y * y.y);
+                        b1 = sg ? f.y * y.y : fmaf(f.x, x.x, -f.y * y.x);
+                    } else {  // two real outputs
+                        const int w2 = max(rw.w, 0);
+                        const float2 x2 = sW[w2 + o.x], y2 = sW[w2 + o2];
+                        a0 = sg ? f.x * x.x : fmaf(f.x, x.x, f.y * y.x);
+                        a1 = sg ? f.y * y.x : fmaf(-f.x, x.y, f.y * y.y);
+                        b0 = sg ? f.x * x2.x : fmaf(f.x, x2.x, f.y * y2.x);
+                        b1 = sg ? f.y * y2.x : fmaf(-f.x, x2.y, f.y * y2.y);
                     }
-                    const uint32_t off = swz16(row, 8 * xq);
-                    *reinterpret_cast<uint4*>(sa + off) = *reinterpret_cast<const uint4*>(hi);
-                    *reinterpret_cast<uint4*>(sa + RT_A_CHUNK + off) = *reinterpret_cast<const uint4*>(lo);
+                    a0 *= rk.x;
+                    a1 *= rk.x;
+                    b0 *= rk.y;
+                    b1 *= rk.y;
+                    ha[e] = __floats2half2_rn(a0, a1);
+                    hb[e] = __floats2half2_rn(b0, b1);
+                    const float2 fa = __half22float2(ha[e]), fb = __half22float2(hb[e]);
+                    la[e] = __floats2half2_rn(a0 - fa.x, a1 - fa.y);
+                    lb[e] = __floats2half2_rn(b0 - fb.x, b1 - fb.y);
+                }
+                // (rows past the last coefficient are never read back)
+                uint32_t off = swz16(rw.x, 8 * xq);
+                *reinterpret_cast<uint4*>(sa + off) = *reinterpret_cast<const uint4*>(ha);
+                *reinterpret_cast<uint4*>(sa + RT_A_CHUNK + off) = *reinterpret_cast<const uint4*>(la);
+                if (rw.y >= 0) {
+                    off = swz16(rw.y, 8 * xq);
+                    *reinterpret_cast<uint4*>(sa + off) = *reinterpret_cast<const uint4*>(hb);
+                    *reinterpret_cast<uint4*>(sa + RT_A_CHUNK + off) = *reinterpret_cast<const uint4*>(lb);
                 }
             }
             cp_async_wait<0>();
@@ -858,7 +912,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
             if (tid == 0) {
                 tc_fence_after();
                 const uint32_t a0 = smem_u32(sa), x0 = smem_u32(sx);
-                const int nks = (nc - kc * TH_KC) > 16 ? 2 : 1;
+                const int nks = (g.nk - kc * TH_KC) > 16 ? 2 : 1;
 #pragma unroll
                 for (int prod = 0; prod < 3; ++prod) {  // a2 x1, a1 x2, a1 x1
                     const uint32_t a = a0 + (prod == 0 ? RT_A_CHUNK : 0);
@@ -958,7 +1012,8 @@ static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
     RTcArgs g;
     g.p = ctx->p;
     g.nc = lf_nc(ctx->p);
-    g.nkc = (g.nc + TH_KC - 1) / TH_KC;
+    g.nk = ctx->tc_nk;
+    g.nkc = (g.nk + TH_KC - 1) / TH_KC;
     g.batches = ctx->m2r_batches.as<int4>();
     g.tables = ctx->m2r_tables.as<double>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
