@@ -151,9 +151,9 @@ struct lfmm_ctx {
     // use_tc: 2 automatic and 1: tensor cores, 0: CUDA cores
     int m2l_tc_ok = 0, m2l_tc_ntiles = 0, use_tc = 2, tc_groups = 0;  // tc_groups 0: automatic
     // FP64 free M2L by digit products (lfmm_m2l_oz.cu)
-    DevBuf oz_A, oz_Ms, oz_cscale, oz_tiles, oz_mseg;
+    DevBuf oz_A, oz_Ms, oz_cscale, oz_perm, oz_emin, oz_tiles, oz_mseg;
     std::vector<int4> oz_tiles_h, oz_mseg_h;
-    int oz_ntiles = 0, oz_ready = 0;
+    int oz_ntiles = 0, oz_ready = 0, oz_nk = 0;
     int m2l_tc_wide = 0;  // tensor-core free M2L in its wide form ((p+1)^2 > 128): no tensor-core M2M / L2L
     // reaction M2L grouped by geometry key on interface-aligned levels
     DevBuf m2r_keys, m2r_order, m2r_tgt, m2r_kstart, m2r_kval, m2r_tables, m2r_levelh, m2r_batches;
@@ -313,7 +313,10 @@ LfErr lf_tc_split(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st);
 // ---- FP64 free M2L by digit products (lfmm_m2l_oz.cu) ----
 bool lf_m2l_oz_ok(const lfmm_ctx* ctx);
+LfErr lf_oz_split(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st);
+void lf_coef_order(int p, std::vector<int>& perm);
+void lf_coef_exponents(int p, std::vector<int>& e);
 int lf_m2l_tc_tile(const lfmm_ctx* ctx);
 LfErr lf_surrogate_alloc(lfmm_ctx* ctx);
 LfErr lf_surrogate_pack(lfmm_ctx* ctx, int comp);

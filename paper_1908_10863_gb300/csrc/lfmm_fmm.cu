@@ -655,10 +655,13 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
     LF_CHECK(cudaMemsetAsync(L, 0, sizeof(R) * ms * nr, st));
     const bool gemm = ctx->m2l_ntiles > 0;
     const bool tc = sizeof(R) == 4 && lf_tc_on(ctx);
+    const bool oz = sizeof(R) == 8 && lf_m2l_oz_ok(ctx);
     if (tc && !(gemm && ctx->m2l_tc_ntiles > 0) && ctx->m2r_nbatch > 0) LF_TRY(lf_tc_split(ctx, st));
+    if (oz && !(gemm && ctx->oz_ntiles > 0) && ctx->m2r_nbatch > 0) LF_TRY(lf_oz_split(ctx, st));
     if (gemm) {
         ph = lf_prof_start(ctx, LFMM_TIME_M2L_FREE, st);
         if (tc && ctx->m2l_tc_ntiles > 0) LF_TRY(lf_tc_split(ctx, st));
+        if (oz && ctx->oz_ntiles > 0) LF_TRY(lf_oz_split(ctx, st));
         if (tc && ctx->m2l_tc_ntiles > 0)
             LF_TRY(lf_m2l_tc(ctx, st));
         else

@@ -63,14 +63,11 @@
         if (!r_.empty()) return r_; \
     } while (0)
 
-#define OZ_S 7                            // digits per operand
-#define OZ_B 9                            // bits per digit
 #define OZ_N LFMM_OZ_TILE                 // targets per tile (MMA N)
 #define OZ_NOFF 189
 #define OZ_NALL 343
 #define OZ_WARPS 8
 #define OZ_THREADS (32 * OZ_WARPS + 32)
-#define OZ_A_BYTES (128 * TC_ROWB)        // one operator digit of a stage
 #define OZ_X_BYTES (OZ_N * TC_ROWB)       // one multipole digit of a stage
 #define OZ_STAGE (OZ_S * (OZ_A_BYTES + OZ_X_BYTES))
 #define OZ_NST 2
@@ -87,32 +84,17 @@ struct OzArgs {
     const int4* mseg;
     const unsigned char* A;  // [343][half][chunk][digit][8 KB], pre-swizzled
     const __half* Ms;        // digits [box][OZ_S][mrow]
-    const double* cscale;    // 2^e per coefficient
+    const double* cscale;    // 2^e per packed coefficient
     const unsigned long long* gmax;  // largest scaled coefficient (double bits), [16] per right-hand side
     double* L;
-    int nc, nkc, nh, mrow, groups, win;
+    int nc, nk, nkc, nh, mrow, groups, win;
     size_t ms_stride, l_stride;
     int* err;
 };
 
-// power of two that takes the largest magnitude (double bits) into [1/4, 1/2)
-__device__ __forceinline__ double oz_scale(unsigned long long bits)
-{
-    if (bits == 0ull || bits >= 0x7ff0000000000000ull) return 1.0;
-    int e = 1021 - (int)(bits >> 52);  // -2 - (biased exponent - 1023)
-    e = e > 1020 ? 1020 : (e < -1020 ? -1020 : e);
-    return __longlong_as_double((long long)(e + 1023) << 52);
-}
-
-// the OZ_S digits of t, |t| < 1/2, as float16 integers, leading digit first.
-// A NaN stays one (in the leading digit).
+// the OZ_S digits of t, |t| < 1/2, as float16 integers, leading digit first
 __device__ __forceinline__ void oz_digits(double t, __half d[OZ_S])
 {
-    if (!(fabs(t) <= 0.5)) {
-        d[0] = __float2half_rn(nanf(""));
-        for (int i = 1; i < OZ_S; ++i) d[i] = __float2half_rn(0.f);
-        return;
-    }
     long long v = __double2ll_rn(t * 9223372036854775808.0);  // 2^63
 #pragma unroll
     for (int i = OZ_S - 1; i > 0; --i) {
@@ -326,7 +308,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(OzArgs g)
                 }
                 tc_fence_after();
                 const uint32_t ab = smem_u32(sm + (size_t)s * OZ_STAGE), xb = ab + OZ_S * OZ_A_BYTES;
-                const int nks = (nc - (it % nkc) * TH_KC) > 16 ? 2 : 1;
+                const int nks = (g.nk - (it % nkc) * TH_KC) > 16 ? 2 : 1;
                 for (int ks = 0; ks < nks; ++ks)
 #pragma unroll
                     for (int i = 0; i < OZ_S; ++i)
@@ -354,18 +336,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(OzArgs g)
 // Operands.
 // ---------------------------------------------------------------------------
 // FP64 operators A [343][KP in][RP out] -> digits, one block per (offset, half,
-// chunk); rows r of the half, K elements k of the chunk.  Entries scaled by
+// chunk); rows r of the half, K elements k of the chunk (inputs in the order of
+// lf_coef_order).  Entries scaled by
 // 2^{-e_in - e_out} / 2 stay below 1/2; a larger one is counted in bad.
-__global__ void __launch_bounds__(256) k_oz_blob(const double* __restrict__ A, int KP, int RP, int nc, int nh, int nkc,
-                                                 const double* __restrict__ cs, unsigned char* __restrict__ blob,
-                                                 int* __restrict__ bad)
+__global__ void __launch_bounds__(256) k_oz_blob(const double* __restrict__ A, int KP, int RP, int nc, int nk, int nh,
+                                                 int nkc, const int* __restrict__ perm, const double* __restrict__ cs, unsigned char* __restrict__ blob, int* __restrict__ bad)
 {
     const int kc = blockIdx.x % nkc, half = (blockIdx.x / nkc) % nh, o = blockIdx.x / (nkc * nh);
     unsigned char* p0 = blob + (size_t)blockIdx.x * (OZ_S * OZ_A_BYTES);
     for (int i = threadIdx.x; i < TH_KC * 128; i += 256) {
-        const int k = i / 128, r = i - k * 128, kin = kc * TH_KC + k, row = 128 * half + r;
+        const int k = i / 128, r = i - k * 128, kp = kc * TH_KC + k, row = 128 * half + r;
+        const int kin = kp < nk ? perm[kp] : -1;
         double v = 0.0;
-        if (kin < nc && row < nc) {
+        if (kin >= 0 && row < nc) {
             v = A[((size_t)o * KP + kin) * RP + row] / cs[kin] / cs[row] * 0.5;
             if (!(fabs(v) < 0.5)) atomicAdd(bad, 1);
         }
@@ -419,9 +402,10 @@ __global__ void __launch_bounds__(256) k_oz_max(const double* __restrict__ M, in
     }
 }
 
-// multipoles [box][nc] -> digits [box][OZ_S][mrow] (zero padded), one thread
-// per pair of coefficients
-__global__ void __launch_bounds__(256) k_oz_split(const double* __restrict__ M, int nbox, int nc, int mrow,
+// multipoles [box][nc] -> digits [box][OZ_S][mrow] in the K order (zero padded),
+// one thread per pair of coefficients
+__global__ void __launch_bounds__(256) k_oz_split(const double* __restrict__ M, int nbox, int nc, int nk,
+                                                  int mrow, const int* __restrict__ perm,
                                                   const double* __restrict__ cs,
                                                   const __grid_constant__ OzLevels lv,
                                                   const unsigned long long* __restrict__ gmax,
@@ -435,8 +419,9 @@ __global__ void __launch_bounds__(256) k_oz_split(const double* __restrict__ M, 
     const int b = (int)(i / per), k = (int)(i % per) * 2;
     const double s = oz_scale(gmax[(size_t)blockIdx.y * 16 + oz_level(lv, b)]);
     __half d0[OZ_S], d1[OZ_S];
-    oz_digits(k < nc ? M[(size_t)b * nc + k] * cs[k] * s : 0.0, d0);
-    oz_digits(k + 1 < nc ? M[(size_t)b * nc + k + 1] * cs[k + 1] * s : 0.0, d1);
+    const int j0 = k < nk ? perm[k] : -1, j1 = k + 1 < nk ? perm[k + 1] : -1;
+    oz_digits(j0 >= 0 ? M[(size_t)b * nc + j0] * cs[j0] * s : 0.0, d0);
+    oz_digits(j1 >= 0 ? M[(size_t)b * nc + j1] * cs[j1] * s : 0.0, d1);
     __half* out = Ms + (size_t)b * OZ_S * mrow + k;
 #pragma unroll
     for (int q = 0; q < OZ_S; ++q) *reinterpret_cast<__half2*>(out + (size_t)q * mrow) = __halves2half2(d0[q], d1[q]);
@@ -447,58 +432,84 @@ __global__ void __launch_bounds__(256) k_oz_split(const double* __restrict__ M, 
 // ---------------------------------------------------------------------------
 bool lf_m2l_oz_ok(const lfmm_ctx* ctx) { return ctx->m2l_rm > 0 && lf_nc(ctx->p) <= 256; }
 
-// operator digits and coefficient scales, once per context (the first FP64
-// evaluation; a captured batch graph never sees it)
+// operator digits, coefficient scales and order, once per context (the first
+// FP64 evaluation; a captured batch graph never sees it)
 static LfErr oz_setup(lfmm_ctx* ctx, cudaStream_t st)
 {
     if (ctx->oz_ready) return LfErr();
-    const int p = ctx->p, nc = lf_nc(p), nh = (nc + 127) / 128, nkc = (nc + TH_KC - 1) / TH_KC, RP = ctx->m2l_rp;
+    const int p = ctx->p, nc = lf_nc(p), nh = (nc + 127) / 128, RP = ctx->m2l_rp, TS = 2 * p + 1;
+    std::vector<int> perm, e;
+    lf_coef_order(p, perm);
+    lf_coef_exponents(p, e);
+    const int nk = (int)perm.size(), nkc = (nk + TH_KC - 1) / TH_KC;
     std::vector<double> cs(nc);
-    for (int j = 0; j < nc; ++j) {
-        int n, m, im;
-        lf_decode(p, j, n, m, im);
-        const double e = 0.5 * (std::lgamma(n - m + 1.0) + std::lgamma(n + m + 1.0)) / std::log(2.0);
-        cs[j] = std::ldexp(1.0, (int)std::lround(e));
-    }
+    for (int j = 0; j < nc; ++j) cs[j] = std::ldexp(1.0, e[j]);
+    // for every (N, mu) the smallest exponent its table value is scaled with:
+    // terms T(n + k, l + m) and T(n + k, |l - m|) of inputs (n, m), outputs (k, l)
+    std::vector<int> emin((size_t)TS * TS, 1000);
+    for (int n = 0; n <= p; ++n)
+        for (int m = 0; m <= n; ++m)
+            for (int k = 0; k <= p; ++k)
+                for (int l = 0; l <= k; ++l) {
+                    const int x = e[lf_re(n, m)] + e[lf_re(k, l)];
+                    int& a = emin[(size_t)(n + k) * TS + l + m];
+                    int& b = emin[(size_t)(n + k) * TS + std::abs(l - m)];
+                    a = std::min(a, x);
+                    b = std::min(b, x);
+                }
     LF_TRY(lf_reserve(ctx->oz_cscale, nc * sizeof(double)));
+    LF_TRY(lf_reserve(ctx->oz_perm, nk * sizeof(int)));
+    LF_TRY(lf_reserve(ctx->oz_emin, emin.size() * sizeof(int)));
     LF_TRY(lf_reserve(ctx->oz_A, (size_t)OZ_NALL * nh * nkc * OZ_S * OZ_A_BYTES));
     LF_CHECK(cudaMemcpyAsync(ctx->oz_cscale.ptr, cs.data(), nc * sizeof(double), cudaMemcpyHostToDevice, st));
+    LF_CHECK(cudaMemcpyAsync(ctx->oz_perm.ptr, perm.data(), nk * sizeof(int), cudaMemcpyHostToDevice, st));
+    LF_CHECK(cudaMemcpyAsync(ctx->oz_emin.ptr, emin.data(), emin.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     int* bad = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_OZ_BAD_OFF);
     LF_CHECK(cudaMemsetAsync(bad, 0, sizeof(int), st));
     LF_CHECK(cudaFuncSetAttribute(k_m2l_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
-    ++ctx->launches, k_oz_blob<<<OZ_NALL * nh * nkc, 256, 0, st>>>(ctx->m2l_A64.as<double>(), RP, RP, nc, nh, nkc,
-                                                                   ctx->oz_cscale.as<double>(),
+    ++ctx->launches, k_oz_blob<<<OZ_NALL * nh * nkc, 256, 0, st>>>(ctx->m2l_A64.as<double>(), RP, RP, nc, nk, nh, nkc,
+                                                                   ctx->oz_perm.as<int>(), ctx->oz_cscale.as<double>(),
                                                                    ctx->oz_A.as<unsigned char>(), bad);
     LF_TRY(lf_cuda(cudaGetLastError(), "operator digits"));
     int n = 0;
     LF_CHECK(lf_d2h(&n, bad, sizeof(int), st));
     if (n) return "internal: free M2L operator out of the digit range";
+    ctx->oz_nk = nk;
     ctx->oz_ready = 1;
     return LfErr();
 }
 
-LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st)
+// the multipoles of every box as digits, for the free M2L and the keyed
+// reaction M2L of this evaluation
+LfErr lf_oz_split(lfmm_ctx* ctx, cudaStream_t st)
 {
-    if (ctx->oz_ntiles == 0) return LfErr();
     LF_TRY(oz_setup(ctx, st));
-    const int nb = ctx->nbox_total, nr = ctx->nrhs_b, nc = lf_nc(ctx->p);
-    OzArgs g;
-    g.nc = nc;
-    g.nh = (nc + 127) / 128;
-    g.nkc = (nc + TH_KC - 1) / TH_KC;
-    g.mrow = g.nkc * TH_KC;
-    g.win = nc <= 128 ? OZ_WIN : OZ_WIN / 2;
-    LF_TRY(lf_reserve(ctx->oz_Ms, (size_t)nb * OZ_S * g.mrow * sizeof(__half) * nr));
+    const int nb = ctx->nbox_total, nr = ctx->nrhs_b, nc = lf_nc(ctx->p), nk = ctx->oz_nk;
+    const int mrow = (nk + TH_KC - 1) / TH_KC * TH_KC;
+    LF_TRY(lf_reserve(ctx->oz_Ms, (size_t)nb * OZ_S * mrow * sizeof(__half) * nr));
     unsigned long long* gm = reinterpret_cast<unsigned long long*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
     OzLevels lv;
     lv.depth = ctx->depth;
     for (int l = 0; l < 17; ++l) lv.off[l] = l <= ctx->depth ? ctx->levels[l].off : 0;
     const double* M = ctx->Mexp.as<double>();
     ++ctx->launches, k_oz_max<<<dim3((nb + 31) / 32, nr), 256, 0, st>>>(M, nb, nc, ctx->oz_cscale.as<double>(), lv, gm);
-    const int64_t tot = (int64_t)nb * (g.mrow / 2);
+    const int64_t tot = (int64_t)nb * (mrow / 2);
     ++ctx->launches, k_oz_split<<<dim3((unsigned)((tot + 255) / 256), nr), 256, 0, st>>>(
-        M, nb, nc, g.mrow, ctx->oz_cscale.as<double>(), lv, gm, ctx->oz_Ms.as<__half>());
-    LF_TRY(lf_cuda(cudaGetLastError(), "multipole digits"));
+        M, nb, nc, nk, mrow, ctx->oz_perm.as<int>(), ctx->oz_cscale.as<double>(), lv, gm, ctx->oz_Ms.as<__half>());
+    return lf_cuda(cudaGetLastError(), "multipole digits");
+}
+
+LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st)
+{
+    if (ctx->oz_ntiles == 0) return LfErr();
+    const int nb = ctx->nbox_total, nr = ctx->nrhs_b, nc = lf_nc(ctx->p);
+    OzArgs g;
+    g.nc = nc;
+    g.nk = ctx->oz_nk;
+    g.nh = (nc + 127) / 128;
+    g.nkc = (g.nk + TH_KC - 1) / TH_KC;
+    g.mrow = g.nkc * TH_KC;
+    g.win = nc <= 128 ? OZ_WIN : OZ_WIN / 2;
     g.tiles = ctx->oz_tiles.as<int4>();
     g.sorted = ctx->m2l_sorted.as<int>();
     g.slots = ctx->m2l_slots.as<int>();
@@ -508,7 +519,7 @@ LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st)
     g.A = ctx->oz_A.as<unsigned char>();
     g.Ms = ctx->oz_Ms.as<__half>();
     g.cscale = ctx->oz_cscale.as<double>();
-    g.gmax = gm;
+    g.gmax = reinterpret_cast<unsigned long long*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
     g.L = ctx->Lexp.as<double>();
     // 27 offsets per CTA amortise its read-back and FP64 atomics; 9 or 3 where
     // the tiles are too few to give every SM several CTAs

@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(TCP_THREADS, 1) k_m2l_tcp(TcArgs g, int nunits
 // positions: Re and Im of (n, m) for m >= 1, and the real (n, 0) of two
 // successive degrees (-1: no coefficient).  The reaction M2L forms its operators
 // pair by pair (lfmm_m2r.cu).
-static void coef_order(int p, std::vector<int>& perm)
+void lf_coef_order(int p, std::vector<int>& perm)
 {
     perm.clear();
     for (int n = 0; n <= p; ++n) {
@@ -681,7 +681,7 @@ static void coef_order(int p, std::vector<int>& perm)
 }
 
 // binary exponent of each packed coefficient's scale: log2 sqrt((n-m)! (n+m)!), rounded
-static void coef_exponents(int p, std::vector<int>& e)
+void lf_coef_exponents(int p, std::vector<int>& e)
 {
     const int nc = lf_nc(p);
     e.assign(nc, 0);
@@ -750,9 +750,9 @@ LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP)
     if (nc > 2 * TC_M || KP < nc || RP < nc) return LfErr();
     const bool wide = nc > TC_M;
     std::vector<int> e;
-    coef_exponents(ctx->p, e);
+    lf_coef_exponents(ctx->p, e);
     std::vector<int> perm;
-    coef_order(ctx->p, perm);
+    lf_coef_order(ctx->p, perm);
     std::vector<float> cs(nc);
     for (int k = 0; k < nc; ++k) cs[k] = std::ldexp(1.f, e[k]);
     LF_TRY(lf_reserve(ctx->tc_cscale, nc * sizeof(float)));

@@ -12,7 +12,8 @@
 // reflection sign (-1)^{n+m} of the multipole (s = -1 maps) and the
 // (-1)^{N+mu} of an a = 2 component belong to A_key.
 // The float32 form with p <= 10 applies the keys on the tensor cores
-// (k_m2r_tc), every other case in the rotated frame (k_m2r_rot).  A level with
+// (k_m2r_tc), the FP64 form with p <= 15 by digit products there (k_m2r_oz),
+// every other case in the rotated frame (k_m2r_rot).  A level with
 // an entry outside the key range, and the coarser ones, keep the per-pair kernel.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -465,7 +466,7 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
 // 0.74 -> 0.83 ms; and orders above 15, which integrated a table per pair
 // before, 27.0 -> 3.0 ms (2,848 charges, 6,910 pairs, p = 20).
 // ---------------------------------------------------------------------------
-#define RR_PH (LFMM_PMAX + 1)
+#define RR_PH 32  // orders m <= 2p of p <= 15 (k_m2r_oz), m <= p of every other
 
 struct RRotArgs {
     int p, nc, cb;          // order, coefficients, columns staged at a time
@@ -481,11 +482,10 @@ struct RRotArgs {
     int nr;
 };
 
-// e^{i m phi}, m <= p, of every lateral key offset, FP64
+// e^{i m phi}, m < RR_PH, of every lateral key offset, FP64
 __global__ void k_m2r_phase64(double* out)
 {
     const int b = blockIdx.x, m = threadIdx.x;
-    if (m >= RR_PH) return;
     const int ox = b / R_OW - R_OR, oy = b % R_OW - R_OR;
     const double phi = (ox == 0 && oy == 0) ? 0.0 : atan2((double)oy, (double)ox);
     double sn, cs;
@@ -965,6 +965,391 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
                      : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// FP64 form, p <= 15: the key's operator applied by digit products on the
+// tensor cores (scheme of lfmm_m2l_oz.cu: seven 9-bit digits per operand, the
+// 28 products of the leading diagonals, exact sums).  One CTA per batch of
+// pairs of one key (and 128-row part of the outputs), 32 columns at a time.
+// The dense operator is formed in FP64 from the table W of the complex
+// reaction coefficient in blocks of 2 x 2 (as k_m2r_tc: one addition per
+// entry), turned into a 64-bit fixed-point number by shifts (the scales are
+// powers of two, so no rounding but the last of 63 bits) and cut into digits;
+// a biased add makes the signed digits plain bit fields, and 1024 + digit in
+// float16 is the bit pattern itself.  The operator's scale comes from the key's
+// largest table value with the smallest scale it meets (emin), so every entry
+// is below 1/2.  The multipoles' digits are those of the free M2L.
+//   Bound: the integer work of the digits (about 50 operations per entry) and
+// the FP64 additions and conversions, which share an SM's 2 per clock; two CTAs
+// per SM hide each other's gathers and read-backs.
+// Measured: 65,536 charges, p = 10 (171,888 pairs): 3.75 ms (k_m2r_rot) -> 0.97 ms;
+// 1,000 charges 0.215 -> 0.082 ms.
+// ---------------------------------------------------------------------------
+#define RZ_T 256
+#define RZ_N 32                          // columns at a time (MMA N: 16 or 32)
+#define RZ_X_BYTES (RZ_N * TC_ROWB)      // one multipole digit of a K chunk
+#define RZ_STAGE (OZ_S * (OZ_A_BYTES + RZ_X_BYTES))
+#define RZ_PAIRS 128                     // row (column) pairs at p = 15
+
+struct ROzArgs {
+    int p, nc, nk, nkc, parts;  // order, coefficients, K positions and chunks, 128-row parts
+    const int4* batches;        // key index, first sorted entry, count | key << 8, table
+    const double* tables;       // [table][TS][TS]
+    const LfmmComp* comps;
+    const double* phase;        // [225 lateral offsets][cos | sin][RR_PH]
+    const int2* pairs;          // (source box, target box) per sorted entry
+    const double* levelh;
+    const __half* Ms;           // digits [box][OZ_S][32 nkc]
+    const double* cscale;       // 2^e per packed coefficient
+    const int* perm;            // packed coefficient of each K position (and row), -1: none
+    const int* emin;            // [TS][TS] smallest exponent of a table value
+    const unsigned long long* gmax;  // largest scaled multipole per level (double bits), [16] per right-hand side
+    double* L;
+    size_t ms_stride, stride;
+    int* err;
+};
+
+// a 2^sh, |a 2^sh| < 1/2, in units of 2^-63 (sign flipped by neg), biased so
+// that its signed digits d_i are the bit fields d_i + 256 (the leading one unmasked)
+__device__ __forceinline__ unsigned long long rz_fixed(double a, int sh, bool neg)
+{
+    constexpr unsigned long long BIAS = 256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36) +
+                                                  (1ull << 45) + (1ull << 54));
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a);
+    const int r = 1022 - (int)((b >> 52) & 0x7ffu) - sh;  // right shift of the significand in bits 62 .. 10
+    const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10;
+    const unsigned long long f = r > 63 ? 0ull : (m + (1ull << (max(r, 1) - 1))) >> max(r, 1);
+    return BIAS + ((((long long)b < 0) != neg) ? 0ull - f : f);
+}
+
+// digit i (0: leading) of two biased numbers as float16
+template <int I>
+__device__ __forceinline__ __half2 rz_digit(unsigned long long a, unsigned long long b)
+{
+    constexpr int S = OZ_B * (OZ_S - 1 - I);
+    uint32_t x = (uint32_t)(a >> S), y = (uint32_t)(b >> S);
+    if (I > 0) {
+        x &= 511u;
+        y &= 511u;
+    }
+    const uint32_t v = (x | y << 16) + 0x64006400u;  // 1024 + field
+    return __hsub2(*reinterpret_cast<const __half2*>(&v), __half2half2(__ushort_as_half(0x6500)));  // - 1280
+}
+
+// the digits of 8 K values of one operator row
+template <int I>
+__device__ __forceinline__ void rz_store(unsigned char* sa, const unsigned long long w[8])
+{
+    __align__(16) __half2 h[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) h[e] = rz_digit<I>(w[2 * e], w[2 * e + 1]);
+    *reinterpret_cast<uint4*>(sa + I * OZ_A_BYTES) = *reinterpret_cast<const uint4*>(h);
+    if constexpr (I + 1 < OZ_S) rz_store<I + 1>(sa, w);
+}
+
+// x or -x by the sign bit (a selected negation ran on the FP64 pipe)
+__device__ __forceinline__ double rz_flip(double x, int neg)
+{
+    return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
+
+__global__ void __launch_bounds__(RZ_T, 2) k_m2r_oz(ROzArgs g)
+{
+    extern __shared__ unsigned char smem_raw[];
+    // 512-byte alignment: the period of the 64-byte swizzle
+    unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 511) &
+                                                         ~(uintptr_t)511);
+    unsigned char* sx = sm + OZ_S * OZ_A_BYTES;
+    double2* sW = reinterpret_cast<double2*>(sm + RZ_STAGE);  // [N][mu + 2p], rows of 4p + 1
+    // column pairs: offsets of the two W terms from the row's; signs of the two
+    // terms (bits 0, 1), two real inputs (bit 2); exponents
+    __shared__ int4 s_co[RZ_PAIRS];
+    __shared__ int s_prow[128];
+    __shared__ double sPh[2 * RR_PH];
+    __shared__ int s_src[R_TB], s_tgt[R_TB];
+    __shared__ unsigned long long s_max;
+    __shared__ double s_unit;  // output unit: 2^{-36 - sc} over the multipoles' scale and h
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_abort;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int p = g.p, nc = g.nc, nkc = g.nkc, TS = 2 * p + 1, WS = 4 * p + 1;
+    const int part = blockIdx.x % g.parts;
+    const int4 b = g.batches[blockIdx.x / g.parts];
+    const int start = b.y, cnt = b.z & 255;
+    if (cnt <= 0 || cnt > R_TB) return;
+    int c, lev, ox, oy, oz;
+    rkey_decode((uint32_t)b.z >> 8, c, lev, ox, oy, oz);
+    const bool refl = g.comps[c].refl != 0;
+    if (tid < RZ_PAIRS) {
+        int4 o = make_int4(0, 0, 4, 0);
+        if (2 * tid < g.nk) {
+            const int j0 = g.perm[2 * tid], j1 = g.perm[2 * tid + 1];
+            int n, m, im;
+            lf_decode(p, j0, n, m, im);
+            const int e0 = ilogb(g.cscale[j0]);
+            // the multipole's reflection sign (-1)^{n+m} for s = -1 maps, and (-1)^m of the second term
+            const int sg = refl && ((n + m) & 1) ? 1 : 0;
+            if (m > 0) {
+                o = make_int4(n * WS + m, n * WS - m, sg | (sg ^ (m & 1)) << 1, e0 | e0 << 16);
+            } else {
+                o = make_int4(n * WS, n * WS, 4 | sg, e0 | e0 << 16);
+                if (j1 >= 0) {
+                    lf_decode(p, j1, n, m, im);
+                    o.y = n * WS;
+                    o.z |= (refl && (n & 1)) ? 2 : 0;
+                    o.w = e0 | ilogb(g.cscale[j1]) << 16;
+                }
+            }
+        }
+        s_co[tid] = o;
+    } else {
+        // rows t and 64 + t: the pair t of this part (so that 8 pairs' stores meet no bank twice)
+        const int r = tid - 128, i = 128 * part + 2 * (r & 63) + (r >> 6);
+        s_prow[r] = i < g.nk ? g.perm[i] : -1;
+    }
+    if (tid < R_TB) {
+        const int2 pr = (tid < cnt) ? g.pairs[start + tid] : make_int2(-1, -1);
+        s_src[tid] = pr.x;
+        s_tgt[tid] = pr.y;
+    } else if (tid < R_TB + 2 * RR_PH) {
+        sPh[tid - R_TB] = g.phase[(size_t)((ox + R_OR) * R_OW + (oy + R_OR)) * 2 * RR_PH + (tid - R_TB)];
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(256)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        mbar_init(&bar, 1);
+        s_abort = 0;
+        s_max = 0ull;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    {
+        const double* Tk = g.tables + (size_t)b.w * TS * TS;
+        unsigned long long mx = 0;
+        for (int j = tid; j < TS * TS; j += RZ_T) {
+            const int N = j / TS, a = j - N * TS;
+            const double t = Tk[j];
+            const int e = g.emin[j];
+            if (e < 1000) {
+                const unsigned long long v = (unsigned long long)__double_as_longlong(
+                    fabs(t) * __longlong_as_double((long long)(1023 - e) << 52));
+                mx = v > mx ? v : mx;
+            }
+            const double wr = t * sPh[a], wi = t * sPh[RR_PH + a];
+            double2* w = sW + N * WS + 2 * p;
+            w[a] = make_double2(wr, wi);
+            w[-a] = (a & 1) ? make_double2(-wr, wi) : make_double2(wr, -wi);
+        }
+        const unsigned h = __reduce_max_sync(0xffffffffu, (unsigned)(mx >> 32));
+        const unsigned l = __reduce_max_sync(0xffffffffu, (unsigned)(mx >> 32) == h ? (unsigned)mx : 0u);
+        if (lane == 0) atomicMax(&s_max, (unsigned long long)h << 32 | l);
+    }
+    __syncthreads();
+    // two table values of at most s_max 2^{e_in + e_out} each make an entry: 2^sc takes it below 1/2
+    const unsigned long long mx = s_max;
+    const bool badt = mx >= 0x7ff0000000000000ull;
+    const int sc = (mx == 0ull || badt) ? 0 : 1020 - (int)(mx >> 52);
+    if (tid == 0) {  // (read after the chunks' barriers)
+        const double u = ldexp(1.0, -36 - sc) / (oz_scale(g.gmax[(size_t)blockIdx.y * 16 + lev]) * g.levelh[lev]);
+        s_unit = badt ? nan64() : u;
+    }
+    // operator unit: row pair xj, quarter xq of every chunk
+    const int xj = tid >> 2, xq = tid & 3;
+    const int r0 = s_prow[xj], r1 = s_prow[64 + xj];
+    int z0 = 0, z1 = 0, er0 = 0, er1 = 0;
+    bool ng0 = false, ng1 = false, cpx = false;  // cpx: Re and Im of one output
+    if (r0 >= 0) {
+        int k, l, im;
+        lf_decode(p, r0, k, l, im);
+        z0 = z1 = k * WS + l + 2 * p;
+        er0 = er1 = ilogb(g.cscale[r0]);
+        ng0 = ng1 = (k & 1) != 0;
+        cpx = l > 0;
+        if (!cpx && r1 >= 0) {
+            lf_decode(p, r1, k, l, im);
+            z1 = k * WS + l + 2 * p;
+            er1 = ilogb(g.cscale[r1]);
+            ng1 = (k & 1) != 0;
+        }
+    }
+    const uint32_t off0 = swz16(xj, 8 * xq), off1 = swz16(64 + xj, 8 * xq);
+    const __half* Ms = g.Ms + (size_t)blockIdx.y * g.ms_stride;
+    double* L = g.L + (size_t)blockIdx.y * g.stride;
+    const int mrow = nkc * TH_KC;
+    bool ok = true;
+    int gr = 0;  // chunks so far
+    for (int q0 = 0; q0 < cnt && ok; q0 += RZ_N) {
+        const int nq = min(RZ_N, cnt - q0), Np = (nq + 15) & ~15;
+        const uint32_t idesc = tc_idesc_f16(128, Np);
+        for (int kc = 0; kc < nkc; ++kc, ++gr) {
+            unsigned long long w[8];
+            const int4* co = s_co + kc * (TH_KC / 2) + 4 * xq;
+            if (r0 >= 0)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int4 o = co[e];
+                    const double2 x = sW[z0 + o.x], y = sW[z0 + o.y];
+                    const double xr = rz_flip(x.x, o.z & 1), yr = rz_flip(y.x, o.z & 2);
+                    const double u0 = (o.z & 4) ? xr : xr + yr;
+                    const double u1 = (o.z & 4) ? yr : rz_flip(y.y, o.z & 2) - rz_flip(x.y, o.z & 1);
+                    w[2 * e] = rz_fixed(u0, sc - (o.w & 0xffff) - er0, ng0);
+                    w[2 * e + 1] = rz_fixed(u1, sc - (o.w >> 16) - er0, ng0);
+                }
+            // the previous chunk's MMAs have read the stage
+            if (gr > 0 && !mbar_wait(&bar, (uint32_t)((gr - 1) & 1))) s_abort = 1;
+            {
+                const int row = (tid & 127) >> 2, q = tid & 3, d0 = tid < 128 ? 0 : 4, d1 = tid < 128 ? 4 : OZ_S;
+                if (row < Np) {
+                    const int src = s_src[q0 + row];
+                    const __half* gs = Ms + (size_t)(src >= 0 ? src : 0) * (OZ_S * mrow) + kc * TH_KC + q * 8;
+                    unsigned char* dst = sx + swz16(row, q * 8);
+                    for (int i = d0; i < d1; ++i) {
+                        if (src >= 0)
+                            cp_async16(smem_u32(dst + i * RZ_X_BYTES), gs + (size_t)i * mrow);
+                        else
+                            *reinterpret_cast<float4*>(dst + i * RZ_X_BYTES) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                }
+            }
+            cp_async_commit();
+            // (rows past the last coefficient are never read back)
+            if (r0 >= 0) rz_store<0>(sm + off0, w);
+            if (r1 >= 0) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int4 o = co[e];
+                    const double2 x = sW[z1 + o.x], y = sW[z1 + o.y];
+                    // the imaginary part of an output, or the second of two real ones
+                    const double xr = rz_flip(cpx ? x.y : x.x, o.z & 1), yr = rz_flip(cpx ? y.y : y.x, o.z & 2);
+                    const double xi = rz_flip(cpx ? x.x : x.y, o.z & 1), yi = rz_flip(cpx ? y.x : y.y, o.z & 2);
+                    const double u0 = (o.z & 4) ? xr : xr + yr;
+                    const double u1 = (o.z & 4) ? yr : (cpx ? xi - yi : yi - xi);
+                    w[2 * e] = rz_fixed(u0, sc - (o.w & 0xffff) - er1, ng1);
+                    w[2 * e + 1] = rz_fixed(u1, sc - (o.w >> 16) - er1, ng1);
+                }
+                rz_store<0>(sm + off1, w);
+            }
+            cp_async_wait<0>();
+            fence_async_smem();
+            tc_fence_before();
+            __syncthreads();
+            if (*(volatile int*)&s_abort) {  // block-uniform after the barrier
+                ok = false;
+                break;
+            }
+            if (tid == 0) {
+                tc_fence_after();
+                const uint32_t ab = smem_u32(sm), xb = smem_u32(sx);
+                const int nks = (g.nk - kc * TH_KC) > 16 ? 2 : 1;
+                for (int ks = 0; ks < nks; ++ks)
+#pragma unroll
+                    for (int i = 0; i < OZ_S; ++i)
+#pragma unroll
+                        for (int j = 0; j < OZ_S - i; ++j)
+                            tc_mma_f16(tmem + (uint32_t)((i + j) * RZ_N), smem_desc(ab + i * OZ_A_BYTES + 32 * ks),
+                                       smem_desc(xb + j * RZ_X_BYTES + 32 * ks), idesc,
+                                       (kc == 0 && ks == 0 && i == 0) ? 0u : 1u);
+                tc_commit(&bar);
+            }
+            __syncwarp();
+        }
+        bool got = false;
+        if (ok) got = mbar_wait(&bar, (uint32_t)((gr - 1) & 1));
+        ok = __syncthreads_and(got) != 0;  // block-uniform
+        tc_fence_after();
+        if (ok) {
+            const int q4 = warp & 3, row = s_prow[32 * q4 + lane], cb = 16 * (warp >> 2);
+            if (cb < Np) {
+                long long hi[16], lo[16];  // units 2^-36 and 2^-72
+#pragma unroll
+                for (int d = 0; d < OZ_S; ++d) {
+                    float v[16];
+                    tc_ld16(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(d * RZ_N + cb), v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const long long n = __float2int_rn(v[i]);
+                        if (d == 0)
+                            hi[i] = n * (1ll << (2 * OZ_B));
+                        else if (d < 3)
+                            hi[i] += n * (1ll << (OZ_B * (2 - d)));
+                        else if (d == 3)
+                            lo[i] = n * (1ll << (3 * OZ_B));
+                        else
+                            lo[i] += n * (1ll << (OZ_B * (6 - d)));
+                    }
+                }
+                if (row >= 0) {
+                    const double sh = g.cscale[row] * s_unit, sl = sh * 0x1p-36;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        if (cb + i >= nq) break;
+                        // carry into hi, then both to FP64 by the bits of 1.5 2^52 + n
+                        const long long h = hi[i] + (lo[i] >> 36), l = lo[i] & 0xfffffffffll;
+                        const double dh = __longlong_as_double(0x4338000000000000ll + h) - 0x1.8p52;
+                        const double dl = __longlong_as_double(0x4338000000000000ll + l) - 0x1.8p52;
+                        atomicAdd(L + (size_t)s_tgt[q0 + cb + i] * nc + row, fma(dh, sh, dl * sl));
+                    }
+                }
+            }
+        } else if (tid == 0) {
+            atomicAdd(g.err, 1);
+        }
+        tc_fence_before();
+        __syncthreads();  // the accumulators are free again
+        tc_fence_after();
+    }
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256) : "memory");
+}
+
+// once per context (the first evaluation; a captured batch graph never sees it)
+static LfErr m2r_phases64(lfmm_ctx* ctx, cudaStream_t st)
+{
+    if (ctx->m2r_phase64_ready) return LfErr();
+    LF_TRY(lf_reserve(ctx->m2r_phase64, (size_t)R_OW * R_OW * 2 * RR_PH * sizeof(double)));
+    ++ctx->launches, k_m2r_phase64<<<R_OW * R_OW, RR_PH, 0, st>>>(ctx->m2r_phase64.as<double>());
+    LF_TRY(lf_cuda(cudaGetLastError(), "m2r phases"));
+    ctx->m2r_phase64_ready = 1;
+    return LfErr();
+}
+
+static LfErr m2r_apply_oz(lfmm_ctx* ctx, cudaStream_t st)
+{
+    LF_TRY(m2r_phases64(ctx, st));
+    ROzArgs g;
+    g.p = ctx->p;
+    g.nc = lf_nc(ctx->p);
+    g.nk = ctx->oz_nk;
+    g.nkc = (g.nk + TH_KC - 1) / TH_KC;
+    g.parts = (g.nk + 127) / 128;
+    g.batches = ctx->m2r_batches.as<int4>();
+    g.tables = ctx->m2r_tables.as<double>();
+    g.comps = ctx->comp_dev.as<LfmmComp>();
+    g.phase = ctx->m2r_phase64.as<double>();
+    g.pairs = ctx->m2r_pairs.as<int2>();
+    g.levelh = ctx->m2r_levelh.as<double>();
+    g.Ms = ctx->oz_Ms.as<__half>();
+    g.cscale = ctx->oz_cscale.as<double>();
+    g.perm = ctx->oz_perm.as<int>();
+    g.emin = ctx->oz_emin.as<int>();
+    g.gmax = reinterpret_cast<unsigned long long*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
+    g.L = ctx->Lexp.as<double>();
+    g.ms_stride = (size_t)ctx->nbox_total * OZ_S * g.nkc * TH_KC;
+    g.stride = (size_t)ctx->nbox_total * g.nc;
+    g.err = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
+    const size_t sm = 512 + RZ_STAGE + sizeof(double2) * (size_t)(2 * g.p + 1) * (4 * g.p + 1);
+    LF_CHECK(cudaFuncSetAttribute(k_m2r_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    ++ctx->launches, k_m2r_oz<<<dim3(ctx->m2r_nbatch * g.parts, ctx->nrhs_b), RZ_T, sm, st>>>(g);
+    return lf_cuda(cudaGetLastError(), "m2r digit products");
+}
+
 template <typename R>
 static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
 {
@@ -976,13 +1361,7 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
     g.batches = ctx->m2r_batches.as<int4>();
     g.tables = ctx->m2r_tables.as<double>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
-    if (!ctx->m2r_phase64_ready) {
-        // once per context (the first evaluation; a captured batch graph never sees it)
-        LF_TRY(lf_reserve(ctx->m2r_phase64, (size_t)R_OW * R_OW * 2 * RR_PH * sizeof(double)));
-        ++ctx->launches, k_m2r_phase64<<<R_OW * R_OW, 32, 0, st>>>(ctx->m2r_phase64.as<double>());
-        LF_TRY(lf_cuda(cudaGetLastError(), "m2r phases"));
-        ctx->m2r_phase64_ready = 1;
-    }
+    LF_TRY(m2r_phases64(ctx, st));
     g.phase = ctx->m2r_phase64.as<double>();
     g.pairs = ctx->m2r_pairs.as<int2>();
     g.levelh = ctx->m2r_levelh.as<double>();
@@ -1050,5 +1429,6 @@ LfErr lf_m2r_apply(lfmm_ctx* ctx, cudaStream_t st)
 {
     if (ctx->m2r_nbatch == 0) return LfErr();
     if (m2r_tc_on(ctx)) return m2r_apply_tc(ctx, st);
-    return ctx->precision ? m2r_apply_rot<float>(ctx, st) : m2r_apply_rot<double>(ctx, st);
+    if (ctx->precision) return m2r_apply_rot<float>(ctx, st);
+    return lf_m2l_oz_ok(ctx) ? m2r_apply_oz(ctx, st) : m2r_apply_rot<double>(ctx, st);
 }

@@ -151,3 +151,21 @@ __host__ __device__ __forceinline__ uint32_t swz16(int row, int k)
     const uint32_t x = (uint32_t)((row >> 1) & 3);
     return (uint32_t)row * TC_ROWB + ((c ^ x) << 4) + (uint32_t)(k & 7) * 2u;
 }
+
+// Digit products of the FP64 form (lfmm_m2l_oz.cu).
+#define OZ_S 7                      // digits per operand
+#define OZ_B 9                      // bits per digit
+#define OZ_A_BYTES (128 * TC_ROWB)  // one digit of 128 operator rows and a K chunk
+__device__ __forceinline__ double nan64() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// power of two that takes the largest magnitude (double bits) into [1/4, 1/2).
+// An infinity or NaN gives NaN: the digits of that level mean nothing, and
+// the scale makes a NaN of every sum it multiplies.
+__device__ __forceinline__ double oz_scale(unsigned long long bits)
+{
+    if (bits == 0ull) return 1.0;
+    if (bits >= 0x7ff0000000000000ull) return nan64();
+    int e = 1021 - (int)(bits >> 52);  // -2 - (biased exponent - 1023)
+    e = e > 1020 ? 1020 : (e < -1020 ? -1020 : e);
+    return __longlong_as_double((long long)(e + 1023) << 52);
+}
