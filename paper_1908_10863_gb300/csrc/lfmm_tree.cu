@@ -136,31 +136,39 @@ LfErr lf_scan_i32(lfmm_ctx* ctx, const int* in, int* out, int64_t n, int64_t* to
 
 // ---------------------------------------------------------------------------
 // Stable LSD radix sort of (key, value) uint32 pairs, 8 bits per pass.  A pass
-// is a histogram per block, [digit][block], and a scatter whose blocks find
-// their own offsets: thread d sums row d (all blocks for the digit's total, the
-// blocks before it for its own part) and the totals are scanned in shared
-// memory.  Up to RS_FUSE blocks that is all; above, one launch of 256 blocks
-// scans the rows first.  (A recursive scan between the two took three more
-// launches per pass, 8 us of 24 at 65,536 keys.)
+// is a histogram per block and a scatter whose blocks find their own offsets:
+// thread d sums digit d over the blocks (all for its total, those before for
+// its own part) and the totals are scanned in shared memory.  Up to RS_FUSE
+// blocks that is all (hist [block][digit]); above, one launch of 256 blocks
+// scans the digits' rows first (hist [digit][block]).  A warp ranks its keys by
+// itself: its run of 32 `rounds` keys counts into its own row of shared
+// memory, so the block meets twice, not five times per 256 keys.
+// Measured, a build of 65,536 charges (sorts of up to 171,888 keys, eight passes'
+// scatters): 138 -> 71 us.
 // ---------------------------------------------------------------------------
 #define RS_T 256
+#define RS_W (RS_T / 32)
 #define RS_ROUNDS 8   // most rounds of RS_T keys per block
-#define RS_FUSE 128   // most blocks whose rows the scatter reads itself
+#define RS_FUSE 128   // most blocks whose counts the scatter reads itself
 
 __global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, int rounds,
-                             int* __restrict__ hist, int nblocks)
+                             int* __restrict__ hist, int sdigit, int sblock)
 {
     __shared__ int h[256];
     const int tid = threadIdx.x;
     h[tid] = 0;
     __syncthreads();
-#pragma unroll 4
-    for (int r = 0; r < rounds; ++r) {
-        int64_t i = ((int64_t)blockIdx.x * rounds + r) * RS_T + tid;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1);
+    uint32_t k[RS_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+        const int64_t i = ((int64_t)blockIdx.x * rounds + r) * RS_T + tid;
+        k[r] = r < rounds && i < n ? (keys[i] >> shift) & 255u : 256u;
     }
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r)
+        if (k[r] < 256u) atomicAdd(&h[k[r]], 1);
     __syncthreads();
-    hist[tid * nblocks + blockIdx.x] = h[tid];
+    hist[(size_t)tid * sdigit + (size_t)blockIdx.x * sblock] = h[tid];
 }
 
 // exclusive prefix sums of the rows of hist, in place, and their totals
@@ -200,68 +208,83 @@ __global__ void __launch_bounds__(RS_T) k_radix_scatter(const uint32_t* __restri
                                                         const int* __restrict__ hist, int nblocks,
                                                         const int* __restrict__ total)
 {
-    __shared__ int s_off[256];
-    __shared__ int s_wcnt[RS_T / 32][256];
-    __shared__ int s_w[RS_T / 32];
+    __shared__ int s_cnt[RS_W][256];
+    __shared__ int s_w[RS_W];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    {
-        // this block's first position of digit tid
-        const int* row = hist + (size_t)tid * nblocks;
-        int tot = 0, pre = 0;
-        if (total) {
-            tot = total[tid];
-            pre = row[blockIdx.x];
-        } else {
-#pragma unroll 8
-            for (int j = 0; j < nblocks; ++j) {
-                const int v = row[j];
-                tot += v;
-                pre += j < (int)blockIdx.x ? v : 0;
+#pragma unroll
+    for (int w = 0; w < RS_W; ++w) s_cnt[w][tid] = 0;
+    uint32_t key[RS_ROUNDS], val[RS_ROUNDS];
+    const int64_t i0 = (int64_t)blockIdx.x * rounds * RS_T + (int64_t)wid * rounds * 32 + lane;
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+        const int64_t i = i0 + 32 * r;
+        const bool in = r < rounds && i < n;
+        key[r] = in ? kin[i] : 0u;
+        val[r] = in ? vin[i] : 0u;
+    }
+    // this block's first position of digit tid
+    int tot = 0, pre = 0;
+    if (total) {
+        tot = total[tid];
+        pre = hist[(size_t)tid * nblocks + blockIdx.x];
+    } else {
+        for (int j0 = 0; j0 < nblocks; j0 += 16) {  // 16 loads in flight
+            int v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = j0 + u < nblocks ? hist[(size_t)(j0 + u) * 256 + tid] : 0;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                tot += v[u];
+                pre += j0 + u < (int)blockIdx.x ? v[u] : 0;
             }
         }
-        int x = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_w[wid] = x;
-        __syncthreads();
-        int before = 0;
-#pragma unroll
-        for (int k = 0; k < RS_T / 32; ++k)
-            if (k < wid) before += s_w[k];
-        s_off[tid] = before + x - tot + pre;
     }
-    for (int r = 0; r < rounds; ++r) {
-        int64_t i = ((int64_t)blockIdx.x * rounds + r) * RS_T + tid;
-        bool valid = i < n;
-        uint32_t key = valid ? kin[i] : 0u;
-        uint32_t val = valid ? vin[i] : 0u;
-        int digit = valid ? (int)((key >> shift) & 255u) : 256;
+    int x = tot;
 #pragma unroll
-        for (int w = 0; w < RS_T / 32; ++w) s_wcnt[w][tid] = 0;
-        __syncthreads();
-        unsigned peers = __match_any_sync(0xffffffffu, digit);
-        int rank = __popc(peers & ((1u << lane) - 1u));
-        int leader = __ffs(peers) - 1;
-        if (valid && lane == leader) s_wcnt[wid][digit] = __popc(peers);
-        __syncthreads();
-        int run = 0;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[wid] = x;
+    __syncthreads();  // counts are zero, s_w complete
+    // rank of each key among this warp's keys of the same digit
+    int rank[RS_ROUNDS];
 #pragma unroll
-        for (int w = 0; w < RS_T / 32; ++w) {
-            int t = s_wcnt[w][tid];
-            s_wcnt[w][tid] = run;
-            run += t;
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+        if (r >= rounds) break;
+        const bool in = i0 + 32 * r < n;
+        const int d = in ? (int)((key[r] >> shift) & 255u) : 256;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const int leader = __ffs(peers) - 1;
+        int old = 0;
+        if (in && lane == leader) {
+            old = s_cnt[wid][d];
+            s_cnt[wid][d] = old + __popc(peers);
         }
-        __syncthreads();
-        if (valid) {
-            int pos = s_off[digit] + s_wcnt[wid][digit] + rank;
-            kout[pos] = key;
-            vout[pos] = val;
+        rank[r] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+    }
+    __syncthreads();
+    int before = 0;
+#pragma unroll
+    for (int k = 0; k < RS_W; ++k)
+        if (k < wid) before += s_w[k];
+    int run = before + x - tot + pre;
+#pragma unroll
+    for (int w = 0; w < RS_W; ++w) {
+        const int t = s_cnt[w][tid];
+        s_cnt[w][tid] = run;
+        run += t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RS_ROUNDS; ++r) {
+        if (r >= rounds) break;
+        if (i0 + 32 * r < n) {
+            const int pos = s_cnt[wid][(key[r] >> shift) & 255u] + rank[r];
+            kout[pos] = key[r];
+            vout[pos] = val[r];
         }
-        __syncthreads();
-        s_off[tid] += run;
     }
 }
 
@@ -284,7 +307,7 @@ LfErr lf_radix_sort(lfmm_ctx* ctx, uint32_t* keys, uint32_t* vals, int64_t n, cu
     int* total = nb > RS_FUSE ? h + (size_t)256 * nb : nullptr;
     for (int pass = first_pass; pass < first_pass + npass; ++pass) {
         int shift = 8 * pass;
-        ++ctx->launches, k_radix_hist<<<nb, RS_T, 0, st>>>(ka, n, shift, rounds, h, nb);
+        ++ctx->launches, k_radix_hist<<<nb, RS_T, 0, st>>>(ka, n, shift, rounds, h, total ? nb : 1, total ? 1 : 256);
         if (total) ++ctx->launches, k_radix_rows<<<256, 256, 0, st>>>(h, nb, total);
         ++ctx->launches, k_radix_scatter<<<nb, RS_T, 0, st>>>(ka, va, kb, vb, n, shift, rounds, h, nb, total);
         LF_TRY(lf_cuda(cudaGetLastError(), "radix pass"));
