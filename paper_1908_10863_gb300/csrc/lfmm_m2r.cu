@@ -11,8 +11,7 @@
 // multipoles), added atomically into the targets' local expansions.  The
 // reflection sign (-1)^{n+m} of the multipole (s = -1 maps) and the
 // (-1)^{N+mu} of an a = 2 component belong to A_key.
-// The float32 form with p <= 10 applies the keys on the tensor cores
-// (k_m2r_tc), the FP64 form with p <= 15 by digit products there (k_m2r_oz),
+// The float32 form applies the keys on the tensor cores (k_m2r_tc), the FP64 form with p <= 15 by digit products there (k_m2r_oz),
 // every other case in the rotated frame (k_m2r_rot).  A level with
 // an entry outside the key range, and the coarser ones, keep the per-pair kernel.
 #include <cuda_fp16.h>
@@ -614,8 +613,10 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 }
 
 // ---------------------------------------------------------------------------
-// Tensor-core form (float32, (p+1)^2 <= 128): one CTA per batch of up to
-// R_TB pairs of one key.  The key's operator is never stored: the CTA forms
+// Tensor-core form (float32, p <= 14): one CTA per batch of up to R_TB pairs
+// of one key, and per 128-row part of the outputs where (p+1)^2 > 128 (the wide
+// form: one vector at a time, the two correction products in an accumulator of
+// their own, as in the free M2L's).  The key's operator is never stored: the CTA forms
 // it in shared memory from the key's Sommerfeld table and the lateral phases,
 // directly as two float16 pieces a1 + a2 in the 64-byte-swizzled K-major layout
 // of the MMA's A operand (M = 128 output coefficients, K = the input
@@ -643,36 +644,42 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 // Measured, p = 10, float16 pieces against TF32 pieces with the operator formed
 // again for every vector: 64 vectors of 262,144 charges 13.8 -> 4.95 ms.  One
 // vector, N = 1M: 0.258 ms with entries formed one at a time, 0.170 ms in blocks.
+// The wide form, 65,536 charges, p = 14: 0.825 ms (k_m2r_rot) -> 0.52 ms, the
+// evaluation's difference from the FP64 form unchanged (3.2e-7).
 // ---------------------------------------------------------------------------
 #define RT_THREADS 256
-#define RT_TS 21                        // table side 2p + 1 for p <= 10
-#define RT_WS 41                        // 4p + 1: orders -2p .. 2p
-#define RT_NKC 4                        // K chunks at most
+#define RT_PH 32                        // stride of the phase table (orders m <= 2p <= 28)
+#define RT_NKC 4                        // K chunks at most where the operator is kept
 #define RT_A_CHUNK (128 * TC_ROWB)      // one K chunk of one operator piece: 128 rows x 64 B
 #define RT_X_CHUNK (R_TB * TC_ROWB)     // one K chunk of one multipole piece and vector: 64 rows x 64 B
 #define RT_ASHIFT 8                     // operators carry 2^8: entries (reflections and image sums included) stay
                                         // far inside float16's range
-template <int V>
+template <int V, bool WIDE>
 struct RtShape {
+    static constexpr int P = WIDE ? 14 : 10;                   // largest order
+    static constexpr int W = (2 * P + 1) * (4 * P + 1);        // entries of the table W
+    static constexpr int CP = WIDE ? 128 : 64;                 // column pairs
+    static constexpr int MROW = WIDE ? 256 : 128;              // halves per box and multipole piece
     static constexpr bool KEEP = V > 1;                        // operator kept for all vectors
     static constexpr int NA = KEEP ? RT_NKC : 2;               // operator chunks in shared memory
     static constexpr int XB = 2 * V * RT_X_CHUNK;              // multipole bytes of a chunk: two pieces
     static constexpr int SMEM = NA * 2 * RT_A_CHUNK + 2 * XB + 512;
     static constexpr int MINB = KEEP ? 2 : 3;                  // resident CTAs per SM
-    static constexpr uint32_t COLS = 64 * V;                   // tensor-memory columns
+    static constexpr uint32_t COLS = WIDE ? 128 : 64 * V;      // tensor-memory columns
 };
 
 struct RTcArgs {
     int p, nc, nk, nkc;     // order, coefficients, K positions, chunks of 32 that hold them
+    int parts;              // 128-row parts of the outputs
     const int4* batches;    // key index, first sorted entry, count | key << 8, table
     const double* tables;   // [table][TS][TS]
     const LfmmComp* comps;
-    const float* phase;     // [225 lateral offsets][cos | sin][RT_TS] (k_m2r_phase)
+    const float* phase;     // [225 lateral offsets][cos | sin][RT_PH] (k_m2r_phase)
     const int2* pairs;      // (source box, target box) per sorted entry (k_m2r_pairs)
     const double* levelh;
-    const __half* Ms;       // split multipoles [box][2 pieces][128]
+    const __half* Ms;       // split multipoles [box][2 pieces][MROW]
     const float* cscale;    // 2^e per packed coefficient
-    const int* perm;        // packed index of each K position
+    const int* perm;        // packed index of each K position (and row), -1: none
     const unsigned* gmax;   // largest scaled multipole per level (float bits), [32] per right-hand side
     float* L;
     size_t ms_stride, stride;  // per right-hand side: halves of Ms, floats of L
@@ -681,7 +688,7 @@ struct RTcArgs {
 };
 
 // e^{i m phi} of every lateral key offset (ox, oy) in [-7, 7]^2, m <= 2p:
-// FP64 sincos rounded to float32, [offset][cos | sin][RT_TS]
+// FP64 sincos rounded to float32, [offset][cos | sin][RT_PH]
 __global__ void k_m2r_phase(int p, float* out)
 {
     const int b = blockIdx.x, m = threadIdx.x;
@@ -690,14 +697,14 @@ __global__ void k_m2r_phase(int p, float* out)
     const double phi = (ox == 0 && oy == 0) ? 0.0 : atan2((double)oy, (double)ox);
     double sn, cs;
     sincos(m * phi, &sn, &cs);
-    out[(size_t)b * 2 * RT_TS + m] = (float)cs;
-    out[(size_t)b * 2 * RT_TS + RT_TS + m] = (float)sn;
+    out[(size_t)b * 2 * RT_PH + m] = (float)cs;
+    out[(size_t)b * 2 * RT_PH + RT_PH + m] = (float)sn;
 }
 
-template <int V>
-__global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs g)
+template <int V, bool WIDE>
+__global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(RTcArgs g)
 {
-    typedef RtShape<V> S;
+    typedef RtShape<V, WIDE> S;
     extern __shared__ unsigned char smem_raw[];
     // 512-byte alignment: the period of the 64-byte swizzle
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 511) &
@@ -705,22 +712,24 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
     unsigned char* smx = sm + S::NA * 2 * RT_A_CHUNK;
     // W(N, mu) = T(N, |mu|) e^{i mu phi} for mu in [-2p, 2p], extended to
     // negative orders by W(N, -mu) = (-1)^mu conj W(N, mu); [N][mu + 2p], rows of 4p + 1
-    __shared__ float2 sW[RT_TS * RT_WS];
-    __shared__ float sPh[2 * RT_TS];
+    __shared__ float2 sW[S::W];
+    __shared__ float sPh[2 * RT_PH];
     // column pairs: offsets of the two W terms from the row's, their signs and
     // scales; y < 0: two real inputs (n, 0), -1 - offset of the second
-    __shared__ int2 s_co[64];
-    __shared__ float2 s_cf[64];
-    // row pairs: packed rows (y = -1: none), offsets; z == w: Re and Im of one (k, l)
+    __shared__ int2 s_co[S::CP];
+    __shared__ float2 s_cf[S::CP];
+    // row pairs (rows t and 64 + t): packed rows (-1: none), offsets; z == w: Re and Im of one (k, l)
     __shared__ int4 s_row[64];
     __shared__ float2 s_rk[64];  // (-1)^k with the rows' scales
+    __shared__ int s_prow[128];
     __shared__ int s_src[R_TB], s_tgt[R_TB];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int p = g.p, nc = g.nc, nkc = g.nkc, TS = 2 * p + 1, WS = 4 * p + 1, TSZ = TS * WS;
-    const int4 b = g.batches[blockIdx.x];
+    const int part = WIDE ? blockIdx.x % g.parts : 0;
+    const int4 b = g.batches[WIDE ? blockIdx.x / g.parts : blockIdx.x];
     // the batch carries its key and table: one dependent load to everything else
     const int start = b.y, cnt = b.z & 255, tab = b.w;
     if (cnt <= 0 || cnt > R_TB) return;
@@ -730,36 +739,35 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
     const bool refl = g.comps[c].refl != 0;
 
     if (tid < 64) {
-        // row pair tid: the (k, l) with l >= 1, then the (k, 0) two at a time
-        const int nl = p * (p + 1) / 2;
+        // row pair of this part: Re and Im of a (k, l), or two (k, 0)
+        const int i = 128 * part + 2 * tid;
         int4 r = make_int4(-1, -1, 0, 0);
         float2 sk = make_float2(0.f, 0.f);
         const float as = (float)(1 << RT_ASHIFT);
-        if (tid < nl) {
-            int k = 1, t = tid;
-            while (t >= k) t -= k++;
-            const int l = t + 1;
-            r = make_int4(lf_re(k, l), lf_im(p, k, l), k * WS + l + 2 * p, k * WS + l + 2 * p);
+        if (i < g.nk) {
+            r.x = g.perm[i];
+            r.y = g.perm[i + 1];
+            int k, l, im;
+            lf_decode(p, r.x, k, l, im);
+            r.z = r.w = k * WS + l + 2 * p;
             sk.x = sk.y = ((k & 1) ? -as : as) / g.cscale[r.x];
-        } else {
-            const int k = 2 * (tid - nl);
-            if (k <= p) {
-                r.x = lf_re(k, 0);
-                r.z = k * WS + 2 * p;
+            if (l == 0) {
                 r.w = -1;  // (not an Re / Im pair)
-                sk.x = as / g.cscale[r.x];
-            }
-            if (k + 1 <= p) {
-                r.y = lf_re(k + 1, 0);
-                r.w = (k + 1) * WS + 2 * p;
-                sk.y = -as / g.cscale[r.y];
+                sk.y = 0.f;
+                if (r.y >= 0) {
+                    lf_decode(p, r.y, k, l, im);
+                    r.w = k * WS + l + 2 * p;
+                    sk.y = ((k & 1) ? -as : as) / g.cscale[r.y];
+                }
             }
         }
         s_row[tid] = r;
         s_rk[tid] = sk;
-    } else if (tid < 128) {
+        s_prow[tid] = r.x;
+        s_prow[64 + tid] = r.y;
+    } else if (tid >= RT_THREADS - S::CP) {
         // column pair: K positions 2c and 2c + 1
-        const int c2 = 2 * (tid - 64);
+        const int cc = tid - (RT_THREADS - S::CP), c2 = 2 * cc;
         int2 o = make_int2(0, 0);
         float2 f = make_float2(0.f, 0.f);
         if (c2 < g.nk) {
@@ -783,16 +791,16 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
                 }
             }
         }
-        s_co[tid - 64] = o;
-        s_cf[tid - 64] = f;
+        s_co[cc] = o;
+        s_cf[cc] = f;
     }
     if (tid < R_TB) {
         const int2 pr = (tid < cnt) ? g.pairs[start + tid] : make_int2(-1, -1);
         s_src[tid] = pr.x;
         s_tgt[tid] = pr.y;
     }
-    if (tid >= 128 && tid < 128 + 2 * RT_TS)
-        sPh[tid - 128] = g.phase[(size_t)((ox + R_OR) * R_OW + (oy + R_OR)) * 2 * RT_TS + (tid - 128)];
+    else if (tid < R_TB + 2 * RT_PH)
+        sPh[tid - R_TB] = g.phase[(size_t)((ox + R_OR) * R_OW + (oy + R_OR)) * 2 * RT_PH + (tid - R_TB)];
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(S::COLS)
@@ -814,7 +822,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
         for (int j = tid; j < TSZ; j += RT_THREADS) {
             const int Nn = j / WS, mu = j - Nn * WS - 2 * p, a = mu < 0 ? -mu : mu;
             const float t = (float)Tk[Nn * TS + a];
-            float wr = t * sPh[a], wi = t * sPh[RT_TS + a];
+            float wr = t * sPh[a], wi = t * sPh[RT_PH + a];
             if (mu < 0) {
                 if (a & 1) wr = -wr; else wi = -wi;
             }
@@ -842,14 +850,14 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
                     if (v >= nv) break;
-                    const __half* gs = g.Ms + (size_t)(r0 + v) * g.ms_stride + (size_t)(src >= 0 ? src : 0) * 256 +
-                                       kc * TH_KC + xq * 8;
+                    const __half* gs = g.Ms + (size_t)(r0 + v) * g.ms_stride +
+                                       (size_t)(src >= 0 ? src : 0) * (2 * S::MROW) + kc * TH_KC + xq * 8;
                     const uint32_t off = swz16(v * Np + xj, xq * 8);
 #pragma unroll
                     for (int piece = 0; piece < 2; ++piece) {
                         unsigned char* dst = sx + piece * V * RT_X_CHUNK + off;
                         if (src >= 0)
-                            cp_async16(smem_u32(dst), gs + piece * 128);
+                            cp_async16(smem_u32(dst), gs + piece * S::MROW);
                         else
                             *reinterpret_cast<float4*>(dst) = make_float4(0.f, 0.f, 0.f, 0.f);
                     }
@@ -892,11 +900,11 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
                     lb[e] = __floats2half2_rn(b0 - fb.x, b1 - fb.y);
                 }
                 // (rows past the last coefficient are never read back)
-                uint32_t off = swz16(rw.x, 8 * xq);
+                uint32_t off = swz16(xj, 8 * xq);
                 *reinterpret_cast<uint4*>(sa + off) = *reinterpret_cast<const uint4*>(ha);
                 *reinterpret_cast<uint4*>(sa + RT_A_CHUNK + off) = *reinterpret_cast<const uint4*>(la);
                 if (rw.y >= 0) {
-                    off = swz16(rw.y, 8 * xq);
+                    off = swz16(64 + xj, 8 * xq);
                     *reinterpret_cast<uint4*>(sa + off) = *reinterpret_cast<const uint4*>(hb);
                     *reinterpret_cast<uint4*>(sa + RT_A_CHUNK + off) = *reinterpret_cast<const uint4*>(lb);
                 }
@@ -917,11 +925,12 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
                 for (int prod = 0; prod < 3; ++prod) {  // a2 x1, a1 x2, a1 x1
                     const uint32_t a = a0 + (prod == 0 ? RT_A_CHUNK : 0);
                     const uint32_t x = x0 + (prod == 1 ? V * RT_X_CHUNK : 0);
+                    const uint32_t acc = tmem + (WIDE && prod < 2 ? 64 : 0);
 #pragma unroll
                     for (int ks = 1; ks >= 0; --ks)
                         if (ks < nks)
-                            tc_mma_f16(tmem, smem_desc(a + 32 * ks), smem_desc(x + 32 * ks), idesc,
-                                       (i == 0 && prod == 0 && ks == nks - 1) ? 0u : 1u);
+                            tc_mma_f16(acc, smem_desc(a + 32 * ks), smem_desc(x + 32 * ks), idesc,
+                                       (i == 0 && (prod == 0 || (WIDE && prod == 2)) && ks == nks - 1) ? 0u : 1u);
                 }
                 tc_commit(&bar[buf]);
             }
@@ -933,8 +942,8 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
         ok = __syncthreads_and(got) != 0;  // block-uniform
         tc_fence_after();
         if (ok) {
-            const int q4 = warp & 3, row = 32 * q4 + lane;
-            const float rs = row < nc ? g.cscale[row] : 0.f;
+            const int q4 = warp & 3, row = s_prow[32 * q4 + lane];
+            const float rs = row >= 0 ? g.cscale[row] : 0.f;
             float sc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v)
@@ -943,7 +952,13 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V>::MINB) k_m2r_tc(RTcArgs
             for (int c0 = 32 * (warp >> 2); c0 < nv * Np; c0 += 64) {
                 float v[32];
                 tc_ld32(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)c0, v);
-                if (row < nc) {
+                if constexpr (WIDE) {
+                    float u[32];
+                    tc_ld32(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)(64 + c0), u);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) v[i] += u[i];
+                }
+                if (row >= 0) {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
                         const int vj = (V > 1 && c0 + i >= Np) ? 1 : 0, j = c0 + i - vj * Np;
@@ -1379,11 +1394,17 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
     return lf_cuda(cudaGetLastError(), "m2r rotated");
 }
 
-// the float32 form with (p+1)^2 <= 128 applies the keys on the tensor cores
-// whenever the free M2L does (tensor-core option)
-static bool m2r_tc_on(const lfmm_ctx* ctx)
+// the float32 form applies the keys on the tensor cores whenever the free M2L
+// does (tensor-core option)
+static bool m2r_tc_on(const lfmm_ctx* ctx) { return ctx->precision == 1 && lf_tc_on(ctx); }
+
+template <int V, bool WIDE>
+static LfErr m2r_launch_tc(lfmm_ctx* ctx, const RTcArgs& g, cudaStream_t st)
 {
-    return ctx->precision == 1 && ctx->p <= 10 && lf_tc_on(ctx);
+    constexpr int sm = RtShape<V, WIDE>::SMEM;
+    LF_CHECK(cudaFuncSetAttribute(k_m2r_tc<V, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    ++ctx->launches, k_m2r_tc<V, WIDE><<<ctx->m2r_nbatch * g.parts, RT_THREADS, sm, st>>>(g);
+    return lf_cuda(cudaGetLastError(), "m2r tensor-core GEMM");
 }
 
 static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
@@ -1402,27 +1423,22 @@ static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
     g.cscale = ctx->tc_cscale.as<float>();
     g.perm = ctx->tc_perm.as<int>();
     g.gmax = reinterpret_cast<unsigned*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
-    g.ms_stride = (size_t)ctx->nbox_total * 256;
+    g.parts = (g.nk + 127) / 128;
+    g.ms_stride = (size_t)ctx->nbox_total * (g.parts > 1 ? 512 : 256);
     g.L = ctx->Lexp.as<float>();
     g.stride = (size_t)ctx->nbox_total * g.nc;
     g.nr = ctx->nrhs_b;
     g.err = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
     if (ctx->m2r_phase_p != ctx->p) {
         // once per context (the first evaluation; a captured batch graph never sees it)
-        LF_TRY(lf_reserve(ctx->m2r_phase, (size_t)R_OW * R_OW * 2 * RT_TS * sizeof(float)));
-        ++ctx->launches, k_m2r_phase<<<R_OW * R_OW, 32, 0, st>>>(ctx->p, ctx->m2r_phase.as<float>());
+        LF_TRY(lf_reserve(ctx->m2r_phase, (size_t)R_OW * R_OW * 2 * RT_PH * sizeof(float)));
+        ++ctx->launches, k_m2r_phase<<<R_OW * R_OW, RT_PH, 0, st>>>(ctx->p, ctx->m2r_phase.as<float>());
         LF_TRY(lf_cuda(cudaGetLastError(), "m2r phases"));
         ctx->m2r_phase_p = ctx->p;
     }
     g.phase = ctx->m2r_phase.as<float>();
-    if (g.nr == 1) {
-        LF_CHECK(cudaFuncSetAttribute(k_m2r_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, RtShape<1>::SMEM));
-        ++ctx->launches, k_m2r_tc<1><<<ctx->m2r_nbatch, RT_THREADS, RtShape<1>::SMEM, st>>>(g);
-    } else {
-        LF_CHECK(cudaFuncSetAttribute(k_m2r_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, RtShape<2>::SMEM));
-        ++ctx->launches, k_m2r_tc<2><<<ctx->m2r_nbatch, RT_THREADS, RtShape<2>::SMEM, st>>>(g);
-    }
-    return lf_cuda(cudaGetLastError(), "m2r tensor-core GEMM");
+    if (g.parts > 1) return m2r_launch_tc<1, true>(ctx, g, st);
+    return g.nr == 1 ? m2r_launch_tc<1, false>(ctx, g, st) : m2r_launch_tc<2, false>(ctx, g, st);
 }
 
 LfErr lf_m2r_apply(lfmm_ctx* ctx, cudaStream_t st)
