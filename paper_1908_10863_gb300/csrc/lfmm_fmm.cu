@@ -211,50 +211,43 @@ __device__ __forceinline__ int lf_octant(LfD4 child, LfD4 parent)
 // ---------------------------------------------------------------------------
 template <typename R>
 __global__ void k_m2m(int off, int p, const LfD4* __restrict__ cen, const int* __restrict__ cbeg,
-                      const int* __restrict__ cend, const R* __restrict__ octU, R* __restrict__ M)
+                      const int* __restrict__ cend, const R* __restrict__ octU, R* __restrict__ M, size_t stride)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nre = lf_nre(p), nc = lf_nc(p);
     R* sM = reinterpret_cast<R*>(smem_raw);
     R* sUr = sM + nc;
     R* sUi = sUr + nre;
-    const int b = off + blockIdx.x;
+    const int b = off + blockIdx.x, ch = cbeg[b] + blockIdx.y;
+    if (ch >= cend[b]) return;
+    M += (size_t)blockIdx.z * stride;
     const int tid = threadIdx.x;
-    int n = 0, m = 0, im = 0;
-    const bool act = tid < nre;
-    if (act) lf_decode(p, tid, n, m, im);
-    R ar = 0, ai = 0;
-    const LfD4 pc = cen[b];
-    for (int ch = cbeg[b]; ch < cend[b]; ++ch) {
-        int o = lf_octant(cen[ch], pc);
-        for (int j = tid; j < nc; j += blockDim.x) sM[j] = M[(size_t)ch * nc + j];
-        for (int j = tid; j < nre; j += blockDim.x) {
-            sUr[j] = octU[(size_t)o * 2 * nre + j];
-            sUi[j] = octU[(size_t)o * 2 * nre + nre + j];
-        }
-        __syncthreads();
-        if (act) {
-            R sc = 1;
-            for (int k = 0; k <= n; ++k) {
-                for (int l = -k; l <= k; ++l) {
-                    int dm = m - l;
-                    if (dm > n - k || dm < -(n - k)) continue;
-                    R mr, mi, ur, ui;
-                    lf_get(sM, p, k, l, mr, mi);
-                    lf_getU(sUr, sUi, n - k, dm, ur, ui);
-                    // M * conj(U)
-                    ar += sc * (mr * ur + mi * ui);
-                    ai += sc * (mi * ur - mr * ui);
-                }
-                sc *= R(0.5);
-            }
-        }
-        __syncthreads();
+    const int o = lf_octant(cen[ch], cen[b]);
+    for (int j = tid; j < nc; j += blockDim.x) sM[j] = M[(size_t)ch * nc + j];
+    for (int j = tid; j < nre; j += blockDim.x) {
+        sUr[j] = octU[(size_t)o * 2 * nre + j];
+        sUi[j] = octU[(size_t)o * 2 * nre + nre + j];
     }
-    if (act) {
-        M[(size_t)b * nc + lf_re(n, m)] = ar;
-        if (m > 0) M[(size_t)b * nc + lf_im(p, n, m)] = ai;
+    __syncthreads();
+    if (tid >= nre) return;
+    int n, m, im;
+    lf_decode(p, tid, n, m, im);
+    R ar = 0, ai = 0, sc = 1;
+    for (int k = 0; k <= n; ++k) {
+        for (int l = -k; l <= k; ++l) {
+            int dm = m - l;
+            if (dm > n - k || dm < -(n - k)) continue;
+            R mr, mi, ur, ui;
+            lf_get(sM, p, k, l, mr, mi);
+            lf_getU(sUr, sUi, n - k, dm, ur, ui);
+            // M * conj(U)
+            ar += sc * (mr * ur + mi * ui);
+            ai += sc * (mi * ur - mr * ui);
+        }
+        sc *= R(0.5);
     }
+    atomicAdd(M + (size_t)b * nc + lf_re(n, m), ar);
+    if (m > 0) atomicAdd(M + (size_t)b * nc + lf_im(p, n, m), ai);
 }
 
 // ---------------------------------------------------------------------------
@@ -263,7 +256,7 @@ __global__ void k_m2m(int off, int p, const LfD4* __restrict__ cen, const int* _
 // ---------------------------------------------------------------------------
 template <typename R>
 __global__ void k_l2l(int off, int p, const LfD4* __restrict__ cen, const int* __restrict__ parent,
-                      const R* __restrict__ octU, R* __restrict__ L)
+                      const R* __restrict__ octU, R* __restrict__ L, size_t stride)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nre = lf_nre(p), nc = lf_nc(p);
@@ -271,6 +264,7 @@ __global__ void k_l2l(int off, int p, const LfD4* __restrict__ cen, const int* _
     R* sUr = sL + nc;
     R* sUi = sUr + nre;
     const int b = off + blockIdx.x;
+    L += (size_t)blockIdx.z * stride;
     const int tid = threadIdx.x;
     const int pb = parent[b];
     const int o = lf_octant(cen[b], cen[pb]);
@@ -284,7 +278,7 @@ __global__ void k_l2l(int off, int p, const LfD4* __restrict__ cen, const int* _
     int jn, im_, mm;
     lf_decode(p, tid, jn, mm, im_);
     R ar = 0, ai = 0;
-    for (int k = jn; k <= p; ++k) {
+    for (int k = jn + blockIdx.y; k <= p; k += gridDim.y) {
         for (int l = -k; l <= k; ++l) {
             int dm = l - mm;
             if (dm > k - jn || dm < -(k - jn)) continue;
@@ -297,8 +291,8 @@ __global__ void k_l2l(int off, int p, const LfD4* __restrict__ cen, const int* _
     }
     R sc = 1;
     for (int q = 0; q < jn; ++q) sc *= R(0.5);
-    L[(size_t)b * nc + lf_re(jn, mm)] += sc * ar;
-    if (mm > 0) L[(size_t)b * nc + lf_im(p, jn, mm)] += sc * ai;
+    atomicAdd(L + (size_t)b * nc + lf_re(jn, mm), sc * ar);
+    if (mm > 0) atomicAdd(L + (size_t)b * nc + lf_im(p, jn, mm), sc * ai);
 }
 
 // ---------------------------------------------------------------------------
@@ -326,6 +320,7 @@ struct M2LArgs {
     const double* gl_t;
     const double* gl_w;
     int Q;
+    size_t stride;  // expansions per right-hand side (blockIdx.z), in elements
 };
 
 // GEN: reaction components of media of four or five layers
@@ -344,8 +339,8 @@ __global__ void k_m2l(M2LArgs a)
     R* sC = sOut + nc;                                   // p+1 (cos m phi)
     R* sS = sC + (p + 1);                                // p+1 (sin m phi)
 
-    const R* M = reinterpret_cast<const R*>(a.M);
-    R* L = reinterpret_cast<R*>(a.L);
+    const R* M = reinterpret_cast<const R*>(a.M) + (size_t)blockIdx.z * a.stride;
+    R* L = reinterpret_cast<R*>(a.L) + (size_t)blockIdx.z * a.stride;
     const R* freeT = reinterpret_cast<const R*>(a.freeT);
 
     const int t = a.level_off + blockIdx.x;
@@ -357,7 +352,11 @@ __global__ void k_m2l(M2LArgs a)
     LfAcc<R> acc;
     const double ih = 1.0 / a.h;
 
-    for (int e = a.mbeg[t]; e < a.mend[t]; ++e) {
+    // (blockIdx.y: an equal share of the entries)
+    const int e0 = a.mbeg[t], ne = a.mend[t] - e0, ny = gridDim.y, y = blockIdx.y;
+    const int eb = e0 + (int)((int64_t)ne * y / ny), ee = e0 + (int)((int64_t)ne * (y + 1) / ny);
+    if (eb == ee) return;
+    for (int e = eb; e < ee; ++e) {
         const uint32_t ent = a.ment[e];
         const int c = (int)(ent >> LFMM_ENT_SHIFT);
         const int s = (int)(ent & LFMM_ENT_MASK);
@@ -435,7 +434,7 @@ __global__ void k_m2l(M2LArgs a)
         }
         __syncthreads();
     }
-    if (act) L[(size_t)t * nc + tid] += acc.get() * (R)ih;
+    if (act) atomicAdd(L + (size_t)t * nc + tid, acc.get() * (R)ih);
 }
 
 // ---------------------------------------------------------------------------
@@ -628,6 +627,10 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
     {
         size_t sm = sizeof(R) * (nc + 2 * (size_t)nre);
         int th = ((nre + 31) / 32) * 32;
+        // (k_m2m adds the children's shares; boxes of the coarser levels follow the leaves)
+        if (!ctx->shift_ready && depth > lmin)
+            LF_CHECK(cudaMemset2DAsync(M + (size_t)leaf.nbox * nc, ms * sizeof(R), 0,
+                                       sizeof(R) * (size_t)(ctx->nbox_total - leaf.nbox) * nc, nr, st));
         for (int l = depth - 1; l >= lmin; --l) {
             const LfmmLevel& lv = ctx->levels[l];
             if (lv.nbox == 0) continue;
@@ -635,8 +638,7 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
             if (ctx->shift_ready)
                 LF_TRY(lf_shift_gemm(ctx, l, false, st));
             else
-                for (int r = 0; r < nr; ++r)
-                    ++ctx->launches, k_m2m<R><<<lv.nbox, th, sm, st>>>(lv.off, p, cen, cbeg, cend, octU, M + r * ms);
+                ++ctx->launches, k_m2m<R><<<dim3(lv.nbox, 8, nr), th, sm, st>>>(lv.off, p, cen, cbeg, cend, octU, M, ms);
             lf_prof_stop(ctx, ph, st);
         }
         LF_TRY(lf_cuda(cudaGetLastError(), "m2m"));
@@ -693,16 +695,15 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
         a.gl_t = ctx->gl_t_m2l.as<double>();
         a.gl_w = ctx->gl_w_m2l.as<double>();
         a.Q = Q;
+        a.stride = ms;
+        // small levels share each box's entries between blocks: about 8 blocks per SM
+        const int split = (int)std::max<int64_t>(1, std::min<int64_t>(16, 8 * 152 / std::max<int64_t>(1, (int64_t)lv.nbox * nr)));
         if (!gemm && lv.m2l_count > 0) {
             a.mbeg = ctx->m2l_off.as<int>();
             a.mend = ctx->m2l_off.as<int>() + ctx->nbox_total;
             a.ment = ctx->m2l_ent.as<uint32_t>();
             ph = lf_prof_start(ctx, LFMM_TIME_M2L_FREE, st);
-            for (int r = 0; r < nr; ++r) {
-                a.M = M + r * ms;
-                a.L = L + r * ms;
-                ++ctx->launches, k_m2l<R, false><<<lv.nbox, mth, msm_f, st>>>(a);
-            }
+            ++ctx->launches, k_m2l<R, false><<<dim3(lv.nbox, split, nr), mth, msm_f, st>>>(a);
             lf_prof_stop(ctx, ph, st);
         }
         if (lv.m2r_count > 0 && l < ctx->m2r_keyed_from) {
@@ -710,14 +711,8 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
             a.mend = ctx->m2r_off.as<int>() + ctx->nbox_total;
             a.ment = ctx->m2r_ent.as<uint32_t>();
             ph = lf_prof_start(ctx, LFMM_TIME_M2L_REACTION, st);
-            for (int r = 0; r < nr; ++r) {
-                a.M = M + r * ms;
-                a.L = L + r * ms;
-                if (general)
-                    ++ctx->launches, k_m2l<R, true, true><<<lv.nbox, mth, msm_r, st>>>(a);
-                else
-                    ++ctx->launches, k_m2l<R, true><<<lv.nbox, mth, msm_r, st>>>(a);
-            }
+            const auto kern = general ? k_m2l<R, true, true> : k_m2l<R, true, false>;
+            ++ctx->launches, kern<<<dim3(lv.nbox, split, nr), mth, msm_r, st>>>(a);
             lf_prof_stop(ctx, ph, st);
         }
         LF_TRY(lf_cuda(cudaGetLastError(), "m2l"));
@@ -729,8 +724,8 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
         if (ctx->shift_ready)
             LF_TRY(lf_shift_gemm(ctx, l, true, st));
         else
-            for (int r = 0; r < nr; ++r)
-                ++ctx->launches, k_l2l<R><<<lv.nbox, lth, lsm, st>>>(lv.off, p, cen, par, octU, L + r * ms);
+            ++ctx->launches, k_l2l<R><<<dim3(lv.nbox, (int64_t)lv.nbox * nr < 8 * 152 ? 4 : 1, nr), lth, lsm, st>>>(
+                lv.off, p, cen, par, octU, L, ms);
         lf_prof_stop(ctx, ph, st);
         LF_TRY(lf_cuda(cudaGetLastError(), "l2l"));
     }

@@ -1386,9 +1386,10 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
     g.nr = ctx->nrhs_b;
     const int TS = 2 * ctx->p + 1;
     const size_t sm = sizeof(R) * ((size_t)2 * lf_nre(ctx->p) * g.cb + (size_t)TS * TS);
-    // few batches (small trees): share the rows of each between blocks
+    // share the rows of each batch between blocks until the longest batch (64
+    // pairs, 15 times the mean in small trees) no longer outlasts the rest
     int parts = 1;
-    while (parts < 8 && (int64_t)ctx->m2r_nbatch * parts < 8 * 152) parts *= 2;
+    while (parts < 8 && (int64_t)ctx->m2r_nbatch * parts < 64 * 152) parts *= 2;
     LF_CHECK(cudaFuncSetAttribute(k_m2r_rot<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     ++ctx->launches, k_m2r_rot<R><<<dim3(ctx->m2r_nbatch, parts), R_T, sm, st>>>(g);
     return lf_cuda(cudaGetLastError(), "m2r rotated");
