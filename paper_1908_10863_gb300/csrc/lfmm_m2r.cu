@@ -38,27 +38,58 @@
 static inline int lf_blocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 #define R_TB 64   // pairs per batch
-#define R_T 256   // threads: 16 row groups x 16 column groups
+#define R_T 256   // threads per block of the rotated form
+#define RR_CB 16  // columns it stages at a time above p = 10
 #define KEY_NONE 0xffffffffu
 
 
 // key = level (4 bits) | comp (7 bits) | offset index (12 bits, offsets in
 // [-7, 7]^3): sorted keys group a level's keys together, so the keys of the
-// levels left to the per-pair kernel are a prefix
+// levels left to the per-pair kernel are a prefix.  The offset index is oz, then
+// the rank of (ox, oy) by rho^2, so the keys that share a table (one oz and
+// rho^2) are neighbours.
 #define R_OR 7
 #define R_OW (2 * R_OR + 1)
+#define R_LAT (R_OW * R_OW)
+struct LatRank {
+    unsigned char rank[R_LAT], lat[R_LAT];  // (ox + 7) 15 + (oy + 7) to rank, and back
+    constexpr LatRank() : rank(), lat()
+    {
+        int n = 0;
+        for (int r2 = 0; r2 <= 2 * R_OR * R_OR; ++r2)
+            for (int i = 0; i < R_LAT; ++i) {
+                const int x = i / R_OW - R_OR, y = i % R_OW - R_OR;
+                if (x * x + y * y == r2) {
+                    rank[i] = (unsigned char)n;
+                    lat[n++] = (unsigned char)i;
+                }
+            }
+    }
+};
+static constexpr LatRank h_lat = LatRank();
+static __device__ const LatRank d_lat = LatRank();
+__host__ __device__ __forceinline__ const LatRank& r_lat()
+{
+#ifdef __CUDA_ARCH__
+    return d_lat;
+#else
+    return h_lat;
+#endif
+}
 __host__ __device__ __forceinline__ uint32_t rkey(int c, int l, int ox, int oy, int oz)
 {
-    return ((uint32_t)l << 19) | ((uint32_t)c << 12) | (uint32_t)(((ox + R_OR) * R_OW + (oy + R_OR)) * R_OW + (oz + R_OR));
+    return ((uint32_t)l << 19) | ((uint32_t)c << 12) |
+           (uint32_t)((oz + R_OR) * R_LAT + r_lat().rank[(ox + R_OR) * R_OW + (oy + R_OR)]);
 }
 __host__ __device__ __forceinline__ void rkey_decode(uint32_t key, int& c, int& l, int& ox, int& oy, int& oz)
 {
     c = (int)((key >> 12) & 127u);
     l = (int)(key >> 19);
     int oi = (int)(key & 4095u);
-    ox = oi / (R_OW * R_OW) - R_OR;
-    oy = (oi / R_OW) % R_OW - R_OR;
-    oz = oi % R_OW - R_OR;
+    const int la = r_lat().lat[oi % R_LAT];
+    ox = la / R_OW - R_OR;
+    oy = la % R_OW - R_OR;
+    oz = oi / R_LAT - R_OR;
 }
 
 // Keys of the reaction M2L entries of one level, from the boxes' grid cells.
@@ -381,10 +412,16 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
     // batches of R_TB pairs of one key: key index, first sorted entry, count | key << 8, table
     std::vector<int4>& batches = ctx->m2r_batches_h;
     batches.clear();
-    for (int64_t k = k0; k < k1; ++k)
-        for (int s = kstart[k]; s < kstart[k + 1]; s += R_TB)
-            batches.push_back(make_int4((int)(k - k0), s, std::min(R_TB, kstart[k + 1] - s) | (int)(kv[k] << 8),
+    // (above p = 15, where only k_m2r_rot applies them: pairs of one table, as
+    // many as it stages at a time, so that no block outlasts the others)
+    const int most = P > 15 ? RR_CB : R_TB;
+    for (int64_t k = k0, k2; k < k1; k = k2) {
+        k2 = k + 1;
+        while (P > 15 && k2 < k1 && ktab[k2 - k0] == ktab[k - k0]) ++k2;
+        for (int s = kstart[k]; s < kstart[k2]; s += most)
+            batches.push_back(make_int4((int)(k - k0), s, std::min(most, kstart[k2] - s) | (int)(kv[k] << 8),
                                         ktab[k - k0]));
+    }
     ctx->m2r_nkeys = (int)nku;
     ctx->m2r_nbatch = (int)batches.size();
     LF_TRY(lf_reserve(ctx->m2r_batches, batches.size() * sizeof(int4) + 16));
@@ -456,14 +493,15 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
 // with s = (-1)^m for m <= l, (-1)^l beyond.  That is half the multiply-adds of
 // the dense (p+1)^2 x (p+1)^2 operator, and the two entries come from two table
 // values, so no operator is stored: the table (a few KB) stays in shared
-// memory, and a pair of additions serves C columns.  One block per batch of
-// pairs of one key (and part of the rows); an item is one (k, l) for C columns,
+// memory, and a pair of additions serves C columns.  The azimuth enters only
+// with the columns, so pairs of every key that shares the table can be columns
+// of one batch (above p = 15 they are).  One block per batch (and part of the rows); an item is one (k, l) for C columns,
 // C the width in {2, 4, 8} that pads the batch least.
-// FP64 (2 multiply-adds per clock and SM) bounds it.  Against one stored dense
-// operator per key (assembled after every build, 720 MB at N = 65,536) and a
-// GEMM: 6.44 + 1.79 ms -> 3.76 ms there, FP64, p = 10; float32, p = 14: 1.04 +
-// 0.74 -> 0.83 ms; and orders above 15, which integrated a table per pair
-// before, 27.0 -> 3.0 ms (2,848 charges, 6,910 pairs, p = 20).
+// FP64 (2 multiply-adds per clock and SM) bounds it.  Orders above 15 integrated a
+// table per pair before: 2,848 charges, 6,910 pairs, p = 20: 27.0 ms -> 3.08 with
+// batches of one key (4.6 pairs) and one block each, 2.53 with the rows in eight
+// shares, 1.98 with the pairs of a table in batches of up to 16 and four shares.
+// Float32, p = 14, 65,536 charges: 1.78 (stored operators and a GEMM) -> 0.83 ms.
 // ---------------------------------------------------------------------------
 #define RR_PH 32  // orders m <= 2p of p <= 15 (k_m2r_oz), m <= p of every other
 
@@ -473,6 +511,7 @@ struct RRotArgs {
     const double* tables;   // [table][TS][TS]
     const LfmmComp* comps;
     const double* phase;    // [225 lateral offsets][cos | sin][RR_PH]
+    const uint32_t* keys;   // key of each sorted entry
     const int2* pairs;      // (source box, target box) per sorted entry
     const double* levelh;
     const void* M;
@@ -496,12 +535,15 @@ __global__ void k_m2r_phase64(double* out)
 // columns [0, cnt) of the staged chunk, rows part of nparts
 template <typename R, int C>
 __device__ __forceinline__ void rr_apply(int p, int nc, const R* sT, const R* sXr, const R* sXi, int cb, int cnt,
-                                         const int* s_tgt, const R* sC, const R* sS, R ih, R* __restrict__ L, int part,
-                                         int nparts)
+                                         const int* s_tgt, const double* __restrict__ phase, const int* s_lat, R ih,
+                                         R* __restrict__ L, int part, int nparts)
 {
     const int nre = lf_nre(p), TS = 2 * p + 1;
     const int ng = (cnt + C - 1) / C, items = nre * ng;
-    for (int it = part * R_T + threadIdx.x; it < items; it += R_T * nparts) {
+    // an equal share of the items; which warps hold them turns with the block
+    // (warps 0 and 1 of every block would share two of the SM's four FP64 units)
+    const int i0 = items * part / nparts, i1 = items * (part + 1) / nparts;
+    for (int it = i0 + (int)((threadIdx.x + 32 * blockIdx.x) & (R_T - 1)); it < i1; it += R_T) {
         const int row = it / ng, c0 = (it - row * ng) * C;
         int k, l, dummy;
         lf_decode(p, row, k, l, dummy);
@@ -535,11 +577,13 @@ __device__ __forceinline__ void rr_apply(int p, int nc, const R* sT, const R* sX
                 xi += cb;
             }
         }
-        const R cr = (k & 1) ? -sC[l] * ih : sC[l] * ih, sr = (k & 1) ? -sS[l] * ih : sS[l] * ih;
+        const R sg = (k & 1) ? -ih : ih;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             if (c0 + c >= cnt) break;
             R* Lt = L + (size_t)s_tgt[c0 + c] * nc;
+            const double* ph = phase + (size_t)s_lat[c0 + c] * 2 * RR_PH + l;
+            const R cr = sg * (R)ph[0], sr = sg * (R)ph[RR_PH];
             atomicAdd(Lt + row, cr * ar[c] - sr * ai[c]);
             if (l > 0) atomicAdd(Lt + lf_im(p, k, l), sr * ar[c] + cr * ai[c]);
         }
@@ -550,8 +594,7 @@ template <typename R>
 __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_src[R_TB], s_tgt[R_TB];
-    __shared__ R sC[RR_PH], sS[RR_PH];
+    __shared__ int s_src[R_TB], s_tgt[R_TB], s_lat[R_TB];
     const int p = g.p, nc = g.nc, nre = lf_nre(p), TS = 2 * p + 1, cb = g.cb, tid = threadIdx.x;
     R* sXr = reinterpret_cast<R*>(smem_raw);  // [(n, m)][cb]
     R* sXi = sXr + nre * cb;
@@ -566,11 +609,9 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
         const int2 pr = (tid < cnt) ? g.pairs[start + tid] : make_int2(-1, -1);
         s_src[tid] = pr.x;
         s_tgt[tid] = pr.y;
-    }
-    if (tid >= 64 && tid < 64 + RR_PH) {
-        const double* ph = g.phase + (size_t)((ox + R_OR) * R_OW + (oy + R_OR)) * 2 * RR_PH + (tid - 64);
-        sC[tid - 64] = (R)ph[0];
-        sS[tid - 64] = (R)ph[RR_PH];
+        int c1, l1;
+        rkey_decode(g.keys[start + min(tid, cnt - 1)], c1, l1, ox, oy, oz);
+        s_lat[tid] = (ox + R_OR) * R_OW + (oy + R_OR);
     }
     const double* Tk = g.tables + (size_t)b.w * TS * TS;
     for (int j = tid; j < TS * TS; j += R_T) sT[j] = (R)Tk[j];
@@ -589,8 +630,10 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
                     lf_decode(p, x, n, m, dummy);
                     const R* Ms = M + (size_t)s_src[q0 + j] * nc;
                     const R mr = Ms[x], mi = m > 0 ? Ms[lf_im(p, n, m)] : R(0);
-                    vr = mr * sC[m] - mi * sS[m];
-                    vi = mr * sS[m] + mi * sC[m];
+                    const double* ph = g.phase + (size_t)s_lat[q0 + j] * 2 * RR_PH + m;
+                    const R cm = (R)ph[0], sm = (R)ph[RR_PH];
+                    vr = mr * cm - mi * sm;
+                    vi = mr * sm + mi * cm;
                     if (refl && ((n + m) & 1)) {
                         vr = -vr;
                         vi = -vi;
@@ -603,11 +646,14 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
             // padded cost of each width: two additions and 2 C multiply-adds per (n, m)
             const int w2 = ((nq + 1) / 2) * 6, w4 = ((nq + 3) / 4) * 10, w8 = ((nq + 7) / 8) * 18;
             if (w8 <= w4 && w8 <= w2)
-                rr_apply<R, 8>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, sC, sS, ih, L, blockIdx.y, gridDim.y);
+                rr_apply<R, 8>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, g.phase, s_lat + q0, ih, L, blockIdx.y,
+                               gridDim.y);
             else if (w4 <= w2)
-                rr_apply<R, 4>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, sC, sS, ih, L, blockIdx.y, gridDim.y);
+                rr_apply<R, 4>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, g.phase, s_lat + q0, ih, L, blockIdx.y,
+                               gridDim.y);
             else
-                rr_apply<R, 2>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, sC, sS, ih, L, blockIdx.y, gridDim.y);
+                rr_apply<R, 2>(p, nc, sT, sXr, sXi, cb, nq, s_tgt + q0, g.phase, s_lat + q0, ih, L, blockIdx.y,
+                               gridDim.y);
         }
     }
 }
@@ -1372,12 +1418,13 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
     g.p = ctx->p;
     g.nc = lf_nc(ctx->p);
     // 32 columns (16 above p = 10) keep several blocks per SM
-    g.cb = ctx->p <= 10 ? 32 : 16;
+    g.cb = ctx->p <= 10 ? 32 : RR_CB;
     g.batches = ctx->m2r_batches.as<int4>();
     g.tables = ctx->m2r_tables.as<double>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
     LF_TRY(m2r_phases64(ctx, st));
     g.phase = ctx->m2r_phase64.as<double>();
+    g.keys = ctx->m2r_keys.as<uint32_t>();
     g.pairs = ctx->m2r_pairs.as<int2>();
     g.levelh = ctx->m2r_levelh.as<double>();
     g.M = ctx->Mexp.ptr;
@@ -1386,10 +1433,12 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
     g.nr = ctx->nrhs_b;
     const int TS = 2 * ctx->p + 1;
     const size_t sm = sizeof(R) * ((size_t)2 * lf_nre(ctx->p) * g.cb + (size_t)TS * TS);
-    // share the rows of each batch between blocks until the longest batch (64
-    // pairs, 15 times the mean in small trees) no longer outlasts the rest
+    // share the rows of each batch between blocks, so that the longest batches
+    // do not outlast the rest; four shares leave every SM quarter a warp
     int parts = 1;
-    while (parts < 8 && (int64_t)ctx->m2r_nbatch * parts < 64 * 152) parts *= 2;
+    while ((parts < 4 && (int64_t)ctx->m2r_nbatch * parts < 64 * 152) ||
+           (parts < 8 && (int64_t)ctx->m2r_nbatch * parts < 8 * 152))
+        parts *= 2;
     LF_CHECK(cudaFuncSetAttribute(k_m2r_rot<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     ++ctx->launches, k_m2r_rot<R><<<dim3(ctx->m2r_nbatch, parts), R_T, sm, st>>>(g);
     return lf_cuda(cudaGetLastError(), "m2r rotated");
