@@ -1250,6 +1250,15 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
         split = 1;
         const int64_t units = (int64_t)leaf.nbox * (list ? list_ny : 1);
         while (split < LFMM_P2P_SPLIT_MAX && units * split * 2 <= want) split *= 2;
+        // long lists in shorter pieces (of 128 sources or more) up to 152 * 256
+        // warps: the far field beside has the higher priority, but its blocks
+        // wait for the near field's to end.  Whole evaluations, split 1 -> 4:
+        // four layers, 262,143 charges 3.07 -> 2.53 ms; 262,144 charges, p = 6 0.588
+        // -> 0.555; interfaces, 50,001 charges (2 -> 4) 1.32 -> 1.25; 65,536 charges
+        // (216 sources per list) gain nothing.
+        const double mean = (double)ctx->levels[ctx->depth].near_count / leaf.nbox * ((double)ctx->n / leaf.nbox);
+        while (warp_kernel && split < LFMM_P2P_SPLIT_MAX && units * split * 2 <= 152 * 256 && mean >= 128.0 * 2 * split)
+            split *= 2;
     }
     a.split = split;
     if (split > 1) {
