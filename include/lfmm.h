@@ -60,10 +60,10 @@ enum {
     LFMM_OPT_TENSOR_CORES = 7,  /* float32 free M2L engine: 2 = automatic (default) and 1: tensor cores (operands
                                    as two float16 pieces, accumulated in order of falling degree; for
                                    11 <= p <= 14 the wide form); 0 = the compensated CUDA-core sums.
-                                   Where (p+1)^2 <= 128 the tensor cores also take the L2L into the
-                                   leaves and the keyed reaction M2L (each key's operator formed in
-                                   shared memory from its Sommerfeld table, eqs. metoleimage1,
-                                   coefintable); 0 puts both on the CUDA cores. */
+                                   The tensor cores also take the keyed reaction M2L (each key's
+                                   operator formed in shared memory from its Sommerfeld table, eqs.
+                                   metoleimage1, coefintable) and, where (p+1)^2 <= 128, the L2L into
+                                   the leaves; 0 puts both on the CUDA cores. */
     LFMM_OPT_P2P_SPLIT = 8,     /* near list of a leaf shared by this many warps/blocks of the P2P kernels:
                                    0 = chosen from the leaf count (default), else 1, 2, 4, 8 or 16 */
     LFMM_OPT_TC_GROUPS = 9,     /* tensor-core free M2L: CTAs per tile of targets (256, or 128 in the wide
