@@ -50,22 +50,27 @@ def fp32_peak_tflops(sm_mhz):
     return SMS * 128 * 2 * sm_mhz * 1e6 / 1e12
 
 
-# Dense TF32 tensor peak: the measured bf16 GEMM rate of the GB300s
-# times the nominal TF32/BF16 ratio (1.1 / 2.25 PFLOP/s); fallback 1.9 PF bf16.
+# Dense tensor peaks: float16 runs at the bf16 rate, the measured bf16 GEMM rate
+# on GB300 (fallback 1.9 PF); TF32 at the nominal TF32/BF16 ratio
+# (1.1 / 2.25 PFLOP/s) of it.
 TF32_PER_BF16 = 1.1 / 2.25
-# DRAM bytes (read + write) of one k_m2l_tc launch per free-space M2L pair,
-# from an ncu capture of the bench's own workload (N=1,048,576, p=10: 245.1 MB
-# read + 33.3 MB written for 10,905,072 pairs), scaled to the bench's pair count.
+# DRAM bytes (read + write) of one k_m2l_tc launch per free-space M2L pair at
+# N=1,048,576, p=10, each from an ncu capture: with TF32 pieces (245.1 MB read +
+# 33.3 MB written for 10,905,072 pairs) and with float16 pieces, the current form
 TC_DRAM_BYTES_PER_PAIR = (245.149952e6 + 33.294592e6) / 10905072
+TC16_DRAM_BYTES_PER_PAIR = (145.3696e6 + 23.028736e6) / 10903404
+
+
+def f16_peak_tflops():
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            return float(json.load(fh)["bf16_tflops"]), "of measured"
+    except Exception:
+        return 1900.0, "of fallback"
 
 
 def tf32_peak_tflops():
-    try:
-        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
-            bf16 = float(json.load(fh)["bf16_tflops"])
-        src = "of measured"
-    except Exception:
-        bf16, src = 1900.0, "of fallback"
+    bf16, src = f16_peak_tflops()
     return bf16 * TF32_PER_BF16, src
 
 
@@ -707,13 +712,13 @@ def main():
     achieved = flops / (m2l_ms / 1e3) / 1e12 if m2l_ms > 0 else None
     tensor_path = results[headline].get("prec", 1) == 1 and (args.p + 1) ** 2 <= 128
     if tensor_path:
-        peak, src = tf32_peak_tflops()
-        roof = {"kernel": "k_m2l_tc (free-space M2L, tcgen05 3xTF32)", "bound": "tensor", "achieved": achieved,
+        peak, src = f16_peak_tflops()
+        roof = {"kernel": "k_m2l_tc (free-space M2L, tcgen05, two float16 pieces per operand)", "bound": "tensor", "achieved": achieved,
                 "peak": peak, "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
-                "traffic": (TC_DRAM_BYTES_PER_PAIR * st["m2l_free"]) if args.p == 10 else None,
-                "peak_note": "dense TF32 = bf16 GEMM burst %s (MEASURED_PEAKS.json) x nominal TF32/BF16 1.1/2.25; "
+                "traffic": (TC16_DRAM_BYTES_PER_PAIR * st["m2l_free"]) if args.p == 10 else None,
+                "peak_note": "dense float16 = the bf16 GEMM burst rate %s (MEASURED_PEAKS.json); "
                              "algorithmic flops = 8 (p+1)^2 (p+1)(p+2)/2 per box pair (the tensor cores execute "
-                             "3 TF32 products of padded 128x128 operators); duration = the stage's CUDA events "
+                             "3 float16 products of padded 128x128 operators); duration = the stage's CUDA events "
                              "inside the timed steps; traffic scaled by pair count from an ncu capture at "
                              "N=1,048,576" % src}
     else:
@@ -747,14 +752,14 @@ def main():
     nc, nre = (args.p + 1) ** 2, (args.p + 1) * (args.p + 2) // 2
     edge = 8 * nc * nre  # flops per parent-child edge (dense complex shift) and per M2L pair
     # the float32 form at (p+1)^2 <= 128 applies the reaction keys on the tensor
-    # cores (k_m2r_tc, 3xTF32): its peak is the dense TF32 rate
+    # cores (k_m2r_tc, float16 pieces): its peak is the dense float16 rate
     r_tc = results[headline].get("prec", 1) == 1 and (args.p + 1) ** 2 <= 128
-    pk_tf32 = tf32_peak_tflops()[0]
+    pk_f16 = f16_peak_tflops()[0]
     work = [("p2m", "k_p2m", st["n"], 20 * nc, "charge", pk32),
             ("m2m", "k_m2l_gemm (M2M)", st["m2m_edges"], edge, "parent-child edge", pk32),
-            ("m2l_reaction", "k_m2r_tc (keyed reaction M2L, tcgen05 3xTF32)" if r_tc
-             else "k_m2r_gemm (keyed reaction M2L)", st["m2l_reaction"], edge, "reaction box pair",
-             pk_tf32 if r_tc else pk32),
+            ("m2l_reaction", "k_m2r_tc (keyed reaction M2L, tcgen05)" if r_tc
+             else "k_m2r_oz / k_m2r_rot (keyed reaction M2L)", st["m2l_reaction"], edge, "reaction box pair",
+             pk_f16 if r_tc else pk32),
             ("l2l", "k_m2l_gemm / k_m2l_tc (L2L)", st["m2m_edges"], edge, "parent-child edge", pk32),
             ("l2p", "k_l2p", st["n"], 20 * nc, "charge", pk32)]
     stage_roofs = []
@@ -765,7 +770,7 @@ def main():
         ach = units * fpu / (ms_s / 1e3) / 1e12
         stage_roofs.append({"stage": stage, "kernel": kern, "units": int(units), "unit": unit,
                             "flops_per_unit": fpu, "ms": ms_s, "achieved_tflops": ach, "peak_tflops": pk,
-                            "peak": "dense TF32 tensor" if pk is pk_tf32 else "FP32 CUDA core",
+                            "peak": "dense float16 tensor" if pk is pk_f16 else "FP32 CUDA core",
                             "frac": ach / pk})
     line = {
         "metric": METRIC,
