@@ -279,7 +279,8 @@ def near_interface_leg(torch, dev, p, flush):
         f.surrogate_train(SURR_SAMPLES, SURR_EPOCHS, SURR_SEED)
         table_err = f.near_tables()
         phis = {}
-        # near-field reaction kernels by quadrature, by the network, by the pre-computed tables
+        # near-field reaction kernels by quadrature (FP64; the float32 form takes its image sums),
+        # by the network, by the pre-computed tables
         for kind, surr, tab in (("quadrature", 0, 0), ("network", 1, 0), ("tables", 0, 1)):
             f.set_option(5, surr)
             f.set_option(10, tab)
