@@ -689,7 +689,7 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 // bounded: on a timeout the CTA counts it in err and skips its read-backs.
 // Measured, p = 10, float16 pieces against TF32 pieces with the operator formed
 // again for every vector: 64 vectors of 262,144 charges 13.8 -> 4.95 ms.  One
-// vector, N = 1M: 0.258 ms with entries formed one at a time, 0.170 ms in blocks.
+// vector, N = 1M: 0.258 ms with entries formed one at a time, 0.17 to 0.19 in blocks.
 // The wide form, 65,536 charges, p = 14: 0.825 ms (k_m2r_rot) -> 0.52 ms, the
 // evaluation's difference from the FP64 form unchanged (3.2e-7).
 // ---------------------------------------------------------------------------
