@@ -895,6 +895,9 @@ static lfmm_status set_option(lfmm_ctx* ctx, int opt, double v)
         int Q = (int)v;
         if (Q < 16 || Q > LFMM_QMAX || (double)Q != v) return fail(ctx, "EINVAL: quadrature nodes out of range");
         ctx->quad_nodes = Q;
+        // the tables of a build are made by the first evaluation; tables made
+        // already are made again by the next one, with the new rule
+        if (ctx->built && ctx->m2r_nbatch > 0) ctx->m2r_dev_pending = 1;
         return fail(ctx, setup_rules(ctx));
     }
     case LFMM_OPT_SURROGATE:

@@ -396,18 +396,16 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
         }
     }
     const int ntab = (int)tdesc.size();
-    const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS, Q = ctx->gl_q_m2l;
+    const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS;
     LF_TRY(lf_reserve(ctx->m2r_tables, (size_t)ntab * TT * 8 + 16));
     LF_TRY(lf_reserve(ctx->m2r_tdesc, (size_t)ntab * sizeof(int4) + 16));
     LF_TRY(lf_reserve(ctx->m2r_ndesc, ndesc.size() * sizeof(int4) + 16));
-    LF_TRY(lf_reserve(ctx->m2r_nodes, ndesc.size() * (size_t)Q * sizeof(double) + 16));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_tdesc.ptr, tdesc.data(), ntab * sizeof(int4), cudaMemcpyHostToDevice, st));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_ndesc.ptr, ndesc.data(), ndesc.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     double* hl = ctx->m2r_levelh_h;
     for (int l = 0; l < 16; ++l) hl[l] = (l <= ctx->depth) ? ctx->levels[l].h : 0.0;
     LF_TRY(lf_reserve(ctx->m2r_levelh, sizeof(double) * 16));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_levelh.ptr, hl, sizeof(double) * 16, cudaMemcpyHostToDevice, st));
-    (void)P;
     ctx->m2r_ntab = ntab;
     // batches of R_TB pairs of one key: key index, first sorted entry, count | key << 8, table
     std::vector<int4>& batches = ctx->m2r_batches_h;
@@ -460,6 +458,8 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
     const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS, Q = ctx->gl_q_m2l;
     size_t sm = sizeof(double) * ((size_t)TT + 2 * (size_t)Q * TS);
     const int nnode = (int)ctx->m2r_ndesc_h.size();
+    // (sized here: LFMM_OPT_QUAD_NODES may have changed Q since the build)
+    LF_TRY(lf_reserve(ctx->m2r_nodes, (size_t)nnode * Q * sizeof(double) + 16));
     auto nodk = (ctx->L >= 3) ? k_m2r_nodes<true> : k_m2r_nodes<false>;
     ++ctx->launches, nodk<<<lf_blocks((int64_t)nnode * Q, 128), 128, 0, st>>>(
         ctx->comp_dev.as<LfmmComp>(), ctx->m2r_ndesc.as<int4>(), nnode, ctx->m2r_levelh.as<double>(),
