@@ -898,7 +898,12 @@ static lfmm_status set_option(lfmm_ctx* ctx, int opt, double v)
         // the tables of a build are made by the first evaluation; tables made
         // already are made again by the next one, with the new rule
         if (ctx->built && ctx->m2r_nbatch > 0) ctx->m2r_dev_pending = 1;
-        return fail(ctx, setup_rules(ctx));
+        // work in flight reads the rule; the uploads run on the legacy stream,
+        // which the context's streams do not wait for
+        LfErr e = lf_cuda(cudaDeviceSynchronize(), "rule in use");
+        if (e.empty()) e = setup_rules(ctx);
+        if (e.empty()) e = lf_cuda(cudaDeviceSynchronize(), "rule upload");
+        return fail(ctx, e);
     }
     case LFMM_OPT_SURROGATE:
         if (v != 0.0 && !ctx->surr_ready) return fail(ctx, "ESTATE: train the surrogate first"), LFMM_ESTATE;

@@ -39,3 +39,24 @@ def test_nodes_changed_between_build_and_evaluation(precision):
     # tables that an evaluation has made already
     assert oracle.err2(ref[128], _phi(w, precision, (16, "build", "evaluate", 128, "evaluate"))) < ROUND[precision]
     assert oracle.err2(ref[16], _phi(w, precision, (128, "build", "evaluate", 16, "evaluate"))) < ROUND[precision]
+
+
+def test_nodes_changed_while_an_evaluation_is_queued():
+    # the option waits for work that reads the rule; the evaluation keeps its own
+    import torch
+    w = workloads.config2(3000, eps=(1.0, 4.5, 1.0))
+    ref = _phi(w, 0, ("build", "evaluate"))
+    q = torch.from_numpy(w.q).cuda()
+    phi = torch.zeros_like(q)
+    side = torch.cuda.Stream()
+    with LayeredFMM(w.d, w.eps, 8, precision=0) as f:
+        f.build(w.xyz, w.layer)
+        f.evaluate(w.q)
+        f.build(w.xyz, w.layer)  # (tables to be made again; every buffer has its size)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(200_000_000)  # ~0.1 s
+            f.evaluate_device(q, phi, stream=side)
+        f.set_option(OPT_QUAD_NODES, 16)
+        torch.cuda.synchronize()
+    assert oracle.err2(ref, phi.cpu().numpy()) < ROUND[0]
