@@ -151,13 +151,15 @@ struct lfmm_ctx {
     // use_tc: 2 automatic and 1: tensor cores, 0: CUDA cores
     int m2l_tc_ok = 0, m2l_tc_ntiles = 0, use_tc = 2, tc_groups = 0;  // tc_groups 0: automatic
     // FP64 free M2L by digit products (lfmm_m2l_oz.cu)
-    DevBuf oz_A, oz_Ms, oz_cscale, oz_perm, oz_emin, oz_tiles, oz_mseg;
+    DevBuf oz_A, oz_Ms, oz_cscale, oz_perm, oz_tiles, oz_mseg;
     std::vector<int4> oz_tiles_h, oz_mseg_h;
     int oz_ntiles = 0, oz_ready = 0, oz_nk = 0;
     int m2l_tc_wide = 0;  // tensor-core free M2L in its wide form ((p+1)^2 > 128): no tensor-core M2M / L2L
     // reaction M2L grouped by geometry key on interface-aligned levels
     DevBuf m2r_keys, m2r_order, m2r_tgt, m2r_kstart, m2r_kval, m2r_tables, m2r_levelh, m2r_batches;
     DevBuf m2r_tdesc;  // table descriptors (component | level << 8, node set, rho^2, oz)
+    DevBuf m2r_emin;    // smallest exponent that scales each value of a table, [2p + 1][2p + 1] (p <= 15)
+    DevBuf m2r_tscale;  // per table: exponent that puts its float16 operators into range
     DevBuf m2r_ndesc, m2r_nodes;  // node sets (component, level, oz) and the remainder at their quadrature nodes
     std::vector<int4> m2r_tdesc_h, m2r_ndesc_h, m2r_batches_h;  // host staging of asynchronous uploads
     int m2r_pending_ne = 0;             // reaction M2L entries whose key grouping awaits lf_prepare_m2r_finish

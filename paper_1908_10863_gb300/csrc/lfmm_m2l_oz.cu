@@ -437,33 +437,18 @@ bool lf_m2l_oz_ok(const lfmm_ctx* ctx) { return ctx->m2l_rm > 0 && lf_nc(ctx->p)
 static LfErr oz_setup(lfmm_ctx* ctx, cudaStream_t st)
 {
     if (ctx->oz_ready) return LfErr();
-    const int p = ctx->p, nc = lf_nc(p), nh = (nc + 127) / 128, RP = ctx->m2l_rp, TS = 2 * p + 1;
+    const int p = ctx->p, nc = lf_nc(p), nh = (nc + 127) / 128, RP = ctx->m2l_rp;
     std::vector<int> perm, e;
     lf_coef_order(p, perm);
     lf_coef_exponents(p, e);
     const int nk = (int)perm.size(), nkc = (nk + TH_KC - 1) / TH_KC;
     std::vector<double> cs(nc);
     for (int j = 0; j < nc; ++j) cs[j] = std::ldexp(1.0, e[j]);
-    // for every (N, mu) the smallest exponent its table value is scaled with:
-    // terms T(n + k, l + m) and T(n + k, |l - m|) of inputs (n, m), outputs (k, l)
-    std::vector<int> emin((size_t)TS * TS, 1000);
-    for (int n = 0; n <= p; ++n)
-        for (int m = 0; m <= n; ++m)
-            for (int k = 0; k <= p; ++k)
-                for (int l = 0; l <= k; ++l) {
-                    const int x = e[lf_re(n, m)] + e[lf_re(k, l)];
-                    int& a = emin[(size_t)(n + k) * TS + l + m];
-                    int& b = emin[(size_t)(n + k) * TS + std::abs(l - m)];
-                    a = std::min(a, x);
-                    b = std::min(b, x);
-                }
     LF_TRY(lf_reserve(ctx->oz_cscale, nc * sizeof(double)));
     LF_TRY(lf_reserve(ctx->oz_perm, nk * sizeof(int)));
-    LF_TRY(lf_reserve(ctx->oz_emin, emin.size() * sizeof(int)));
     LF_TRY(lf_reserve(ctx->oz_A, (size_t)OZ_NALL * nh * nkc * OZ_S * OZ_A_BYTES));
     LF_CHECK(cudaMemcpyAsync(ctx->oz_cscale.ptr, cs.data(), nc * sizeof(double), cudaMemcpyHostToDevice, st));
     LF_CHECK(cudaMemcpyAsync(ctx->oz_perm.ptr, perm.data(), nk * sizeof(int), cudaMemcpyHostToDevice, st));
-    LF_CHECK(cudaMemcpyAsync(ctx->oz_emin.ptr, emin.data(), emin.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     int* bad = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_OZ_BAD_OFF);
     LF_CHECK(cudaMemsetAsync(bad, 0, sizeof(int), st));
     LF_CHECK(cudaFuncSetAttribute(k_m2l_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));

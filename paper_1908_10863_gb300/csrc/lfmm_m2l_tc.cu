@@ -757,6 +757,22 @@ LfErr lf_setup_m2l_tc(lfmm_ctx* ctx, int KP, int RP)
     for (int k = 0; k < nc; ++k) cs[k] = std::ldexp(1.f, e[k]);
     LF_TRY(lf_reserve(ctx->tc_cscale, nc * sizeof(float)));
     LF_CHECK(cudaMemcpy(ctx->tc_cscale.ptr, cs.data(), nc * sizeof(float), cudaMemcpyHostToDevice));
+    // for every (N, mu) the smallest exponent its reaction table value is scaled
+    // with: terms T(n + k, l + m) and T(n + k, |l - m|) of inputs (n, m), outputs (k, l)
+    const int p = ctx->p, TS = 2 * p + 1;
+    std::vector<int> emin((size_t)TS * TS, 1000);
+    for (int n = 0; n <= p; ++n)
+        for (int m = 0; m <= n; ++m)
+            for (int k = 0; k <= p; ++k)
+                for (int l = 0; l <= k; ++l) {
+                    const int x = e[lf_re(n, m)] + e[lf_re(k, l)];
+                    int& a = emin[(size_t)(n + k) * TS + l + m];
+                    int& b = emin[(size_t)(n + k) * TS + std::abs(l - m)];
+                    a = std::min(a, x);
+                    b = std::min(b, x);
+                }
+    LF_TRY(lf_reserve(ctx->m2r_emin, emin.size() * sizeof(int)));
+    LF_CHECK(cudaMemcpy(ctx->m2r_emin.ptr, emin.data(), emin.size() * sizeof(int), cudaMemcpyHostToDevice));
     ctx->tc_nk = (int)perm.size();
     LF_TRY(lf_reserve(ctx->tc_perm, perm.size() * sizeof(int)));
     LF_CHECK(cudaMemcpy(ctx->tc_perm.ptr, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice));

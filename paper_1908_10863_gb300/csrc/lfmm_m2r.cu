@@ -173,12 +173,16 @@ __global__ void __launch_bounds__(128) k_m2r_nodes(const LfmmComp* __restrict__ 
 // One Sommerfeld table per (component, level, rho^2, oz): the table depends on
 // the lateral distance only; the azimuth enters through the phases applied
 // when the operator is formed.  tdesc: component | level << 8, node set, rho^2, oz.
+// tscale (p <= 15): the exponent s for which no entry of an operator made of the
+// table, two values at most with their scales 2^{-e} (emin), reaches 2^{15 - s}.
 __global__ void __launch_bounds__(128) k_m2r_tables(const LfmmComp* __restrict__ comps, const int4* __restrict__ tdesc,
                                                     int ntab, const double* __restrict__ levelh,
                                                     const double* __restrict__ zfrac, int P,
                                                     const double* __restrict__ gt, const double* __restrict__ gw, int Q,
-                                                    const double* __restrict__ nodes, double* __restrict__ tables)
+                                                    const double* __restrict__ nodes, double* __restrict__ tables,
+                                                    const int* __restrict__ emin, int* __restrict__ tscale)
 {
+    __shared__ int s_exp;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int TS = 2 * P + 1, TT = TS * TS;
     double* sT = reinterpret_cast<double*>(smem_raw);
@@ -192,16 +196,25 @@ __global__ void __launch_bounds__(128) k_m2r_tables(const LfmmComp* __restrict__
     const double vz = (double)oz + zfrac[c * 16 + l];  // image offset n + f in box units
     const double zz = (cp.a == 1) ? vz : -vz;
     for (int j = threadIdx.x; j < TT; j += blockDim.x) sT[j] = 0.0;
+    if (threadIdx.x == 0) s_exp = -4096;
     __syncthreads();
     lf_sommerfeld_table_block<false>(cp, rho, zz, levelh[l], 2 * P, sT, TS, Q, gt, gw, sJ, sA,
                                      nodes + (size_t)d.y * Q);
     double* out = tables + (size_t)k * TT;
+    int ex = -4096;  // largest binary exponent of a scaled value
     for (int j = threadIdx.x; j < TT; j += blockDim.x) {
         int N = j / TS, mu = j - N * TS;
         double v = (mu <= N) ? sT[j] : 0.0;
         if (cp.a == 2 && ((N + mu) & 1)) v = -v;
         out[j] = v;
+        if (emin && mu <= N && v != 0.0)
+            ex = max(ex, (int)(((unsigned)__double2hiint(v) >> 20) & 0x7ffu) - 1023 - emin[j]);
     }
+    if (!emin) return;
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_exp, ex);
+    __syncthreads();
+    if (threadIdx.x == 0) tscale[k] = max(-100, min(100, 13 - s_exp));  // (float32 powers of two)
 }
 
 // ---------------------------------------------------------------------------
@@ -399,6 +412,7 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
     const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS;
     LF_TRY(lf_reserve(ctx->m2r_tables, (size_t)ntab * TT * 8 + 16));
     LF_TRY(lf_reserve(ctx->m2r_tdesc, (size_t)ntab * sizeof(int4) + 16));
+    LF_TRY(lf_reserve(ctx->m2r_tscale, (size_t)ntab * sizeof(int) + 16));
     LF_TRY(lf_reserve(ctx->m2r_ndesc, ndesc.size() * sizeof(int4) + 16));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_tdesc.ptr, tdesc.data(), ntab * sizeof(int4), cudaMemcpyHostToDevice, st));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_ndesc.ptr, ndesc.data(), ndesc.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
@@ -468,7 +482,8 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
     ++ctx->launches, k_m2r_tables<<<ntab, 128, sm, st>>>(
         ctx->comp_dev.as<LfmmComp>(), ctx->m2r_tdesc.as<int4>(), ntab, ctx->m2r_levelh.as<double>(),
         ctx->m2r_zfrac.as<double>(), P, ctx->gl_t_m2l.as<double>(), ctx->gl_w_m2l.as<double>(), Q,
-        ctx->m2r_nodes.as<double>(), ctx->m2r_tables.as<double>());
+        ctx->m2r_nodes.as<double>(), ctx->m2r_tables.as<double>(), ctx->m2r_emin.as<int>(),
+        ctx->m2r_tscale.as<int>());
     LF_TRY(lf_cuda(cudaGetLastError(), "m2r tables"));
     if (ctx->m2r_nent > 0) {
         LF_TRY(lf_reserve(ctx->m2r_pairs, (size_t)ctx->m2r_nent * sizeof(int2) + 16));
@@ -668,7 +683,9 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 // of the MMA's A operand (M = 128 output coefficients, K = the input
 // coefficients by falling degree in chunks of 32), scaled like the free M2L's
 // operators (lfmm_m2l_tc.cu: 2^{-e} per coefficient, folded into the signs
-// below).  The source multipoles (B operand) are the scaled float16 pieces
+// below) and by a power of two of the table's own (tscale): the image series of
+// a thin layer of high permittivity adds up to thousands, weak reflections to
+// little, and float16 has five exponent bits.  The source multipoles (B operand) are the scaled float16 pieces
 // which that M2L split once per evaluation, gathered by 16-byte cp.async;
 // products a2 x1 + a1 x2 + a1 x1.  Operator entries come from a table W of the
 // complex reaction coefficient extended to negative orders.  They are formed in
@@ -698,8 +715,6 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 #define RT_NKC 4                        // K chunks at most where the operator is kept
 #define RT_A_CHUNK (128 * TC_ROWB)      // one K chunk of one operator piece: 128 rows x 64 B
 #define RT_X_CHUNK (R_TB * TC_ROWB)     // one K chunk of one multipole piece and vector: 64 rows x 64 B
-#define RT_ASHIFT 8                     // operators carry 2^8: entries (reflections and image sums included) stay
-                                        // far inside float16's range
 template <int V, bool WIDE>
 struct RtShape {
     static constexpr int P = WIDE ? 14 : 10;                   // largest order
@@ -719,6 +734,7 @@ struct RTcArgs {
     int parts;              // 128-row parts of the outputs
     const int4* batches;    // key index, first sorted entry, count | key << 8, table
     const double* tables;   // [table][TS][TS]
+    const int* tscale;      // per table: its operators carry 2^tscale (k_m2r_tables)
     const LfmmComp* comps;
     const float* phase;     // [225 lateral offsets][cos | sin][RT_PH] (k_m2r_phase)
     const int2* pairs;      // (source box, target box) per sorted entry (k_m2r_pairs)
@@ -747,6 +763,8 @@ __global__ void k_m2r_phase(int p, float* out)
     out[(size_t)b * 2 * RT_PH + RT_PH + m] = (float)sn;
 }
 
+__device__ __forceinline__ float rt_pow2(int e) { return __int_as_float((e + 127) << 23); }  // |e| <= 126
+
 template <int V, bool WIDE>
 __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(RTcArgs g)
 {
@@ -756,7 +774,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 511) &
                                                          ~(uintptr_t)511);
     unsigned char* smx = sm + S::NA * 2 * RT_A_CHUNK;
-    // W(N, mu) = T(N, |mu|) e^{i mu phi} for mu in [-2p, 2p], extended to
+    // W(N, mu) = 2^tscale T(N, |mu|) e^{i mu phi} for mu in [-2p, 2p], extended to
     // negative orders by W(N, -mu) = (-1)^mu conj W(N, mu); [N][mu + 2p], rows of 4p + 1
     __shared__ float2 sW[S::W];
     __shared__ float sPh[2 * RT_PH];
@@ -772,6 +790,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
+    __shared__ float s_as;  // 2^-tscale
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int p = g.p, nc = g.nc, nkc = g.nkc, TS = 2 * p + 1, WS = 4 * p + 1, TSZ = TS * WS;
     const int part = WIDE ? blockIdx.x % g.parts : 0;
@@ -779,6 +798,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
     // the batch carries its key and table: one dependent load to everything else
     const int start = b.y, cnt = b.z & 255, tab = b.w;
     if (cnt <= 0 || cnt > R_TB) return;
+    const int te = g.tscale[tab];  // (used once W is formed)
     const int Np = (cnt + 15) & ~15;  // columns per vector
     int c, lev, ox, oy, oz;
     rkey_decode((uint32_t)b.z >> 8, c, lev, ox, oy, oz);
@@ -789,21 +809,20 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
         const int i = 128 * part + 2 * tid;
         int4 r = make_int4(-1, -1, 0, 0);
         float2 sk = make_float2(0.f, 0.f);
-        const float as = (float)(1 << RT_ASHIFT);
         if (i < g.nk) {
             r.x = g.perm[i];
             r.y = g.perm[i + 1];
             int k, l, im;
             lf_decode(p, r.x, k, l, im);
             r.z = r.w = k * WS + l + 2 * p;
-            sk.x = sk.y = ((k & 1) ? -as : as) / g.cscale[r.x];
+            sk.x = sk.y = ((k & 1) ? -1.f : 1.f) / g.cscale[r.x];
             if (l == 0) {
                 r.w = -1;  // (not an Re / Im pair)
                 sk.y = 0.f;
                 if (r.y >= 0) {
                     lf_decode(p, r.y, k, l, im);
                     r.w = k * WS + l + 2 * p;
-                    sk.y = ((k & 1) ? -as : as) / g.cscale[r.y];
+                    sk.y = ((k & 1) ? -1.f : 1.f) / g.cscale[r.y];
                 }
             }
         }
@@ -865,9 +884,11 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
     const uint32_t tmem = s_tmem;
     {
         const double* Tk = g.tables + (size_t)tab * TS * TS;
+        const float as = rt_pow2(te);
+        if (tid == 0) s_as = rt_pow2(-te);
         for (int j = tid; j < TSZ; j += RT_THREADS) {
             const int Nn = j / WS, mu = j - Nn * WS - 2 * p, a = mu < 0 ? -mu : mu;
-            const float t = (float)Tk[Nn * TS + a];
+            const float t = (float)Tk[Nn * TS + a] * as;
             float wr = t * sPh[a], wi = t * sPh[RT_PH + a];
             if (mu < 0) {
                 if (a & 1) wr = -wr; else wi = -wi;
@@ -994,7 +1015,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
 #pragma unroll
             for (int v = 0; v < V; ++v)
                 sc[v] = rs * (float)(1.0 / hl) /
-                        (tc_scale(g.gmax[(size_t)min(r0 + v, g.nr - 1) * 32 + lev]) * (float)(1 << RT_ASHIFT));
+                        tc_scale(g.gmax[(size_t)min(r0 + v, g.nr - 1) * 32 + lev]) * s_as;
             for (int c0 = 32 * (warp >> 2); c0 < nv * Np; c0 += 64) {
                 float v[32];
                 tc_ld32(tmem + ((uint32_t)(32 * q4) << 16) + (uint32_t)c0, v);
@@ -1399,7 +1420,7 @@ static LfErr m2r_apply_oz(lfmm_ctx* ctx, cudaStream_t st)
     g.Ms = ctx->oz_Ms.as<__half>();
     g.cscale = ctx->oz_cscale.as<double>();
     g.perm = ctx->oz_perm.as<int>();
-    g.emin = ctx->oz_emin.as<int>();
+    g.emin = ctx->m2r_emin.as<int>();
     g.gmax = reinterpret_cast<unsigned long long*>(ctx->counts.as<char>() + LFMM_TCMAX_OFF);
     g.L = ctx->Lexp.as<double>();
     g.ms_stride = (size_t)ctx->nbox_total * OZ_S * g.nkc * TH_KC;
@@ -1466,6 +1487,7 @@ static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
     g.nkc = (g.nk + TH_KC - 1) / TH_KC;
     g.batches = ctx->m2r_batches.as<int4>();
     g.tables = ctx->m2r_tables.as<double>();
+    g.tscale = ctx->m2r_tscale.as<int>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
     g.pairs = ctx->m2r_pairs.as<int2>();
     g.levelh = ctx->m2r_levelh.as<double>();
