@@ -881,7 +881,8 @@ static lfmm_status set_option(lfmm_ctx* ctx, int opt, double v)
         if (v != 0.0 && v != 1.0) return fail(ctx, "EINVAL: precision must be 0 or 1");
         if (v == 1.0 && ctx->p > 14) return fail(ctx, "EINVAL: the FP32 form supports p <= 14");
         ctx->precision = (int)v;
-        const LfErr e = auto_near_tables(ctx);
+        LfErr e = auto_near_tables(ctx);
+        if (e.empty() && ctx->built) e = lf_oz_prepare(ctx, ctx->s_main);
         return e.empty() ? LFMM_OK : fail(ctx, e);
     }
     case LFMM_OPT_LEAF_CAP:
@@ -991,6 +992,7 @@ lfmm_status lf_build_dev(lfmm_ctx* ctx, int64_t n, const double* xyz_dev, const 
     ctx->built = true;
     ++ctx->serial;
     e = auto_near_tables(ctx);
+    if (e.empty()) e = lf_oz_prepare(ctx, ctx->s_main);
     if (!e.empty()) return fail(ctx, e);
     return LFMM_OK;
 }

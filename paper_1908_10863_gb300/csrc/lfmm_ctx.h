@@ -315,6 +315,7 @@ LfErr lf_tc_split(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2l_tc(lfmm_ctx* ctx, cudaStream_t st);
 // ---- FP64 free M2L by digit products (lfmm_m2l_oz.cu) ----
 bool lf_m2l_oz_ok(const lfmm_ctx* ctx);
+LfErr lf_oz_prepare(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_oz_split(lfmm_ctx* ctx, cudaStream_t st);
 LfErr lf_m2l_oz(lfmm_ctx* ctx, cudaStream_t st);
 void lf_coef_order(int p, std::vector<int>& perm);

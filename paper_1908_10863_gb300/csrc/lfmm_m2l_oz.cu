@@ -432,11 +432,14 @@ __global__ void __launch_bounds__(256) k_oz_split(const double* __restrict__ M, 
 // ---------------------------------------------------------------------------
 bool lf_m2l_oz_ok(const lfmm_ctx* ctx) { return ctx->m2l_rm > 0 && lf_nc(ctx->p) <= 256; }
 
-// operator digits, coefficient scales and order, once per context (the first
-// FP64 evaluation; a captured batch graph never sees it)
-static LfErr oz_setup(lfmm_ctx* ctx, cudaStream_t st)
+// operator digits, coefficient scales and order, once per context: at the end of
+// the first build of the FP64 form that has M2L pairs, or when a built context
+// takes that form.  It reads the range check back, so no evaluation may be the
+// first to come here (lfmm_evaluate_device does not wait for the device).
+LfErr lf_oz_prepare(lfmm_ctx* ctx, cudaStream_t st)
 {
-    if (ctx->oz_ready) return LfErr();
+    if (ctx->oz_ready || ctx->precision || !lf_m2l_oz_ok(ctx)) return LfErr();
+    if (!(ctx->m2l_ntiles > 0 && ctx->oz_ntiles > 0) && ctx->m2r_nbatch == 0) return LfErr();
     const int p = ctx->p, nc = lf_nc(p), nh = (nc + 127) / 128, RP = ctx->m2l_rp;
     std::vector<int> perm, e;
     lf_coef_order(p, perm);
@@ -468,7 +471,7 @@ static LfErr oz_setup(lfmm_ctx* ctx, cudaStream_t st)
 // reaction M2L of this evaluation
 LfErr lf_oz_split(lfmm_ctx* ctx, cudaStream_t st)
 {
-    LF_TRY(oz_setup(ctx, st));
+    LF_TRY(lf_oz_prepare(ctx, st));  // (done already, unless that failed)
     const int nb = ctx->nbox_total, nr = ctx->nrhs_b, nc = lf_nc(ctx->p), nk = ctx->oz_nk;
     const int mrow = (nk + TH_KC - 1) / TH_KC * TH_KC;
     LF_TRY(lf_reserve(ctx->oz_Ms, (size_t)nb * OZ_S * mrow * sizeof(__half) * nr));
