@@ -263,7 +263,8 @@ def run_form(f, xyz_d, lay_d, q_d, phi_d, fld_d, torch, steps, warmup, flush):
 
 
 def near_interface_leg(torch, dev, p, flush):
-    """P2P stage and whole step on the near-interface workload: quadrature vs network."""
+    """P2P stage and whole step on the near-interface workload: the default of a
+    context without networks (image sums), the quadrature, the network, the tables."""
     from paper_1908_10863_gb300 import LayeredFMM, workloads
     import oracle
     w = workloads.near_interface(1 << 18)
@@ -276,12 +277,13 @@ def near_interface_leg(torch, dev, p, flush):
                        "q~U[-1,1], p=%d, leaf 40" % (w.n, p)}
     for prec, pname in ((0, "fp64"), (1, "fp32")):
         f = LayeredFMM(w.d, w.eps, p, precision=prec)
-        f.surrogate_train(SURR_SAMPLES, SURR_EPOCHS, SURR_SEED)
-        table_err = f.near_tables()
         phis = {}
-        # near-field reaction kernels by quadrature (FP64; the float32 form takes its image sums),
-        # by the network, by the pre-computed tables
-        for kind, surr, tab in (("quadrature", 0, 0), ("network", 1, 0), ("tables", 0, 1)):
+        # near-field reaction kernels by image sums (before the context holds networks), by
+        # quadrature, by the network, by the pre-computed tables
+        for kind, surr, tab in (("images", 0, 2), ("quadrature", 0, 0), ("network", 1, 2), ("tables", 0, 1)):
+            if kind == "quadrature":
+                f.surrogate_train(SURR_SAMPLES, SURR_EPOCHS, SURR_SEED)
+                table_err = f.near_tables()
             f.set_option(5, surr)
             f.set_option(10, tab)
             times, launches, stages = run_form(f, xyz_d, lay_d, q_d, phi_d, fld_d, torch, 2, 1, flush)
@@ -289,8 +291,8 @@ def near_interface_leg(torch, dev, p, flush):
             out[pname + "_" + kind] = {"ms_per_step": sum(times) / len(times), "p2p_ms": stages["p2p"],
                                        "pairs_network": st["surr_net_pairs"], "pairs_quadrature": st["surr_quad_pairs"]}
             phis[kind] = phi_d.cpu().numpy().copy()
-        f.set_option(10, 0)
-        for kind in ("network", "tables"):
+        f.set_option(10, 2)
+        for kind in ("images", "network", "tables"):
             out[pname + "_" + kind]["err2_phi_vs_quadrature"] = oracle.err2(phis["quadrature"], phis[kind])
             out[pname + "_" + kind + "_p2p_speedup"] = (out[pname + "_quadrature"]["p2p_ms"] /
                                                         out[pname + "_" + kind]["p2p_ms"])

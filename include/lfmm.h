@@ -72,12 +72,14 @@ enum {
                                    21, i.e. 9 offsets per accumulation; 63 in the wide form) */
     LFMM_OPT_NEAR_TABLES = 10,  /* near-field reaction kernels: 2 = automatic (default): image sums where the
                                    medium's remainders have them (up to three layers whose reflections'
-                                   product stays below ~0.97), else the float32 form takes the remainder
+                                   product stays below ~0.97; in the float32 form while the rule has at
+                                   most 20 images), else the float32 form takes the remainder
                                    from pre-computed tables (deviation from the quadrature ~2e-8 to 1e-5,
                                    see lfmm_near_tables) once a build's near lists hold reaction pairs,
                                    building them at the end of that build (once per context), and the
-                                   FP64 form the quadrature; 1 = tables in both forms (built on first
-                                   use); 0 = image sums or the quadrature, no tables */
+                                   FP64 form the quadrature (as does an FP64 context that holds trained
+                                   networks); 1 = tables in both forms (built on first
+                                   use); 0 = quadrature */
     LFMM_OPT_TC_PERSISTENT = 11, /* tensor-core free M2L: 1 = one persistent CTA per SM walking the
                                    (tile, offset group) units with a double-buffered accumulator, for
                                    launches of at least 4 units per SM; 0 = one CTA per unit, two CTAs per
@@ -148,8 +150,9 @@ lfmm_status lfmm_evaluate_device(lfmm_ctx* ctx, int nrhs, const double* q_dev, d
  * interpolated kernels from the quadrature at 2048 seeded points per
  * component, relative to |I_00| (field kernels times the distance), to
  * *max_rel_err (may be NULL).  Does not change LFMM_OPT_NEAR_TABLES: with its
- * automatic default the float32 form uses built tables wherever the near
- * lists hold reaction pairs; the float32 kernels read a float32 copy. */
+ * automatic default the float32 form uses built tables where the near lists
+ * hold reaction pairs and the medium has no (short) image rule; the float32
+ * kernels read a float32 copy. */
 lfmm_status lfmm_near_tables(lfmm_ctx* ctx, double* max_rel_err);
 
 /* Self-check of failure detection (the paper has no counterpart).  Every
@@ -248,10 +251,9 @@ lfmm_status lfmm_batch_info(lfmm_batch* b, int64_t* out, int nout);
  *   1. tensor-core free M2L (float32 form) for every member, for none, or for
  *      the members of at least 20,000 / 60,000 charges;
  *   2. near-list split of the P2P kernels: automatic, 1, 2, 4, 8;
- *   3. near-field reaction kernels by quadrature (0) or from the pre-computed
- *      tables (1; members whose near lists hold reaction pairs; see
- *      lfmm_near_tables).  The members' automatic default already takes the
- *      tables in the float32 form.
+ *   3. near-field reaction kernels by the automatic choice of
+ *      LFMM_OPT_NEAR_TABLES (0) or from the pre-computed tables (1; members
+ *      whose near lists hold reaction pairs; see lfmm_near_tables).
  * A member tuned alone picks the settings that fill the GPU with its own
  * work; in a batch the members fill it together, which is what this times.
  * Afterwards every member holds the winner.  Needs use_graph = 1.

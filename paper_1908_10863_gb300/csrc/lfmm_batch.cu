@@ -249,8 +249,8 @@ lfmm_status lfmm_batch_evaluate(lfmm_batch* b, const double* q, double* phi, dou
 
 // One candidate setting applied to every member: tensor-core free M2L for the
 // members with at least tc_min charges (float32 form), near-list split, and
-// the pre-computed near-field tables for members whose near lists hold
-// reaction pairs.
+// the pre-computed near-field tables in place of the automatic choice for
+// members whose near lists hold reaction pairs.
 struct BatchSetting {
     int64_t tc_min;
     int split;
@@ -264,7 +264,7 @@ static lfmm_status apply_setting(lfmm_batch* b, const BatchSetting& s)
         lfmm_status st = lfmm_set_option(c, LFMM_OPT_TENSOR_CORES, c->n >= s.tc_min ? 1.0 : 0.0);
         if (st == LFMM_OK) st = lfmm_set_option(c, LFMM_OPT_P2P_SPLIT, (double)s.split);
         const bool tab = s.tables && c->near_reaction_entries > 0;
-        if (st == LFMM_OK) st = lfmm_set_option(c, LFMM_OPT_NEAR_TABLES, tab ? 1.0 : 0.0);
+        if (st == LFMM_OK) st = lfmm_set_option(c, LFMM_OPT_NEAR_TABLES, tab ? 1.0 : 2.0);
         if (st != LFMM_OK) return bfail(b, "problem " + std::to_string(i) + ": " + c->err, st);
     }
     return LFMM_OK;

@@ -145,7 +145,7 @@ struct lfmm_ctx {
     DevBuf near_tab;            // remainder tables of the near-field reaction kernels
     DevBuf near_tab4;           // their float32 copy, one float4 per grid point (float32 kernels)
     int near_tab_ready = 0;
-    int use_near_tab = 2;       // 0 quadrature, 1 tables, 2 tables in the float32 form (default)
+    int use_near_tab = 2;       // 0 quadrature, 1 tables, 2 image sums, else tables (float32) or quadrature (default)
     double near_tab_err = -1.0;  // largest relative deviation from the quadrature at the check points
     double m2l_levelh_h[16] = {0};
     // use_tc: 2 automatic and 1: tensor cores, 0: CUDA cores
@@ -249,13 +249,13 @@ LfErr lf_p2p_pair_stats(lfmm_ctx* ctx);
 inline bool lf_tc_on(const lfmm_ctx* ctx) { return ctx->m2l_tc_ok && ctx->use_tc != 0; }
 
 // whether the float32 near field takes its reaction remainders from the image
-// rule: unless the tables are asked for, and while the rule is short.  A pair
+// rule: by the automatic setting, and while the rule is short.  A pair
 // costs ~9 instructions per image against 16 gathered loads and ~100
 // instructions of the tables.
 #define LFMM_IMG32_MAX 20
 inline bool lf_img32_on(const lfmm_ctx* ctx)
 {
-    return ctx->img_ok && ctx->use_near_tab != 1 && (ctx->img32.n <= LFMM_IMG32_MAX || ctx->use_near_tab == 0);
+    return ctx->img_ok && ctx->use_near_tab == 2 && ctx->img32.n <= LFMM_IMG32_MAX;
 }
 
 // ---- free-space M2L GEMM (lfmm_m2l.cu) ----

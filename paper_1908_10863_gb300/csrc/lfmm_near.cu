@@ -1232,13 +1232,13 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
     // Float32: reaction pairs in k_p2p_list, by the image rule where it is
     // short (lf_img32_on), else from the tables (media of four and five layers,
     // slow image series) or the quadrature.  FP64: by the image rule in the same
-    // kernel, unless the tables are asked for or the medium has no rule; the
+    // kernel, unless the tables or the quadrature are asked for or the medium has no rule; the
     // FP64 form of a context that holds trained networks keeps the quadrature
     // for the pairs outside the network runs (test_surrogate_gain_in_near_field
     // states the network's gain over it).  Lists without reaction pairs take
     // k_p2p_list in FP64 and with several charge vectors.
     const bool react = ctx->near_reaction_entries > 0;
-    const bool img = ctx->precision ? lf_img32_on(ctx) : ctx->img_ok && ctx->use_near_tab != 1 && !ctx->surr_ready;
+    const bool img = ctx->precision ? lf_img32_on(ctx) : ctx->img_ok && ctx->use_near_tab == 2 && !ctx->surr_ready;
     const bool list = !net && (ctx->precision ? react || nr > 1 : !react || (img && !general));
     const int list_rb = nr == 1 ? 1 : (nr == 2 ? 2 : (nr <= 4 ? 4 : 8));  // right-hand sides per batch
     const int list_ny = (nr + list_rb - 1) / list_rb;
@@ -1269,7 +1269,7 @@ LfErr lf_near_field(lfmm_ctx* ctx, cudaStream_t st)
     LfImgRule<float> net32 = ctx->img32;
     LfImgRule<double> net64 = ctx->img64;
     if (!lf_img32_on(ctx)) net32.n = -1;
-    if (!ctx->img_ok || ctx->use_near_tab == 1) net64.n = -1;
+    if (!ctx->img_ok || ctx->use_near_tab != 2) net64.n = -1;
     if (list) {
         const dim3 g(lf_blocks((int64_t)leaf.nbox * split, PL_WARPS), list_ny);
         const int T = 32 * PL_WARPS, nb = leaf.nbox, nc = ctx->ncomp;
