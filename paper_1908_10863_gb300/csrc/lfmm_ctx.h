@@ -232,6 +232,16 @@ inline T* lf_pin(const lfmm_ctx* ctx, size_t off)
 {
     return reinterpret_cast<T*>(static_cast<char*>(ctx->host_pin) + off);
 }
+// Dynamic shared memory that a kernel may ask for.  The limit belongs to the
+// process and launches of other contexts read it at the same time (one host
+// thread per context), so every caller of a kernel sets the same limit, the
+// most that any launch of it needs, not its own launch's size.
+template <typename K>
+inline LfErr lf_smem_limit(K* kern, size_t most)
+{
+    return lf_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most),
+                   "shared memory limit");
+}
 // device-to-host copy ordered after the work queued on st, complete on return
 inline cudaError_t lf_d2h(void* dst, const void* src, size_t bytes, cudaStream_t st)
 {

@@ -686,11 +686,11 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
     // downward pass: all M2L into zeroed L, then L2L top-down (child += shifted parent)
     const int Q = ctx->gl_q_m2l;
     const size_t msm_f = m2l_smem<R>(p, Q, false), msm_r = m2l_smem<R>(p, Q, true);
-    LF_CHECK(cudaFuncSetAttribute(k_m2l<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm_f));
-    LF_CHECK(cudaFuncSetAttribute(k_m2l<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm_r));
+    const size_t most_r = m2l_smem<R>(LFMM_PMAX, LFMM_QMAX, true);
+    LF_TRY(lf_smem_limit(k_m2l<R, false>, m2l_smem<R>(LFMM_PMAX, LFMM_QMAX, false)));
+    LF_TRY(lf_smem_limit(k_m2l<R, true>, most_r));
     const bool general = ctx->L >= 3;
-    if (general)
-        LF_CHECK(cudaFuncSetAttribute(k_m2l<R, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm_r));
+    if (general) LF_TRY(lf_smem_limit(k_m2l<R, true, true>, most_r));
     const int mth = ((nc + 31) / 32) * 32;
     const size_t lsm = sizeof(R) * (nc + 2 * (size_t)nre);
     const int lth = ((nre + 31) / 32) * 32;
@@ -779,7 +779,8 @@ static LfErr far_field(lfmm_ctx* ctx, cudaStream_t st)
         const int nleaf = (int)std::max<size_t>(1, std::min<size_t>(span, L2P_SMEM / per));
         const auto kern = walk_parts > 1 ? (nr == 1 ? k_l2p<R, 1, 4> : k_l2p<R, 4, 4>)
                                          : (nr == 1 ? k_l2p<R, 1, 1> : k_l2p<R, 4, 1>);
-        LF_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per * nleaf)));
+        static_assert((LFMM_PMAX + 1) * (LFMM_PMAX + 2) / 2 * 4 * sizeof(L2PFac<R>) <= L2P_SMEM, "one leaf fits");
+        LF_TRY(lf_smem_limit(kern, L2P_SMEM));
         ++ctx->launches, kern<<<dim3(lf_blocks(ctx->n, charges), (nr + rb - 1) / rb), L2P_T, per * nleaf, st>>>(
             ctx->n, p, ctx->leaf_of.as<int>(), cen, ctx->xs.as<double>(), ctx->ys.as<double>(),
             ctx->zs.as<double>(), 1.0 / leaf.h, L, ctx->phi_far.as<double>(), ctx->fld_far.as<double>(), nr, ms,

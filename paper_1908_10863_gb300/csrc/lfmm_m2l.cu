@@ -758,7 +758,7 @@ static LfErr launch_one(lfmm_ctx* ctx, cudaStream_t st, const GemmArgs& g, int n
 {
     const size_t sm = sizeof(R) * ((size_t)G_KC * 16 * RM + (size_t)G_TB * (RP + 1));
     const auto kern = k_m2l_gemm<R, RP, RM, COMPF, TRI>;
-    LF_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LF_TRY(lf_smem_limit(kern, sm));
     ++ctx->launches, kern<<<dim3(nblk, ctx->nrhs_b, RP / (16 * RM)), G_T, sm, st>>>(g);
     return lf_cuda(cudaGetLastError(), "gathered gemm");
 }

@@ -470,7 +470,8 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
     }
     const int ntab = ctx->m2r_ntab;
     const int P = ctx->p, TS = 2 * P + 1, TT = TS * TS, Q = ctx->gl_q_m2l;
-    size_t sm = sizeof(double) * ((size_t)TT + 2 * (size_t)Q * TS);
+    const size_t sm = sizeof(double) * ((size_t)TT + 2 * (size_t)Q * TS);
+    constexpr int MS = 2 * LFMM_PMAX + 1;
     const int nnode = (int)ctx->m2r_ndesc_h.size();
     // (sized here: LFMM_OPT_QUAD_NODES may have changed Q since the build)
     LF_TRY(lf_reserve(ctx->m2r_nodes, (size_t)nnode * Q * sizeof(double) + 16));
@@ -478,7 +479,7 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
     ++ctx->launches, nodk<<<lf_blocks((int64_t)nnode * Q, 128), 128, 0, st>>>(
         ctx->comp_dev.as<LfmmComp>(), ctx->m2r_ndesc.as<int4>(), nnode, ctx->m2r_levelh.as<double>(),
         ctx->m2r_zfrac.as<double>(), ctx->gl_t_m2l.as<double>(), Q, ctx->m2r_nodes.as<double>());
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_tables, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LF_TRY(lf_smem_limit(k_m2r_tables, sizeof(double) * (MS * MS + 2 * LFMM_QMAX * MS)));
     ++ctx->launches, k_m2r_tables<<<ntab, 128, sm, st>>>(
         ctx->comp_dev.as<LfmmComp>(), ctx->m2r_tdesc.as<int4>(), ntab, ctx->m2r_levelh.as<double>(),
         ctx->m2r_zfrac.as<double>(), P, ctx->gl_t_m2l.as<double>(), ctx->gl_w_m2l.as<double>(), Q,
@@ -1070,7 +1071,8 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
 #define RZ_N 32                          // columns at a time (MMA N: 16 or 32)
 #define RZ_X_BYTES (RZ_N * TC_ROWB)      // one multipole digit of a K chunk
 #define RZ_STAGE (OZ_S * (OZ_A_BYTES + RZ_X_BYTES))
-#define RZ_PAIRS 128                     // row (column) pairs at p = 15
+#define RZ_PMAX 15                       // largest order
+#define RZ_PAIRS 128                     // row (column) pairs at that order
 
 struct ROzArgs {
     int p, nc, nk, nkc, parts;  // order, coefficients, K positions and chunks, 128-row parts
@@ -1427,7 +1429,7 @@ static LfErr m2r_apply_oz(lfmm_ctx* ctx, cudaStream_t st)
     g.stride = (size_t)ctx->nbox_total * g.nc;
     g.err = reinterpret_cast<int*>(ctx->counts.as<char>() + LFMM_TIMEOUT_OFF);
     const size_t sm = 512 + RZ_STAGE + sizeof(double2) * (size_t)(2 * g.p + 1) * (4 * g.p + 1);
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LF_TRY(lf_smem_limit(k_m2r_oz, 512 + RZ_STAGE + sizeof(double2) * (2 * RZ_PMAX + 1) * (4 * RZ_PMAX + 1)));
     ++ctx->launches, k_m2r_oz<<<dim3(ctx->m2r_nbatch * g.parts, ctx->nrhs_b), RZ_T, sm, st>>>(g);
     return lf_cuda(cudaGetLastError(), "m2r digit products");
 }
@@ -1454,13 +1456,15 @@ static LfErr m2r_apply_rot(lfmm_ctx* ctx, cudaStream_t st)
     g.nr = ctx->nrhs_b;
     const int TS = 2 * ctx->p + 1;
     const size_t sm = sizeof(R) * ((size_t)2 * lf_nre(ctx->p) * g.cb + (size_t)TS * TS);
+    constexpr int MS = 2 * LFMM_PMAX + 1;  // (more than p = 10 takes with its 32 columns)
+    constexpr size_t most = sizeof(R) * (2 * ((LFMM_PMAX + 1) * (LFMM_PMAX + 2) / 2) * RR_CB + MS * MS);
     // share the rows of each batch between blocks, so that the longest batches
     // do not outlast the rest; four shares leave every SM quarter a warp
     int parts = 1;
     while ((parts < 4 && (int64_t)ctx->m2r_nbatch * parts < 64 * 152) ||
            (parts < 8 && (int64_t)ctx->m2r_nbatch * parts < 8 * 152))
         parts *= 2;
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_rot<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LF_TRY(lf_smem_limit(k_m2r_rot<R>, most));
     ++ctx->launches, k_m2r_rot<R><<<dim3(ctx->m2r_nbatch, parts), R_T, sm, st>>>(g);
     return lf_cuda(cudaGetLastError(), "m2r rotated");
 }
@@ -1473,7 +1477,7 @@ template <int V, bool WIDE>
 static LfErr m2r_launch_tc(lfmm_ctx* ctx, const RTcArgs& g, cudaStream_t st)
 {
     constexpr int sm = RtShape<V, WIDE>::SMEM;
-    LF_CHECK(cudaFuncSetAttribute(k_m2r_tc<V, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    LF_TRY(lf_smem_limit(k_m2r_tc<V, WIDE>, sm));
     ++ctx->launches, k_m2r_tc<V, WIDE><<<ctx->m2r_nbatch * g.parts, RT_THREADS, sm, st>>>(g);
     return lf_cuda(cudaGetLastError(), "m2r tensor-core GEMM");
 }

@@ -1501,7 +1501,8 @@ LfErr lf_sommerfeld_tables_dev(lfmm_ctx* ctx, int comp, int npts, const double* 
     const int Q = ctx->gl_q_m2l;
     size_t sm = sizeof(double) * ((size_t)TS * TS + 2 * (size_t)Q * TS);
     auto kern = (ctx->L >= 3) ? k_som_tables<true> : k_som_tables<false>;
-    LF_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    constexpr int MS = 2 * LFMM_PMAX + 1;
+    LF_TRY(lf_smem_limit(kern, sizeof(double) * (MS * MS + 2 * LFMM_QMAX * MS)));
     ++ctx->launches, kern<<<npts, 128, sm, ctx->s_main>>>(ctx->comp[comp], npts, rho, z, S, P, ctx->gl_t_m2l.as<double>(),
                                                   ctx->gl_w_m2l.as<double>(), Q, out);
     return lf_cuda(cudaGetLastError(), "sommerfeld tables");
