@@ -1,5 +1,9 @@
 // lfmm_m2l_oz.cu -- free-space M2L (eq. metole) of the FP64 form on the tcgen05
-// tensor cores, by error-free digit products.
+// tensor cores, by digit products.  The idea, to split the operands of a matrix
+// product into pieces whose products a fast unit adds without rounding, is
+// K. Ozaki, T. Ogita, S. Oishi, S. M. Rump, "Error-free transformations of
+// matrix multiplication by using fast routines of matrix multiplication and its
+// applications", Numer. Algorithms 59 (2012), 95-118.
 //
 // The same tiles, offset classes and operators A_o as the float32 tensor-core
 // M2L (lfmm_m2l_tc.cu), in FP64 accuracy.  Operands are scaled by powers of
@@ -10,17 +14,28 @@
 // integer contraction, exact in the float32 accumulator while its sums stay
 // below 2^24 in magnitude, and
 //   A X = sum_d 2^{-9 d} sum_{i + j = d} A_i X_j,
-// of which the diagonals d = 2 .. 8 are kept (28 products; the rest is below
-// 2^-72 per term, under the rounding of an FP64 sum: the relative error of an
-// offset's contribution measures 7e-17 against 3.5e-16 for FP64
-// multiply-adds).  Seven accumulators, one per diagonal, 64 columns each, take
-// 448 of the 512 tensor-memory columns.
+// of which the diagonals d = 2 .. 8 are kept (28 products).  What is dropped is
+// at most 2^-62.4 per term (six products of up to 2^16, weight 2^-81), 2^-65.3
+// in the mean square of random operands: the relative error of an offset's
+// contribution measures 7e-17 against 3.5e-16 for FP64 multiply-adds.  That is
+// relative to the level's largest multipole: boxes within 2^-10 of it are finer
+// than in FP64, smaller ones coarser.  A target sees the large boxes too, so
+// what it loses stays below its own rounding unless their charges cancel.
+// Measured, superposition in the worst of 512 cells, 20,000 charges of size 1
+// and a few large ones: a lone charge of 1e9 2.5e-15 (FP64 multiply-adds
+// 3.0e-15), a pair of +-1e9 8.9e-13 (9.1e-14), a quadrupole of them 2.2e-10
+// (1.4e-10).  Seven accumulators, one per diagonal, 64 columns each, take 448 of
+// the 512 tensor-memory columns.
 //   Size of the sums: the leading digits follow the operands' own magnitudes
-// (row sums of |A| below about 3, so d = 2 stays near 2^19); a full-range
-// product of trailing digits is bounded by (p+1)^2 2^16, and the sums of up to
-// 7 such products over a window of OZ_WIN offsets have a standard deviation
-// below 2^20.5 (digits are as good as uniform), 11 deviations under 2^24;
-// beyond it a sum would only be rounded in its last bit.
+// (row sums of |A| below about 3, so d = 2 stays near 2^19).  A full diagonal of
+// trailing digits over a window of OZ_WIN offsets could reach
+// 4 (p+1)^2 7 2^16 = 2^27.7, four bits past exact; its standard deviation, digits
+// being as good as uniform, is below 2^20.5, so that 2^24 is eleven deviations
+// away.  Exact is therefore a matter of probability, not of a bound: operands
+// whose digits line up in sign over hundreds of terms with those of an
+// operator's row would be rounded.  Equal multipoles in every box and charges
+// of repeating digits do not come near (the results of 1, 1/3, 1/511 and 255/511
+// on a lattice agree to rounding).
 // Every window the accumulators are read back, converted to integers and added
 // with their weights into two 64-bit integers per output (units 2^-36, 2^-72);
 // the sum of all a CTA's offsets becomes one FP64 number and one atomic.
