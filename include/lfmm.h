@@ -50,8 +50,10 @@ typedef enum {
 
 /* Options for lfmm_set_option. */
 enum {
-    LFMM_OPT_PRECISION = 1, /* 0 = plain FP64 (default); 1 = FP32 P2P/M2L/L2P with
-                               compensated far-field sums, FP64 Sommerfeld tables */
+    LFMM_OPT_PRECISION = 1, /* 0 = FP64 (default; for p <= 15 both M2Ls on the tensor cores, by products
+                               of nine-bit digits of 63-bit operands, as accurate as FP64 sums);
+                               1 = FP32 P2P/M2L/L2P with compensated sums at the charges, FP64 Sommerfeld
+                               tables */
     LFMM_OPT_LEAF_CAP = 2,  /* octree leaf capacity (default 40) */
     LFMM_OPT_PROFILE = 3,   /* 1 = time every stage with CUDA events (lfmm_get_timings) */
     LFMM_OPT_QUAD_NODES = 4, /* Gauss-Laguerre nodes of the M2L remainder integrals (16..128, default 64) */

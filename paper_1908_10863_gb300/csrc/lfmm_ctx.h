@@ -223,7 +223,7 @@ LfErr lf_cuda(cudaError_t e, const char* what);
 #define LFMM_PIN_SCAN 512       // a scan's last input and output (2 ints)
 #define LFMM_PIN_LIST 1024      // list statistics, overflow, counters, per-level snapshots (< 1 KB)
 #define LFMM_PIN_M2L 2048       // free M2L class counts (144 ints)
-#define LFMM_PIN_ROOT 2688      // (end of the class counts)
+#define LFMM_PIN_M2L_END 2688
 #define LFMM_PIN_BOUNDS 4096    // bounding-box partials (256 blocks x 6 doubles)
 #define LFMM_PIN_UP 4096        // later in the build: root lists and list counters to upload (12 KB)
 #define LFMM_PIN_M2R 16384      // reaction M2L key starts and values (the rest)

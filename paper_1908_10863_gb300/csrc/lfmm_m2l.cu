@@ -396,7 +396,7 @@ LfErr lf_prepare_m2l_classes(lfmm_ctx* ctx, cudaStream_t st)
     if (nsort > 0)
         ++ctx->launches, k_class_keys<<<lf_blocks(nsort, 256), 256, 0, st>>>(
             cl, nsort, ctx->box_key.as<uint32_t>(), ctx->m2l_keys.as<uint32_t>(), ctx->m2l_sorted.as<uint32_t>(), cnt);
-    static_assert(LFMM_PIN_M2L + (16 + 16 * 8) * sizeof(int) <= LFMM_PIN_ROOT, "pinned regions");
+    static_assert(LFMM_PIN_M2L + (16 + 16 * 8) * sizeof(int) <= LFMM_PIN_M2L_END, "pinned regions");
     LF_CHECK(cudaMemcpyAsync(lf_pin<int>(ctx, LFMM_PIN_M2L) + 16, cnt, 16 * 8 * sizeof(int), cudaMemcpyDeviceToHost,
                              st));
     // M2M slots: children of each parent by octant (every box of levels
@@ -831,9 +831,10 @@ static LfErr shift_gemm_t(lfmm_ctx* ctx, int level, bool l2l, cudaStream_t st)
 {
     // The L2L into the leaves runs on the tensor cores in the float32 form
     // (the CUDA-core gather of parent locals is latency-bound there).  The
-    // other translations stay on the CUDA cores: at N = 1M, p = 10 the
-    // tensor-core M2M saved 0.05 ms, and chaining 3xTF32 L2L over every level
-    // raised Err2(phi) from 2.0e-6 to 3.2e-6.
+    // other translations stay on the CUDA cores: with the TF32 pieces used
+    // before, tensor-core M2M saved 0.05 ms at N = 1M, p = 10, and L2L chained
+    // over every level raised Err2(phi) from 2.0e-6 to 3.2e-6 (not measured again
+    // with float16 pieces).
     if (sizeof(R) == 4 && l2l && level == ctx->depth && lf_tc_on(ctx) && !ctx->m2l_tc_wide)
         return lf_l2l_tc(ctx, level, st);
     GemmArgs g;

@@ -122,11 +122,11 @@
 
 struct TcArgs {
     const int4* tiles;      // level, class, start, count
-    const int* sorted;      // target boxes grouped by (level, class), or null: targets start .. start + count - 1
+    const int* sorted;      // target boxes grouped by (level, class)
     const int* slots;       // [box][noff] source box at each offset of the class, or -1
     const int* cls;         // [class][noff] operator index of each class position
-    int noff;               // offsets per class: 189 (M2L), 8 (M2M: children), 1 (L2L: parent)
-    int unit_scale;         // 1: add D as it is (M2M, L2L); 0: add D / h_level (M2L)
+    int noff;               // offsets per class: 189 (M2L), 1 (L2L: parent)
+    int unit_scale;         // 1: add D as it is (L2L); 0: add D / h_level (M2L)
     const double* levelh;   // box size per level
     const int4* mseg;       // merged tiles' runs [merged tile][TC_MSEG]: (level, start, count, 0)
     const unsigned char* A; // [343][4 chunks][2 pieces x 8 KB], pre-swizzled
@@ -145,7 +145,7 @@ struct TcArgs {
 };
 
 // Target t of a tile (a box id, or -1 past the tile's count) and its output
-// scale (1 for M2M and L2L, 1/h of the target's level for M2L).  A tile with
+// scale (1 for L2L, 1/h of the target's level for M2L).  A tile with
 // level < 0 is a merged tile: the leftover runs (fewer targets than a tile)
 // of one octant class on several levels, listed at mseg[-1 - level] with
 // tile.z runs; its columns take the runs in order, each with its level's
@@ -162,7 +162,7 @@ __device__ __forceinline__ int tc_tile_target(const TcArgs& g, const int4& tile,
     if (t >= tile.w) return -1;
     if (tile.x >= 0) {
         ih = tc_out_scale(g, tile.x);
-        return g.sorted ? g.sorted[tile.z + t] : tile.z + t;
+        return g.sorted[tile.z + t];
     }
     const int4* sg = g.mseg + (size_t)(-1 - tile.x) * TC_MSEG;
     for (int k = 0; k < tile.z; ++k) {

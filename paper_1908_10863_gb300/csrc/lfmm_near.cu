@@ -6,10 +6,14 @@
 //   I_00 = int J0(k rho) e^{-k h} sigma(k) dk,
 // and the field needs I_10 = int k J0 e^{-kh} sigma, I_11' = int k J1 e^{-kh} sigma.
 // Each is the closed form of the leading exponential C e^{-k zeta} of sigma
-// (C/R, C H/R^3, C rho/R^3 with H = h + zeta) plus the remainder by
-// Gauss-Laguerre quadrature in t = k (h + zeta_r).
-// One block per leaf target box; sources of each near box are staged in
-// shared memory relative to the target box centre.
+// (C/R, C H/R^3, C rho/R^3 with H = h + zeta) plus the remainder: by a rule of
+// images (LfImgRule), from tables, by Gauss-Laguerre quadrature in
+// t = k (h + zeta_r), or by a trained network.
+// Sources are staged in shared memory relative to the target box centre:
+// k_p2p_list by one warp per target leaf (or part of its list), whatever the
+// remainder's form in float32 and by images in FP64; k_p2p_free_staged and
+// k_p2p_warp for one float32 vector without reaction pairs; k_p2p by one block
+// per leaf for FP64 quadrature and tables; k_p2p_net for the networks.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -173,8 +177,9 @@ __device__ __forceinline__ void p2p_store(const P2PArgs& a, int i, const P2PAcc<
     }
 }
 
-// One block per target leaf (FP64 form), a batch of RB right-hand sides.
-// GEN: media of four or five layers (both forms, one right-hand side per launch).
+// One block per target leaf, a batch of RB right-hand sides: the FP64 form's
+// reaction pairs by quadrature or tables.
+// GEN: media of four or five layers (one right-hand side per launch).
 template <typename R, int RB, bool GEN = false>
 __global__ void __launch_bounds__(P2P_T) k_p2p(P2PArgs a)
 {
@@ -222,8 +227,7 @@ __global__ void __launch_bounds__(P2P_T) k_p2p(P2PArgs a)
                 } else {
                     for (int u = 0; u < cnt; ++u)
                         p2p_reaction_add<R, RB, GEN>(cp, xi - sx[u], yi - sy[u], zi - sz[u], &sq[0][u], P2P_T,
-                                                     a.nr, a.Qn, a.gl_t, a.gl_w, A, LF_CTAB(a, c),
-                                                     sizeof(R) == 4 ? LF_CTAB4(a, c) : nullptr);
+                                                     a.nr, a.Qn, a.gl_t, a.gl_w, A, LF_CTAB(a, c));
                 }
             }
         }
@@ -371,13 +375,13 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_p2p_warp(P2PArgs a, const flo
 // per clock and SM) bounds the FP64 form, so what counts there is that every
 // lane of a warp instruction holds a pair.
 // Measured, eps (1, 5, 10): 1,000 charges in FP64, 86k reaction pairs, 6.27 ms
-// by one block of 128 threads per leaf and the quadrature, 0.48 ms here; 2,848
-// charges at p = 20, 538k reaction pairs, 33.0 and 1.67 ms; float32, 50,001
+// by one block of 128 threads per leaf and the quadrature, 0.34 ms here; 2,848
+// charges at p = 20, 538k reaction pairs, 33.0 and 1.24 ms; float32, 50,001
 // charges beside the interfaces, 30M reaction pairs, 0.95 ms by the tables
-// (k_p2p_warp), 0.57 ms here.  Several vectors share a pair's kernels: eight
+// (k_p2p_warp), 0.37 ms here.  Several vectors share a pair's kernels: eight
 // per batch in float32 (four multiply-adds per pair and vector, charges read
 // as float4s), all batches in one launch; 64 vectors of 262,144 charges,
-// 21.4 ms (k_p2p_warp, batches of 4, one source box at a time) -> 6.95 ms.
+// 21.4 ms (k_p2p_warp, batches of 4, one source box at a time) -> 6.99 ms.
 #define PL_CAP 64
 #define PL_WARPS 4
 
