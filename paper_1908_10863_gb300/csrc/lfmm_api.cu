@@ -1159,7 +1159,7 @@ void lfmm_destroy(lfmm_ctx* ctx)
                       &ctx->m2r_tgt, &ctx->m2r_phase64, &ctx->m2r_phase, &ctx->m2r_pairs, &ctx->m2r_kstart, &ctx->m2r_kval, &ctx->m2r_tables, &ctx->m2r_levelh, &ctx->m2r_zfrac, &ctx->m2r_zbase,
                       &ctx->m2r_batches, &ctx->m2r_tdesc, &ctx->m2r_ndesc, &ctx->m2r_nodes, &ctx->surr_theta, &ctx->surr_grad, &ctx->surr_m1,
                       &ctx->surr_m2, &ctx->surr_w, &ctx->surr_b, &ctx->surr_meta, &ctx->surr_err, &ctx->surr_comps,
-                      &ctx->surr_xoff, &ctx->surr_counters, &ctx->m2l_Atc, &ctx->tc_cscale, &ctx->tc_perm, &ctx->oz_A, &ctx->oz_Ms, &ctx->oz_cscale, &ctx->oz_perm, &ctx->m2r_emin, &ctx->m2r_tscale, &ctx->oz_tiles, &ctx->oz_mseg, &ctx->l2l_Atc, &ctx->tc_shift_tiles, &ctx->m2l_tc_tiles, &ctx->tc_mseg, &ctx->m2l_Ms, &ctx->m2m_A64, &ctx->m2m_A32,
+                      &ctx->surr_xoff, &ctx->surr_counters, &ctx->m2l_Atc, &ctx->tc_cscale, &ctx->tc_perm, &ctx->oz_A, &ctx->oz_Ms, &ctx->oz_cscale, &ctx->oz_perm, &ctx->m2r_emin, &ctx->m2r_tscale, &ctx->m2r_tabf, &ctx->oz_tiles, &ctx->oz_mseg, &ctx->l2l_Atc, &ctx->tc_shift_tiles, &ctx->m2l_tc_tiles, &ctx->tc_mseg, &ctx->m2l_Ms, &ctx->m2m_A64, &ctx->m2m_A32,
                       &ctx->l2l_A64, &ctx->l2l_A32, &ctx->shift_cls, &ctx->m2m_slots, &ctx->shift_tiles};
     for (DevBuf* b : bufs) lf_free(*b);
     for (cudaEvent_t e : ctx->prof_pool) cudaEventDestroy(e);

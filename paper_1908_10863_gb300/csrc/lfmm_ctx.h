@@ -159,7 +159,7 @@ struct lfmm_ctx {
     DevBuf m2r_keys, m2r_order, m2r_tgt, m2r_kstart, m2r_kval, m2r_tables, m2r_levelh, m2r_batches;
     DevBuf m2r_tdesc;  // table descriptors (component | level << 8, node set, rho^2, oz)
     DevBuf m2r_emin;    // smallest exponent that scales each value of a table, [2p + 1][2p + 1] (p <= 15)
-    DevBuf m2r_tscale;  // per table: exponent that puts its float16 operators into range
+    DevBuf m2r_tscale, m2r_tabf;  // per table: exponent that puts its float16 operators into range; scaled float32 copy
     DevBuf m2r_ndesc, m2r_nodes;  // node sets (component, level, oz) and the remainder at their quadrature nodes
     std::vector<int4> m2r_tdesc_h, m2r_ndesc_h, m2r_batches_h;  // host staging of asynchronous uploads
     int m2r_pending_ne = 0;             // reaction M2L entries whose key grouping awaits lf_prepare_m2r_finish

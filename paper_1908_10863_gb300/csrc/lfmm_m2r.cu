@@ -40,6 +40,7 @@ static inline int lf_blocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 #define R_TB 64   // pairs per batch
 #define R_T 256   // threads per block of the rotated form
 #define RR_CB 16  // columns it stages at a time above p = 10
+#define RT_PMAX 14  // largest order of the float32 form
 #define KEY_NONE 0xffffffffu
 
 
@@ -174,13 +175,16 @@ __global__ void __launch_bounds__(128) k_m2r_nodes(const LfmmComp* __restrict__ 
 // the lateral distance only; the azimuth enters through the phases applied
 // when the operator is formed.  tdesc: component | level << 8, node set, rho^2, oz.
 // tscale (p <= 15): the exponent s for which no entry of an operator made of the
-// table, two values at most with their scales 2^{-e} (emin), reaches 2^{15 - s}.
+// table, two values at most with their scales 2^{-e} (emin), reaches 2^{15 - s};
+// tabf (p <= 14): the table times 2^s in float32, which k_m2r_tc reads (half the
+// bytes, and no conversions on the FP64 pipe: applying s there instead cost it 1%).
 __global__ void __launch_bounds__(128) k_m2r_tables(const LfmmComp* __restrict__ comps, const int4* __restrict__ tdesc,
                                                     int ntab, const double* __restrict__ levelh,
                                                     const double* __restrict__ zfrac, int P,
                                                     const double* __restrict__ gt, const double* __restrict__ gw, int Q,
                                                     const double* __restrict__ nodes, double* __restrict__ tables,
-                                                    const int* __restrict__ emin, int* __restrict__ tscale)
+                                                    const int* __restrict__ emin, int* __restrict__ tscale,
+                                                    float* __restrict__ tabf)
 {
     __shared__ int s_exp;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -214,7 +218,15 @@ __global__ void __launch_bounds__(128) k_m2r_tables(const LfmmComp* __restrict__
     ex = __reduce_max_sync(0xffffffffu, ex);
     if ((threadIdx.x & 31) == 0) atomicMax(&s_exp, ex);
     __syncthreads();
-    if (threadIdx.x == 0) tscale[k] = max(-100, min(100, 13 - s_exp));  // (float32 powers of two)
+    const int ts = max(-100, min(100, 13 - s_exp));  // (float32 powers of two)
+    if (threadIdx.x == 0) tscale[k] = ts;
+    if (!tabf) return;
+    const double s = __hiloint2double((1023 + ts) << 20, 0);
+    for (int j = threadIdx.x; j < TT; j += blockDim.x) {
+        const int N = j / TS, mu = j - N * TS;
+        const double v = (mu <= N) ? sT[j] * s : 0.0;
+        tabf[(size_t)k * TT + j] = (float)((cp.a == 2 && ((N + mu) & 1)) ? -v : v);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -413,6 +425,7 @@ LfErr lf_prepare_m2r_finish(lfmm_ctx* ctx, cudaStream_t st)
     LF_TRY(lf_reserve(ctx->m2r_tables, (size_t)ntab * TT * 8 + 16));
     LF_TRY(lf_reserve(ctx->m2r_tdesc, (size_t)ntab * sizeof(int4) + 16));
     LF_TRY(lf_reserve(ctx->m2r_tscale, (size_t)ntab * sizeof(int) + 16));
+    if (P <= RT_PMAX) LF_TRY(lf_reserve(ctx->m2r_tabf, (size_t)ntab * TT * sizeof(float) + 16));
     LF_TRY(lf_reserve(ctx->m2r_ndesc, ndesc.size() * sizeof(int4) + 16));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_tdesc.ptr, tdesc.data(), ntab * sizeof(int4), cudaMemcpyHostToDevice, st));
     LF_CHECK(cudaMemcpyAsync(ctx->m2r_ndesc.ptr, ndesc.data(), ndesc.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
@@ -484,7 +497,7 @@ LfErr lf_m2r_device(lfmm_ctx* ctx, cudaStream_t st)
         ctx->comp_dev.as<LfmmComp>(), ctx->m2r_tdesc.as<int4>(), ntab, ctx->m2r_levelh.as<double>(),
         ctx->m2r_zfrac.as<double>(), P, ctx->gl_t_m2l.as<double>(), ctx->gl_w_m2l.as<double>(), Q,
         ctx->m2r_nodes.as<double>(), ctx->m2r_tables.as<double>(), ctx->m2r_emin.as<int>(),
-        ctx->m2r_tscale.as<int>());
+        ctx->m2r_tscale.as<int>(), P <= RT_PMAX ? ctx->m2r_tabf.as<float>() : nullptr);
     LF_TRY(lf_cuda(cudaGetLastError(), "m2r tables"));
     if (ctx->m2r_nent > 0) {
         LF_TRY(lf_reserve(ctx->m2r_pairs, (size_t)ctx->m2r_nent * sizeof(int2) + 16));
@@ -718,7 +731,7 @@ __global__ void __launch_bounds__(R_T) k_m2r_rot(RRotArgs g)
 #define RT_X_CHUNK (R_TB * TC_ROWB)     // one K chunk of one multipole piece and vector: 64 rows x 64 B
 template <int V, bool WIDE>
 struct RtShape {
-    static constexpr int P = WIDE ? 14 : 10;                   // largest order
+    static constexpr int P = WIDE ? RT_PMAX : 10;                   // largest order
     static constexpr int W = (2 * P + 1) * (4 * P + 1);        // entries of the table W
     static constexpr int CP = WIDE ? 128 : 64;                 // column pairs
     static constexpr int MROW = WIDE ? 256 : 128;              // halves per box and multipole piece
@@ -734,8 +747,8 @@ struct RTcArgs {
     int p, nc, nk, nkc;     // order, coefficients, K positions, chunks of 32 that hold them
     int parts;              // 128-row parts of the outputs
     const int4* batches;    // key index, first sorted entry, count | key << 8, table
-    const double* tables;   // [table][TS][TS]
-    const int* tscale;      // per table: its operators carry 2^tscale (k_m2r_tables)
+    const float* tables;    // [table][TS][TS], times 2^tscale (k_m2r_tables)
+    const int* tscale;      // per table
     const LfmmComp* comps;
     const float* phase;     // [225 lateral offsets][cos | sin][RT_PH] (k_m2r_phase)
     const int2* pairs;      // (source box, target box) per sorted entry (k_m2r_pairs)
@@ -799,7 +812,6 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
     // the batch carries its key and table: one dependent load to everything else
     const int start = b.y, cnt = b.z & 255, tab = b.w;
     if (cnt <= 0 || cnt > R_TB) return;
-    const int te = g.tscale[tab];  // (used once W is formed)
     const int Np = (cnt + 15) & ~15;  // columns per vector
     int c, lev, ox, oy, oz;
     rkey_decode((uint32_t)b.z >> 8, c, lev, ox, oy, oz);
@@ -877,6 +889,7 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
         s_abort = 0;
+        s_as = rt_pow2(-g.tscale[tab]);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
@@ -884,12 +897,10 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     {
-        const double* Tk = g.tables + (size_t)tab * TS * TS;
-        const float as = rt_pow2(te);
-        if (tid == 0) s_as = rt_pow2(-te);
+        const float* Tk = g.tables + (size_t)tab * TS * TS;
         for (int j = tid; j < TSZ; j += RT_THREADS) {
             const int Nn = j / WS, mu = j - Nn * WS - 2 * p, a = mu < 0 ? -mu : mu;
-            const float t = (float)Tk[Nn * TS + a] * as;
+            const float t = Tk[Nn * TS + a];
             float wr = t * sPh[a], wi = t * sPh[RT_PH + a];
             if (mu < 0) {
                 if (a & 1) wr = -wr; else wi = -wi;
@@ -1490,7 +1501,7 @@ static LfErr m2r_apply_tc(lfmm_ctx* ctx, cudaStream_t st)
     g.nk = ctx->tc_nk;
     g.nkc = (g.nk + TH_KC - 1) / TH_KC;
     g.batches = ctx->m2r_batches.as<int4>();
-    g.tables = ctx->m2r_tables.as<double>();
+    g.tables = ctx->m2r_tabf.as<float>();
     g.tscale = ctx->m2r_tscale.as<int>();
     g.comps = ctx->comp_dev.as<LfmmComp>();
     g.pairs = ctx->m2r_pairs.as<int2>();
