@@ -1061,8 +1061,8 @@ __global__ void __launch_bounds__(RT_THREADS, RtShape<V, WIDE>::MINB) k_m2r_tc(R
 
 // ---------------------------------------------------------------------------
 // FP64 form, p <= 15: the key's operator applied by digit products on the
-// tensor cores (scheme of lfmm_m2l_oz.cu: seven 9-bit digits per operand, the
-// 28 products of the leading diagonals, exact sums).  One CTA per batch of
+// tensor cores (scheme and bounds of lfmm_m2l_oz.cu: seven 9-bit digits per
+// operand, the 28 products of the leading diagonals, one offset per sum).  One CTA per batch of
 // pairs of one key (and 128-row part of the outputs), 32 columns at a time.
 // The dense operator is formed in FP64 from the table W of the complex
 // reaction coefficient in blocks of 2 x 2 (as k_m2r_tc: one addition per
